@@ -94,7 +94,7 @@ struct ra_ctx {
     cudaEvent_t fork_ev = nullptr, plan_ev = nullptr;
     bool plan_pending = false;
     int parity = 0;
-    bool no_early_once = false;  // the next attention launch follows the whole-stack compaction
+    bool no_early_once = false;  // the next fused launches follow the whole-stack compaction, or a copy into the caches
     bool step_open = false;  // a step's prologue ran (plans launched, stack evicted) and its end has not
     int step_cur = 0;        // the plan half that step reads
     std::vector<int32_t> plan_g, plan_n;
@@ -737,8 +737,10 @@ int ra_prefill(ra_ctx* ctx, int layer, const uint16_t* k, const uint16_t* v, int
     p.v = v;
     p.row_stride = row_stride;
     p.only_seq = -1;
+    p.layers = 1;
     for (int b = 0; b < ctx->B; ++b) p.n_rows[b] = ctx->lp[b];
     cudaError_t e = launch_prefill(p, (cudaStream_t)stream);
+    ctx->no_early_once = true;
     return e == cudaSuccess ? RA_OK : cuda_fail(ctx, e, "prefill launch");
 }
 
@@ -766,8 +768,10 @@ int ra_restore(ra_ctx* ctx, int layer, const int32_t* g_host, const int32_t* c_h
     p.pos = pos;
     p.row_stride = row_stride;
     p.only_seq = -1;
+    p.layers = 1;
     for (int b = 0; b < ctx->B; ++b) p.n_rows[b] = c_host[b];
     cudaError_t e;
+    ctx->no_early_once = true;
     if (maxc > 0 && (e = launch_restore(p, s)) != cudaSuccess) return cuda_fail(ctx, e, "restore launch");
     for (int b = 0; b < ctx->B; ++b) {
         const size_t i = (size_t)layer * ctx->B + b;
@@ -887,12 +891,9 @@ int ra_admit(ra_ctx* ctx, int seq, int prompt_len, const uint16_t* k, const uint
         p.row_stride = row_stride;
         p.only_seq = seq;
         p.n_rows[seq] = prompt_len;
-        for (int l = 0; l < ctx->L; ++l) {
-            p.layer = l;
-            p.k = k + (size_t)l * ctx->KVH * row_stride * kHeadDim;
-            p.v = v + (size_t)l * ctx->KVH * row_stride * kHeadDim;
-            if ((e = launch_prefill(p, s)) != cudaSuccess) return cuda_fail(ctx, e, "admit prefill launch");
-        }
+        p.layers = ctx->L;
+        if ((e = launch_prefill(p, s)) != cudaSuccess) return cuda_fail(ctx, e, "admit prefill launch");
+        ctx->no_early_once = true;
     }
     // a fresh request: nothing generated, nothing cached, its own random stream
     for (int l = 0; l < ctx->L; ++l) {
@@ -1282,8 +1283,9 @@ int decode_layer_impl(ra_ctx* ctx, int layer, const uint16_t* q, const uint16_t*
     // needs no input, and positions were last written by this layer's previous step, which has
     // completed (every kernel before the predecessor has).  The scored policy reads scores its
     // predecessor computes, and with one layer the predecessor is this layer's previous step.
-    ep.early = (ctx->policy != RA_POLICY_SNAPKV && ctx->L >= 2) ? 1 : 0;
-    const int score_early = ctx->L >= 2 ? 1 : 0;  // the scoring pass reads only older kernels' output
+    // Neither starts early right after rows were loaded: the predecessor may have written this layer.
+    ep.early = (ctx->policy != RA_POLICY_SNAPKV && ctx->L >= 2 && !ctx->no_early_once) ? 1 : 0;
+    const int score_early = (ctx->L >= 2 && !ctx->no_early_once) ? 1 : 0;  // the scoring pass reads only older kernels' output
     ep.pending = 1;  // the step's token is appended by the attention launch below
     int n = 0;
     double moved = 0;

@@ -149,7 +149,8 @@ struct CopyRowsParams {
     const uint16_t* v;
     const int32_t* pos; // restore only: [B][KVH][row_stride]
     int row_stride;
-    int only_seq;       // >= 0: the launch copies that sequence alone (one CTA per KV head)
+    int only_seq;       // >= 0: the launch copies that sequence alone
+    int layers;         // layers from `layer` on, their sources one after the other
     int32_t n_rows[RA_MAX_BATCH];  // rows to copy per sequence
 };
 

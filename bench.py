@@ -530,7 +530,7 @@ def attention_roofline(a, clean, steps, layers, peaks, peak_src, traffic):
         us_launch = 1000.0 * win_ms / win_n
         timing = (f"CUDA events at the step boundaries on the launching stream, over the {len(clean)} of "
                   f"{steps} steps of a third pass in which no sequence evicts: such a step launches "
-                  f"only the {layers} layers' attention kernels, overlapped as in the timed region; "
+                  f"only the attention of its {layers} layers, as in the timed region; "
                   f"duration = their device time / {win_n} launches")
     else:  # every step evicts somewhere (ragged phases): the per-launch events are all there is
         by_launch, us_launch, timing = a["bytes_per_launch"], a["us_per_launch"], serialized["timing"]

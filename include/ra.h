@@ -346,7 +346,8 @@ int ra_decode_layer(ra_ctx* ctx, int layer, const uint16_t* q, const uint16_t* k
  * joined to it at its end, by events: once `stream` completes, so has all the
  * step's work) computes the next step's evicted sets in every layer, and at that step one
  * launch compacts every layer of the sequences that fire (ordered or order-free,
- * in place) before the first layer runs.  Sets computed ahead are used only
+ * in place) before the first layer runs.  The attention of all layers is one launch
+ * too, where their counters are alike (unless compaction is inside the attention pass).  Sets computed ahead are used only
  * where the counters they were computed from still hold; elsewhere the layers
  * select as ra_decode_layer does.
  */

@@ -56,7 +56,7 @@ struct ra_ctx {
     long long total_rows = 0;
     long long gen_rows = 0;
     int regions = 0;
-    size_t partial_records = 0;  // split-K partial records the arena holds
+    size_t max_chunks = 0;       // chunks of the attention split the arena holds partial records for
     // arena layout (byte offsets)
     size_t off_k, off_v, off_pos, off_region, off_spare, off_lp, off_pages, off_plan, off_partial, off_arrive,
         off_err, off_evplan, bytes;
@@ -239,13 +239,15 @@ void fill_active(const ra_ctx* ctx, uint32_t* mask)
         if (ctx->active[b]) mask[b >> 5] |= 1u << (b & 31);
 }
 
-// Work split of one layer's attention from the host mirror, in tiles: a head has
-// ceil(lp / TILE) prompt tiles and ceil(gen / TILE) tiles of generated rows, where gen is
-// the cached generated rows plus one for a fused new token; the tiles are cut into one equal
-// chunk per warp.  *slots = rows attended.
-int plan_attention(ra_ctx* ctx, int layer, int fused, AttnParams* p, int* n_active, int* ctas, double* slots,
+// Work split of the attention of `layers` layers from `layer` on (counters alike), from the host
+// mirror, in tiles: a head has ceil(lp / TILE) prompt tiles and ceil(gen / TILE) tiles of generated
+// rows, where gen is the cached generated rows plus one for a fused new token; the tiles are cut
+// into one equal chunk per warp.  *slots = rows attended.
+int plan_attention(ra_ctx* ctx, int layer, int layers, int fused, AttnParams* p, int* n_active, int* ctas, double* slots,
                    int* shape, const std::vector<int32_t>* old_rows = nullptr)
 {
+    p->layer = layer;
+    p->layers = layers;
     fill_active(ctx, p->active);
     // sequences whose compaction the launch does: their cached rows are the old region's
     for (int i = 0; i < RA_MAX_BATCH / 32; ++i) p->compacting[i] = 0u;
@@ -269,7 +271,7 @@ int plan_attention(ra_ctx* ctx, int layer, int fused, AttnParams* p, int* n_acti
         for (int j = 1; j < np && consecutive; ++j) consecutive = pg[j] == pg[0] + j;
         p->seq_page0[b] = np == 0 ? 0 : (consecutive ? pg[0] : -1);
         if (ctx->active[b]) {
-            rows += (long long)ctx->KVH * (ctx->lp[b] + gen);
+            rows += (long long)layers * ctx->KVH * (ctx->lp[b] + gen);
             ++na;
         }
     }
@@ -284,6 +286,8 @@ int plan_attention(ra_ctx* ctx, int layer, int fused, AttnParams* p, int* n_acti
         if (ctx->active[b]) acc += (long long)ctx->KVH * ((ctx->lp[b] + T - 1) / T + (p->seq_gen[b] + T - 1) / T);
         p->seq_base[b + 1] = (int32_t)acc;
     }
+    p->layer_tiles = (int)acc;
+    acc *= layers;
     if (acc >= (1LL << 31)) return fail(ctx, RA_ERR_UNSUPPORTED, "layer holds more than 2^31 tiles");
     p->total = (int)acc;
     const int wpc = attn_warps_per_cta(*shape, ctx->G), cps = attn_ctas_per_sm(*shape);
@@ -296,8 +300,7 @@ int plan_attention(ra_ctx* ctx, int layer, int fused, AttnParams* p, int* n_acti
     p->nwarps = *ctas * wpc;
     *n_active = na;
     *slots = (double)rows;
-    // partial records are indexed chunk + head: both bounded by what the arena holds
-    if ((size_t)p->nchunks + (size_t)ctx->B * ctx->KVH > ctx->partial_records)
+    if ((size_t)p->nchunks > ctx->max_chunks)
         return fail(ctx, RA_ERR_STATE, "attention split needs more partial records than the arena holds");
     return RA_OK;
 }
@@ -336,9 +339,9 @@ int layout_base(ra_ctx* ctx)
     const size_t max_chunks =
         (size_t)kMaxSMs * std::max(attn_warps_per_cta(kAttnWide, ctx->G) * attn_ctas_per_sm(kAttnWide),
                                    attn_warps_per_cta(kAttnNarrow, ctx->G) * attn_ctas_per_sm(kAttnNarrow)) + 1;
-    ctx->partial_records = max_chunks + (size_t)batch * kv_heads;
-    ctx->off_partial = take(ctx->partial_records * partial_stride(ctx->G) * 4);
-    ctx->off_arrive = take((size_t)batch * kv_heads * 4);
+    ctx->max_chunks = max_chunks;
+    ctx->off_partial = take(2 * max_chunks * partial_stride(ctx->G) * 4);
+    ctx->off_arrive = take(max_chunks * 4);
     ctx->off_err = take(256);
     ctx->off_evplan = take((size_t)2 * layers * batch * kv_heads * (r + 1) * 4);
     ctx->base_bytes = o;
@@ -671,7 +674,7 @@ int ra_bind(ra_ctx* ctx, void* device_arena, size_t bytes, void* stream)
         (e = cudaMemcpyAsync(Ly.pages, ctx->pages.data(), ctx->pages.size() * 4, cudaMemcpyHostToDevice, s)) !=
             cudaSuccess ||
         (e = cudaMemcpyAsync(Ly.err, &zero, 4, cudaMemcpyHostToDevice, s)) != cudaSuccess ||
-        (e = cudaMemsetAsync(Ly.arrive, 0, (size_t)BH * 4, s)) != cudaSuccess)
+        (e = cudaMemsetAsync(Ly.arrive, 0, ctx->max_chunks * 4, s)) != cudaSuccess)
         return cuda_fail(ctx, e, "table initialisation");
     // rows that were never written (past a head's cached slots) then read as zeros, never as stale NaNs
     if ((e = cudaMemsetAsync(a, 0, ctx->off_pos, s)) != cudaSuccess) return cuda_fail(ctx, e, "cache clear");
@@ -1065,7 +1068,7 @@ int ra_decode_attn(ra_ctx* ctx, int layer, const uint16_t* q, uint16_t* out, flo
     int ctas = 0;
     double rows = 0;
     int shape = kAttnWide;
-    if ((rc = plan_attention(ctx, layer, 0, &p, &n_active, &ctas, &rows, &shape)) != RA_OK) return rc;
+    if ((rc = plan_attention(ctx, layer, 1, 0, &p, &n_active, &ctas, &rows, &shape)) != RA_OK) return rc;
     if (n_active == 0) return RA_OK;
     set_scale(&p, scale);
     cudaStream_t s = (cudaStream_t)stream;
@@ -1258,21 +1261,19 @@ int ra_decode_layer(ra_ctx* ctx, int layer, const uint16_t* q, const uint16_t* k
 namespace {
 // plan_parity >= 0: evicted sets computed ahead into that half of the plan buffer may be used
 // (inside a step whose prologue has ordered the stream after their computation)
-int decode_layer_impl(ra_ctx* ctx, int layer, const uint16_t* q, const uint16_t* k_new, const uint16_t* v_new,
-                      uint16_t* out, float scale, void* stream, int plan_parity)
+//
+// Eviction of one layer, with the step's token pending: it is the newest slot, so it is never a
+// candidate, and evicting before writing it gives the same state as append-then-evict.  With
+// compaction in the attention pass only the selection runs here: that pass reads the old region
+// anyway and writes the survivors to the new one as it goes; old_rows [B] then receives the rows
+// of the sequences it compacts and *compacted the rows it writes.  *n_fired: sequences that evict.
+int evict_pending(ra_ctx* ctx, int layer, cudaStream_t s, int plan_parity, std::vector<int32_t>& old_rows,
+                  double* compacted, int* n_fired)
 {
     int rc;
-    if ((rc = check_layer_call(ctx, layer, q, k_new, v_new, out)) != RA_OK) return rc;
     const size_t base = (size_t)layer * ctx->B;
-    cudaStream_t s = (cudaStream_t)stream;
-    cudaError_t e;
-    std::vector<int32_t> old_rows((size_t)ctx->B, -1);  // sequences the attention launch compacts: rows before
     // The attention pass compacts (time order kept) when each tile's evicted rows fit its 64-bit mask.
     const bool fuse_compaction = ctx->compaction == RA_COMPACT_FUSED && ctx->r <= 64;  // tiles have <= 64 rows
-    // 1. Eviction first, with the step's token pending: it is the newest slot, so it is never a
-    //    candidate, and evicting before writing it gives the same state as append-then-evict.
-    //    With ordered compaction only the selection runs here: the attention pass below reads
-    //    the old region anyway and writes the survivors to the new one as it goes.
     EvictParams ep{};
     ep.lay = ctx->lay;
     ep.layer = layer;
@@ -1301,7 +1302,7 @@ int decode_layer_impl(ra_ctx* ctx, int layer, const uint16_t* q, const uint16_t*
             moved += (double)(ctx->K + ctx->r - 1) * ctx->KVH;
         }
     }
-    double compacted = 0;  // rows the attention launch writes as compaction
+    *n_fired = n;
     if (n > 0 && plan_parity >= 0 && !ep.holefill && !fuse_compaction && plan_usable(ctx)) {
         bool all = true;  // every triggered sequence's evicted sets were computed ahead for this round
         for (int i = 0; i < n && all; ++i) {
@@ -1321,15 +1322,25 @@ int decode_layer_impl(ra_ctx* ctx, int layer, const uint16_t* q, const uint16_t*
             ctx->nev[base + b] += 1;
             if (fuse_compaction) {
                 old_rows[b] = ep.trig_c[i];
-                compacted += (double)(ctx->K + ctx->r) * ctx->KVH;
+                *compacted += (double)(ctx->K + ctx->r) * ctx->KVH;
             }
             ctx->c[base + b] = ctx->K + ctx->r - 1;  // rows left before the token is written (last)
         }
     }
-    // 2. Fused append + attention (+ merge of the split pieces).
+    return RA_OK;
+}
+
+// Fused append + attention (+ merge of the split pieces) of `layers` layers from `layer` on, whose
+// counters are alike, in one launch; q, k_new, v_new, out: [layers][...].  `evicted`: the launches
+// before it evicted in one of them.
+int attend_pending(ra_ctx* ctx, int layer, int layers, const uint16_t* q, const uint16_t* k_new, const uint16_t* v_new,
+                   uint16_t* out, float scale, cudaStream_t s, bool evicted, const std::vector<int32_t>& old_rows,
+                   double compacted)
+{
+    int rc;
+    cudaError_t e;
     AttnParams p{};
     p.lay = ctx->lay;
-    p.layer = layer;
     p.q = q;
     p.out = out;
     p.k_new = k_new;
@@ -1341,36 +1352,61 @@ int decode_layer_impl(ra_ctx* ctx, int layer, const uint16_t* q, const uint16_t*
     int n_active = 0, ctas = 0;
     double rows = 0;
     int shape = kAttnWide;
-    if ((rc = plan_attention(ctx, layer, 1, &p, &n_active, &ctas, &rows, &shape, &old_rows)) != RA_OK)
+    if ((rc = plan_attention(ctx, layer, layers, 1, &p, &n_active, &ctas, &rows, &shape, &old_rows)) != RA_OK)
         return rc;
     if (n_active == 0) return RA_OK;
     set_scale(&p, scale);
     // The kernel may request its first K/V tiles before its predecessor finishes when that
     // predecessor cannot be writing this layer's cache or tables: no eviction of this layer at
-    // this step (else it is this layer's compaction) and more than one layer (else it is this
-    // layer's previous step).  Kernels let successors start only after their own wait, so
+    // this step (else it is this layer's compaction) and layers outside this launch (else it is
+    // these layers' previous step).  Kernels let successors start only after their own wait, so
     // everything older than the predecessor has completed.
-    p.early = (n == 0 && ctx->L >= 2 && !ctx->no_early_once) ? 1 : 0;
-    ctx->no_early_once = false;
+    p.early = (!evicted && layers < ctx->L && !ctx->no_early_once) ? 1 : 0;
+    ctx->no_early_once = layers > 1;  // the next launch's predecessor then writes every layer's newest row
     {
         // rows read (a new token's from the caller), a new token's row written, q read, out written
         int n_pending = 0;
         for (int b = 0; b < ctx->B; ++b) n_pending += (int)((p.pending[b >> 5] >> (b & 31)) & 1u);
         // (a compacting head's survivors are written once more, with their positions)
         ProfScope ps(ctx, RA_KERNEL_ATTN,
-                     rows * 2 * kRowBytes + 2.0 * n_active * ctx->H * kRowBytes +
-                         (double)n_pending * ctx->KVH * 2 * kRowBytes + compacted * (2 * kRowBytes + 8),
+                     rows * 2 * kRowBytes + 2.0 * layers * n_active * ctx->H * kRowBytes +
+                         (double)layers * n_pending * ctx->KVH * 2 * kRowBytes + compacted * (2 * kRowBytes + 8),
                      s);
         e = launch_attention(shape, p, &ctx->tmap_k[shape], &ctx->tmap_v[shape], ctas, s);
         ps.done();
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "attention launch");
-    for (int b = 0; b < ctx->B; ++b) {
-        if (!ctx->active[b]) continue;
-        ctx->c[base + b] += 1;
-        ctx->g[base + b] += 1;
-    }
+    for (int l = layer; l < layer + layers; ++l)
+        for (int b = 0; b < ctx->B; ++b) {
+            if (!ctx->active[b]) continue;
+            ctx->c[(size_t)l * ctx->B + b] += 1;
+            ctx->g[(size_t)l * ctx->B + b] += 1;
+        }
     return RA_OK;
+}
+
+int decode_layer_impl(ra_ctx* ctx, int layer, const uint16_t* q, const uint16_t* k_new, const uint16_t* v_new,
+                      uint16_t* out, float scale, void* stream, int plan_parity)
+{
+    int rc, n = 0;
+    if ((rc = check_layer_call(ctx, layer, q, k_new, v_new, out)) != RA_OK) return rc;
+    cudaStream_t s = (cudaStream_t)stream;
+    std::vector<int32_t> old_rows((size_t)ctx->B, -1);  // sequences the attention launch compacts: rows before
+    double compacted = 0;  // rows the attention launch writes as compaction
+    if ((rc = evict_pending(ctx, layer, s, plan_parity, old_rows, &compacted, &n)) != RA_OK) return rc;
+    return attend_pending(ctx, layer, 1, q, k_new, v_new, out, scale, s, n > 0, old_rows, compacted);
+}
+
+// Every active sequence's counters are the same in every layer (they are unless layers were
+// restored or evicted on their own).
+bool layers_alike(const ra_ctx* ctx)
+{
+    for (int l = 1; l < ctx->L; ++l)
+        for (int b = 0; b < ctx->B; ++b) {
+            const size_t i = (size_t)l * ctx->B + b;
+            if (ctx->active[b] && (ctx->g[i] != ctx->g[b] || ctx->c[i] != ctx->c[b])) return false;
+        }
+    return true;
 }
 
 }  // namespace
@@ -1381,6 +1417,8 @@ int ra_decode_step(ra_ctx* ctx, const uint16_t* q_all, const uint16_t* k_all, co
     int rc;
     if ((rc = check_bound(ctx)) != RA_OK) return rc;
     if (!q_all || !k_all || !v_all || !out_all) return fail(ctx, RA_ERR_INVALID_ARG, "NULL argument");
+    if (!aligned16(q_all) || !aligned16(k_all) || !aligned16(v_all) || !aligned16(out_all))
+        return fail(ctx, RA_ERR_INVALID_ARG, "q/k_new/v_new/out must be non-NULL and 16-byte aligned");
     // validate every layer's capacity first so that a failing step changes nothing
     for (int l = 0; l < ctx->L; ++l)
         for (int b = 0; b < ctx->B; ++b)
@@ -1390,6 +1428,20 @@ int ra_decode_step(ra_ctx* ctx, const uint16_t* q_all, const uint16_t* k_all, co
     cudaStream_t s = (cudaStream_t)stream;
     if (ctx->step_open && (rc = step_epilogue(ctx, s)) != RA_OK) return rc;  // a per-layer step left open
     if ((rc = step_prologue(ctx, s)) != RA_OK) return rc;
+    // All the step's inputs are here, so the layers' attention runs as one launch: first the rounds
+    // left to the layers (sequences that fire with no set computed ahead; they need cached rows
+    // only), then every layer at once.  With compaction inside the attention pass, or with
+    // counters that differ between layers, layer by layer.
+    if (ctx->L > 1 && layers_alike(ctx) && !(ctx->compaction == RA_COMPACT_FUSED && ctx->r <= 64)) {
+        std::vector<int32_t> old_rows((size_t)ctx->B, -1);
+        double compacted = 0;
+        int n = 0;
+        for (int l = 0; l < ctx->L && rc == RA_OK; ++l) rc = evict_pending(ctx, l, s, ctx->step_cur, old_rows, &compacted, &n);
+        if (rc == RA_OK)
+            rc = attend_pending(ctx, 0, ctx->L, q_all, k_all, v_all, out_all, scale, s, true, old_rows, 0.0);
+        const int rc_end = step_epilogue(ctx, s);
+        return rc != RA_OK ? rc : rc_end;
+    }
     for (int l = 0; l < ctx->L; ++l)
         if ((rc = decode_layer_impl(ctx, l, q_all + l * qs, k_all + l * ks, v_all + l * ks, out_all + l * qs, scale,
                                     stream, ctx->step_cur)) != RA_OK)
@@ -1631,13 +1683,15 @@ extern "C" int ra_decode_attn_noalloc(ra_ctx* ctx, int layer, const uint16_t* q,
     int n_active = 0, ctas = 0;
     double rows = 0;
     int shape = kAttnWide;
-    if ((rc = plan_attention(ctx, layer, 0, &p, &n_active, &ctas, &rows, &shape)) != RA_OK) return rc;
+    if ((rc = plan_attention(ctx, layer, 1, 0, &p, &n_active, &ctas, &rows, &shape)) != RA_OK) return rc;
     if (n_active == 0) return RA_OK;
     set_scale(&p, scale);
-    // [arrival counters, one int per (seq, KV head)][partial records, one per (chunk, head) piece]
-    const size_t counters = align_up((size_t)ctx->B * ctx->KVH * sizeof(int32_t), kAlign);
-    const size_t need =
-        counters + (size_t)(p.nchunks + (long long)ctx->B * ctx->KVH) * partial_stride(ctx->G) * sizeof(float);
+    // [arrival counters, one int per chunk][partial records, two per chunk].  The limit that the
+    // interface states counts a record per warp and per head.
+    const size_t counters = align_up((size_t)p.nchunks * sizeof(int32_t), kAlign), record = partial_stride(ctx->G) * sizeof(float);
+    const size_t heads = (size_t)ctx->B * ctx->KVH;
+    const size_t need = std::max(align_up(heads * sizeof(int32_t), kAlign) + (p.nchunks + heads) * record,
+                                 counters + 2 * (size_t)p.nchunks * record);
     if (need > kNoAllocScratchBytes)
         return fail(ctx, RA_ERR_CAPACITY, "layer needs %zu bytes of split-K scratch; the fixed array holds %zu", need,
                     kNoAllocScratchBytes);

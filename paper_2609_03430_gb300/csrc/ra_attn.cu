@@ -10,18 +10,23 @@
 // consumes that tile.
 //
 // Work split: every head is cut into tiles of TILE rows (its prompt rows, then
-// its generated rows); the tiles of all heads of the layer are laid end to end
-// (sequence-major, then KV head) and cut into equal chunks of W tiles, one per
-// warp, so every warp makes the same number of pipeline trips.  A
+// its generated rows); the tiles of all heads of the launch are laid end to end
+// (layer-major, then sequence, then KV head) and cut into equal chunks of W
+// tiles, one per warp, so every warp makes the same number of pipeline trips.
+// A launch takes one layer, or every layer of a stacked step: its ramp and its
+// tail (about 10 us together, during which the memory idles) then come once a
+// step instead of once a layer.  36 layers of 174 MB, one launch each: 1340 us
+// a step, in one launch 921 us; 64 layers of 8.7 MB: 1747 and 95 us.  A
 // warp runs its own pipeline: lane 0 streams the tiles of K and V -- each as
 // two 64-channel boxes stored with the 128-byte swizzle -- plus, at the first
 // tile of each head piece, the G query rows, into a ring of SPW shared-memory
 // stages with 2-D TMA loads completing on per-stage mbarriers; all 32 lanes
 // consume.  A head that fits in one chunk is finished in registers.  Otherwise
 // each (head, chunk) piece writes an fp32 partial (unnormalised o, running max
-// m, sum l) to record `chunk + head` -- unique because chunks and heads both
-// advance monotonically through the tile order -- and the last warp to finish
-// a piece of that head (an arrival counter per head) merges all of them.
+// m, sum l) to one of its chunk's two records -- record 1 for the head that
+// starts in the chunk and goes on in the next, record 0 for the head that
+// began before it -- and the last warp to finish a piece of that head (an
+// arrival counter per chunk, that of the head's first) merges all of them.
 //
 // With the scored comparator's buffers bound, the warp that consumes a head's
 // first tile also copies the head's G query rows into the query window, and
@@ -117,6 +122,11 @@ struct Cfg {
     static_assert(SMEM <= 232448, "fits the 227 KB opt-in shared memory of sm_100+");
 };
 
+// What a launch does: one layer; one layer with the compaction of the heads in p.compacting; several
+// layers.  Instantiations of their own, so that plain launches run code free of the others' branches
+// and registers (with the layer walk in it, a layer of one sequence took 6% longer).
+constexpr int kModePlain = 0, kModeCompact = 1, kModeStack = 2;
+
 // Tile header flags; the chunk index sits above them (<< kFlagBits).
 constexpr int kFirst = 1, kLast = 2, kNewTok = 4, kHead0 = 8, kCompact = 16, kFlagBits = 5;
 
@@ -124,7 +134,7 @@ constexpr int kFirst = 1, kLast = 2, kNewTok = 4, kHead0 = 8, kCompact = 16, kFl
 struct TileIter {
     int chunk;                       // this warp's chunk (-1: not started)
     int f, end;                      // flattened tile cursor and end of the current chunk
-    int b, h, k;                     // current sequence, KV head, tile within the head
+    int l, b, h, k;                  // current layer (of the launch), sequence, KV head, tile within the head
     int nt, tp;                      // tiles in the head, prompt tiles among them
     int lp, gen;                     // prompt rows, generated rows (incl. a fused new token)
     bool comp;                       // the head compacts in this launch: its generated rows are the old region's
@@ -132,6 +142,7 @@ struct TileIter {
     const int32_t* ptab;             // the sequence's page table (null: its pages are page0, page0 + 1, ...)
     int page0;
     int pg_i, pg_cur, pg_next;       // page-table entry i of the current prompt tile, and entry i + 1 (read ahead)
+    int reg_hid, reg_next;           // several layers: the head whose region was read ahead, and that region
     bool piece_start;
 };
 
@@ -140,19 +151,37 @@ struct TileDesc {
     int n, hid, flags, chunk;
 };
 
+// The sequence of head `hid` of the launch, (layer * B + sequence) * KVH + KV head.
+template <int MODE>
+__device__ __forceinline__ int hid_seq(const AttnParams& p, int hid)
+{
+    const int lb = hid / p.lay.KVH;
+    return MODE == kModeStack ? lb % p.lay.B : lb;
+}
+
 __device__ __forceinline__ int seq_head_tiles(const AttnParams& p, int b)
 {
     return (p.seq_base[b + 1] - p.seq_base[b]) / p.lay.KVH;
 }
 
-template <bool COMPACT>
+// First tile of head `hid` in the launch's tile order, and the head's tiles.
+template <int MODE>
+__device__ __forceinline__ long long head_tile0(const AttnParams& p, int hid, int* nth)
+{
+    const int lb = hid / p.lay.KVH, h = hid - lb * p.lay.KVH;
+    const int l = MODE == kModeStack ? lb / p.lay.B : 0, b = lb - l * p.lay.B;
+    *nth = seq_head_tiles(p, b);
+    return (long long)l * p.layer_tiles + p.seq_base[b] + (long long)h * *nth;
+}
+
+template <int MODE>
 __device__ __forceinline__ void enter_head(TileIter& it, const AttnParams& p)
 {
     const DevLayout& L = p.lay;
     it.lp = p.seq_lp[it.b];
     it.gen = p.seq_gen[it.b];
     it.tp = (it.lp + p.tile - 1) / p.tile;
-    it.pbase = prompt_row(L, p.layer, 0, it.h, 0);
+    it.pbase = prompt_row(L, p.layer + (MODE == kModeStack ? it.l : 0), 0, it.h, 0);
     it.page0 = p.seq_page0[it.b];
     it.ptab = it.page0 >= 0 ? nullptr : L.pages + (size_t)it.b * L.max_pages;
     it.pg_i = 0;
@@ -160,48 +189,60 @@ __device__ __forceinline__ void enter_head(TileIter& it, const AttnParams& p)
         it.pg_cur = it.ptab ? __ldg(it.ptab) : it.page0;
         it.pg_next = it.lp > kPromptPage ? (it.ptab ? __ldg(it.ptab + 1) : it.page0 + 1) : 0;
     }
-    it.comp = COMPACT && ((p.compacting[it.b >> 5] >> (it.b & 31)) & 1u);
-    const int reg = it.comp ? L.plan[(size_t)(it.b * L.KVH + it.h) * (kPlanHeader + L.r)]  // the old region
-                            : p.seq_region[it.b] * L.KVH + it.h;
+    it.comp = MODE == kModeCompact && ((p.compacting[it.b >> 5] >> (it.b & 31)) & 1u);
+    int reg;
+    if (MODE == kModeStack) {  // the next head's region is read one head ahead
+        const int hid = (it.l * L.B + it.b) * L.KVH + it.h, last = p.layers * L.B * L.KVH - 1;
+        const int32_t* tab = L.region + (size_t)p.layer * L.B * L.KVH;
+        reg = it.reg_hid == hid ? it.reg_next : __ldcg(tab + hid);
+        it.reg_hid = hid + 1;
+        it.reg_next = hid < last ? __ldcg(tab + hid + 1) : 0;
+    } else {
+        reg = it.comp ? L.plan[(size_t)(it.b * L.KVH + it.h) * (kPlanHeader + L.r)]  // the old region
+                      : p.seq_region[it.b] * L.KVH + it.h;
+    }
     it.grow = L.gen_row0 + (long long)reg * L.Cmax;
     it.piece_start = true;
 }
 
-template <bool COMPACT>
+template <int MODE>
 __device__ void iter_init(TileIter& it, const AttnParams& p, int R0, int R1)
 {
     it.f = R0;
     it.end = R1;
-    int lo = 0, hi = p.lay.B - 1;  // largest b with seq_base[b] <= R0 (empty sequences skipped below)
+    it.reg_hid = -1;
+    it.l = MODE == kModeStack ? R0 / p.layer_tiles : 0;
+    const int F = R0 - it.l * p.layer_tiles;
+    int lo = 0, hi = p.lay.B - 1;  // largest b with seq_base[b] <= F (empty sequences skipped below)
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if (p.seq_base[mid] <= R0) lo = mid; else hi = mid - 1;
+        if (p.seq_base[mid] <= F) lo = mid; else hi = mid - 1;
     }
     int b = lo;
-    while (b < p.lay.B && p.seq_base[b + 1] <= R0) ++b;
+    while (b < p.lay.B && p.seq_base[b + 1] <= F) ++b;
     it.b = b;
     it.nt = seq_head_tiles(p, b);
-    const int off = R0 - p.seq_base[b];
+    const int off = F - p.seq_base[b];
     it.h = off / it.nt;
     it.k = off - it.h * it.nt;
-    enter_head<COMPACT>(it, p);
+    enter_head<MODE>(it, p);
 }
 
 // The warp's chunk (its index): false once it is done.
-template <bool COMPACT>
+template <int MODE>
 __device__ bool iter_next_chunk(TileIter& it, const AttnParams& p, int warp_id)
 {
     if (it.chunk >= 0 || warp_id >= p.nchunks) return false;
     it.chunk = warp_id;
     const int R0 = warp_id * p.W;
-    iter_init<COMPACT>(it, p, R0, min(p.total, R0 + p.W));
+    iter_init<MODE>(it, p, R0, min(p.total, R0 + p.W));
     return true;
 }
 
-template <bool COMPACT>
+template <int MODE>
 __device__ bool iter_next(TileIter& it, const AttnParams& p, TileDesc& d, int warp_id)
 {
-    if (it.f >= it.end && !iter_next_chunk<COMPACT>(it, p, warp_id)) return false;
+    if (it.f >= it.end && !iter_next_chunk<MODE>(it, p, warp_id)) return false;
     const int T = p.tile;
     d.flags = (it.piece_start ? kFirst : 0) | (it.k == 0 ? kHead0 : 0);
     if (it.k < it.tp) {  // a prompt tile lies inside one page (kPromptPage is a multiple of T)
@@ -219,10 +260,10 @@ __device__ bool iter_next(TileIter& it, const AttnParams& p, TileDesc& d, int wa
         d.n = min(T, it.gen - kg * T);
         if (p.k_new && ((p.pending[it.b >> 5] >> (it.b & 31)) & 1u) && kg * T + d.n == it.gen)
             d.flags |= kNewTok;  // its last row is the step's new token
-        if (COMPACT && it.comp) d.flags |= kCompact;
+        if (MODE == kModeCompact && it.comp) d.flags |= kCompact;
     }
     if (it.k + 1 == it.nt || it.f + 1 == it.end) d.flags |= kLast;
-    d.hid = it.b * p.lay.KVH + it.h;
+    d.hid = ((MODE == kModeStack ? it.l * p.lay.B : 0) + it.b) * p.lay.KVH + it.h;
     d.chunk = it.chunk;
     it.piece_start = false;
     ++it.k;
@@ -232,11 +273,15 @@ __device__ bool iter_next(TileIter& it, const AttnParams& p, TileDesc& d, int wa
             it.h = 0;
             do {
                 ++it.b;
+                if (MODE == kModeStack && it.b == p.lay.B) {  // (only with layers left: it.f < it.end)
+                    it.b = 0;
+                    ++it.l;
+                }
             } while (seq_head_tiles(p, it.b) == 0);
             it.nt = seq_head_tiles(p, it.b);
         }
         it.k = 0;
-        enter_head<COMPACT>(it, p);
+        enter_head<MODE>(it, p);
     }
     return true;
 }
@@ -307,31 +352,32 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
            ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(hi)) << 16);
 }
 
-// The scored policy's window: the softmax normaliser of query head g of (b, KV head h) at this
+// The scored policy's window: the softmax normaliser of query head g of head `hid` at this
 // step, as (scale * log2 e, log2 sum_i exp2(scale * log2 e * q.k_i)), beside its query rows.
-template <int G>
-__device__ __forceinline__ void record_stats(const AttnParams& p, int b, int h, int g, float lse2)
+template <int G, int MODE>
+__device__ __forceinline__ void record_stats(const AttnParams& p, int hid, int g, float lse2)
 {
     const int r = p.lay.r;
-    int slot = (p.seq_g[b] + p.ring_off) % r;
+    int slot = (p.seq_g[hid_seq<MODE>(p, hid)] + p.ring_off) % r;
     if (slot < 0) slot += r;
-    p.lay.qstats[((((size_t)p.layer * p.lay.B + b) * p.lay.KVH + h) * r + slot) * G + g] =
+    p.lay.qstats[(((size_t)p.layer * p.lay.B * p.lay.KVH + hid) * r + slot) * G + g] =
         make_float2(p.qk_scale_log2, lse2);
 }
 
-// Merge every piece of head `hid` (pieces are partial records c0 + q + hid, q < P) into the
-// bf16 output rows of its G query heads.  One warp, two rounds of L2 reads: first every lane
+// Merge every piece of head `hid` (P chunks from w0 on: record 1 of chunk w0, record 0 of the
+// others) into the bf16 output rows of its G query heads.  One warp, two rounds of L2 reads: first every lane
 // reads the statistics of its pieces (lane q: piece q, q + 32, ...) and the warp reduces them
 // to each query head's max M and normaliser L; then lanes split as (query head g, channel
 // group), and for every piece load its max (one address per head: a broadcast) and their
 // channels together, so the loads of all pieces are independent.  Partials come from other
 // SMs: read through L2.
-template <int G>
-__device__ void merge_head(const AttnParams& p, int hid, int c0, int P, int lane)
+template <int G, int MODE>
+__device__ void merge_head(const AttnParams& p, int hid, int w0, int P, int lane)
 {
     using C = Cfg<G>;
-    const size_t rs = (size_t)partial_stride(G);
-    const float* base = p.partial + (size_t)(c0 + hid) * rs;
+    constexpr int rs = partial_stride(G);
+    const float* base = p.partial + (size_t)w0 * 2 * rs;
+    auto piece = [&](int q) { return base + (size_t)(q == 0 ? rs : 2 * q * rs); };
     float M[G], Lh[G];
 #pragma unroll
     for (int g = 0; g < G; ++g) {
@@ -340,7 +386,7 @@ __device__ void merge_head(const AttnParams& p, int hid, int c0, int P, int lane
     }
     for (int q = lane; q < P; q += 32)
 #pragma unroll
-        for (int g = 0; g < G; ++g) M[g] = fmaxf(M[g], __ldcg(base + q * rs + G * kHeadDim + g));
+        for (int g = 0; g < G; ++g) M[g] = fmaxf(M[g], __ldcg(piece(q) + G * kHeadDim + g));
 #pragma unroll
     for (int g = 0; g < G; ++g)
 #pragma unroll
@@ -348,7 +394,7 @@ __device__ void merge_head(const AttnParams& p, int hid, int c0, int P, int lane
     for (int q = lane; q < P; q += 32)
 #pragma unroll
         for (int g = 0; g < G; ++g) {
-            const float* st = base + q * rs + G * kHeadDim;
+            const float* st = piece(q) + G * kHeadDim;
             Lh[g] = fmaf(exp2f(__ldcg(st + g) - M[g]), __ldcg(st + G + g), Lh[g]);
         }
 #pragma unroll
@@ -371,7 +417,7 @@ __device__ void merge_head(const AttnParams& p, int hid, int c0, int P, int lane
     for (int j = 0; j < C::MCH / 4; ++j) acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
     for (int q = 0; q < P; ++q) {
-        const float* rec = base + q * rs;
+        const float* rec = piece(q);
         const float a = exp2f(__ldcg(rec + G * kHeadDim + gg) - Mg);
         const float4* o = reinterpret_cast<const float4*>(rec + gg * kHeadDim + ch0);
 #pragma unroll
@@ -385,9 +431,8 @@ __device__ void merge_head(const AttnParams& p, int hid, int c0, int P, int lane
     }
     if (g >= G) return;
     const float inv = 1.f / Lg;
-    const int b = hid / p.lay.KVH, h = hid - b * p.lay.KVH;
-    if (p.qring && sub == 0) record_stats<G>(p, b, h, g, Mg + log2f(Lg));
-    uint16_t* out = p.out + ((size_t)b * p.lay.H + (size_t)h * G + g) * kHeadDim + ch0;
+    if (p.qring && sub == 0) record_stats<G, MODE>(p, hid, g, Mg + log2f(Lg));
+    uint16_t* out = p.out + ((size_t)hid * G + g) * kHeadDim + ch0;
 #pragma unroll
     for (int k = 0; k < C::MCH / 4; ++k) {
         const uint2 w = make_uint2(pack_bf16x2(acc[k].x * inv, acc[k].y * inv), pack_bf16x2(acc[k].z * inv, acc[k].w * inv));
@@ -395,9 +440,7 @@ __device__ void merge_head(const AttnParams& p, int hid, int c0, int P, int lane
     }
 }
 
-// COMPACT: the launch also does the compaction of the heads in p.compacting (a separate
-// instantiation, so that launches without it run code free of its branches and registers).
-template <int G, bool COMPACT>
+template <int G, int MODE>
 __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
     attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtensorMap tk,
                 const __grid_constant__ CUtensorMap tv)
@@ -439,19 +482,18 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
     auto issue_inputs = [&](int s) {
         const int4 hd = hdrs[s];
         uint8_t* st = wstage + (size_t)s * C::STAGE_BYTES;
-        const int b = hd.z / p.lay.KVH, h = hd.z - b * p.lay.KVH;
         if (hd.y & kNewTok) {
-            const size_t src = ((size_t)b * p.lay.KVH + h) * kHeadDim;
+            const size_t src = (size_t)hd.z * kHeadDim;
             bulk_load(st + C::NT_OFF, p.k_new + src, (uint32_t)kRowBytes, &bars[s]);
             bulk_load(st + C::NT_OFF + kRowBytes, p.v_new + src, (uint32_t)kRowBytes, &bars[s]);
         }
         if (hd.y & kFirst)
-            bulk_load(st + 2 * C::KV_BYTES, p.q + ((size_t)b * p.lay.H + (size_t)h * G) * kHeadDim,
+            bulk_load(st + 2 * C::KV_BYTES, p.q + (size_t)hd.z * G * kHeadDim,
                       (uint32_t)C::Q_BYTES, &bars[s]);
     };
     auto issue = [&](int t, bool inputs) -> bool {
         TileDesc d;
-        if (!iter_next<COMPACT>(it, p, d, gw)) return false;
+        if (!iter_next<MODE>(it, p, d, gw)) return false;
         const int s = t % C::SPW;
         if (lane == 0) {
             uint8_t* st = wstage + (size_t)s * C::STAGE_BYTES;
@@ -520,11 +562,11 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
                 qa[kk][1] = gq < G ? *reinterpret_cast<const uint32_t*>(Qs + gq * kRowBytes + (16 * kk + 8 + 2 * tq) * 2) : 0u;
             }
             if ((hd.y & kHead0) && p.qring) {  // the scored policy's window: this step's query rows of the head
-                const int b = hd.z / p.lay.KVH, h = hd.z - b * p.lay.KVH, r = p.lay.r;
-                int slot = (p.seq_g[b] + p.ring_off) % r;
+                const int r = p.lay.r;
+                int slot = (p.seq_g[hid_seq<MODE>(p, hd.z)] + p.ring_off) % r;
                 if (slot < 0) slot += r;
                 uint4* dst = reinterpret_cast<uint4*>(
-                    p.qring + ((((size_t)p.layer * p.lay.B + b) * p.lay.KVH + h) * r + slot) * (size_t)(G * kHeadDim));
+                    p.qring + (((size_t)p.layer * p.lay.B * p.lay.KVH + hd.z) * r + slot) * (size_t)(G * kHeadDim));
                 for (int i = lane; i < G * 16; i += 32) dst[i] = lds128(Qs + i * 16);
             }
         }
@@ -532,7 +574,7 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
         // mask, from the ascending list of at most 64 evicted ordinals) and how many before it.
         uint32_t ev_lo = 0u, ev_hi = 0u;
         int ev_before = 0, j0 = 0;
-        if (COMPACT && (hd.y & kCompact)) {
+        if (MODE == kModeCompact && (hd.y & kCompact)) {
             const int32_t* plan = p.lay.plan + (size_t)hd.z * (kPlanHeader + p.lay.r);
             const int m = plan[3];
             j0 = (int)((long long)hd.w - p.lay.gen_row0 - (long long)plan[0] * p.lay.Cmax);
@@ -545,11 +587,11 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
             ev_hi = __reduce_or_sync(0xffffffffu, hi);
         }
         if (hd.y & kNewTok) {  // fused append: put the new token in row n-1 of the tile and into the cache
-            const int b = hd.z / p.lay.KVH;
+            const int b = hid_seq<MODE>(p, hd.z);
             const int c = lane & 15;
             const uint4 v = lds128(Ks + C::NT_OFF + (lane >> 4) * kRowBytes + c * 16);
             *reinterpret_cast<uint4*>((lane < 16 ? Ks : Vs) + swz<G>(n - 1, c)) = v;
-            if (!(COMPACT && (hd.y & kCompact))) {  // (a compacting head writes it with its survivors)
+            if (!(MODE == kModeCompact && (hd.y & kCompact))) {  // (a compacting head writes it with its survivors)
                 const long long row = (long long)hd.w + n - 1;
                 reinterpret_cast<uint4*>((lane < 16 ? p.lay.kpool : p.lay.vpool) + row * kHeadDim)[c] = v;
                 if (lane == 0) p.lay.pos[row - p.lay.gen_row0] = p.seq_lp[b] + p.seq_g[b];
@@ -580,7 +622,7 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
             }
             const int r0 = bs + gq, r1 = r0 + 8;  // this lane's rows; heads hA, hB
             bool v0 = r0 < n, v1 = r1 < n;
-            if (COMPACT && (hd.y & kCompact)) {  // evicted rows get no weight
+            if (MODE == kModeCompact && (hd.y & kCompact)) {  // evicted rows get no weight
                 v0 = v0 && !(((r0 < 32 ? ev_lo >> r0 : ev_hi >> (r0 - 32)) & 1u));
                 v1 = v1 && !(((r1 < 32 ? ev_lo >> r1 : ev_hi >> (r1 - 32)) & 1u));
             }
@@ -611,7 +653,7 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const float m = (e & 1) ? mB : mA;
-                pr[e] = (COMPACT && sv[e] == -INFINITY) ? 0.f : exp2f(sv[e] - m);
+                pr[e] = (MODE == kModeCompact && sv[e] == -INFINITY) ? 0.f : exp2f(sv[e] - m);
             }
             lA += pr[0] + pr[2];
             lB += pr[1] + pr[3];
@@ -632,17 +674,16 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
                 lb += __shfl_xor_sync(0xffffffffu, lb, o);
             }
             const int hid = hd.z;
-            const int b = hid / p.lay.KVH, h = hid - b * p.lay.KVH;
-            const int nth = seq_head_tiles(p, b);
-            const long long A = p.seq_base[b] + (long long)h * nth;
+            int nth;
+            const long long A = head_tile0<MODE>(p, hid, &nth);
             const int w0 = (int)(A / p.W), w1 = (int)((A + nth - 1) / p.W);
             if (w0 == w1) {  // the whole head was this warp's: normalise and write the output
                 if (p.qring && gq == 0) {
-                    if (hA < G) record_stats<G>(p, b, h, hA, mA + log2f(la));
-                    if (hB < G) record_stats<G>(p, b, h, hB, mB + log2f(lb));
+                    if (hA < G) record_stats<G, MODE>(p, hid, hA, mA + log2f(la));
+                    if (hB < G) record_stats<G, MODE>(p, hid, hB, mB + log2f(lb));
                 }
                 const float iA = 1.f / la, iB = 1.f / lb;
-                __nv_bfloat16* ob = reinterpret_cast<__nv_bfloat16*>(p.out + ((size_t)b * p.lay.H + (size_t)h * G) * kHeadDim);
+                __nv_bfloat16* ob = reinterpret_cast<__nv_bfloat16*>(p.out + (size_t)hid * G * kHeadDim);
 #pragma unroll
                 for (int mt = 0; mt < 8; ++mt) {
                     const int ch = 16 * mt + gq;
@@ -656,7 +697,8 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
                     }
                 }
             } else {
-                float* rec = p.partial + (size_t)((hd.y >> kFlagBits) + hid) * partial_stride(G);
+                const int chunk = hd.y >> kFlagBits;
+                float* rec = p.partial + (size_t)(2 * chunk + (chunk == w0 ? 1 : 0)) * partial_stride(G);
 #pragma unroll
                 for (int mt = 0; mt < 8; ++mt) {
                     const int ch = 16 * mt + gq;
@@ -682,12 +724,12 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
                 __threadfence();
                 __syncwarp();
                 int old = 0;
-                if (lane == 0) old = atomicAdd(p.arrive + hid, 1);
+                if (lane == 0) old = atomicAdd(p.arrive + w0, 1);
                 old = __shfl_sync(0xffffffffu, old, 0);
                 if (old == w1 - w0) {  // every other piece of this head is already written
                     __threadfence();
-                    merge_head<G>(p, hid, w0, w1 - w0 + 1, lane);
-                    if (lane == 0) p.arrive[hid] = 0;  // ready for the next launch
+                    merge_head<G, MODE>(p, hid, w0, w1 - w0 + 1, lane);
+                    if (lane == 0) p.arrive[w0] = 0;  // ready for the next launch
                 }
             }
             mA = mB = -INFINITY;
@@ -711,7 +753,7 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
             const float sl = p.qk_scale_log2;
             float sc[4] = {r0 < n ? s0a * sl : -INFINITY, r0 + 1 < n ? s0b * sl : -INFINITY,
                            r0 + 8 < n ? s1a * sl : -INFINITY, r0 + 9 < n ? s1b * sl : -INFINITY};
-            if (COMPACT && (hd.y & kCompact)) {  // evicted rows get no weight
+            if (MODE == kModeCompact && (hd.y & kCompact)) {  // evicted rows get no weight
                 const int rr[4] = {r0, r0 + 1, r0 + 8, r0 + 9};
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
@@ -736,7 +778,7 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
 #pragma unroll
             // masked rows: exp2(-inf) = 0; a compacting head can have a whole batch evicted, with
             // m_run still -inf (the difference would be NaN), so there a masked row weighs 0 outright
-            for (int e = 0; e < 4; ++e) pr[e] = (COMPACT && sc[e] == -INFINITY) ? 0.f : exp2f(sc[e] - m_run);
+            for (int e = 0; e < 4; ++e) pr[e] = (MODE == kModeCompact && sc[e] == -INFINITY) ? 0.f : exp2f(sc[e] - m_run);
             l_run += (pr[0] + pr[1]) + (pr[2] + pr[3]);
             const uint32_t pa0 = pack_bf16x2(pr[0], pr[1]), pa2 = pack_bf16x2(pr[2], pr[3]);
             // O += P V: 16 n-tiles of 8 channels, k = the 16 rows
@@ -754,20 +796,20 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
             l += __shfl_xor_sync(0xffffffffu, l, 1);
             l += __shfl_xor_sync(0xffffffffu, l, 2);
             const int hid = hd.z;
-            const int b = hid / p.lay.KVH, h = hid - b * p.lay.KVH;
-            const int nth = seq_head_tiles(p, b);
-            const long long A = p.seq_base[b] + (long long)h * nth;
+            int nth;
+            const long long A = head_tile0<MODE>(p, hid, &nth);
             const int w0 = (int)(A / p.W), w1 = (int)((A + nth - 1) / p.W);
             if (w0 == w1) {  // the whole head was this warp's: normalise and write the output
                 if (gq < G) {
-                    if (p.qring && tq == 0) record_stats<G>(p, b, h, gq, m_run + log2f(l));
+                    if (p.qring && tq == 0) record_stats<G, MODE>(p, hid, gq, m_run + log2f(l));
                     const float inv = 1.f / l;
-                    uint32_t* out = reinterpret_cast<uint32_t*>(p.out + ((size_t)b * p.lay.H + (size_t)h * G + gq) * kHeadDim);
+                    uint32_t* out = reinterpret_cast<uint32_t*>(p.out + ((size_t)hid * G + gq) * kHeadDim);
 #pragma unroll
                     for (int nt = 0; nt < 16; ++nt) out[nt * 4 + tq] = pack_bf16x2(O[nt][0] * inv, O[nt][1] * inv);
                 }
             } else {
-                float* rec = p.partial + (size_t)((hd.y >> kFlagBits) + hid) * partial_stride(G);
+                const int chunk = hd.y >> kFlagBits;
+                float* rec = p.partial + (size_t)(2 * chunk + (chunk == w0 ? 1 : 0)) * partial_stride(G);
                 if (gq < G) {
 #pragma unroll
                     for (int nt = 0; nt < 16; ++nt)
@@ -780,12 +822,12 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
                 __threadfence();
                 __syncwarp();
                 int old = 0;
-                if (lane == 0) old = atomicAdd(p.arrive + hid, 1);
+                if (lane == 0) old = atomicAdd(p.arrive + w0, 1);
                 old = __shfl_sync(0xffffffffu, old, 0);
                 if (old == w1 - w0) {  // every other piece of this head is already written
                     __threadfence();
-                    merge_head<G>(p, hid, w0, w1 - w0 + 1, lane);
-                    if (lane == 0) p.arrive[hid] = 0;  // ready for the next launch
+                    merge_head<G, MODE>(p, hid, w0, w1 - w0 + 1, lane);
+                    if (lane == 0) p.arrive[w0] = 0;  // ready for the next launch
                 }
             }
             m_run = -INFINITY;
@@ -795,7 +837,7 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
         }
 #endif
 
-        if (COMPACT && (hd.y & kCompact)) {
+        if (MODE == kModeCompact && (hd.y & kCompact)) {
             // Compaction fused into the pass: every surviving row of the tile (the new token
             // included) goes from the staged tile to its slot in the new region, ordinal
             // j - (evicted before j); positions follow.  One row per step, 16-byte lanes
@@ -819,7 +861,7 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
             }
             for (int jj = lane; jj < n; jj += 32) {
                 if (evicted(jj)) continue;
-                const int b = hd.z / p.lay.KVH;
+                const int b = hid_seq<MODE>(p, hd.z);
                 const bool newtok = (hd.y & kNewTok) && jj == n - 1;
                 dpos[dest(jj)] = newtok ? p.seq_lp[b] + p.seq_g[b] : __ldg(spos + j0 + jj);
             }
@@ -853,17 +895,18 @@ cudaError_t launch_attn_g(const AttnParams& p, const CUtensorMap* tk, const CUte
     using C = Cfg<G>;
     bool compact = false;
     for (int i = 0; i < RA_MAX_BATCH / 32; ++i) compact |= p.compacting[i] != 0u;
-    if (compact) return launch_pdl(attn_kernel<G, true>, dim3(ctas), dim3(C::WARPS * 32), C::SMEM, s, p, *tk, *tv);
-    return launch_pdl(attn_kernel<G, false>, dim3(ctas), dim3(C::WARPS * 32), C::SMEM, s, p, *tk, *tv);
+    auto kernel = p.layers > 1 ? attn_kernel<G, kModeStack> : compact ? attn_kernel<G, kModeCompact> : attn_kernel<G, kModePlain>;
+    return launch_pdl(kernel, dim3(ctas), dim3(C::WARPS * 32), C::SMEM, s, p, *tk, *tv);
 }
 
 template <int G>
 cudaError_t prepare_g()
 {
-    cudaError_t e = cudaFuncSetAttribute(attn_kernel<G, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)Cfg<G>::SMEM);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(attn_kernel<G, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<G>::SMEM);
+    for (auto kernel : {attn_kernel<G, kModePlain>, attn_kernel<G, kModeCompact>, attn_kernel<G, kModeStack>}) {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<G>::SMEM);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace

@@ -38,7 +38,7 @@ struct DevLayout {
     int32_t* pages;        // [B][max_pages] page of each kPromptPage-position block of a sequence's prompt
     int32_t* plan;         // [B*KVH][kPlanHeader + r] eviction plan of the current layer
     float* partial;        // attention split partials
-    int32_t* arrive;       // [B*KVH] split-piece arrival counters
+    int32_t* arrive;       // split-piece arrival counters, one per chunk of the attention split
     int32_t* err;          // device error word
     int32_t* evplan;       // [2][L][B][KVH][r + 1] evicted sets computed ahead (plan_kernel)
     // scored policy (null when the context was bound without its buffers)
@@ -107,18 +107,22 @@ constexpr int kScoreMaxCandidates = 16384;  // K + r bound of the scored policy 
 
 // Attention work is counted in tiles of TILE rows: a head has ceil(lp / TILE) prompt tiles and
 // ceil(gen / TILE) tiles of generated rows (gen includes a fused new token, its last row).
+// A launch takes `layers` layers from `layer` on, their counters alike (the per-sequence arrays below
+// serve every layer): their heads and tiles are laid end to end, layer-major.
 struct AttnParams {
     DevLayout lay;
-    int layer;
+    int layer;              // first layer
+    int layers;             // layers of the launch (more than one: the region tables are read from memory)
+    int layer_tiles;        // tiles of one layer
     int tile;               // rows per tile
-    const uint16_t* q;      // [B][H][128]
-    uint16_t* out;          // [B][H][128]
-    const uint16_t* k_new;  // fused append: the step's new rows [B][KVH][128]; null = attention only
+    const uint16_t* q;      // [layers][B][H][128]
+    uint16_t* out;          // [layers][B][H][128]
+    const uint16_t* k_new;  // fused append: the step's new rows [layers][B][KVH][128]; null = attention only
     const uint16_t* v_new;
-    float* partial;         // split-K partial records (arena or the no-alloc array)
-    int32_t* arrive;        // [B*KVH] pieces merged so far per head; zero between launches
+    float* partial;         // split-K partial records, two per chunk (arena or the no-alloc array)
+    int32_t* arrive;        // per chunk: pieces merged so far of the head that starts there; zero between launches
     int W;                  // tiles per chunk of the split: warp w takes tiles [w W, (w + 1) W)
-    int total;              // total tiles of the layer
+    int total;              // total tiles of the launch
     int nchunks;            // ceil(total / W)
     int nwarps;             // warps launched
     float qk_scale_log2;    // scale * log2(e)

@@ -28,6 +28,15 @@
 // began before it -- and the last warp to finish a piece of that head (an
 // arrival counter per chunk, that of the head's first) merges all of them.
 //
+// The narrow build merges inside the CTA first.  Small layers have more warps
+// than heads: one sequence's 8 heads of 2.7K rows were 85 one-tile pieces each,
+// 177 KB of partials that one warp merged, 20.6 us a layer.  A CTA's warps hold
+// consecutive chunks, so their pieces of a head are deposited in shared memory
+// and merged there by the last of them; at most two records per CTA (the head it
+// shares with the CTA before and the one it shares with the next) go to global
+// memory, announced at the CTA's end, and the last CTA merges a head with all
+// its threads.  8.5 us a layer of one sequence, 33.1 instead of 36.6 us one of 16.
+//
 // With the scored comparator's buffers bound, the warp that consumes a head's
 // first tile also copies the head's G query rows into the query window, and
 // whoever finishes a head records each query's softmax normaliser beside it:
@@ -72,7 +81,11 @@ namespace {
 
 constexpr float kTau = 8.0f;                       // lazy-rescale threshold (log2 units)
 constexpr uint64_t kWaitLimitNs = 2000000000ull;   // bounded mbarrier waits: 2 s
+#if RA_ATTN_CTA_MERGE
+constexpr int kSmemBudget = 232448 - 1024 - 256;  // all an SM gives, but the alignment and the statics
+#else
 constexpr int kSmemBudget = 220 * 1024;
+#endif
 constexpr int kHalfCh = 64;                        // channels per swizzled TMA box (128 bytes)
 
 // Kernel shape: rows per stage (a multiple of 16), stages per warp, warps per CTA
@@ -96,20 +109,39 @@ constexpr int kHalfCh = 64;                        // channels per swizzled TMA 
 #ifndef RA_ATTN_TRANSPOSED
 #define RA_ATTN_TRANSPOSED 0
 #endif
+// 1: a CTA merges its warps' pieces of a head in shared memory before anything goes to global memory
+// (the narrow shape; see the comment at the top of the file).
+#define RA_ATTN_CTA_MERGE RA_ATTN_TRANSPOSED
 
 template <int G>
 struct Cfg {
     static constexpr int TILE = RA_ATTN_TILE;                                // rows per stage
     static constexpr int HALF_BYTES = TILE * 128;                            // one 64-channel half of K or V
     static constexpr int KV_BYTES = 2 * HALF_BYTES;                          // a K (or V) tile
-    static constexpr int Q_BYTES = G * kRowBytes;
-    static constexpr int NT_OFF = 2 * KV_BYTES + Q_BYTES;  // the fused new token's K and V rows (unswizzled)
-    static constexpr int STAGE_BYTES = (NT_OFF + 2 * kRowBytes + 1023) / 1024 * 1024;
+    static constexpr int STAGE_BYTES = 2 * KV_BYTES;
     static constexpr int SPW = RA_ATTN_SPW;
-    static constexpr int WARPS_FIT = kSmemBudget / (SPW * STAGE_BYTES);
+    // Beside the stages, per warp: the query rows of a piece and the fused new token's K and V rows
+    // (unswizzled).  A slot per stage, or with RA_ATTN_CTA_MERGE one per warp (a second piece start or
+    // new token among the tiles on the way is then read straight from global memory), which leaves
+    // room for the deposits: O (rows DEP_ROW floats apart: no bank conflicts), m and l of a piece.
+    static constexpr bool CTA_MERGE = RA_ATTN_CTA_MERGE;
+    static constexpr int SLOTS = CTA_MERGE ? 1 : SPW;
+    static constexpr int Q_BYTES = G * kRowBytes;
+    static constexpr int SLOT_BYTES = Q_BYTES + 2 * kRowBytes;
+    static constexpr int DEP_ROW = kHeadDim + 4;
+    static constexpr int DEP_FLOATS = G * DEP_ROW + (2 * G + 3) / 4 * 4;
+    static constexpr int DEP_BYTES = CTA_MERGE ? DEP_FLOATS * 4 : 0;
+    static constexpr int WARP_BYTES = SPW * (STAGE_BYTES + 16 + 8) + SLOTS * SLOT_BYTES + DEP_BYTES;
+    static constexpr int WARPS_FIT = kSmemBudget / WARP_BYTES;
     static constexpr int WARPS = WARPS_FIT < RA_ATTN_WARPS ? WARPS_FIT : RA_ATTN_WARPS;
     static constexpr int NSTAGE = WARPS * SPW;
-    static constexpr size_t SMEM = 1024 + (size_t)NSTAGE * STAGE_BYTES + (size_t)NSTAGE * (16 + 8);
+    // [stages][slots][deposits][tile headers][mbarriers]
+    static constexpr int SLOT_OFF = NSTAGE * STAGE_BYTES;
+    static constexpr int DEP_OFF = SLOT_OFF + WARPS * SLOTS * SLOT_BYTES;
+    static constexpr int HDR_OFF = DEP_OFF + WARPS * DEP_BYTES;
+    static constexpr int BAR_OFF = HDR_OFF + NSTAGE * 16;
+    static constexpr size_t SMEM = 1024 + (size_t)BAR_OFF + NSTAGE * 8;
+    static_assert(DEP_BYTES <= STAGE_BYTES && DEP_BYTES % 16 == 0, "a deposit fits a stage");
     // merge layout: LG lanes per query head, MCH channels per lane
     static constexpr int GP = G <= 1 ? 1 : (G <= 2 ? 2 : (G <= 4 ? 4 : 8));
     static constexpr int LG = 32 / GP;
@@ -119,7 +151,7 @@ struct Cfg {
     static_assert(kPromptPage % TILE == 0, "a prompt tile lies inside one page");
     static_assert(HALF_BYTES % 1024 == 0, "128-byte-swizzled TMA boxes start 1024-byte aligned");
     static_assert(WARPS >= 2, "shared-memory budget too small");
-    static_assert(SMEM <= 232448, "fits the 227 KB opt-in shared memory of sm_100+");
+    static_assert(SMEM + (CTA_MERGE ? 256 : 0) <= 232448, "fits the 227 KB opt-in shared memory of sm_100+");
 };
 
 // What a launch does: one layer; one layer with the compaction of the heads in p.compacting; several
@@ -128,7 +160,8 @@ struct Cfg {
 constexpr int kModePlain = 0, kModeCompact = 1, kModeStack = 2;
 
 // Tile header flags; the chunk index sits above them (<< kFlagBits).
-constexpr int kFirst = 1, kLast = 2, kNewTok = 4, kHead0 = 8, kCompact = 16, kFlagBits = 5;
+// kQDirect, kNtDirect: the query rows, the new token's rows are read straight from global memory.
+constexpr int kFirst = 1, kLast = 2, kNewTok = 4, kHead0 = 8, kCompact = 16, kQDirect = 32, kNtDirect = 64, kFlagBits = 7;
 
 // Producer-side walk over the warp's chunks (chunks and cursors count tiles).
 struct TileIter {
@@ -364,6 +397,7 @@ __device__ __forceinline__ void record_stats(const AttnParams& p, int hid, int g
         make_float2(p.qk_scale_log2, lse2);
 }
 
+#if !RA_ATTN_CTA_MERGE
 // Merge every piece of head `hid` (P chunks from w0 on: record 1 of chunk w0, record 0 of the
 // others) into the bf16 output rows of its G query heads.  One warp, two rounds of L2 reads: first every lane
 // reads the statistics of its pieces (lane q: piece q, q + 32, ...) and the warp reduces them
@@ -439,6 +473,158 @@ __device__ void merge_head(const AttnParams& p, int hid, int w0, int P, int lane
         *reinterpret_cast<uint2*>(out + 4 * k) = w;
     }
 }
+#else
+// The CTA's own merge.  A warp that ends its piece of a head which other warps of the CTA hold too
+// deposits it in shared memory; the last of them to do so merges the deposits, into the output or,
+// where the head goes on in another CTA, into one of the CTA's two global records (0: the head began
+// in an earlier CTA, 1: it starts here).
+struct CtaMerge {
+    int arrived[8];            // deposits made, by the first warp that holds a piece of the head (one head each)
+    int stage[8];              // the stage a warp's last piece ended in
+    struct Part {
+        int hid, c0, P;        // the record's head, the first CTA that holds a piece, how many do (0: no record)
+    } part[2];
+    int last[2];
+};
+
+// Where a warp deposits: its last piece goes to its stage other than `s` (nothing is on the way there any
+// more), a piece that ends before its chunk does to the warp's deposit slot.
+template <int G>
+__device__ __forceinline__ uint8_t* deposit(uint8_t* smem, int warp, bool last_piece, int s)
+{
+    using C = Cfg<G>;
+    static_assert(C::SPW == 2 || !C::CTA_MERGE, "the other stage");
+    return last_piece ? smem + (size_t)(warp * C::SPW + (s ^ 1)) * C::STAGE_BYTES : smem + C::DEP_OFF + (size_t)warp * C::DEP_BYTES;
+}
+
+// Warps a .. z of the CTA have deposited head `hid`, whose chunks are w0 .. w1.  One warp: lanes split
+// as (query head g, channel group).
+template <int G, int MODE>
+__device__ void merge_deposits(const AttnParams& p, CtaMerge& cm, uint8_t* smem, int hid, int w0, int w1, int a, int z, int lane)
+{
+    using C = Cfg<G>;
+    const int cta0 = (int)blockIdx.x * C::WARPS;
+    const int g = lane / C::LG, sub = lane % C::LG, ch0 = sub * C::MCH;
+    if (g < G) {
+        auto piece = [&](int w) { return reinterpret_cast<const float*>(deposit<G>(smem, w, cta0 + w < w1, cm.stage[w])); };
+        float M = -INFINITY, l = 0.f;
+        for (int w = a; w <= z; ++w) M = fmaxf(M, piece(w)[G * C::DEP_ROW + g]);
+        float4 acc[C::MCH / 4];
+#pragma unroll
+        for (int j = 0; j < C::MCH / 4; ++j) acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int w = a; w <= z; ++w) {
+            const float* rec = piece(w);
+            const float m = rec[G * C::DEP_ROW + g];
+            const float e = m == -INFINITY ? 0.f : exp2f(m - M);  // (a piece whose rows are all evicted weighs nothing)
+            l = fmaf(e, rec[G * C::DEP_ROW + G + g], l);
+            const float4* o = reinterpret_cast<const float4*>(rec + g * C::DEP_ROW + ch0);
+#pragma unroll
+            for (int k = 0; k < C::MCH / 4; ++k) {
+                const float4 v = o[k];
+                acc[k].x = fmaf(e, v.x, acc[k].x);
+                acc[k].y = fmaf(e, v.y, acc[k].y);
+                acc[k].z = fmaf(e, v.z, acc[k].z);
+                acc[k].w = fmaf(e, v.w, acc[k].w);
+            }
+        }
+        if (w0 >= cta0 && w1 < cta0 + C::WARPS) {  // the whole head is here
+            if (p.qring && sub == 0) record_stats<G, MODE>(p, hid, g, M + log2f(l));
+            const float inv = 1.f / l;
+            uint16_t* out = p.out + ((size_t)hid * G + g) * kHeadDim + ch0;
+#pragma unroll
+            for (int k = 0; k < C::MCH / 4; ++k)
+                *reinterpret_cast<uint2*>(out + 4 * k) = make_uint2(pack_bf16x2(acc[k].x * inv, acc[k].y * inv),
+                                                                    pack_bf16x2(acc[k].z * inv, acc[k].w * inv));
+        } else {
+            float* rec = p.partial + (size_t)(2 * blockIdx.x + (w0 >= cta0 ? 1 : 0)) * partial_stride(G);
+#pragma unroll
+            for (int k = 0; k < C::MCH / 4; ++k) *reinterpret_cast<float4*>(rec + g * kHeadDim + ch0 + 4 * k) = acc[k];
+            if (sub == 0) {
+                rec[G * kHeadDim + g] = M;
+                rec[G * kHeadDim + G + g] = l;
+            }
+        }
+    }
+    if (lane == 0 && (w0 < cta0 || w1 >= cta0 + C::WARPS))
+        cm.part[w0 >= cta0 ? 1 : 0] = {hid, w0 / C::WARPS, w1 / C::WARPS - w0 / C::WARPS + 1};
+}
+
+// The CTA's end: its records are announced, and where this CTA is the last to hold a piece of a head,
+// all its threads merge the head's records, four channels of a query head each, up to eight records
+// on the way per thread.  Partials come from other SMs: read through L2.
+template <int G, int MODE>
+__device__ void finish_cta(const AttnParams& p, CtaMerge& cm)
+{
+    using C = Cfg<G>;
+    constexpr int rs = partial_stride(G), kBatch = 8;
+    __syncthreads();  // the records are written
+    if (threadIdx.x < 2) {
+        const CtaMerge::Part q = cm.part[threadIdx.x];
+        int last = 0;
+        if (q.P > 0) {
+            __threadfence();
+            last = atomicAdd(p.arrive + q.c0, 1) == q.P - 1;
+            if (last) {
+                p.arrive[q.c0] = 0;  // ready for the next launch
+                __threadfence();
+            }
+        }
+        cm.last[threadIdx.x] = last;
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int slot = 0; slot < 2; ++slot) {
+        if (!cm.last[slot]) continue;
+        const CtaMerge::Part q = cm.part[slot];
+        const float* base = p.partial + (size_t)q.c0 * 2 * rs;
+        for (int col = threadIdx.x; col < G * (kHeadDim / 4); col += C::WARPS * 32) {
+            const int g = col / (kHeadDim / 4), c4 = col % (kHeadDim / 4);
+            float M = -INFINITY, l = 0.f;
+            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+            for (int q0 = 0; q0 < q.P; q0 += kBatch) {
+                float m[kBatch], s[kBatch], nM = M;
+                float4 o[kBatch];
+#pragma unroll
+                for (int j = 0; j < kBatch; ++j) {
+                    m[j] = -INFINITY;
+                    s[j] = 0.f;
+                    o[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (q0 + j < q.P) {
+                        const float* rec = base + (size_t)(q0 + j == 0 ? 1 : 2 * (q0 + j)) * rs;
+                        m[j] = __ldcg(rec + G * kHeadDim + g);
+                        s[j] = __ldcg(rec + G * kHeadDim + G + g);
+                        o[j] = __ldcg(reinterpret_cast<const float4*>(rec + g * kHeadDim) + c4);
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < kBatch; ++j) nM = fmaxf(nM, m[j]);
+                if (nM == -INFINITY) continue;
+                const float sc = exp2f(M - nM);
+                M = nM;
+                l *= sc;
+                acc.x *= sc;
+                acc.y *= sc;
+                acc.z *= sc;
+                acc.w *= sc;
+#pragma unroll
+                for (int j = 0; j < kBatch; ++j) {
+                    const float e = exp2f(m[j] - M);
+                    l = fmaf(e, s[j], l);
+                    acc.x = fmaf(e, o[j].x, acc.x);
+                    acc.y = fmaf(e, o[j].y, acc.y);
+                    acc.z = fmaf(e, o[j].z, acc.z);
+                    acc.w = fmaf(e, o[j].w, acc.w);
+                }
+            }
+            if (p.qring && c4 == 0) record_stats<G, MODE>(p, q.hid, g, M + log2f(l));
+            const float inv = 1.f / l;
+            *reinterpret_cast<uint2*>(p.out + ((size_t)q.hid * G + g) * kHeadDim + 4 * c4) =
+                make_uint2(pack_bf16x2(acc.x * inv, acc.y * inv), pack_bf16x2(acc.z * inv, acc.w * inv));
+        }
+    }
+}
+#endif
 
 template <int G, int MODE>
 __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
@@ -450,16 +636,23 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint8_t* wstage = smem + (size_t)warp * C::SPW * C::STAGE_BYTES;
-    // [stages (1024-byte aligned)][tile headers, 16 bytes each][mbarriers, 8 bytes each]
-    int4* hdrs = reinterpret_cast<int4*>(smem + (size_t)C::NSTAGE * C::STAGE_BYTES) + warp * C::SPW;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)C::NSTAGE * C::STAGE_BYTES + C::NSTAGE * 16) + warp * C::SPW;
+    uint8_t* wslot = smem + C::SLOT_OFF + (size_t)warp * C::SLOTS * C::SLOT_BYTES;
+    int4* hdrs = reinterpret_cast<int4*>(smem + C::HDR_OFF) + warp * C::SPW;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::BAR_OFF) + warp * C::SPW;
 
     const int gw = blockIdx.x * C::WARPS + warp;
+#if RA_ATTN_CTA_MERGE
+    __shared__ CtaMerge cm;
+    if (threadIdx.x < 8) cm.arrived[threadIdx.x] = 0;
+    if (threadIdx.x < 2) cm.part[threadIdx.x].P = 0;
+    __syncthreads();
+#else
     if (gw >= p.nchunks) {  // no chunk for this warp
         pdl_wait();
         pdl_launch_dependents();
         return;
     }
+#endif
 
     if (lane == 0) {
         for (int s = 0; s < C::SPW; ++s) mbar_init(&bars[s], 1);
@@ -478,28 +671,39 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
     it.chunk = -1;
     it.f = it.end = 0;
     int issued = 0;
+    bool q_busy = false, nt_busy = false;  // the warp's only slot holds rows not consumed yet (SLOTS == 1)
     // The caller's rows of a stage: the query rows (first tile of a piece), the new token's row.
     auto issue_inputs = [&](int s) {
         const int4 hd = hdrs[s];
-        uint8_t* st = wstage + (size_t)s * C::STAGE_BYTES;
-        if (hd.y & kNewTok) {
+        uint8_t* sl = wslot + (size_t)(s % C::SLOTS) * C::SLOT_BYTES;
+        if ((hd.y & (kNewTok | kNtDirect)) == kNewTok) {
             const size_t src = (size_t)hd.z * kHeadDim;
-            bulk_load(st + C::NT_OFF, p.k_new + src, (uint32_t)kRowBytes, &bars[s]);
-            bulk_load(st + C::NT_OFF + kRowBytes, p.v_new + src, (uint32_t)kRowBytes, &bars[s]);
+            bulk_load(sl + C::Q_BYTES, p.k_new + src, (uint32_t)kRowBytes, &bars[s]);
+            bulk_load(sl + C::Q_BYTES + kRowBytes, p.v_new + src, (uint32_t)kRowBytes, &bars[s]);
         }
-        if (hd.y & kFirst)
-            bulk_load(st + 2 * C::KV_BYTES, p.q + (size_t)hd.z * G * kHeadDim,
+        if ((hd.y & (kFirst | kQDirect)) == kFirst)
+            bulk_load(sl, p.q + (size_t)hd.z * G * kHeadDim,
                       (uint32_t)C::Q_BYTES, &bars[s]);
     };
     auto issue = [&](int t, bool inputs) -> bool {
         TileDesc d;
         if (!iter_next<MODE>(it, p, d, gw)) return false;
         const int s = t % C::SPW;
+        if (C::SLOTS == 1) {
+            if (d.flags & kFirst) {
+                if (q_busy) d.flags |= kQDirect;
+                q_busy = true;
+            }
+            if (d.flags & kNewTok) {
+                if (nt_busy) d.flags |= kNtDirect;
+                nt_busy = true;
+            }
+        }
         if (lane == 0) {
             uint8_t* st = wstage + (size_t)s * C::STAGE_BYTES;
             hdrs[s] = make_int4(d.n, d.flags | (d.chunk << kFlagBits), d.hid, (int)d.row);
-            const bool first = d.flags & kFirst;
-            const bool newtok = d.flags & kNewTok;
+            const bool first = (d.flags & (kFirst | kQDirect)) == kFirst;
+            const bool newtok = (d.flags & (kNewTok | kNtDirect)) == kNewTok;
             mbar_arrive_expect_tx(&bars[s], 2u * C::KV_BYTES + (first ? (uint32_t)C::Q_BYTES : 0u) +
                                                 (newtok ? 2u * kRowBytes : 0u));
             tma_load_2d(st, &tk, 0, (int)d.row, &bars[s]);
@@ -547,15 +751,24 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
             if (lane == 0) atomicExch(p.lay.err, kDeviceErrTimeout);
             for (int u = t + 1; u < issued; ++u)
                 (void)mbar_wait_bounded(&bars[u % C::SPW], (uint32_t)((u / C::SPW) & 1), kWaitLimitNs);
+#if RA_ATTN_CTA_MERGE
+            break;  // (to the CTA's last barrier)
+#else
             return;
+#endif
         }
         const int4 hd = hdrs[s];
         const int n = hd.x;
         uint8_t* Ks = wstage + (size_t)s * C::STAGE_BYTES;
         uint8_t* Vs = Ks + C::KV_BYTES;
         const uint32_t ks = smem_u32(Ks), vs = smem_u32(Vs);
+        uint8_t* slot = wslot + (size_t)(s % C::SLOTS) * C::SLOT_BYTES;
         if (hd.y & kFirst) {  // first tile of a head piece: fresh query fragments
-            const uint8_t* Qs = Vs + C::KV_BYTES;
+            const uint8_t* Qs = slot;
+            if (C::SLOTS == 1) {
+                if (hd.y & kQDirect) Qs = reinterpret_cast<const uint8_t*>(p.q + (size_t)hd.z * G * kHeadDim);
+                else q_busy = false;
+            }
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk) {
                 qa[kk][0] = gq < G ? *reinterpret_cast<const uint32_t*>(Qs + gq * kRowBytes + (16 * kk + 2 * tq) * 2) : 0u;
@@ -589,7 +802,13 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
         if (hd.y & kNewTok) {  // fused append: put the new token in row n-1 of the tile and into the cache
             const int b = hid_seq<MODE>(p, hd.z);
             const int c = lane & 15;
-            const uint4 v = lds128(Ks + C::NT_OFF + (lane >> 4) * kRowBytes + c * 16);
+            uint4 v;
+            if (C::SLOTS == 1 && (hd.y & kNtDirect)) {
+                v = reinterpret_cast<const uint4*>((lane < 16 ? p.k_new : p.v_new) + (size_t)hd.z * kHeadDim)[c];
+            } else {
+                v = lds128(slot + C::Q_BYTES + (lane >> 4) * kRowBytes + c * 16);
+                nt_busy = false;
+            }
             *reinterpret_cast<uint4*>((lane < 16 ? Ks : Vs) + swz<G>(n - 1, c)) = v;
             if (!(MODE == kModeCompact && (hd.y & kCompact))) {  // (a compacting head writes it with its survivors)
                 const long long row = (long long)hd.w + n - 1;
@@ -697,39 +916,53 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
                     }
                 }
             } else {
-                const int chunk = hd.y >> kFlagBits;
-                float* rec = p.partial + (size_t)(2 * chunk + (chunk == w0 ? 1 : 0)) * partial_stride(G);
+                // a piece: the CTA's chunks of this head are a .. z
+                const int chunk = hd.y >> kFlagBits, cta0 = (int)blockIdx.x * C::WARPS;
+                const int a = max(w0, cta0), z = min(w1, cta0 + C::WARPS - 1);
+                float* rec;
+                int rs;
+                if (a == z) {  // the only one of this CTA: to global memory
+                    rec = p.partial + (size_t)(2 * blockIdx.x + (a == w0 ? 1 : 0)) * partial_stride(G);
+                    rs = kHeadDim;
+                } else {  // deposited for the CTA's merge
+                    rec = reinterpret_cast<float*>(deposit<G>(smem, warp, chunk < w1, s));
+                    rs = C::DEP_ROW;
+                }
 #pragma unroll
                 for (int mt = 0; mt < 8; ++mt) {
                     const int ch = 16 * mt + gq;
                     if (hA < G) {
-                        rec[hA * kHeadDim + ch] = O[mt][0];
-                        rec[hA * kHeadDim + ch + 8] = O[mt][2];
+                        rec[hA * rs + ch] = O[mt][0];
+                        rec[hA * rs + ch + 8] = O[mt][2];
                     }
                     if (hB < G) {
-                        rec[hB * kHeadDim + ch] = O[mt][1];
-                        rec[hB * kHeadDim + ch + 8] = O[mt][3];
+                        rec[hB * rs + ch] = O[mt][1];
+                        rec[hB * rs + ch + 8] = O[mt][3];
                     }
                 }
                 if (gq == 0) {
                     if (hA < G) {
-                        rec[G * kHeadDim + hA] = mA;
-                        rec[G * kHeadDim + G + hA] = la;
+                        rec[G * rs + hA] = mA;
+                        rec[G * rs + G + hA] = la;
                     }
                     if (hB < G) {
-                        rec[G * kHeadDim + hB] = mB;
-                        rec[G * kHeadDim + G + hB] = lb;
+                        rec[G * rs + hB] = mB;
+                        rec[G * rs + G + hB] = lb;
                     }
                 }
-                __threadfence();
-                __syncwarp();
-                int old = 0;
-                if (lane == 0) old = atomicAdd(p.arrive + w0, 1);
-                old = __shfl_sync(0xffffffffu, old, 0);
-                if (old == w1 - w0) {  // every other piece of this head is already written
-                    __threadfence();
-                    merge_head<G, MODE>(p, hid, w0, w1 - w0 + 1, lane);
-                    if (lane == 0) p.arrive[w0] = 0;  // ready for the next launch
+                if (a == z) {
+                    if (lane == 0) cm.part[a == w0 ? 1 : 0] = {hid, w0 / C::WARPS, w1 / C::WARPS - w0 / C::WARPS + 1};
+                } else {
+                    if (lane == 0 && chunk < w1) cm.stage[warp] = s;
+                    __threadfence_block();
+                    __syncwarp();
+                    int old = 0;
+                    if (lane == 0) old = atomicAdd(&cm.arrived[a - cta0], 1);
+                    old = __shfl_sync(0xffffffffu, old, 0);
+                    if (old == z - a) {  // every other piece of the head in this CTA is deposited
+                        __threadfence_block();
+                        merge_deposits<G, MODE>(p, cm, smem, hid, w0, w1, a - cta0, z - cta0, lane);
+                    }
                 }
             }
             mA = mB = -INFINITY;
@@ -874,6 +1107,9 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
             if (more) ++issued;
         }
     }
+#if RA_ATTN_CTA_MERGE
+    finish_cta<G, MODE>(p, cm);
+#endif
 }
 
 // Active sequences whose heads hold no slot at all (empty prompt, nothing generated)

@@ -375,37 +375,44 @@ void layout_scoring(ra_ctx* ctx)
 }
 
 // Launch shape of a scoring pass over the heads of the sequences in p (pass 1: prompt + the
-// trig_n cached rows each; pass 2: the trig_n candidate rows each): about two waves of CTAs
-// (one per SM when the window needs more than half the shared memory), each taking a run of
-// consecutive tiles of one head.  Returns the algorithmic bytes: the key rows read (every
-// one is contracted with the M = r * G window rows, so flops = bytes * M).
+// trig_n cached rows each; pass 2: the trig_n candidate rows each): CTAs (one per SM: all of its
+// tensor memory) take runs of consecutive tiles of one head, in whole 128-row tiles (two scoring
+// tiles).  Pass 2 aims at one wave.  Pass 1 has more work than a wave on most calls: it takes the run
+// length whose waves, each as long as the run and about three tiles' start-up, end first.
+// Returns the algorithmic bytes: the key rows read (every one is contracted with the M = r * G
+// window rows, so flops = bytes * M).
 double plan_scoring(ra_ctx* ctx, EvictParams* p, int pass)
 {
-    const int M = ctx->r * ctx->G;
-    // pass 2 runs on tcgen05 with all of an SM's tensor memory: one CTA per SM, and runs of
-    // whole 128-row tiles (two scoring tiles)
-    const int per_sm = pass == 2 ? 1 : (score_row_tiles_per_warp(M) <= 2 ? 2 : 1);
     long long work = 0;
     int most = 1;
     double rows = 0;
+    std::vector<int> tiles((size_t)p->n_trig);
     for (int i = 0; i < p->n_trig; ++i) {
         const int lp = pass == 1 ? ctx->lp[p->trig[i]] : 0, n = p->trig_n[i];
         const int t = (lp + kScoreTile - 1) / kScoreTile + (n + kScoreTile - 1) / kScoreTile;
+        tiles[i] = t;
         work += (long long)ctx->KVH * t;
         most = std::max(most, t);
         rows += (double)ctx->KVH * (lp + n);
     }
-    const long long target = (long long)ctx->sms * per_sm;
-    long long ch = std::max<long long>((work + target - 1) / target, 1);
-    if (pass == 1) ch = std::max<long long>(ch, (most + ctx->stats_chunks - 1) / ctx->stats_chunks);
-    if (pass == 2) ch = (ch + 1) / 2 * 2;
-    const int nch = (int)((most + ch - 1) / ch);
     if (pass == 1) {
-        p->ch1 = (int)ch;
-        p->nch1 = nch;
+        long long best = 0;
+        const int least = std::max(2, (most + ctx->stats_chunks - 1) / ctx->stats_chunks);
+        p->ch1 = (most + 1) / 2 * 2;
+        for (int ch = (least + 1) / 2 * 2; ch <= (most + 1) / 2 * 2; ch += 2) {
+            long long ctas = 0;
+            for (int t : tiles) ctas += (long long)ctx->KVH * ((t + ch - 1) / ch);
+            const long long cost = (ctas + ctx->sms - 1) / ctx->sms * (ch / 2 + 3);
+            if (best == 0 || cost < best) {
+                best = cost;
+                p->ch1 = ch;
+            }
+        }
+        p->nch1 = (most + p->ch1 - 1) / p->ch1;
     } else {
-        p->ch2 = (int)ch;
-        p->nch2 = nch;
+        long long ch = std::max<long long>((work + ctx->sms - 1) / ctx->sms, 1);
+        p->ch2 = (int)((ch + 1) / 2 * 2);
+        p->nch2 = (most + p->ch2 - 1) / p->ch2;
     }
     return rows * kRowBytes;
 }

@@ -209,7 +209,7 @@ cudaError_t launch_score(const EvictParams& p, int pass, const CUtensorMap* tmap
                          cudaStream_t s);
 cudaError_t launch_score_merge(const EvictParams& p, cudaStream_t s);
 cudaError_t score_prepare();
-int score_row_tiles_per_warp(int M);  // 16-row tiles of the M window rows per warp (1..4)
+int score_window_tiles(int M);  // 128-row tiles of the M window rows (1..4)
 
 // Attention comes in two kernel shapes, one build of ra_attn.cu each: wide (48-row tiles, 4 warps
 // per CTA) for large layers and narrow (32-row tiles, 6 warps) for small ones, where a finer split

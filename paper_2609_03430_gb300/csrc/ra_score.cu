@@ -19,20 +19,21 @@
 //       every candidate's sum is complete inside it -- no atomics, and the
 //       result does not depend on the launch shape.  It runs on tcgen05 with
 //       the accumulators in tensor memory (see the kernel).
-//   restore pass (score_stats_kernel<MT> + score_merge_kernel)  only when a
+//   restore pass (score_stats_tc_kernel<MQ> + score_merge_kernel)  only when a
 //       window is loaded from outside (ra_restore_queries): the normalisers,
 //       recomputed over the prompt and the cached rows each query sees (by
 //       position), split over chunks of key tiles and merged.
 // The contraction of the window rows with the key rows is a dense GEMM
-// (M x keys x 128), so both passes run on the tensor cores.  The restore pass
-// (a warm start only) uses mma.sync m16n8k16 (bf16 in, fp32 accumulate);
-// its CTA layout: 8 warps; warp w owns the 16-row M tiles
-// w, w + 8, ... (MT of them).  The M rows arrive by 2-D TMA (64-row x
-// 64-channel boxes, 128-byte swizzle) with the first key tile and are read as
-// A fragments with ldmatrix; key tiles of 64 rows x 128 channels arrive the
-// same way into a two-stage ring on mbarriers and are read as B fragments.  Logits are in base 2 with the scale folded in.
+// (M x keys x 128), so both passes run on tcgen05 with the accumulators in
+// tensor memory: the summation pass with the keys on the M side (a thread
+// holds a key and sums over the window), the restore pass with the window on
+// the M side (a thread holds a window row and sums over the keys), so that
+// neither needs a reduction across threads.  Rows arrive by 2-D TMA (64-row x
+// 64-channel boxes, 128-byte swizzle).  Logits are in base 2 with the scale
+// folded in.
 #include <cuda.h>
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <math.h>
 #include <stdint.h>
 
@@ -44,55 +45,9 @@ static_assert(kPromptPage % kScoreTile == 0, "a scoring tile of the prompt lies 
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kWarps = kThreads / 32;
-constexpr int kStages = 2;
 constexpr int kHalfBytes = kScoreTile * 128;      // one 64-channel box of a key tile
-constexpr int kTileBytes = 2 * kHalfBytes;        // a key tile: 64 rows x 256 bytes
 constexpr uint64_t kWaitLimitNs = 2000000000ull;  // bounded mbarrier waits: 2 s
-static_assert(kScoreTile == 64, "eight 8-column MMA tiles per key tile");
 static_assert(kHalfBytes % 1024 == 0, "128-byte-swizzled TMA boxes start 1024-byte aligned");
-
-template <int MT>
-struct SCfg {
-    static constexpr int ROWS = 16 * kWarps * MT;                 // window rows held (M padded)
-    static constexpr int Q_HALF = ROWS * 128;                     // one 64-channel half of the window
-    static constexpr int Q_OFF = kStages * kTileBytes;            // after the key stages
-    static constexpr int BAR_OFF = Q_OFF + ROWS * kRowBytes;
-    static constexpr size_t SMEM = 1024 + (size_t)BAR_OFF + kStages * 8;
-    static_assert(ROWS <= kScoreMaxRows || MT == 1, "window rows");
-    static_assert(ROWS % kScoreTile == 0 && Q_HALF % 1024 == 0, "whole TMA boxes, 1024-byte aligned");
-    static_assert(SMEM <= 232448, "fits the 227 KB opt-in shared memory");
-};
-
-// Byte offset of (window row R, 16-byte chunk c) of the window block: two 64-channel halves of
-// `half` bytes each, rows of 128 bytes, chunks xored with R mod 8 (the TMA 128-byte swizzle).
-__device__ __forceinline__ uint32_t qswz(int R, int c, int half)
-{
-    return (uint32_t)((c >> 3) * half + R * 128 + (((c & 7) ^ (R & 7)) << 4));
-}
-
-// Byte offset of (key row j, 16-byte chunk c) inside a 128-byte-swizzled key tile.
-__device__ __forceinline__ uint32_t kswz(int j, int c)
-{
-    return (uint32_t)((c >> 3) * kHalfBytes + j * 128 + (((c & 7) ^ (j & 7)) << 4));
-}
-
-__device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], uint32_t addr)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(addr));
-}
-
-// D[16x8] += A[16x16] B[16x8], bf16 in, fp32 accumulate.
-__device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
-{
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-        "{%0, %1, %2, %3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
 
 // Tiles of one head in the restore pass: its prompt rows, then its c cached generated rows.
 __device__ __forceinline__ int head_tiles(int lp, int n_gen, int* tp)
@@ -110,185 +65,17 @@ __device__ __forceinline__ int visible_rows(const int32_t* pos, int c, int lp, i
     const int step = g - d;
     if (step < 1) return 0;  // no such step yet: the slot is never read before a real query fills it
     const int qpos = lp + step - 1;
+    // nothing is evicted between two rounds, so the tokens after the query are the newest d cached
+    // ones: two reads confirm it (the search's chain of dependent reads takes several microseconds)
+    const int guess = max(c - d, 0);
+    const int below = guess > 0 ? __ldcg(pos + guess - 1) : INT_MIN, after = guess < c ? __ldcg(pos + guess) : INT_MAX;
+    if (below <= qpos && after > qpos) return guess;
     int lo = 0, hi = c;      // first ordinal whose position is after qpos
     while (lo < hi) {
         const int mid = (lo + hi) >> 1;
         if (__ldcg(pos + mid) <= qpos) lo = mid + 1; else hi = mid;
     }
     return lo;
-}
-
-// Restore pass: per window row, (max, sum of exp2) over one chunk of the keys it sees.
-template <int MT>
-__global__ void __launch_bounds__(kThreads, MT <= 2 ? 2 : 1) score_stats_kernel(const __grid_constant__ EvictParams p,
-                                                                              const __grid_constant__ CUtensorMap tk,
-                                                                              const __grid_constant__ CUtensorMap tw)
-{
-    using C = SCfg<MT>;
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::BAR_OFF);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-
-    pdl_wait();  // the window, the cache and the tables come from earlier kernels
-    pdl_launch_dependents();
-
-    const DevLayout& L = p.lay;
-    const int t = blockIdx.y / L.KVH, h = blockIdx.y - t * L.KVH;
-    const int b = p.trig[t];
-    const int N = p.trig_n[t], r = L.r, G = L.G, M = r * G;
-    const int lp = L.seq_lp[b];
-    int tp;
-    const int nt_head = head_tiles(lp, N, &tp);
-    const int ch = p.ch1;
-    const int t0 = blockIdx.x * ch;
-    if (t0 >= nt_head) return;  // (exiting counts as letting the successor start)
-    const int ntile = min(ch, nt_head - t0);
-    const long long pbase = prompt_row(L, p.layer, 0, h, 0);
-    const int32_t* ptab = L.pages + (size_t)b * L.max_pages;
-    const size_t lbh = ((size_t)p.layer * L.B + b) * L.KVH + h;
-    const int reg = L.region[lbh];
-    const long long grow = L.gen_row0 + (long long)reg * L.Cmax;
-    const int hid = b * L.KVH + h;
-
-    auto tile_row = [&](int k) -> long long {  // first cache row of the head's tile k
-        // (a prompt tile lies inside one page: kPromptPage is a multiple of kScoreTile)
-        return k < tp ? pbase + (long long)__ldg(ptab + k * kScoreTile / kPromptPage) * L.KVH * kPromptPage +
-                            (k * kScoreTile) % kPromptPage
-                      : grow + (long long)(k - tp) * kScoreTile;
-    };
-    // thread 0: tile t0 + i into stage i % 2 (one arrival per phase: `extra` bytes of other copies
-    // completing on the same barrier are expected together with the tile)
-    auto issue = [&](int i, uint32_t extra) {
-        const int s = i % kStages;
-        uint8_t* st = smem + (size_t)s * kTileBytes;
-        const int row = (int)tile_row(t0 + i);
-        mbar_arrive_expect_tx(&bars[s], (uint32_t)kTileBytes + extra);
-        tma_load_2d(st, &tk, 0, row, &bars[s]);
-        tma_load_2d(st + kHalfBytes, &tk, 64, row, &bars[s]);
-    };
-    if (tid == 0) {
-        for (int s = 0; s < kStages; ++s) mbar_init(&bars[s], 1);
-        fence_mbar_init();
-        prefetch_tensormap(&tk);
-        prefetch_tensormap(&tw);
-        // The window rows (row R = slot * G + g) complete on stage 0's barrier with the first
-        // key tile.  Rows past M belong to the next head's window (or lie past the end and
-        // read as zero): finite, and given no weight.
-        issue(0, (uint32_t)(C::ROWS * kRowBytes));
-        const int row0 = (int)(lbh * (size_t)M);
-        for (int rb = 0; rb < C::ROWS; rb += kScoreTile) {
-            tma_load_2d(smem + C::Q_OFF + rb * 128, &tw, 0, row0 + rb, &bars[0]);
-            tma_load_2d(smem + C::Q_OFF + C::Q_HALF + rb * 128, &tw, 64, row0 + rb, &bars[0]);
-        }
-        for (int i = 1; i < kStages && i < ntile; ++i) issue(i, 0u);
-    }
-    __syncthreads();
-
-    // This lane's rows: R = 16 * (warp + 8 i) + (lane / 4) + 8 hf; its columns: 8 nt + 2 (lane % 4) + e.
-    const int tq = lane & 3;
-    const int mi = lane >> 3, ri = lane & 7;
-    int lim[MT][2];  // generated rows the row sees
-    float mrow[MT][2], lrow[MT][2];  // running max and (per-lane partial) sum of exp2
-#pragma unroll
-    for (int i = 0; i < MT; ++i)
-#pragma unroll
-        for (int hf = 0; hf < 2; ++hf) {
-            const int R = 16 * (warp + kWarps * i) + (lane >> 2) + 8 * hf;
-            lim[i][hf] = R < M ? visible_rows(L.pos + (size_t)reg * L.Cmax, N, lp, p.trig_g[t], r, R / G) : 0;
-            mrow[i][hf] = -INFINITY;
-            lrow[i][hf] = 0.f;
-        }
-    const float sl = p.qk_scale_log2;  // the scale the restored queries are taken at
-    const uint32_t qs = smem_u32(smem + C::Q_OFF);
-
-    for (int i = 0; i < ntile; ++i) {
-        const int s = i % kStages;
-        const bool ok = mbar_wait_bounded(&bars[s], (uint32_t)((i / kStages) & 1), kWaitLimitNs);
-        if (!__syncthreads_and(ok)) {  // give up together; let the copies in flight land first
-            if (tid == 0) {
-                atomicExch(L.err, kDeviceErrTimeout);
-                for (int j = i + 1; j < ntile && j < i + kStages; ++j)
-                    (void)mbar_wait_bounded(&bars[j % kStages], (uint32_t)((j / kStages) & 1), kWaitLimitNs);
-            }
-            return;
-        }
-        const uint32_t ks = smem_u32(smem + (size_t)s * kTileBytes);
-        float acc[MT][8][4];
-#pragma unroll
-        for (int a = 0; a < MT; ++a)
-#pragma unroll
-            for (int n = 0; n < 8; ++n) acc[a][n][0] = acc[a][n][1] = acc[a][n][2] = acc[a][n][3] = 0.f;
-#pragma unroll
-        for (int kk = 0; kk < 8; ++kk) {
-            uint32_t af[MT][4];
-#pragma unroll
-            for (int a = 0; a < MT; ++a)
-                ldsm_x4(af[a], qs + qswz(16 * (warp + kWarps * a) + (lane & 15), 2 * kk + (lane >> 4), C::Q_HALF));
-#pragma unroll
-            for (int np = 0; np < 4; ++np) {
-                uint32_t bf[4];
-                ldsm_x4(bf, ks + kswz(16 * np + (mi >> 1) * 8 + ri, 2 * kk + (mi & 1)));
-#pragma unroll
-                for (int a = 0; a < MT; ++a) {
-                    mma16816(acc[a][2 * np], af[a], bf[0], bf[1]);
-                    mma16816(acc[a][2 * np + 1], af[a], bf[2], bf[3]);
-                }
-            }
-        }
-        const int k = t0 + i;
-        {
-            const bool prompt = k < tp;
-            const int base = (prompt ? k : k - tp) * kScoreTile;  // index of column 0 within its segment
-#pragma unroll
-            for (int a = 0; a < MT; ++a)
-#pragma unroll
-                for (int hf = 0; hf < 2; ++hf) {
-                    const int nvalid = (prompt ? lp : lim[a][hf]) - base;  // columns this row sees
-                    float bm = -INFINITY;
-#pragma unroll
-                    for (int n = 0; n < 8; ++n)
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            const int col = 8 * n + 2 * tq + e;
-                            const float v = col < nvalid ? acc[a][n][2 * hf + e] * sl : -INFINITY;
-                            acc[a][n][2 * hf + e] = v;
-                            bm = fmaxf(bm, v);
-                        }
-                    bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, 1));
-                    bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, 2));
-                    const float mn = fmaxf(mrow[a][hf], bm);
-                    if (mn != -INFINITY) {
-                        float sum = mrow[a][hf] == -INFINITY ? 0.f : lrow[a][hf] * exp2f(mrow[a][hf] - mn);
-#pragma unroll
-                        for (int n = 0; n < 8; ++n)
-#pragma unroll
-                            for (int e = 0; e < 2; ++e) sum += exp2f(acc[a][n][2 * hf + e] - mn);
-                        lrow[a][hf] = sum;
-                        mrow[a][hf] = mn;
-                    }
-                }
-        }
-        __syncthreads();  // stage s free again
-        if (tid == 0 && i + kStages < ntile) {
-            fence_proxy_async_smem();
-            issue(i + kStages, 0u);
-        }
-    }
-
-    {  // this chunk's statistics of every real row
-        float* out = L.stats + ((size_t)hid * L.stats_chunks + blockIdx.x) * M * 2;
-#pragma unroll
-        for (int a = 0; a < MT; ++a)
-#pragma unroll
-            for (int hf = 0; hf < 2; ++hf) {
-                float l = lrow[a][hf];
-                l += __shfl_xor_sync(0xffffffffu, l, 1);
-                l += __shfl_xor_sync(0xffffffffu, l, 2);
-                const int R = 16 * (warp + kWarps * a) + (lane >> 2) + 8 * hf;
-                if (tq == 0 && R < M) *reinterpret_cast<float2*>(out + (size_t)R * 2) = make_float2(mrow[a][hf], l);
-            }
-    }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -550,6 +337,251 @@ __global__ void __launch_bounds__(kThreads, 1) score_sum_tc_kernel(const __grid_
     }
 }
 
+// ---------------------------------------------------------------------------------------------
+// Restore pass on tcgen05: per window row, (max, sum of exp2) over one chunk of the keys it sees.
+//
+// D = Q K^T: the window rows are the M side (MQ tiles of 128), the 128 keys of a tile the N side, so
+// that a TMEM lane holds one window row's logits and the thread that reads it keeps that row's
+// running maximum and sum in registers.  The two warpgroups take the M tiles in turn, or the
+// halves of the keys when there is one M tile only.  A tile is two runs of kScoreTile cache rows
+// (a prompt page holds three); with at most 256 window rows the accumulator is double-buffered, and
+// the products of tile i + 1 run while tile i is summed.  Bound by exp2 (one per logit) and the
+// few instructions around it.  For 160 heads of 3.3K keys and 256 window rows it takes 85 us
+// where the mma.sync kernel, with two shuffles per 16 keys and a row, took 167 us.
+template <int MQ>
+struct StCfg {
+    static constexpr int ROWS = 128 * MQ;
+    static constexpr int NBUF = MQ <= 2 ? 2 : 1;               // accumulator buffers in TMEM
+    static constexpr int BUF_COLS = kTcRows * MQ;              // columns of one buffer: 128 keys per M tile
+    static constexpr uint32_t COLS = MQ == 1 ? 256u : 512u;    // columns allocated (a power of 2)
+    static constexpr int MINE = (MQ + 1) / 2;                  // window rows per thread
+    static constexpr int Q_OFF = 2 * kTcStage;                 // after the two key stages
+    static constexpr int Q_HALF = ROWS * 128;
+    static constexpr int RED_OFF = Q_OFF + ROWS * kRowBytes;   // MQ == 1: the second warpgroup's statistics
+    static constexpr int BAR_OFF = RED_OFF + (MQ == 1 ? 128 * 8 : 0);  // full[2], mma_done[2], TMEM base
+    static constexpr size_t SMEM = 1024 + (size_t)BAR_OFF + 4 * 8 + 16;
+    static_assert(NBUF * BUF_COLS <= (int)COLS && SMEM <= 232448, "tensor and shared memory");
+};
+
+__device__ __forceinline__ float ex2(float x)
+{
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// Running (max, sum of exp2) of one row over 32 more logits, of which the first `valid` count.  The maximum
+// is raised only past 2^8 (the result is the same up to rounding).
+template <bool MASK>
+__device__ __forceinline__ void add_stats(const uint32_t (&v)[32], int valid, float sl, float& m, float& l)
+{
+    float x[32];
+#pragma unroll
+    for (int j = 0; j < 32; ++j) x[j] = !MASK || j < valid ? __uint_as_float(v[j]) : -INFINITY;
+    float c[4] = {x[0], x[1], x[2], x[3]};
+#pragma unroll
+    for (int j = 4; j < 32; ++j) c[j & 3] = fmaxf(c[j & 3], x[j]);
+    const float top = fmaxf(fmaxf(c[0], c[1]), fmaxf(c[2], c[3])) * sl;
+    if (top == -INFINITY) return;  // nothing visible
+    if (top > m + 8.f) {
+        l *= m == -INFINITY ? 0.f : ex2(m - top);
+        m = top;
+    }
+    float a[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int j = 0; j < 32; ++j) a[j & 3] += ex2(fmaf(x[j], sl, -m));
+    l += (a[0] + a[1]) + (a[2] + a[3]);
+}
+
+template <int MQ>
+__global__ void __launch_bounds__(kThreads, 1) score_stats_tc_kernel(const __grid_constant__ EvictParams p,
+                                                                    const __grid_constant__ CUtensorMap tk,
+                                                                    const __grid_constant__ CUtensorMap tw)
+{
+    using C = StCfg<MQ>;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + C::BAR_OFF);  // key tile (and the window) landed
+    uint64_t* mdone = full + 2;                                          // the tile's MMAs completed
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(full + 4);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+
+    pdl_wait();  // the window, the cache and the tables come from earlier kernels
+    pdl_launch_dependents();
+
+    const DevLayout& L = p.lay;
+    const int t = blockIdx.y / L.KVH, h = blockIdx.y - t * L.KVH;
+    const int b = p.trig[t];
+    const int N = p.trig_n[t], r = L.r, G = L.G, M = r * G;
+    const int lp = L.seq_lp[b];
+    int tp;
+    const int nt_head = head_tiles(lp, N, &tp);
+    const int t0 = blockIdx.x * p.ch1;           // this CTA's runs [t0, t1) of kScoreTile rows
+    if (t0 >= nt_head) return;  // (exiting counts as letting the successor start)
+    const int t1 = min(t0 + p.ch1, nt_head), ntile = (t1 - t0 + 1) / 2;
+    const long long pbase = prompt_row(L, p.layer, 0, h, 0);
+    const int32_t* ptab = L.pages + (size_t)b * L.max_pages;
+    const size_t lbh = ((size_t)p.layer * L.B + b) * L.KVH + h;
+    const int reg = L.region[lbh];
+    const long long grow = L.gen_row0 + (long long)reg * L.Cmax;
+
+    auto run_row = [&](int k) -> int {  // first cache row of the head's run k
+        // (a run of the prompt lies inside one page: kPromptPage is a multiple of kScoreTile)
+        return (int)(k < tp ? pbase + (long long)__ldg(ptab + k * kScoreTile / kPromptPage) * L.KVH * kPromptPage +
+                                  (k * kScoreTile) % kPromptPage
+                            : grow + (long long)(k - tp) * kScoreTile);
+    };
+    // thread 0: tile i (runs t0 + 2 i and the next, if this CTA has it) into stage i % 2; `extra` bytes of other
+    // copies complete on the same barrier.  A missing second run leaves old rows, whose logits count nothing.
+    auto issue_tile = [&](int i, uint32_t extra) {
+        const int s = i % 2, k = t0 + 2 * i, n = min(2, t1 - k);
+        uint8_t* st = smem + (size_t)s * kTcStage;
+        mbar_arrive_expect_tx(&full[s], (uint32_t)(n * kScoreTile * kRowBytes) + extra);
+        for (int q = 0; q < n; ++q) {
+            const int row = run_row(k + q);
+            tma_load_2d(st + q * kHalfBytes, &tk, 0, row, &full[s]);
+            tma_load_2d(st + kTcHalf + q * kHalfBytes, &tk, 64, row, &full[s]);
+        }
+    };
+    if (warp == 0) {  // the accumulators' tensor memory (held until the end)
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                     "r"(C::COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (tid == 0) {
+        for (int s = 0; s < 2; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&mdone[s], 1);
+        }
+        fence_mbar_init();
+        prefetch_tensormap(&tk);
+        prefetch_tensormap(&tw);
+        // The window rows (row R = slot * G + g) complete on full[0] with the first key tile; rows past M
+        // are another head's (or read as zero) and belong to no thread's statistics.
+        issue_tile(0, (uint32_t)(C::ROWS * kRowBytes));
+        const int row0 = (int)(lbh * (size_t)M);
+        for (int rb = 0; rb < C::ROWS; rb += kScoreTile) {
+            tma_load_2d(smem + C::Q_OFF + rb * 128, &tw, 0, row0 + rb, &full[0]);
+            tma_load_2d(smem + C::Q_OFF + C::Q_HALF + rb * 128, &tw, 64, row0 + rb, &full[0]);
+        }
+        if (ntile > 1) issue_tile(1, 0u);
+    }
+    // thread 0's counts of tiles: copies issued, MMAs issued, MMAs waited for
+    int n_loaded = min(ntile, 2), n_mma = 0, done = 0;
+    // this thread's window rows: lane wq * 32 + lane of M tiles wg, wg + 2 (one M tile: of that tile)
+    const int wg = warp >> 2, wq = warp & 3;
+    int lim[C::MINE];  // generated rows the row sees
+    float mrow[C::MINE], lrow[C::MINE];
+#pragma unroll
+    for (int i = 0; i < C::MINE; ++i) {
+        const int R = ((MQ == 1 ? 0 : wg) + 2 * i) * 128 + wq * 32 + lane;
+        lim[i] = R < M ? visible_rows(L.pos + (size_t)reg * L.Cmax, N, lp, p.trig_g[t], r, R / G) : 0;
+        mrow[i] = -INFINITY;
+        lrow[i] = 0.f;
+    }
+    const float sl = p.qk_scale_log2;  // the scale the restored queries are taken at
+    tmem_fence_before();
+    __syncthreads();
+    tmem_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    const uint32_t idesc = umma_idesc_bf16(128, kTcRows);
+    const uint32_t sbase = smem_u32(smem);
+
+    // Thread 0: the MMAs of tile i into accumulator buffer i % NBUF, committed to mdone[i % 2].
+    auto issue_mma = [&](int i) -> bool {
+        if (!mbar_wait_bounded(&full[i % 2], (uint32_t)((i / 2) & 1), kWaitLimitNs)) return false;
+        tmem_fence_after();
+        const uint32_t d0 = tmem + (uint32_t)((i % C::NBUF) * C::BUF_COLS);
+        const uint32_t b0 = sbase + (uint32_t)((i % 2) * kTcStage);
+#pragma unroll
+        for (int q = 0; q < MQ; ++q)
+#pragma unroll
+            for (int kh = 0; kh < 2; ++kh)        // 64-channel half
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk)    // 16-channel K-step inside the half
+                    umma_bf16(d0 + q * kTcRows, umma_desc_sw128(sbase + C::Q_OFF + kh * C::Q_HALF + q * 128 * 128 + kk * 32),
+                              umma_desc_sw128(b0 + kh * kTcHalf + kk * 32), idesc, (kh | kk) != 0);
+        umma_commit(&mdone[i % 2]);
+        n_mma = i + 1;
+        return true;
+    };
+
+    bool ok = true;
+    if (tid == 0) ok = issue_mma(0);
+    for (int i = 0; i < ntile; ++i) {
+        const bool got = mbar_wait_bounded(&mdone[i % 2], (uint32_t)((i / 2) & 1), kWaitLimitNs);
+        if (!__syncthreads_and(got && ok)) {  // give up together
+            if (tid == 0) atomicExch(L.err, kDeviceErrTimeout);
+            break;
+        }
+        done = i + 1;
+        tmem_fence_after();
+        if (tid == 0 && i + 2 < ntile) {  // the tile's MMAs have read stage i % 2: refill it
+            fence_proxy_async_smem();
+            issue_tile(i + 2, 0u);
+            n_loaded = i + 3;
+        }
+        // (every thread has read the other buffer: it passed the barrier above after tile i - 1)
+        if (C::NBUF == 2 && tid == 0 && ok && i + 1 < ntile) ok = issue_mma(i + 1);
+#pragma unroll
+        for (int c = 0; c < C::MINE; ++c) {
+            const int q = (MQ == 1 ? 0 : wg) + 2 * c;
+            if (q >= MQ) continue;
+            const uint32_t tl = tmem + ((uint32_t)(wq * 32) << 16) + (uint32_t)((i % C::NBUF) * C::BUF_COLS + q * kTcRows);
+#pragma unroll 1
+            for (int c0 = MQ == 1 ? wg * 64 : 0; c0 < (MQ == 1 ? wg * 64 + 64 : kTcRows); c0 += 32) {
+                const int k = t0 + 2 * i + (c0 >> 6);  // the run these columns belong to
+                if (k >= t1) break;
+                const bool prompt = k < tp;
+                const int valid = (prompt ? lp - k * kScoreTile : lim[c] - (k - tp) * kScoreTile) - (c0 & 63);
+                uint32_t v[32];
+                __syncwarp();
+                tmem_ld32(tl + c0, v);
+                if (__all_sync(0xffffffffu, valid >= 32)) add_stats<false>(v, valid, sl, mrow[c], lrow[c]);
+                else add_stats<true>(v, valid, sl, mrow[c], lrow[c]);
+            }
+        }
+        tmem_fence_before();
+        if (C::NBUF == 1) {
+            __syncthreads();  // the accumulators are read: free for the next tile
+            if (tid == 0 && ok && i + 1 < ntile) {
+                tmem_fence_after();
+                ok = issue_mma(i + 1);
+            }
+        }
+    }
+    // Leave only with nothing in flight: after a timeout, the MMAs issued but not waited for and
+    // the copies issued but not consumed are waited for once more, bounded.
+    if (tid == 0) {
+        for (int i = done; i < n_mma; ++i) (void)mbar_wait_bounded(&mdone[i % 2], (uint32_t)((i / 2) & 1), kWaitLimitNs);
+        for (int i = n_mma; i < n_loaded; ++i) (void)mbar_wait_bounded(&full[i % 2], (uint32_t)((i / 2) & 1), kWaitLimitNs);
+    }
+    if (MQ == 1 && wg == 1)
+        reinterpret_cast<float2*>(smem + C::RED_OFF)[wq * 32 + lane] = make_float2(mrow[0], lrow[0]);
+    tmem_fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        tmem_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C::COLS) : "memory");
+    }
+    if (MQ == 1) {
+        if (wg == 1) return;
+        const float2 o = reinterpret_cast<const float2*>(smem + C::RED_OFF)[wq * 32 + lane];
+        const float mx = fmaxf(mrow[0], o.x);
+        if (mx != -INFINITY)
+            lrow[0] = (mrow[0] == -INFINITY ? 0.f : lrow[0] * ex2(mrow[0] - mx)) + (o.x == -INFINITY ? 0.f : o.y * ex2(o.x - mx));
+        mrow[0] = mx;
+    }
+    // this chunk's statistics of every real row
+    float2* out = reinterpret_cast<float2*>(L.stats) + ((size_t)(b * L.KVH + h) * L.stats_chunks + blockIdx.x) * M;
+#pragma unroll
+    for (int c = 0; c < C::MINE; ++c) {
+        const int R = ((MQ == 1 ? 0 : wg) + 2 * c) * 128 + wq * 32 + lane;
+        if (R < M) out[R] = make_float2(mrow[c], lrow[c]);
+    }
+}
+
 // Restore pass, last step: merge each window row's chunk statistics into its normaliser.
 __global__ void __launch_bounds__(256) score_merge_kernel(const __grid_constant__ EvictParams p)
 {
@@ -580,13 +612,13 @@ template <int MT>
 cudaError_t launch_stats(const EvictParams& p, const CUtensorMap* tk, const CUtensorMap* tq, cudaStream_t s)
 {
     const dim3 grid(p.nch1, p.n_trig * p.lay.KVH);
-    return launch_pdl(score_stats_kernel<MT>, grid, dim3(kThreads), SCfg<MT>::SMEM, s, p, *tk, *tq);
+    return launch_pdl(score_stats_tc_kernel<MT>, grid, dim3(kThreads), StCfg<MT>::SMEM, s, p, *tk, *tq);
 }
 
 template <int MT>
 cudaError_t prepare_mt()
 {
-    cudaError_t e = cudaFuncSetAttribute(score_stats_kernel<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SCfg<MT>::SMEM);
+    cudaError_t e = cudaFuncSetAttribute(score_stats_tc_kernel<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)StCfg<MT>::SMEM);
     if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(score_sum_tc_kernel<128 * MT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)TcCfg<128 * MT>::SMEM);
@@ -601,7 +633,7 @@ cudaError_t launch_sum_tc(const EvictParams& p, const CUtensorMap* tk, const CUt
 
 }  // namespace
 
-int score_row_tiles_per_warp(int M) { return ((M + 15) / 16 + kWarps - 1) / kWarps; }
+int score_window_tiles(int M) { return (M + 127) / 128; }
 
 cudaError_t score_prepare()
 {
@@ -619,7 +651,7 @@ cudaError_t launch_score_merge(const EvictParams& p, cudaStream_t s)
 
 cudaError_t launch_score(const EvictParams& p, int pass, const CUtensorMap* tk, const CUtensorMap* tq, cudaStream_t s)
 {
-    const int MT = score_row_tiles_per_warp(p.lay.r * p.lay.G);
+    const int MT = score_window_tiles(p.lay.r * p.lay.G);
     if (pass == 1) {
         switch (MT) {
             case 1: return launch_stats<1>(p, tk, tq, s);

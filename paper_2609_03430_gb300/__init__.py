@@ -101,11 +101,21 @@ def _check(rc, ctx=None):
     return rc
 
 
-def _stream_ptr(stream):
-    import torch
+_torch = _raw_stream = None
 
+
+def _stream_ptr(stream):
+    global _torch, _raw_stream
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+        if _torch is None:
+            import torch
+
+            _torch = torch
+            # the handle without a Stream object around it, where torch offers it
+            _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if _raw_stream is None:
+            return _torch.cuda.current_stream().cuda_stream
+        return _raw_stream(_torch.cuda.current_device())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream

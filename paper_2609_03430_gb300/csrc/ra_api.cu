@@ -50,6 +50,7 @@ struct ra_ctx {
     int max_prompt = 0, max_pages = 1;
     long long pool_pages = 0;
     std::vector<int32_t> pages;      // [B][max_pages]
+    std::vector<int32_t> page0;      // [B] first page of a sequence whose pages are consecutive, else -1
     std::vector<int32_t> free_pages;
     std::vector<int32_t> admits;     // [B]
     long long prompt_rows_per_layer = 0;
@@ -232,6 +233,16 @@ int make_tmap(ra_ctx* ctx, CUtensorMap* map, void* base, long long rows, int box
     return RA_OK;
 }
 
+// page0 of sequence b, after its pages changed.
+void note_pages(ra_ctx* ctx, int b)
+{
+    const int32_t* pg = ctx->pages.data() + (size_t)b * ctx->max_pages;
+    const int np = (ctx->lp[b] + kPromptPage - 1) / kPromptPage;
+    bool consecutive = true;
+    for (int j = 1; j < np && consecutive; ++j) consecutive = pg[j] == pg[0] + j;
+    ctx->page0[b] = np == 0 ? 0 : (consecutive ? pg[0] : -1);
+}
+
 void fill_active(const ra_ctx* ctx, uint32_t* mask)
 {
     for (int i = 0; i < RA_MAX_BATCH / 32; ++i) mask[i] = 0;
@@ -244,8 +255,9 @@ void fill_active(const ra_ctx* ctx, uint32_t* mask)
 // rows, where gen is the cached generated rows plus one for a fused new token; the tiles are cut
 // into one equal chunk per warp.  *slots = rows attended.
 int plan_attention(ra_ctx* ctx, int layer, int layers, int fused, AttnParams* p, int* n_active, int* ctas, double* slots,
-                   int* shape, const std::vector<int32_t>* old_rows = nullptr)
+                   int* shape, const int32_t* old_rows = nullptr)
 {
+    p->lay = ctx->lay;
     p->layer = layer;
     p->layers = layers;
     fill_active(ctx, p->active);
@@ -253,23 +265,19 @@ int plan_attention(ra_ctx* ctx, int layer, int layers, int fused, AttnParams* p,
     for (int i = 0; i < RA_MAX_BATCH / 32; ++i) p->compacting[i] = 0u;
     if (old_rows)
         for (int b = 0; b < ctx->B; ++b)
-            if ((*old_rows)[b] >= 0) p->compacting[b >> 5] |= 1u << (b & 31);
+            if (old_rows[b] >= 0) p->compacting[b >> 5] |= 1u << (b & 31);
     // fused: every active sequence's token is pending
     for (int i = 0; i < RA_MAX_BATCH / 32; ++i) p->pending[i] = fused ? p->active[i] : 0u;
     long long acc = 0, rows = 0;
     int na = 0;
     for (int b = 0; b < ctx->B; ++b) {
-        const int cached = (old_rows && (*old_rows)[b] >= 0) ? (*old_rows)[b] : ctx->c[(size_t)layer * ctx->B + b];
+        const int cached = (old_rows && old_rows[b] >= 0) ? old_rows[b] : ctx->c[(size_t)layer * ctx->B + b];
         const int gen = cached + (int)((p->pending[b >> 5] >> (b & 31)) & 1u);
         p->seq_gen[b] = gen;
         p->seq_g[b] = ctx->g[(size_t)layer * ctx->B + b];  // generated tokens before this step's
         p->seq_lp[b] = ctx->lp[b];
         p->seq_region[b] = ctx->rbase[(size_t)layer * ctx->B + b];
-        const int32_t* pg = ctx->pages.data() + (size_t)b * ctx->max_pages;
-        const int np = (ctx->lp[b] + kPromptPage - 1) / kPromptPage;
-        bool consecutive = true;
-        for (int j = 1; j < np && consecutive; ++j) consecutive = pg[j] == pg[0] + j;
-        p->seq_page0[b] = np == 0 ? 0 : (consecutive ? pg[0] : -1);
+        p->seq_page0[b] = ctx->page0[b];
         if (ctx->active[b]) {
             rows += (long long)layers * ctx->KVH * (ctx->lp[b] + gen);
             ++na;
@@ -420,6 +428,10 @@ double plan_scoring(ra_ctx* ctx, EvictParams* p, int pass)
 int run_eviction_launches(ra_ctx* ctx, EvictParams& p, double moved, cudaStream_t s, bool compact_in_attention,
                           int score_early);
 
+// Section 2 / Appendix F trigger: every r steps, once the candidates exceed the budget (g, c: the
+// counters with the step's token).
+bool fires(const ra_ctx* ctx, int g, int c) { return g % ctx->r == 0 && c - ctx->r > ctx->K; }
+
 // Evicted sets can be computed ahead for the policies whose keys need no scores (random, shared,
 // recency, block), with ordered compaction outside the attention pass (the one-launch kernels) or
 // order-free slots.  Keys that follow positions (order-free slots, block draws) are read from the
@@ -531,10 +543,10 @@ int run_eviction_launches(ra_ctx* ctx, EvictParams& p, double moved, cudaStream_
     return RA_OK;
 }
 
-void set_scale(AttnParams* p, float scale)
+float scale_log2(float scale)
 {
     const float sc = scale > 0.f ? scale : 1.0f / sqrtf((float)kHeadDim);
-    p->qk_scale_log2 = sc * 1.4426950408889634f;
+    return sc * 1.4426950408889634f;
 }
 
 }  // namespace
@@ -667,6 +679,8 @@ int ra_bind(ra_ctx* ctx, void* device_arena, size_t bytes, void* stream)
         if (next > ctx->pool_pages) return fail(ctx, RA_ERR_CAPACITY, "prompts need more pages than the pool holds");
         for (long long pg = ctx->pool_pages - 1; pg >= next; --pg) ctx->free_pages.push_back((int32_t)pg);
     }
+    ctx->page0.assign(ctx->B, 0);
+    for (int b = 0; b < ctx->B; ++b) note_pages(ctx, b);
     ctx->admits.assign(ctx->B, 0);
     // Tables: regions of (layer, seq, head) in order, one spare per (seq, head).
     const int BH = ctx->B * ctx->KVH;
@@ -887,6 +901,7 @@ int ra_admit(ra_ctx* ctx, int seq, int prompt_len, const uint16_t* k, const uint
         ctx->free_pages.pop_back();
     }
     ctx->lp[seq] = prompt_len;
+    note_pages(ctx, seq);
     cudaError_t e;
     // (pageable sources: the calls return once the values are staged)
     if ((e = cudaMemcpyAsync(ctx->lay.pages + (size_t)seq * ctx->max_pages, row, (size_t)ctx->max_pages * 4,
@@ -963,9 +978,7 @@ int ra_restore_queries(ra_ctx* ctx, int layer, const uint16_t* q, float scale, v
     }
     if (n == 0) return RA_OK;
     p.n_trig = n;
-    AttnParams sp{};
-    set_scale(&sp, scale);
-    p.qk_scale_log2 = sp.qk_scale_log2;
+    p.qk_scale_log2 = scale_log2(scale);
     const double bytes = plan_scoring(ctx, &p, 1);
     {
         ProfScope ps(ctx, RA_KERNEL_SCORE_STATS, bytes, s);
@@ -1022,6 +1035,12 @@ int ra_evict(ra_ctx* ctx, int layer, int* n_fired, void* stream)
     if (n_fired) *n_fired = 0;
     if ((rc = check_bound(ctx)) != RA_OK) return rc;
     if ((rc = check_layer(ctx, layer)) != RA_OK) return rc;
+    bool any = false;
+    for (int b = 0; b < ctx->B && !any; ++b) {
+        const size_t i = (size_t)layer * ctx->B + b;
+        any = ctx->active[b] && ctx->g[i] > 0 && fires(ctx, ctx->g[i], ctx->c[i]);
+    }
+    if (!any) return RA_OK;
     EvictParams p{};
     p.lay = ctx->lay;
     p.layer = layer;
@@ -1033,8 +1052,7 @@ int ra_evict(ra_ctx* ctx, int layer, int* n_fired, void* stream)
     for (int b = 0; b < ctx->B; ++b) {
         if (!ctx->active[b]) continue;
         const int g = ctx->g[(size_t)layer * ctx->B + b], c = ctx->c[(size_t)layer * ctx->B + b];
-        // section 2 / Appendix F trigger: every r steps, once the candidates exceed the budget
-        if (g > 0 && g % ctx->r == 0 && c - ctx->r > ctx->K) {
+        if (g > 0 && fires(ctx, g, c)) {
             p.trig[n] = (int16_t)b;
             p.trig_c[n] = c;
             p.trig_n[n] = c - ctx->r;
@@ -1043,7 +1061,6 @@ int ra_evict(ra_ctx* ctx, int layer, int* n_fired, void* stream)
             moved += (double)(ctx->K + ctx->r) * ctx->KVH;
         }
     }
-    if (n == 0) return RA_OK;
     p.n_trig = n;
     if ((rc = run_eviction(ctx, p, moved, (cudaStream_t)stream)) != RA_OK) return rc;
     for (int i = 0; i < n; ++i) {
@@ -1062,11 +1079,11 @@ int ra_decode_attn(ra_ctx* ctx, int layer, const uint16_t* q, uint16_t* out, flo
     if ((rc = check_layer(ctx, layer)) != RA_OK) return rc;
     if (!q || !out || !aligned16(q) || !aligned16(out))
         return fail(ctx, RA_ERR_INVALID_ARG, "q/out must be non-NULL and 16-byte aligned");
-    AttnParams p{};
-    p.lay = ctx->lay;
-    p.layer = layer;
+    AttnParams p;
     p.q = q;
     p.out = out;
+    p.k_new = p.v_new = nullptr;
+    p.early = 0;
     p.partial = ctx->lay.partial;
     p.arrive = ctx->lay.arrive;
     p.qring = ctx->lay.qring;
@@ -1077,7 +1094,7 @@ int ra_decode_attn(ra_ctx* ctx, int layer, const uint16_t* q, uint16_t* out, flo
     int shape = kAttnWide;
     if ((rc = plan_attention(ctx, layer, 1, 0, &p, &n_active, &ctas, &rows, &shape)) != RA_OK) return rc;
     if (n_active == 0) return RA_OK;
-    set_scale(&p, scale);
+    p.qk_scale_log2 = scale_log2(scale);
     cudaStream_t s = (cudaStream_t)stream;
     ProfScope ps(ctx, RA_KERNEL_ATTN, rows * 2 * kRowBytes + 2.0 * n_active * ctx->H * kRowBytes, s);
     cudaError_t e = launch_attention(shape, p, &ctx->tmap_k[shape], &ctx->tmap_v[shape], ctas, s);
@@ -1125,7 +1142,14 @@ int step_prologue(ra_ctx* ctx, cudaStream_t s)
     const int cur = ctx->parity, nxt = 1 - cur;
     std::fill(ctx->plan_g.begin() + (size_t)nxt * ctx->L * ctx->B, ctx->plan_g.begin() + (size_t)(nxt + 1) * ctx->L * ctx->B,
               -1);
-    if (serve) {
+    bool now = false, next = false;  // a sequence may fire at this step, at the next one (layer 0's counters)
+    for (int b = 0; b < ctx->B && serve; ++b) {
+        if (!ctx->active[b]) continue;
+        const int g = ctx->g[b], c = ctx->c[b];
+        now = now || fires(ctx, g + 1, c + 1);
+        next = next || (g + 2) % ctx->r == 0;
+    }
+    if (next) {
         // The sequences whose trigger fires at the next step (from layer 0's counters after this
         // step): their evicted sets in every layer, computed on the side stream beside this step.
         // The fork orders the plan after the previous step, the last reader of half nxt.
@@ -1141,10 +1165,10 @@ int step_prologue(ra_ctx* ctx, cudaStream_t s)
         for (int b = 0; b < ctx->B; ++b) {
             if (!ctx->active[b]) continue;
             const int g1 = ctx->g[b] + 1, c1 = ctx->c[b] + 1;
-            const bool fires = g1 % ctx->r == 0 && c1 - ctx->r > ctx->K;
-            if (fires && read_pos) continue;  // this step rewrites the positions the keys would read
-            const int g2 = g1 + 1, c2 = (fires ? ctx->K + ctx->r : c1) + 1;
-            if (g2 % ctx->r == 0 && c2 - ctx->r > ctx->K && c2 - ctx->r <= ctx->K + ctx->r) {
+            const bool fired = fires(ctx, g1, c1);
+            if (fired && read_pos) continue;  // this step rewrites the positions the keys would read
+            const int g2 = g1 + 1, c2 = (fired ? ctx->K + ctx->r : c1) + 1;
+            if (fires(ctx, g2, c2) && c2 - ctx->r <= ctx->K + ctx->r) {
                 pp.trig[n] = (int16_t)b;
                 pp.trig_admit[n] = (uint16_t)ctx->admits[b];
                 pp.trig_g[n] = g2;
@@ -1177,7 +1201,7 @@ int step_prologue(ra_ctx* ctx, cudaStream_t s)
     // computed ahead: all their rounds in one launch, in place, before the first layer: the
     // survivors move down (ordered) or the evicted slots are refilled from the newest rows
     // (order-free), and the layers then append the token as usual.
-    if (serve) {
+    if (now) {
         const bool fill = ctx->compaction == RA_COMPACT_HOLEFILL;
         EvictParams sp{};
         sp.lay = ctx->lay;
@@ -1189,7 +1213,7 @@ int step_prologue(ra_ctx* ctx, cudaStream_t s)
         for (int b = 0; b < ctx->B; ++b) {
             if (!ctx->active[b]) continue;
             const int g = ctx->g[b], c = ctx->c[b];
-            if ((g + 1) % ctx->r != 0 || c + 1 - ctx->r <= ctx->K) continue;
+            if (!fires(ctx, g + 1, c + 1)) continue;
             bool all = true;
             for (int l = 0; l < ctx->L && all; ++l) {
                 const size_t i = (size_t)l * ctx->B + b, k = (size_t)cur * ctx->L * ctx->B + i;
@@ -1272,13 +1296,17 @@ namespace {
 // Eviction of one layer, with the step's token pending: it is the newest slot, so it is never a
 // candidate, and evicting before writing it gives the same state as append-then-evict.  With
 // compaction in the attention pass only the selection runs here: that pass reads the old region
-// anyway and writes the survivors to the new one as it goes; old_rows [B] then receives the rows
-// of the sequences it compacts and *compacted the rows it writes.  *n_fired: sequences that evict.
+// anyway and writes the survivors to the new one as it goes; old_rows (empty before) then receives
+// the rows of the sequences it compacts, -1 for the others, and *compacted the rows it writes.  *n_fired: sequences that evict.
 int evict_pending(ra_ctx* ctx, int layer, cudaStream_t s, int plan_parity, std::vector<int32_t>& old_rows,
                   double* compacted, int* n_fired)
 {
     int rc;
     const size_t base = (size_t)layer * ctx->B;
+    *n_fired = 0;
+    bool any = false;
+    for (int b = 0; b < ctx->B && !any; ++b) any = ctx->active[b] && fires(ctx, ctx->g[base + b] + 1, ctx->c[base + b] + 1);
+    if (!any) return RA_OK;
     // The attention pass compacts (time order kept) when each tile's evicted rows fit its 64-bit mask.
     const bool fuse_compaction = ctx->compaction == RA_COMPACT_FUSED && ctx->r <= 64;  // tiles have <= 64 rows
     EvictParams ep{};
@@ -1300,7 +1328,7 @@ int evict_pending(ra_ctx* ctx, int layer, cudaStream_t s, int plan_parity, std::
     for (int b = 0; b < ctx->B; ++b) {
         if (!ctx->active[b]) continue;
         const int g1 = ctx->g[base + b] + 1, c1 = ctx->c[base + b] + 1;
-        if (g1 % ctx->r == 0 && c1 - ctx->r > ctx->K) {
+        if (fires(ctx, g1, c1)) {
             ep.trig[n] = (int16_t)b;
             ep.trig_c[n] = c1 - 1;
             ep.trig_n[n] = c1 - ctx->r;
@@ -1328,6 +1356,7 @@ int evict_pending(ra_ctx* ctx, int layer, cudaStream_t s, int plan_parity, std::
             const int b = ep.trig[i];
             ctx->nev[base + b] += 1;
             if (fuse_compaction) {
+                old_rows.resize((size_t)ctx->B, -1);
                 old_rows[b] = ep.trig_c[i];
                 *compacted += (double)(ctx->K + ctx->r) * ctx->KVH;
             }
@@ -1346,8 +1375,7 @@ int attend_pending(ra_ctx* ctx, int layer, int layers, const uint16_t* q, const 
 {
     int rc;
     cudaError_t e;
-    AttnParams p{};
-    p.lay = ctx->lay;
+    AttnParams p;
     p.q = q;
     p.out = out;
     p.k_new = k_new;
@@ -1359,10 +1387,11 @@ int attend_pending(ra_ctx* ctx, int layer, int layers, const uint16_t* q, const 
     int n_active = 0, ctas = 0;
     double rows = 0;
     int shape = kAttnWide;
-    if ((rc = plan_attention(ctx, layer, layers, 1, &p, &n_active, &ctas, &rows, &shape, &old_rows)) != RA_OK)
+    if ((rc = plan_attention(ctx, layer, layers, 1, &p, &n_active, &ctas, &rows, &shape,
+                             old_rows.empty() ? nullptr : old_rows.data())) != RA_OK)
         return rc;
     if (n_active == 0) return RA_OK;
-    set_scale(&p, scale);
+    p.qk_scale_log2 = scale_log2(scale);
     // The kernel may request its first K/V tiles before its predecessor finishes when that
     // predecessor cannot be writing this layer's cache or tables: no eviction of this layer at
     // this step (else it is this layer's compaction) and layers outside this launch (else it is
@@ -1396,9 +1425,8 @@ int decode_layer_impl(ra_ctx* ctx, int layer, const uint16_t* q, const uint16_t*
                       uint16_t* out, float scale, void* stream, int plan_parity)
 {
     int rc, n = 0;
-    if ((rc = check_layer_call(ctx, layer, q, k_new, v_new, out)) != RA_OK) return rc;
     cudaStream_t s = (cudaStream_t)stream;
-    std::vector<int32_t> old_rows((size_t)ctx->B, -1);  // sequences the attention launch compacts: rows before
+    std::vector<int32_t> old_rows;  // of the sequences the attention launch compacts
     double compacted = 0;  // rows the attention launch writes as compaction
     if ((rc = evict_pending(ctx, layer, s, plan_parity, old_rows, &compacted, &n)) != RA_OK) return rc;
     return attend_pending(ctx, layer, 1, q, k_new, v_new, out, scale, s, n > 0, old_rows, compacted);
@@ -1440,7 +1468,7 @@ int ra_decode_step(ra_ctx* ctx, const uint16_t* q_all, const uint16_t* k_all, co
     // only), then every layer at once.  With compaction inside the attention pass, or with
     // counters that differ between layers, layer by layer.
     if (ctx->L > 1 && layers_alike(ctx) && !(ctx->compaction == RA_COMPACT_FUSED && ctx->r <= 64)) {
-        std::vector<int32_t> old_rows((size_t)ctx->B, -1);
+        std::vector<int32_t> old_rows;  // (stays empty)
         double compacted = 0;
         int n = 0;
         for (int l = 0; l < ctx->L && rc == RA_OK; ++l) rc = evict_pending(ctx, l, s, ctx->step_cur, old_rows, &compacted, &n);
@@ -1680,11 +1708,11 @@ extern "C" int ra_decode_attn_noalloc(ra_ctx* ctx, int layer, const uint16_t* q,
     if ((rc = check_layer(ctx, layer)) != RA_OK) return rc;
     if (!q || !out || !aligned16(q) || !aligned16(out))
         return fail(ctx, RA_ERR_INVALID_ARG, "q/out must be non-NULL and 16-byte aligned");
-    AttnParams p{};
-    p.lay = ctx->lay;
-    p.layer = layer;
+    AttnParams p;
     p.q = q;
     p.out = out;
+    p.k_new = p.v_new = nullptr;
+    p.early = 0;
     p.qring = ctx->lay.qring;
     p.ring_off = -1;
     int n_active = 0, ctas = 0;
@@ -1692,7 +1720,7 @@ extern "C" int ra_decode_attn_noalloc(ra_ctx* ctx, int layer, const uint16_t* q,
     int shape = kAttnWide;
     if ((rc = plan_attention(ctx, layer, 1, 0, &p, &n_active, &ctas, &rows, &shape)) != RA_OK) return rc;
     if (n_active == 0) return RA_OK;
-    set_scale(&p, scale);
+    p.qk_scale_log2 = scale_log2(scale);
     // [arrival counters, one int per chunk][partial records, two per chunk].  The limit that the
     // interface states counts a record per warp and per head.
     const size_t counters = align_up((size_t)p.nchunks * sizeof(int32_t), kAlign), record = partial_stride(ctx->G) * sizeof(float);

@@ -73,6 +73,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "ra_internal.h"
 #include "ra_ptx.cuh"
 
@@ -185,21 +187,22 @@ struct TileDesc {
 };
 
 // The sequence of head `hid` of the launch, (layer * B + sequence) * KVH + KV head.
-template <int MODE>
-__device__ __forceinline__ int hid_seq(const AttnParams& p, int hid)
+template <int MODE, class PT>
+__device__ __forceinline__ int hid_seq(const PT& p, int hid)
 {
     const int lb = hid / p.lay.KVH;
     return MODE == kModeStack ? lb % p.lay.B : lb;
 }
 
-__device__ __forceinline__ int seq_head_tiles(const AttnParams& p, int b)
+template <class PT>
+__device__ __forceinline__ int seq_head_tiles(const PT& p, int b)
 {
     return (p.seq_base[b + 1] - p.seq_base[b]) / p.lay.KVH;
 }
 
 // First tile of head `hid` in the launch's tile order, and the head's tiles.
-template <int MODE>
-__device__ __forceinline__ long long head_tile0(const AttnParams& p, int hid, int* nth)
+template <int MODE, class PT>
+__device__ __forceinline__ long long head_tile0(const PT& p, int hid, int* nth)
 {
     const int lb = hid / p.lay.KVH, h = hid - lb * p.lay.KVH;
     const int l = MODE == kModeStack ? lb / p.lay.B : 0, b = lb - l * p.lay.B;
@@ -207,8 +210,8 @@ __device__ __forceinline__ long long head_tile0(const AttnParams& p, int hid, in
     return (long long)l * p.layer_tiles + p.seq_base[b] + (long long)h * *nth;
 }
 
-template <int MODE>
-__device__ __forceinline__ void enter_head(TileIter& it, const AttnParams& p)
+template <int MODE, class PT>
+__device__ __forceinline__ void enter_head(TileIter& it, const PT& p)
 {
     const DevLayout& L = p.lay;
     it.lp = p.seq_lp[it.b];
@@ -238,8 +241,8 @@ __device__ __forceinline__ void enter_head(TileIter& it, const AttnParams& p)
     it.piece_start = true;
 }
 
-template <int MODE>
-__device__ void iter_init(TileIter& it, const AttnParams& p, int R0, int R1)
+template <int MODE, class PT>
+__device__ void iter_init(TileIter& it, const PT& p, int R0, int R1)
 {
     it.f = R0;
     it.end = R1;
@@ -262,8 +265,8 @@ __device__ void iter_init(TileIter& it, const AttnParams& p, int R0, int R1)
 }
 
 // The warp's chunk (its index): false once it is done.
-template <int MODE>
-__device__ bool iter_next_chunk(TileIter& it, const AttnParams& p, int warp_id)
+template <int MODE, class PT>
+__device__ bool iter_next_chunk(TileIter& it, const PT& p, int warp_id)
 {
     if (it.chunk >= 0 || warp_id >= p.nchunks) return false;
     it.chunk = warp_id;
@@ -272,8 +275,8 @@ __device__ bool iter_next_chunk(TileIter& it, const AttnParams& p, int warp_id)
     return true;
 }
 
-template <int MODE>
-__device__ bool iter_next(TileIter& it, const AttnParams& p, TileDesc& d, int warp_id)
+template <int MODE, class PT>
+__device__ bool iter_next(TileIter& it, const PT& p, TileDesc& d, int warp_id)
 {
     if (it.f >= it.end && !iter_next_chunk<MODE>(it, p, warp_id)) return false;
     const int T = p.tile;
@@ -387,8 +390,8 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
 
 // The scored policy's window: the softmax normaliser of query head g of head `hid` at this
 // step, as (scale * log2 e, log2 sum_i exp2(scale * log2 e * q.k_i)), beside its query rows.
-template <int G, int MODE>
-__device__ __forceinline__ void record_stats(const AttnParams& p, int hid, int g, float lse2)
+template <int G, int MODE, class PT>
+__device__ __forceinline__ void record_stats(const PT& p, int hid, int g, float lse2)
 {
     const int r = p.lay.r;
     int slot = (p.seq_g[hid_seq<MODE>(p, hid)] + p.ring_off) % r;
@@ -405,8 +408,8 @@ __device__ __forceinline__ void record_stats(const AttnParams& p, int hid, int g
 // group), and for every piece load its max (one address per head: a broadcast) and their
 // channels together, so the loads of all pieces are independent.  Partials come from other
 // SMs: read through L2.
-template <int G, int MODE>
-__device__ void merge_head(const AttnParams& p, int hid, int w0, int P, int lane)
+template <int G, int MODE, class PT>
+__device__ void merge_head(const PT& p, int hid, int w0, int P, int lane)
 {
     using C = Cfg<G>;
     constexpr int rs = partial_stride(G);
@@ -499,8 +502,8 @@ __device__ __forceinline__ uint8_t* deposit(uint8_t* smem, int warp, bool last_p
 
 // Warps a .. z of the CTA have deposited head `hid`, whose chunks are w0 .. w1.  One warp: lanes split
 // as (query head g, channel group).
-template <int G, int MODE>
-__device__ void merge_deposits(const AttnParams& p, CtaMerge& cm, uint8_t* smem, int hid, int w0, int w1, int a, int z, int lane)
+template <int G, int MODE, class PT>
+__device__ void merge_deposits(const PT& p, CtaMerge& cm, uint8_t* smem, int hid, int w0, int w1, int a, int z, int lane)
 {
     using C = Cfg<G>;
     const int cta0 = (int)blockIdx.x * C::WARPS;
@@ -552,8 +555,8 @@ __device__ void merge_deposits(const AttnParams& p, CtaMerge& cm, uint8_t* smem,
 // The CTA's end: its records are announced, and where this CTA is the last to hold a piece of a head,
 // all its threads merge the head's records, four channels of a query head each, up to eight records
 // on the way per thread.  Partials come from other SMs: read through L2.
-template <int G, int MODE>
-__device__ void finish_cta(const AttnParams& p, CtaMerge& cm)
+template <int G, int MODE, class PT>
+__device__ void finish_cta(const PT& p, CtaMerge& cm)
 {
     using C = Cfg<G>;
     constexpr int rs = partial_stride(G), kBatch = 8;
@@ -626,9 +629,9 @@ __device__ void finish_cta(const AttnParams& p, CtaMerge& cm)
 }
 #endif
 
-template <int G, int MODE>
+template <int G, int MODE, int NB>
 __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
-    attn_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtensorMap tk,
+    attn_kernel(const __grid_constant__ AttnParamsN<NB> p, const __grid_constant__ CUtensorMap tk,
                 const __grid_constant__ CUtensorMap tv)
 {
     using C = Cfg<G>;
@@ -1131,18 +1134,39 @@ cudaError_t launch_attn_g(const AttnParams& p, const CUtensorMap* tk, const CUte
     using C = Cfg<G>;
     bool compact = false;
     for (int i = 0; i < RA_MAX_BATCH / 32; ++i) compact |= p.compacting[i] != 0u;
-    auto kernel = p.layers > 1 ? attn_kernel<G, kModeStack> : compact ? attn_kernel<G, kModeCompact> : attn_kernel<G, kModePlain>;
-    return launch_pdl(kernel, dim3(ctas), dim3(C::WARPS * 32), C::SMEM, s, p, *tk, *tv);
+    const dim3 grid(ctas), block(C::WARPS * 32);
+    if (p.layers == 1 && !compact && p.lay.B <= kSmallBatch) {
+        AttnParamsN<kSmallBatch> sp;
+        static_cast<AttnScalars&>(sp) = p;
+        auto take = [&](auto& to, const auto& from, int n) { std::copy(from, from + n, to); };
+        const int B = p.lay.B, words = (B + 31) / 32;
+        take(sp.active, p.active, words);
+        take(sp.pending, p.pending, words);
+        take(sp.seq_base, p.seq_base, B + 1);
+        take(sp.seq_gen, p.seq_gen, B);
+        take(sp.seq_g, p.seq_g, B);
+        take(sp.seq_lp, p.seq_lp, B);
+        take(sp.seq_page0, p.seq_page0, B);
+        take(sp.seq_region, p.seq_region, B);
+        return launch_pdl(attn_kernel<G, kModePlain, kSmallBatch>, grid, block, C::SMEM, s, sp, *tk, *tv);
+    }
+    auto kernel = p.layers > 1 ? attn_kernel<G, kModeStack, RA_MAX_BATCH>
+                  : compact    ? attn_kernel<G, kModeCompact, RA_MAX_BATCH>
+                               : attn_kernel<G, kModePlain, RA_MAX_BATCH>;
+    return launch_pdl(kernel, grid, block, C::SMEM, s, p, *tk, *tv);
 }
 
 template <int G>
 cudaError_t prepare_g()
 {
-    for (auto kernel : {attn_kernel<G, kModePlain>, attn_kernel<G, kModeCompact>, attn_kernel<G, kModeStack>}) {
-        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<G>::SMEM);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    auto set = [](auto* kernel) {
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<G>::SMEM);
+    };
+    cudaError_t e = set(attn_kernel<G, kModePlain, kSmallBatch>);
+    if (e == cudaSuccess) e = set(attn_kernel<G, kModePlain, RA_MAX_BATCH>);
+    if (e == cudaSuccess) e = set(attn_kernel<G, kModeCompact, RA_MAX_BATCH>);
+    if (e == cudaSuccess) e = set(attn_kernel<G, kModeStack, RA_MAX_BATCH>);
+    return e;
 }
 
 }  // namespace

@@ -109,7 +109,7 @@ constexpr int kScoreMaxCandidates = 16384;  // K + r bound of the scored policy 
 // ceil(gen / TILE) tiles of generated rows (gen includes a fused new token, its last row).
 // A launch takes `layers` layers from `layer` on, their counters alike (the per-sequence arrays below
 // serve every layer): their heads and tiles are laid end to end, layer-major.
-struct AttnParams {
+struct AttnScalars {
     DevLayout lay;
     int layer;              // first layer
     int layers;             // layers of the launch (more than one: the region tables are read from memory)
@@ -127,24 +127,33 @@ struct AttnParams {
     int nwarps;             // warps launched
     float qk_scale_log2;    // scale * log2(e)
     int early;              // 1: the first tiles' K/V may be loaded before the predecessor kernel finishes
-    uint32_t active[RA_MAX_BATCH / 32];
-    int32_t seq_base[RA_MAX_BATCH + 1];  // KVH * prefix of tiles per head over active sequences
-    int32_t seq_gen[RA_MAX_BATCH];       // generated rows attended per head (incl. a fused new token)
-    int32_t seq_g[RA_MAX_BATCH];         // tokens generated before this step's (fused) / up to it (separate)
-    // From the host mirror, so that entering a head needs no load from memory: the prompt length,
-    // the first prompt page when the sequence's pages are consecutive (-1: walk the page table), and
-    // this layer's region base (the region of KV head h is base * KVH + h)
-    int32_t seq_lp[RA_MAX_BATCH];
-    int32_t seq_page0[RA_MAX_BATCH];
-    int32_t seq_region[RA_MAX_BATCH];
-    uint32_t pending[RA_MAX_BATCH / 32]; // fused step: sequences whose new token this kernel appends
+    uint16_t* qring;        // record each head's query rows in the scored policy's window (or null)
+    int ring_off;           // window slot of sequence b = (seq_g[b] + ring_off) mod r
+};
+
+// The per-sequence part, for NB sequences.  Launch parameters are copied three times on their way (into
+// the launch, to the device, into every SM's constant cache), so a layer's launch of a batch of at
+// most kSmallBatch takes 2.3 KB instead of 14.9 KB.
+constexpr int kSmallBatch = 64;
+template <int NB>
+struct AttnParamsN : AttnScalars {
+    uint32_t active[NB / 32];
+    uint32_t pending[NB / 32];    // fused step: sequences whose new token this kernel appends
     // fused step: sequences that evicted this step and whose compaction this kernel does -- it reads
     // their old regions (plan header), masks the evicted rows and writes every survivor (and the new
     // token) to its slot in the new region (time order kept)
-    uint32_t compacting[RA_MAX_BATCH / 32];
-    uint16_t* qring;                     // record each head's query rows in the scored policy's window (or null)
-    int ring_off;                        // window slot of sequence b = (seq_g[b] + ring_off) mod r
+    uint32_t compacting[NB / 32];
+    int32_t seq_base[NB + 1];     // KVH * prefix of tiles per head over active sequences
+    int32_t seq_gen[NB];          // generated rows attended per head (incl. a fused new token)
+    int32_t seq_g[NB];            // tokens generated before this step's (fused) / up to it (separate)
+    // From the host mirror, so that entering a head needs no load from memory: the prompt length,
+    // the first prompt page when the sequence's pages are consecutive (-1: walk the page table), and
+    // this layer's region base (the region of KV head h is base * KVH + h)
+    int32_t seq_lp[NB];
+    int32_t seq_page0[NB];
+    int32_t seq_region[NB];
 };
+using AttnParams = AttnParamsN<RA_MAX_BATCH>;
 
 struct CopyRowsParams {
     DevLayout lay;

@@ -230,8 +230,9 @@ int ra_get_scores(ra_ctx* ctx, int layer, int seq, int kv_head, float* host_scor
  * Tuning: the decode-attention kernel shape.  RA_ATTN_SHAPE_AUTO (default)
  * picks per launch: layers attending fewer than 2^20 cache rows take the
  * narrow shape (32-row tiles, 6 warps per SM: a finer split of a short layer),
- * larger ones the wide shape (48-row tiles, 4 warps).  Outputs agree within
- * fp32 rounding (the split, hence the summation order, differs).
+ * larger ones the wide shape (48-row tiles, 4 warps); layers of so few heads
+ * that each can have a cluster of CTAs of its own (one or a few sequences) take
+ * that.  Outputs agree within fp32 rounding (the split, hence the summation order, differs).
  */
 #define RA_ATTN_SHAPE_AUTO 0
 #define RA_ATTN_SHAPE_WIDE 1

@@ -14,7 +14,7 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libra.so")
-SOURCES = ["ra_api.cu", "ra_evict.cu", "ra_attn.cu", "ra_score.cu"]
+SOURCES = ["ra_api.cu", "ra_evict.cu", "ra_attn.cu", "ra_attn_cluster.cu", "ra_score.cu"]
 # (source, object, extra flags): the attention file is built twice, once per kernel shape.
 UNITS = [
     ("ra_api.cu", "ra_api.o", []),
@@ -22,9 +22,10 @@ UNITS = [
     ("ra_attn.cu", "ra_attn_wide.o", ["-DRA_ATTN_NS=attn_wide", "-DRA_ATTN_TILE=48", "-DRA_ATTN_WARPS=4"]),
     ("ra_attn.cu", "ra_attn_narrow.o",
      ["-DRA_ATTN_NS=attn_narrow", "-DRA_ATTN_TILE=32", "-DRA_ATTN_WARPS=6", "-DRA_ATTN_TRANSPOSED=1"]),
+    ("ra_attn_cluster.cu", "ra_attn_cluster.o", []),
     ("ra_score.cu", "ra_score.o", []),
 ]
-HEADERS = ["ra_internal.h", "ra_ptx.cuh"]
+HEADERS = ["ra_internal.h", "ra_ptx.cuh", "ra_attn_tile.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I" + os.path.join(ROOT, "include"), "-I" + CSRC]
 # Extra nvcc flags, e.g. -DRA_ATTN_S_LPS=16 ... to build another attention kernel shape.

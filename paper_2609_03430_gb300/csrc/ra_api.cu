@@ -70,6 +70,7 @@ struct ra_ctx {
     int device = -1;
     int sms = 0;
     int evict_active[kEvMaxCluster + 1] = {0};  // clusters of each size the device runs at once
+    int attn_active[17] = {0};                  // the same of the attention's cluster kernel
     uint8_t* arena = nullptr;
     DevLayout lay{};
     CUtensorMap tmap_k[kAttnShapes]{}, tmap_v[kAttnShapes]{};  // per attention shape (tile rows)
@@ -95,7 +96,10 @@ struct ra_ctx {
     cudaEvent_t fork_ev = nullptr, plan_ev = nullptr;
     bool plan_pending = false;
     int parity = 0;
-    bool no_early_once = false;  // the next fused launches follow the whole-stack compaction, or a copy into the caches
+    bool no_early_once = false;  // the next fused launches follow an eviction, or a copy into the caches
+    // The last launch that touched the caches was ra_append_kv's (everything before it has completed when
+    // a kernel behind it starts): its successor may read all rows but the newest ahead of it.
+    bool appended = false;
     bool step_open = false;  // a step's prologue ran (plans launched, stack evicted) and its end has not
     int step_cur = 0;        // the plan half that step reads
     std::vector<int32_t> plan_g, plan_n;
@@ -250,6 +254,8 @@ void fill_active(const ra_ctx* ctx, uint32_t* mask)
         if (ctx->active[b]) mask[b >> 5] |= 1u << (b & 31);
 }
 
+int cluster_size(const ra_ctx* ctx, int heads, int longest, int W);
+
 // Work split of the attention of `layers` layers from `layer` on (counters alike), from the host
 // mirror, in tiles: a head has ceil(lp / TILE) prompt tiles and ceil(gen / TILE) tiles of generated
 // rows, where gen is the cached generated rows plus one for a fused new token; the tiles are cut
@@ -308,9 +314,39 @@ int plan_attention(ra_ctx* ctx, int layer, int layers, int fused, AttnParams* p,
     p->nwarps = *ctas * wpc;
     *n_active = na;
     *slots = (double)rows;
+    // A layer of few heads takes a cluster per head: see cluster_size.
+    p->cluster = 0;
+    p->cluster_heads = 0;
+    if (layers == 1 && !old_rows && ctx->attn_shape == RA_ATTN_SHAPE_AUTO && *shape == kAttnNarrow && ctx->B <= kSmallBatch && acc > 0) {
+        int holding = 0, longest = 0;
+        for (int b = 0; b < ctx->B; ++b) {
+            const int t = (p->seq_base[b + 1] - p->seq_base[b]) / ctx->KVH;
+            holding += t > 0;
+            longest = std::max(longest, t);
+        }
+        p->cluster_heads = holding * ctx->KVH;
+        p->cluster = cluster_size(ctx, p->cluster_heads, longest, (int)W);
+    }
     if ((size_t)p->nchunks > ctx->max_chunks)
         return fail(ctx, RA_ERR_STATE, "attention split needs more partial records than the arena holds");
     return RA_OK;
+}
+
+// CTAs per head of the cluster kernel for `heads` heads of at most `longest` tiles, or 0 where the
+// split over all CTAs (W tiles per warp) is the better one.  The largest cluster that leaves every head
+// its own and all of them running at once, but no more CTAs than the longest head fills.  The line:
+// the cluster kernel saves 2 to 4 us a layer, about as long as a warp takes for two tiles, but heads
+// that do not divide the SMs (or are uneven) give its warps more tiles than W.  Measured, with 8 KV heads
+// and G = 4 (tiles per warp here / with the split): 1/1 5.7 against 8.3 us, 4/3 12.4 and 14.8, 7/6
+// 19.6 and 21.4, 13/11 30.8 and 31.9, 17/16 42.0 and 41.7, 14/12 34.7 and 33.3, 14/9 30.4 and 27.1.
+int cluster_size(const ra_ctx* ctx, int heads, int longest, int W)
+{
+    int cl = std::min(16, ctx->sms / heads);
+    cl = std::min(cl, (longest + kClusterWarps - 1) / kClusterWarps);
+    while (cl > 1 && ctx->attn_active[cl] < heads) --cl;
+    if (cl < 1 || ctx->attn_active[cl] < heads) return 0;
+    const int Wc = (longest + cl * kClusterWarps - 1) / (cl * kClusterWarps);
+    return W <= 20 && Wc <= W + (W <= 11 ? 2 : 1) ? cl : 0;
 }
 
 void layout_scoring(ra_ctx* ctx);
@@ -460,6 +496,7 @@ int run_eviction(ra_ctx* ctx, EvictParams& p, double moved, cudaStream_t s, bool
         p.trig_dst[i] = ctx->sbase[p.trig[i]];
         p.trig_admit[i] = (uint16_t)ctx->admits[p.trig[i]];
     }
+    ctx->appended = false;
     int rc = run_eviction_launches(ctx, p, moved, s, compact_in_attention, score_early);
     if (rc == RA_OK && !p.holefill)  // every ordered compaction (any kernel) swaps region and spare
         for (int i = 0; i < p.n_trig; ++i)
@@ -711,6 +748,7 @@ int ra_bind(ra_ctx* ctx, void* device_arena, size_t bytes, void* stream)
         if ((rc = make_tmap(ctx, &ctx->tmap_v[sh], Ly.vpool, ctx->total_rows, tile)) != RA_OK) return rc;
         if ((e = attn_prepare(sh, ctx->G)) != cudaSuccess) return cuda_fail(ctx, e, "attention kernel attributes");
     }
+    if ((e = attn_cluster_prepare(ctx->G, ctx->attn_active)) != cudaSuccess) return cuda_fail(ctx, e, "attention kernel attributes");
     if ((e = evict_prepare(ctx->evict_active)) != cudaSuccess) return cuda_fail(ctx, e, "eviction kernel attributes");
     if (ctx->scoring) {
         if ((rc = make_tmap(ctx, &ctx->tmap_ks, Ly.kpool, ctx->total_rows, kScoreTile)) != RA_OK) return rc;
@@ -765,6 +803,7 @@ int ra_prefill(ra_ctx* ctx, int layer, const uint16_t* k, const uint16_t* v, int
     for (int b = 0; b < ctx->B; ++b) p.n_rows[b] = ctx->lp[b];
     cudaError_t e = launch_prefill(p, (cudaStream_t)stream);
     ctx->no_early_once = true;
+    ctx->appended = false;
     return e == cudaSuccess ? RA_OK : cuda_fail(ctx, e, "prefill launch");
 }
 
@@ -796,6 +835,7 @@ int ra_restore(ra_ctx* ctx, int layer, const int32_t* g_host, const int32_t* c_h
     for (int b = 0; b < ctx->B; ++b) p.n_rows[b] = c_host[b];
     cudaError_t e;
     ctx->no_early_once = true;
+    ctx->appended = false;
     if (maxc > 0 && (e = launch_restore(p, s)) != cudaSuccess) return cuda_fail(ctx, e, "restore launch");
     for (int b = 0; b < ctx->B; ++b) {
         const size_t i = (size_t)layer * ctx->B + b;
@@ -919,6 +959,7 @@ int ra_admit(ra_ctx* ctx, int seq, int prompt_len, const uint16_t* k, const uint
         p.layers = ctx->L;
         if ((e = launch_prefill(p, s)) != cudaSuccess) return cuda_fail(ctx, e, "admit prefill launch");
         ctx->no_early_once = true;
+        ctx->appended = false;
     }
     // a fresh request: nothing generated, nothing cached, its own random stream
     for (int l = 0; l < ctx->L; ++l) {
@@ -1021,6 +1062,7 @@ int ra_append_kv(ra_ctx* ctx, int layer, const uint16_t* k_new, const uint16_t* 
     cudaError_t e = launch_append(p, ctx->B, s);
     ps.done();
     if (e != cudaSuccess) return cuda_fail(ctx, e, "append launch");
+    ctx->appended = true;
     for (int b = 0; b < ctx->B; ++b) {
         if (!ctx->active[b]) continue;
         ctx->c[(size_t)layer * ctx->B + b] += 1;
@@ -1062,6 +1104,7 @@ int ra_evict(ra_ctx* ctx, int layer, int* n_fired, void* stream)
         }
     }
     p.n_trig = n;
+    ctx->no_early_once = true;
     if ((rc = run_eviction(ctx, p, moved, (cudaStream_t)stream)) != RA_OK) return rc;
     for (int i = 0; i < n; ++i) {
         const int b = p.trig[i];
@@ -1083,7 +1126,7 @@ int ra_decode_attn(ra_ctx* ctx, int layer, const uint16_t* q, uint16_t* out, flo
     p.q = q;
     p.out = out;
     p.k_new = p.v_new = nullptr;
-    p.early = 0;
+    p.early = ctx->appended ? kEarlyButNewest : kEarlyNone;
     p.partial = ctx->lay.partial;
     p.arrive = ctx->lay.arrive;
     p.qring = ctx->lay.qring;
@@ -1243,6 +1286,7 @@ int step_prologue(ra_ctx* ctx, cudaStream_t s)
                     ctx->nev[k] += 1;
                 }
             ctx->no_early_once = true;
+            ctx->appended = false;
         }
     }
     ctx->step_open = true;
@@ -1320,8 +1364,9 @@ int evict_pending(ra_ctx* ctx, int layer, cudaStream_t s, int plan_parity, std::
     // completed (every kernel before the predecessor has).  The scored policy reads scores its
     // predecessor computes, and with one layer the predecessor is this layer's previous step.
     // Neither starts early right after rows were loaded: the predecessor may have written this layer.
-    ep.early = (ctx->policy != RA_POLICY_SNAPKV && ctx->L >= 2 && !ctx->no_early_once) ? 1 : 0;
-    const int score_early = (ctx->L >= 2 && !ctx->no_early_once) ? 1 : 0;  // the scoring pass reads only older kernels' output
+    const bool clean = ctx->L >= 2 && !ctx->no_early_once && !ctx->appended;
+    ep.early = (ctx->policy != RA_POLICY_SNAPKV && clean) ? 1 : 0;
+    const int score_early = clean ? 1 : 0;  // the scoring pass reads only older kernels' output
     ep.pending = 1;  // the step's token is appended by the attention launch below
     int n = 0;
     double moved = 0;
@@ -1394,10 +1439,15 @@ int attend_pending(ra_ctx* ctx, int layer, int layers, const uint16_t* q, const 
     p.qk_scale_log2 = scale_log2(scale);
     // The kernel may request its first K/V tiles before its predecessor finishes when that
     // predecessor cannot be writing this layer's cache or tables: no eviction of this layer at
-    // this step (else it is this layer's compaction) and layers outside this launch (else it is
-    // these layers' previous step).  Kernels let successors start only after their own wait, so
+    // this step (else it is this layer's compaction) and more than one layer (else it is this
+    // layer's previous step), or but for each head's newest cached row.  Kernels let successors start only after their own wait, so
     // everything older than the predecessor has completed.
-    p.early = (!evicted && layers < ctx->L && !ctx->no_early_once) ? 1 : 0;
+    // With one layer in all (its previous step) or after a call that appended on its own, the newest
+    // cached rows are the ones that the predecessor may be writing.
+    p.early = evicted || ctx->no_early_once || layers > 1 ? kEarlyNone
+              : ctx->L > 1 && !ctx->appended              ? kEarlyAll
+                                                          : kEarlyButNewest;
+    ctx->appended = false;
     ctx->no_early_once = layers > 1;  // the next launch's predecessor then writes every layer's newest row
     {
         // rows read (a new token's from the caller), a new token's row written, q read, out written
@@ -1712,7 +1762,7 @@ extern "C" int ra_decode_attn_noalloc(ra_ctx* ctx, int layer, const uint16_t* q,
     p.q = q;
     p.out = out;
     p.k_new = p.v_new = nullptr;
-    p.early = 0;
+    p.early = kEarlyNone;
     p.qring = ctx->lay.qring;
     p.ring_off = -1;
     int n_active = 0, ctas = 0;

@@ -75,20 +75,18 @@
 
 #include <algorithm>
 
+#include "ra_attn_tile.cuh"
 #include "ra_internal.h"
 #include "ra_ptx.cuh"
 
 namespace ra {
 namespace {
 
-constexpr float kTau = 8.0f;                       // lazy-rescale threshold (log2 units)
-constexpr uint64_t kWaitLimitNs = 2000000000ull;   // bounded mbarrier waits: 2 s
 #if RA_ATTN_CTA_MERGE
 constexpr int kSmemBudget = 232448 - 1024 - 256;  // all an SM gives, but the alignment and the statics
 #else
 constexpr int kSmemBudget = 220 * 1024;
 #endif
-constexpr int kHalfCh = 64;                        // channels per swizzled TMA box (128 bytes)
 
 // Kernel shape: rows per stage (a multiple of 16), stages per warp, warps per CTA
 // (one CTA per SM; the warp count is capped by what fits in shared memory).  The library
@@ -162,8 +160,9 @@ struct Cfg {
 constexpr int kModePlain = 0, kModeCompact = 1, kModeStack = 2;
 
 // Tile header flags; the chunk index sits above them (<< kFlagBits).
-// kQDirect, kNtDirect: the query rows, the new token's rows are read straight from global memory.
-constexpr int kFirst = 1, kLast = 2, kNewTok = 4, kHead0 = 8, kCompact = 16, kQDirect = 32, kNtDirect = 64, kFlagBits = 7;
+// kNewest: the tile holds the newest cached row or rows past it.  kQDirect, kNtDirect: the query rows, the new token's rows are read straight from global memory.
+constexpr int kFirst = 1, kLast = 2, kNewTok = 4, kHead0 = 8, kCompact = 16, kQDirect = 32, kNtDirect = 64,
+              kNewest = 128, kFlagBits = 8;
 
 // Producer-side walk over the warp's chunks (chunks and cursors count tiles).
 struct TileIter {
@@ -294,8 +293,9 @@ __device__ bool iter_next(TileIter& it, const PT& p, TileDesc& d, int warp_id)
         const int kg = it.k - it.tp;
         d.row = it.grow + (long long)kg * T;
         d.n = min(T, it.gen - kg * T);
-        if (p.k_new && ((p.pending[it.b >> 5] >> (it.b & 31)) & 1u) && kg * T + d.n == it.gen)
-            d.flags |= kNewTok;  // its last row is the step's new token
+        const bool pending = p.k_new && ((p.pending[it.b >> 5] >> (it.b & 31)) & 1u);
+        if (pending && kg * T + d.n == it.gen) d.flags |= kNewTok;  // its last row is the step's new token
+        if (kg * T + d.n > it.gen - (pending ? 2 : 1)) d.flags |= kNewest;
         if (MODE == kModeCompact && it.comp) d.flags |= kCompact;
     }
     if (it.k + 1 == it.nt || it.f + 1 == it.end) d.flags |= kLast;
@@ -322,26 +322,10 @@ __device__ bool iter_next(TileIter& it, const PT& p, TileDesc& d, int warp_id)
     return true;
 }
 
-// Byte offset of (row j, 16-byte chunk c of 16) inside a swizzled K or V tile:
-// two boxes of 64 channels; within a box the chunk index is xored with j mod 8.
 template <int G>
 __device__ __forceinline__ uint32_t swz(int j, int c)
 {
-    return (uint32_t)((c >> 3) * Cfg<G>::HALF_BYTES + j * 128 + (((c & 7) ^ (j & 7)) << 4));
-}
-
-__device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], uint32_t addr)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(addr));
-}
-
-__device__ __forceinline__ void ldsm_x4_t(uint32_t (&r)[4], uint32_t addr)
-{
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(addr));
+    return swz_tile<Cfg<G>::HALF_BYTES>(j, c);
 }
 
 #if !RA_ATTN_TRANSPOSED
@@ -361,32 +345,6 @@ __device__ __forceinline__ void mma_rows8(float& c0, float& c1, uint32_t a0, uin
 }
 #pragma nv_diag_default 550
 #endif
-
-#if RA_ATTN_TRANSPOSED
-// C[16x8] += A[16x16] B[16x8], bf16 inputs, fp32 accumulators (register-only: not volatile, so the
-// compiler may interleave independent products).
-__device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
-{
-    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
-        "{%0, %1, %2, %3};"
-        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-// Transpose of an 8x8 bf16 matrix held in fragment layout (lane l: row l / 4, columns 2 (l % 4) + {0, 1}).
-__device__ __forceinline__ uint32_t movtrans(uint32_t x)
-{
-    uint32_t y;
-    asm("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
-    return y;
-}
-#endif
-
-__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
-{
-    return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(lo)) |
-           ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(hi)) << 16);
-}
 
 // The scored policy's window: the softmax normaliser of query head g of head `hid` at this
 // step, as (scale * log2 e, log2 sum_i exp2(scale * log2 e * q.k_i)), beside its query rows.
@@ -666,9 +624,11 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
     __syncwarp();
     // The cache, the region table and the inputs may come from the previous kernel.  With
     // p.early (the host has checked that the previous kernel writes none of this layer's
-    // cache or tables) the first tiles' K and V are requested before waiting; the query
-    // rows and the new token's row, which the caller may have just produced, come after.
-    if (!p.early) pdl_wait();
+    // cache or tables, or only each head's newest cached row) the first tiles' K and V are requested
+    // before waiting; the query rows and the new token's row, which the caller may have just
+    // produced, come after.
+    bool waited = p.early == kEarlyNone;
+    if (waited) pdl_wait();
 
     TileIter it;
     it.chunk = -1;
@@ -688,10 +648,16 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
             bulk_load(sl, p.q + (size_t)hd.z * G * kHeadDim,
                       (uint32_t)C::Q_BYTES, &bars[s]);
     };
-    auto issue = [&](int t, bool inputs) -> bool {
+    auto issue = [&](int t) -> bool {
         TileDesc d;
         if (!iter_next<MODE>(it, p, d, gw)) return false;
         const int s = t % C::SPW;
+        if (!waited && p.early == kEarlyButNewest && (d.flags & kNewest)) {
+            waited = true;
+            pdl_wait();
+            if (lane == 0)
+                for (int u = 0; u < t; ++u) issue_inputs(u);
+        }
         if (C::SLOTS == 1) {
             if (d.flags & kFirst) {
                 if (q_busy) d.flags |= kQDirect;
@@ -713,16 +679,17 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
             tma_load_2d(st + C::HALF_BYTES, &tk, kHalfCh, (int)d.row, &bars[s]);
             tma_load_2d(st + C::KV_BYTES, &tv, 0, (int)d.row, &bars[s]);
             tma_load_2d(st + C::KV_BYTES + C::HALF_BYTES, &tv, kHalfCh, (int)d.row, &bars[s]);
-            if (inputs) issue_inputs(s);
+            if (waited) issue_inputs(s);
         }
         return true;
     };
     bool more = true;
     for (int t = 0; t < C::SPW && more; ++t) {
-        more = issue(t, !p.early);
+        more = issue(t);
         if (more) ++issued;
     }
-    if (p.early) {
+    if (!waited) {
+        waited = true;
         pdl_wait();
         if (lane == 0)
             for (int t = 0; t < issued; ++t) issue_inputs(t);
@@ -731,16 +698,13 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
 
     const int gq = lane >> 2;  // this lane's query head (rows >= G are padding)
     const int tq = lane & 3;
-    const int mi = lane >> 3, ri = lane & 7;  // ldmatrix: matrix and row this lane addresses
-
     uint32_t qa[8][2];  // fragments of Q (rows 0..7) for the 8 k-steps of 16 channels (A, or B of Q^T)
 #if RA_ATTN_TRANSPOSED
     const int hA = 2 * tq, hB = 2 * tq + 1;  // the query heads of this lane's accumulator columns
-    float O[8][4];      // O^T: m-tile mt = channels 16 mt..; {ch 16mt+gq: hA, hB; ch 16mt+gq+8: hA, hB}
-    float mA = -INFINITY, mB = -INFINITY, lA = 0.f, lB = 0.f;  // running max and (lane-partial) sum per head
-#pragma unroll
-    for (int mt = 0; mt < 8; ++mt) O[mt][0] = O[mt][1] = O[mt][2] = O[mt][3] = 0.f;
+    PieceT acc;
+    acc.clear();
 #else
+    const int mi = lane >> 3, ri = lane & 7;  // ldmatrix: matrix and row this lane addresses
     float O[16][2];     // O[head gq][n-tile * 8 + 2 tq + {0, 1}]
     float m_run = -INFINITY, l_run = 0.f;
 #pragma unroll
@@ -830,79 +794,19 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
         }
 
 #if RA_ATTN_TRANSPOSED
-        // per 16-row batch: S^T = K Q^T (two accumulator chains), online softmax, O^T += V^T P^T
-        const float sl = p.qk_scale_log2;
-        for (int bs = 0; bs < n; bs += 16) {
-            float x[4] = {0.f, 0.f, 0.f, 0.f}, y[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-            for (int kk = 0; kk < 8; kk += 2) {
-                uint32_t a0[4], a1[4];
-                ldsm_x4(a0, ks + swz<G>(bs + (mi & 1) * 8 + ri, 2 * kk + (mi >> 1)));
-                ldsm_x4(a1, ks + swz<G>(bs + (mi & 1) * 8 + ri, 2 * kk + 2 + (mi >> 1)));
-                mma16816(x, a0, qa[kk][0], qa[kk][1]);
-                mma16816(y, a1, qa[kk + 1][0], qa[kk + 1][1]);
-            }
-            const int r0 = bs + gq, r1 = r0 + 8;  // this lane's rows; heads hA, hB
-            bool v0 = r0 < n, v1 = r1 < n;
-            if (MODE == kModeCompact && (hd.y & kCompact)) {  // evicted rows get no weight
-                v0 = v0 && !(((r0 < 32 ? ev_lo >> r0 : ev_hi >> (r0 - 32)) & 1u));
-                v1 = v1 && !(((r1 < 32 ? ev_lo >> r1 : ev_hi >> (r1 - 32)) & 1u));
-            }
-            float sv[4] = {v0 ? (x[0] + y[0]) * sl : -INFINITY, v0 ? (x[1] + y[1]) * sl : -INFINITY,
-                           v1 ? (x[2] + y[2]) * sl : -INFINITY, v1 ? (x[3] + y[3]) * sl : -INFINITY};
-            float xA = fmaxf(sv[0], sv[2]), xB = fmaxf(sv[1], sv[3]);
-            if (__any_sync(0xffffffffu, xA > mA + kTau || xB > mB + kTau)) {
-#pragma unroll
-                for (int o = 4; o < 32; o <<= 1) {  // over the 8 lanes that share a head pair
-                    xA = fmaxf(xA, __shfl_xor_sync(0xffffffffu, xA, o));
-                    xB = fmaxf(xB, __shfl_xor_sync(0xffffffffu, xB, o));
-                }
-                const float nA = xA > mA + kTau ? xA : mA, nB = xB > mB + kTau ? xB : mB;
-                const float aA = (nA == mA) ? 1.f : exp2f(mA - nA), aB = (nB == mB) ? 1.f : exp2f(mB - nB);
-                mA = nA;
-                mB = nB;
-                lA *= aA;
-                lB *= aB;
-#pragma unroll
-                for (int mt = 0; mt < 8; ++mt) {
-                    O[mt][0] *= aA;
-                    O[mt][2] *= aA;
-                    O[mt][1] *= aB;
-                    O[mt][3] *= aB;
-                }
-            }
-            float pr[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const float m = (e & 1) ? mB : mA;
-                pr[e] = (MODE == kModeCompact && sv[e] == -INFINITY) ? 0.f : exp2f(sv[e] - m);
-            }
-            lA += pr[0] + pr[2];
-            lB += pr[1] + pr[3];
-            const uint32_t b0 = movtrans(pack_bf16x2(pr[0], pr[1])), b1 = movtrans(pack_bf16x2(pr[2], pr[3]));
-#pragma unroll
-            for (int mt = 0; mt < 8; ++mt) {
-                uint32_t v4[4];
-                ldsm_x4_t(v4, vs + swz<G>(bs + (mi >> 1) * 8 + ri, 2 * mt + (mi & 1)));
-                mma16816(O[mt], v4, b0, b1);
-            }
-        }
+        attend_tile<C::HALF_BYTES, MODE == kModeCompact>(acc, ks, vs, n, qa, p.qk_scale_log2, ev_lo, ev_hi, lane);
 
         if (hd.y & kLast) {  // last tile of the piece
-            float la = lA, lb = lB;
-#pragma unroll
-            for (int o = 4; o < 32; o <<= 1) {
-                la += __shfl_xor_sync(0xffffffffu, la, o);
-                lb += __shfl_xor_sync(0xffffffffu, lb, o);
-            }
+            float la, lb;
+            acc.sum_lanes(la, lb);
             const int hid = hd.z;
             int nth;
             const long long A = head_tile0<MODE>(p, hid, &nth);
             const int w0 = (int)(A / p.W), w1 = (int)((A + nth - 1) / p.W);
             if (w0 == w1) {  // the whole head was this warp's: normalise and write the output
                 if (p.qring && gq == 0) {
-                    if (hA < G) record_stats<G, MODE>(p, hid, hA, mA + log2f(la));
-                    if (hB < G) record_stats<G, MODE>(p, hid, hB, mB + log2f(lb));
+                    if (hA < G) record_stats<G, MODE>(p, hid, hA, acc.mA + log2f(la));
+                    if (hB < G) record_stats<G, MODE>(p, hid, hB, acc.mB + log2f(lb));
                 }
                 const float iA = 1.f / la, iB = 1.f / lb;
                 __nv_bfloat16* ob = reinterpret_cast<__nv_bfloat16*>(p.out + (size_t)hid * G * kHeadDim);
@@ -910,12 +814,12 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
                 for (int mt = 0; mt < 8; ++mt) {
                     const int ch = 16 * mt + gq;
                     if (hA < G) {
-                        ob[hA * kHeadDim + ch] = __float2bfloat16_rn(O[mt][0] * iA);
-                        ob[hA * kHeadDim + ch + 8] = __float2bfloat16_rn(O[mt][2] * iA);
+                        ob[hA * kHeadDim + ch] = __float2bfloat16_rn(acc.O[mt][0] * iA);
+                        ob[hA * kHeadDim + ch + 8] = __float2bfloat16_rn(acc.O[mt][2] * iA);
                     }
                     if (hB < G) {
-                        ob[hB * kHeadDim + ch] = __float2bfloat16_rn(O[mt][1] * iB);
-                        ob[hB * kHeadDim + ch + 8] = __float2bfloat16_rn(O[mt][3] * iB);
+                        ob[hB * kHeadDim + ch] = __float2bfloat16_rn(acc.O[mt][1] * iB);
+                        ob[hB * kHeadDim + ch + 8] = __float2bfloat16_rn(acc.O[mt][3] * iB);
                     }
                 }
             } else {
@@ -931,28 +835,7 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
                     rec = reinterpret_cast<float*>(deposit<G>(smem, warp, chunk < w1, s));
                     rs = C::DEP_ROW;
                 }
-#pragma unroll
-                for (int mt = 0; mt < 8; ++mt) {
-                    const int ch = 16 * mt + gq;
-                    if (hA < G) {
-                        rec[hA * rs + ch] = O[mt][0];
-                        rec[hA * rs + ch + 8] = O[mt][2];
-                    }
-                    if (hB < G) {
-                        rec[hB * rs + ch] = O[mt][1];
-                        rec[hB * rs + ch + 8] = O[mt][3];
-                    }
-                }
-                if (gq == 0) {
-                    if (hA < G) {
-                        rec[G * rs + hA] = mA;
-                        rec[G * rs + G + hA] = la;
-                    }
-                    if (hB < G) {
-                        rec[G * rs + hB] = mB;
-                        rec[G * rs + G + hB] = lb;
-                    }
-                }
+                acc.store<G>(rec, rs, la, lb, lane);
                 if (a == z) {
                     if (lane == 0) cm.part[a == w0 ? 1 : 0] = {hid, w0 / C::WARPS, w1 / C::WARPS - w0 / C::WARPS + 1};
                 } else {
@@ -968,10 +851,7 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
                     }
                 }
             }
-            mA = mB = -INFINITY;
-            lA = lB = 0.f;
-#pragma unroll
-            for (int mt = 0; mt < 8; ++mt) O[mt][0] = O[mt][1] = O[mt][2] = O[mt][3] = 0.f;
+            acc.clear();
         }
 #else
         for (int bs = 0; bs < n; bs += 16) {
@@ -1106,7 +986,7 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
         __syncwarp();
         if (more) {
             if (lane == 0) fence_proxy_async_smem();
-            more = issue(t + C::SPW, true);
+            more = issue(t + C::SPW);
             if (more) ++issued;
         }
     }
@@ -1135,7 +1015,7 @@ cudaError_t launch_attn_g(const AttnParams& p, const CUtensorMap* tk, const CUte
     bool compact = false;
     for (int i = 0; i < RA_MAX_BATCH / 32; ++i) compact |= p.compacting[i] != 0u;
     const dim3 grid(ctas), block(C::WARPS * 32);
-    if (p.layers == 1 && !compact && p.lay.B <= kSmallBatch) {
+    if (p.layers == 1 && !compact && p.lay.B <= kSmallBatch) {  // (p.cluster implies it)
         AttnParamsN<kSmallBatch> sp;
         static_cast<AttnScalars&>(sp) = p;
         auto take = [&](auto& to, const auto& from, int n) { std::copy(from, from + n, to); };
@@ -1148,6 +1028,7 @@ cudaError_t launch_attn_g(const AttnParams& p, const CUtensorMap* tk, const CUte
         take(sp.seq_lp, p.seq_lp, B);
         take(sp.seq_page0, p.seq_page0, B);
         take(sp.seq_region, p.seq_region, B);
+        if (p.cluster > 0) return launch_attn_cluster(sp, tk, tv, p.cluster_heads, p.cluster, s);
         return launch_pdl(attn_kernel<G, kModePlain, kSmallBatch>, grid, block, C::SMEM, s, sp, *tk, *tv);
     }
     auto kernel = p.layers > 1 ? attn_kernel<G, kModeStack, RA_MAX_BATCH>

@@ -1,0 +1,184 @@
+// ra_attn_tile.cuh -- one tile of cache rows against a head's query rows on mma.sync, shared by the
+// attention kernels of ra_attn.cu and ra_attn_cluster.cu.
+#pragma once
+
+#include <cuda_bf16.h>
+#include <math.h>
+#include <stdint.h>
+
+#include "ra_internal.h"
+#include "ra_ptx.cuh"
+
+namespace ra {
+namespace {
+
+constexpr float kTau = 8.0f;                       // lazy-rescale threshold (log2 units)
+constexpr uint64_t kWaitLimitNs = 2000000000ull;   // bounded mbarrier waits: 2 s
+constexpr int kHalfCh = 64;                        // channels per swizzled TMA box (128 bytes)
+
+// Byte offset of (row j, 16-byte chunk c of 16) inside a swizzled K or V tile: two boxes of 64
+// channels, HALF bytes each; within a box the chunk index is xored with j mod 8.
+template <int HALF>
+__device__ __forceinline__ uint32_t swz_tile(int j, int c)
+{
+    return (uint32_t)((c >> 3) * HALF + j * 128 + (((c & 7) ^ (j & 7)) << 4));
+}
+
+__device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr));
+}
+
+__device__ __forceinline__ void ldsm_x4_t(uint32_t (&r)[4], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr));
+}
+
+// C[16x8] += A[16x16] B[16x8], bf16 inputs, fp32 accumulators (register-only: not volatile, so the
+// compiler may interleave independent products).
+__device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+{
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+        "{%0, %1, %2, %3};"
+        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// Transpose of an 8x8 bf16 matrix held in fragment layout (lane l: row l / 4, columns 2 (l % 4) + {0, 1}).
+__device__ __forceinline__ uint32_t movtrans(uint32_t x)
+{
+    uint32_t y;
+    asm("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
+    return y;
+}
+
+__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
+{
+    return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(lo)) |
+           ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(hi)) << 16);
+}
+
+// The transposed products' running state of a head piece, per lane: O^T (m-tile mt = channels 16 mt..:
+// {ch 16 mt + gq: heads hA, hB; ch 16 mt + gq + 8: hA, hB}, gq = lane / 4, hA = 2 (lane % 4), hB = hA + 1), the
+// running max and the (lane-partial) sum of the two heads.
+struct PieceT {
+    float O[8][4];
+    float mA, mB, lA, lB;
+    __device__ __forceinline__ void clear()
+    {
+        mA = mB = -INFINITY;
+        lA = lB = 0.f;
+#pragma unroll
+        for (int mt = 0; mt < 8; ++mt) O[mt][0] = O[mt][1] = O[mt][2] = O[mt][3] = 0.f;
+    }
+    __device__ __forceinline__ void sum_lanes(float& la, float& lb) const  // over the 8 lanes of a head pair
+    {
+        la = lA;
+        lb = lB;
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) {
+            la += __shfl_xor_sync(0xffffffffu, la, o);
+            lb += __shfl_xor_sync(0xffffffffu, lb, o);
+        }
+    }
+    // O, m and l to a record: heads `stride` floats apart, then m [G], l [G].
+    template <int G>
+    __device__ __forceinline__ void store(float* rec, int stride, float la, float lb, int lane) const
+    {
+        const int gq = lane >> 2, hA = 2 * (lane & 3), hB = hA + 1;
+#pragma unroll
+        for (int mt = 0; mt < 8; ++mt) {
+            const int ch = 16 * mt + gq;
+            if (hA < G) {
+                rec[hA * stride + ch] = O[mt][0];
+                rec[hA * stride + ch + 8] = O[mt][2];
+            }
+            if (hB < G) {
+                rec[hB * stride + ch] = O[mt][1];
+                rec[hB * stride + ch + 8] = O[mt][3];
+            }
+        }
+        if (gq == 0) {
+            if (hA < G) {
+                rec[G * stride + hA] = mA;
+                rec[G * stride + G + hA] = la;
+            }
+            if (hB < G) {
+                rec[G * stride + hB] = mB;
+                rec[G * stride + G + hB] = lb;
+            }
+        }
+    }
+};
+
+// n rows of a tile (K at shared address ks, V at vs): per 16-row batch S^T = K Q^T (two accumulator
+// chains), online softmax, O^T += V^T P^T.  qa: the head's query rows as B fragments of the 8 k-steps.
+// MASK: rows whose bit of ev_hi:ev_lo is set get no weight.
+template <int HALF, bool MASK>
+__device__ __forceinline__ void attend_tile(PieceT& s, uint32_t ks, uint32_t vs, int n, const uint32_t (&qa)[8][2], float sl,
+                                            uint32_t ev_lo, uint32_t ev_hi, int lane)
+{
+    const int gq = lane >> 2, mi = lane >> 3, ri = lane & 7;  // ldmatrix: matrix and row this lane addresses
+    for (int bs = 0; bs < n; bs += 16) {
+        float x[4] = {0.f, 0.f, 0.f, 0.f}, y[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int kk = 0; kk < 8; kk += 2) {
+            uint32_t a0[4], a1[4];
+            ldsm_x4(a0, ks + swz_tile<HALF>(bs + (mi & 1) * 8 + ri, 2 * kk + (mi >> 1)));
+            ldsm_x4(a1, ks + swz_tile<HALF>(bs + (mi & 1) * 8 + ri, 2 * kk + 2 + (mi >> 1)));
+            mma16816(x, a0, qa[kk][0], qa[kk][1]);
+            mma16816(y, a1, qa[kk + 1][0], qa[kk + 1][1]);
+        }
+        const int r0 = bs + gq, r1 = r0 + 8;  // this lane's rows; heads hA, hB
+        bool v0 = r0 < n, v1 = r1 < n;
+        if (MASK) {
+            v0 = v0 && !(((r0 < 32 ? ev_lo >> r0 : ev_hi >> (r0 - 32)) & 1u));
+            v1 = v1 && !(((r1 < 32 ? ev_lo >> r1 : ev_hi >> (r1 - 32)) & 1u));
+        }
+        float sv[4] = {v0 ? (x[0] + y[0]) * sl : -INFINITY, v0 ? (x[1] + y[1]) * sl : -INFINITY,
+                       v1 ? (x[2] + y[2]) * sl : -INFINITY, v1 ? (x[3] + y[3]) * sl : -INFINITY};
+        float xA = fmaxf(sv[0], sv[2]), xB = fmaxf(sv[1], sv[3]);
+        if (__any_sync(0xffffffffu, xA > s.mA + kTau || xB > s.mB + kTau)) {
+#pragma unroll
+            for (int o = 4; o < 32; o <<= 1) {  // over the 8 lanes that share a head pair
+                xA = fmaxf(xA, __shfl_xor_sync(0xffffffffu, xA, o));
+                xB = fmaxf(xB, __shfl_xor_sync(0xffffffffu, xB, o));
+            }
+            const float nA = xA > s.mA + kTau ? xA : s.mA, nB = xB > s.mB + kTau ? xB : s.mB;
+            const float aA = (nA == s.mA) ? 1.f : exp2f(s.mA - nA), aB = (nB == s.mB) ? 1.f : exp2f(s.mB - nB);
+            s.mA = nA;
+            s.mB = nB;
+            s.lA *= aA;
+            s.lB *= aB;
+#pragma unroll
+            for (int mt = 0; mt < 8; ++mt) {
+                s.O[mt][0] *= aA;
+                s.O[mt][2] *= aA;
+                s.O[mt][1] *= aB;
+                s.O[mt][3] *= aB;
+            }
+        }
+        float pr[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const float m = (e & 1) ? s.mB : s.mA;
+            pr[e] = (MASK && sv[e] == -INFINITY) ? 0.f : exp2f(sv[e] - m);
+        }
+        s.lA += pr[0] + pr[2];
+        s.lB += pr[1] + pr[3];
+        const uint32_t b0 = movtrans(pack_bf16x2(pr[0], pr[1])), b1 = movtrans(pack_bf16x2(pr[2], pr[3]));
+#pragma unroll
+        for (int mt = 0; mt < 8; ++mt) {
+            uint32_t v4[4];
+            ldsm_x4_t(v4, vs + swz_tile<HALF>(bs + (mi >> 1) * 8 + ri, 2 * mt + (mi & 1)));
+            mma16816(s.O[mt], v4, b0, b1);
+        }
+    }
+}
+
+}  // namespace
+}  // namespace ra

@@ -107,6 +107,10 @@ constexpr int kScoreMaxCandidates = 16384;  // K + r bound of the scored policy 
 
 // Attention work is counted in tiles of TILE rows: a head has ceil(lp / TILE) prompt tiles and
 // ceil(gen / TILE) tiles of generated rows (gen includes a fused new token, its last row).
+// What the predecessor kernel may write of the layer's cache: anything, nothing, or the newest cached
+// row of each head (an append, or the layer's attention of the step before).
+constexpr int kEarlyNone = 0, kEarlyAll = 1, kEarlyButNewest = 2;
+
 // A launch takes `layers` layers from `layer` on, their counters alike (the per-sequence arrays below
 // serve every layer): their heads and tiles are laid end to end, layer-major.
 struct AttnScalars {
@@ -126,7 +130,9 @@ struct AttnScalars {
     int nchunks;            // ceil(total / W)
     int nwarps;             // warps launched
     float qk_scale_log2;    // scale * log2(e)
-    int early;              // 1: the first tiles' K/V may be loaded before the predecessor kernel finishes
+    int early;              // kEarly*: the first tiles' K/V may be loaded before the predecessor kernel finishes
+    int cluster;            // CTAs per head of the cluster kernel (0: the split over all CTAs), its heads
+    int cluster_heads;
     uint16_t* qring;        // record each head's query rows in the scored policy's window (or null)
     int ring_off;           // window slot of sequence b = (seq_g[b] + ring_off) mod r
 };
@@ -233,6 +239,13 @@ int score_window_tiles(int M);  // 128-row tiles of the M window rows (1..4)
 namespace attn_wide { RA_ATTN_API }
 namespace attn_narrow { RA_ATTN_API }
 #undef RA_ATTN_API
+
+// A cluster of `cl` CTAs per head (ra_attn_cluster.cu; the narrow shape's tensor maps), for layers of few
+// heads: clusters of each size 1..16 the device runs at once, and the launch.
+constexpr int kClusterWarps = 6;
+cudaError_t attn_cluster_prepare(int G, int* active);
+cudaError_t launch_attn_cluster(const AttnParamsN<kSmallBatch>& p, const CUtensorMap* tk, const CUtensorMap* tv, int heads,
+                                int cl, cudaStream_t s);
 
 enum AttnShape { kAttnWide = 0, kAttnNarrow = 1, kAttnShapes = 2 };
 #ifndef RA_ATTN_NARROW_ROWS

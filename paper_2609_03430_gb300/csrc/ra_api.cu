@@ -419,45 +419,39 @@ void layout_scoring(ra_ctx* ctx)
 }
 
 // Launch shape of a scoring pass over the heads of the sequences in p (pass 1: prompt + the
-// trig_n cached rows each; pass 2: the trig_n candidate rows each): CTAs (one per SM: all of its
-// tensor memory) take runs of consecutive tiles of one head, in whole 128-row tiles (two scoring
-// tiles).  Pass 2 aims at one wave.  Pass 1 has more work than a wave on most calls: it takes the run
-// length whose waves, each as long as the run and about three tiles' start-up, end first.
-// Returns the algorithmic bytes: the key rows read (every one is contracted with the M = r * G
-// window rows, so flops = bytes * M).
+// trig_n cached rows each; pass 2: the trig_n candidate rows each, in p->layers layers): CTAs (one per
+// SM: all of its tensor memory) take runs of consecutive tiles of one head, in whole 128-row tiles
+// (two scoring tiles), of the length whose waves, each as long as the run and about three tiles'
+// start-up, end first.  Returns the algorithmic bytes: the key rows read (every one is contracted
+// with the M = r * G window rows, so flops = bytes * M).
 double plan_scoring(ra_ctx* ctx, EvictParams* p, int pass)
 {
-    long long work = 0;
+    const int layers = pass == 1 ? 1 : p->layers;
     int most = 1;
     double rows = 0;
     std::vector<int> tiles((size_t)p->n_trig);
     for (int i = 0; i < p->n_trig; ++i) {
         const int lp = pass == 1 ? ctx->lp[p->trig[i]] : 0, n = p->trig_n[i];
-        const int t = (lp + kScoreTile - 1) / kScoreTile + (n + kScoreTile - 1) / kScoreTile;
-        tiles[i] = t;
-        work += (long long)ctx->KVH * t;
-        most = std::max(most, t);
-        rows += (double)ctx->KVH * (lp + n);
+        tiles[i] = (lp + kScoreTile - 1) / kScoreTile + (n + kScoreTile - 1) / kScoreTile;
+        most = std::max(most, tiles[i]);
+        rows += (double)layers * ctx->KVH * (lp + n);
     }
-    if (pass == 1) {
-        long long best = 0;
-        const int least = std::max(2, (most + ctx->stats_chunks - 1) / ctx->stats_chunks);
-        p->ch1 = (most + 1) / 2 * 2;
-        for (int ch = (least + 1) / 2 * 2; ch <= (most + 1) / 2 * 2; ch += 2) {
-            long long ctas = 0;
-            for (int t : tiles) ctas += (long long)ctx->KVH * ((t + ch - 1) / ch);
-            const long long cost = (ctas + ctx->sms - 1) / ctx->sms * (ch / 2 + 3);
-            if (best == 0 || cost < best) {
-                best = cost;
-                p->ch1 = ch;
-            }
+    // (pass 1 keeps a record per run: as many as the arena has)
+    const int least = pass == 1 ? std::max(2, (most + ctx->stats_chunks - 1) / ctx->stats_chunks) : 2;
+    const int whole = (most + 1) / 2 * 2;
+    int run = whole;
+    long long best = 0;
+    for (int ch = (least + 1) / 2 * 2; ch <= whole; ch += 2) {
+        long long ctas = 0;
+        for (int t : tiles) ctas += (long long)layers * ctx->KVH * ((t + ch - 1) / ch);
+        const long long cost = (ctas + ctx->sms - 1) / ctx->sms * (ch / 2 + 3);
+        if (best == 0 || cost < best) {
+            best = cost;
+            run = ch;
         }
-        p->nch1 = (most + p->ch1 - 1) / p->ch1;
-    } else {
-        long long ch = std::max<long long>((work + ctx->sms - 1) / ctx->sms, 1);
-        p->ch2 = (int)((ch + 1) / 2 * 2);
-        p->nch2 = (most + p->ch2 - 1) / p->ch2;
     }
+    (pass == 1 ? p->ch1 : p->ch2) = run;
+    (pass == 1 ? p->nch1 : p->nch2) = (most + run - 1) / run;
     return rows * kRowBytes;
 }
 
@@ -486,6 +480,16 @@ bool plan_usable(const ra_ctx* ctx)
     return ctx->compaction == RA_COMPACT_ORDERED && ctx->evict_active[1] > 0;
 }
 
+// The scored policy's rounds of a step's start, every layer in one launch each of scores, selection
+// and in-place compaction (a window holds the queries of earlier steps only, so no layer of this step is
+// needed): with ordered compaction of its own, and more than one layer (one layer's round compacts out
+// of place, over all CTAs).
+bool scored_stack_usable(const ra_ctx* ctx)
+{
+    return ctx->policy == RA_POLICY_SNAPKV && ctx->compaction == RA_COMPACT_ORDERED && ctx->L > 1 && ctx->L <= 65535 && ctx->r <= kEvMaxEvicted &&
+           (ctx->evict_mode & ~RA_EVICT_EXACT) != RA_EVICT_TWO_KERNELS;
+}
+
 // One eviction round of the triggered sequences in p: [score passes,] select, compact (unless
 // the caller's attention launch does the compaction).
 int run_eviction(ra_ctx* ctx, EvictParams& p, double moved, cudaStream_t s, bool compact_in_attention = false,
@@ -508,6 +512,8 @@ int run_eviction_launches(ra_ctx* ctx, EvictParams& p, double moved, cudaStream_
                           int score_early)
 {
     cudaError_t e;
+    p.layers = 1;
+    p.to_plan = 0;
     if (p.policy == RA_POLICY_SNAPKV) {  // window scores with the normalisers recorded at decode time
         for (int i = 0; i < p.n_trig; ++i) ctx->score_n[(size_t)p.layer * ctx->B + p.trig[i]] = p.trig_n[i];
         const double bytes = plan_scoring(ctx, &p, 2);
@@ -1185,12 +1191,13 @@ int step_prologue(ra_ctx* ctx, cudaStream_t s)
     const int cur = ctx->parity, nxt = 1 - cur;
     std::fill(ctx->plan_g.begin() + (size_t)nxt * ctx->L * ctx->B, ctx->plan_g.begin() + (size_t)(nxt + 1) * ctx->L * ctx->B,
               -1);
+    const bool scored = scored_stack_usable(ctx);
     bool now = false, next = false;  // a sequence may fire at this step, at the next one (layer 0's counters)
-    for (int b = 0; b < ctx->B && serve; ++b) {
+    for (int b = 0; b < ctx->B && (serve || scored); ++b) {
         if (!ctx->active[b]) continue;
         const int g = ctx->g[b], c = ctx->c[b];
         now = now || fires(ctx, g + 1, c + 1);
-        next = next || (g + 2) % ctx->r == 0;
+        next = next || (serve && (g + 2) % ctx->r == 0);
     }
     if (next) {
         // The sequences whose trigger fires at the next step (from layer 0's counters after this
@@ -1241,7 +1248,7 @@ int step_prologue(ra_ctx* ctx, cudaStream_t s)
         }
     }
     // The sequences that fire at this step in every layer alike, with every layer's evicted set
-    // computed ahead: all their rounds in one launch, in place, before the first layer: the
+    // computed ahead, or from scores computed now: all their rounds in one launch, in place, before the first layer: the
     // survivors move down (ordered) or the evicted slots are refilled from the newest rows
     // (order-free), and the layers then append the token as usual.
     if (now) {
@@ -1260,7 +1267,8 @@ int step_prologue(ra_ctx* ctx, cudaStream_t s)
             bool all = true;
             for (int l = 0; l < ctx->L && all; ++l) {
                 const size_t i = (size_t)l * ctx->B + b, k = (size_t)cur * ctx->L * ctx->B + i;
-                all = ctx->g[i] == g && ctx->c[i] == c && ctx->plan_g[k] == g + 1 && ctx->plan_n[k] == c + 1 - ctx->r;
+                all = ctx->g[i] == g && ctx->c[i] == c &&
+                      (scored || (ctx->plan_g[k] == g + 1 && ctx->plan_n[k] == c + 1 - ctx->r));
             }
             if (!all) continue;
             sp.trig[n] = (int16_t)b;
@@ -1273,9 +1281,29 @@ int step_prologue(ra_ctx* ctx, cudaStream_t s)
         }
         if (n > 0) {
             sp.n_trig = n;
+            if (scored) {
+                sp.policy = ctx->policy;
+                sp.layers = ctx->L;
+                sp.to_plan = 1;
+                for (int i = 0; i < n; ++i)
+                    for (int l = 0; l < ctx->L; ++l) ctx->score_n[(size_t)l * ctx->B + sp.trig[i]] = sp.trig_n[i];
+                {
+                    const double bytes = plan_scoring(ctx, &sp, 2);
+                    ProfScope ps(ctx, RA_KERNEL_SCORE_SUM, bytes, s);
+                    e = launch_score(sp, 2, &ctx->tmap_ks, &ctx->tmap_q, s);
+                    ps.done();
+                }
+                if (e != cudaSuccess) return cuda_fail(ctx, e, "score launch");
+                {
+                    ProfScope ps(ctx, RA_KERNEL_SELECT, 0.0, s);
+                    e = launch_select(sp, s);
+                    ps.done();
+                }
+                if (e != cudaSuccess) return cuda_fail(ctx, e, "select launch");
+            }
             {
                 ProfScope ps(ctx, RA_KERNEL_STACK, moved * 2.0 * (2 * kRowBytes + 4), s);
-                e = fill ? launch_fill_stack(sp, ctx->L, s) : launch_compact_stack(sp, ctx->L, s);
+                e = fill ? launch_fill_stack(sp, ctx->L, s) : launch_compact_stack(sp, ctx->L, ctx->sms, s);
                 ps.done();
             }
             if (e != cudaSuccess) return cuda_fail(ctx, e, "whole-stack compaction launch");

@@ -10,7 +10,9 @@
 //                   the K smallest (score, ordinal) -- Eq. 1 -- and a
 //                   ballot-compacted, ascending list of the evicted ordinals.
 //                   Under the scored comparator the score is the max-pooled
-//                   window attention that ra_score.cu computed; with order-free
+//                   window attention that ra_score.cu computed (at a step's
+//                   start for every layer in one launch, into the sets that
+//                   compact_stack_kernel takes); with order-free
 //                   slots every key follows the candidate's position.
 //                   With order-free slots the select CTA also refills the
 //                   evicted slots in place from the newest ones (no compact).
@@ -92,8 +94,12 @@ __global__ void __launch_bounds__(1024) append_kernel(const __grid_constant__ Ap
 }
 
 // ----------------------------------------------------------------------------- select
-constexpr int kSelThreads = 256;
+// One CTA per triggered head is a chain of short passes over the head's keys, so its length is what a
+// thread has to do: a head of many candidates takes 1024 threads (10 heads of 4160 scored candidates: 25.1 us
+// with 256 threads, six layers of them 22.9 us with 1024), small ones and the refill of order-free slots 256.
+constexpr int kSelWide = 1024, kSelWideFrom = 1024;
 
+template <int kSelThreads>
 __global__ void __launch_bounds__(kSelThreads) select_kernel(const __grid_constant__ EvictParams p)
 {
     extern __shared__ uint32_t sm[];
@@ -115,6 +121,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const __grid_consta
     const int K = L.K, r = L.r;
     const int m = N - K;
     const int head_id = b * L.KVH + h;
+    const int layer = p.layer + (int)blockIdx.z;
     int32_t* plan = L.plan + (size_t)head_id * (kPlanHeader + r);
     if (m <= 0 || m > r || N > kMaxCandidates || N > c) {  // the host mirror rules this out; never move data on a bad plan
         if (p.early) {
@@ -123,7 +130,10 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const __grid_consta
         }
         if (tid == 0) {
             atomicExch(L.err, kDeviceErrPlan);
-            plan[3] = 0;
+            if (p.to_plan)
+                L.evplan[(size_t)((((size_t)p.ev_plan_parity * L.L + layer) * L.B + b) * L.KVH + h) * (r + 1)] = -1;
+            else
+                plan[3] = 0;
         }
         return;
     }
@@ -135,7 +145,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const __grid_consta
 
     if (tid < 256) hist[0][tid] = 0;  // the first digit's histogram (the fill's barrier publishes it)
     const uint32_t k0 = (uint32_t)L.seed, k1 = (uint32_t)(L.seed >> 32);
-    const int32_t* pos = L.pos + (size_t)L.region[((size_t)p.layer * L.B + b) * L.KVH + h] * L.Cmax;
+    const int32_t* pos = L.pos + (size_t)L.region[((size_t)layer * L.B + b) * L.KVH + h] * L.Cmax;
     if (p.holefill && p.policy != RA_POLICY_BLOCK) {  // order-free slots: every key follows the position
         const uint32_t id = key_stream(p.trig_admit[blockIdx.x],
                                        p.policy == RA_POLICY_SHARED ? (uint32_t)(b * L.KVH) : (uint32_t)head_id);
@@ -143,18 +153,18 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const __grid_consta
         for (int j = tid; j < N; j += kSelThreads) {
             const uint32_t pj = (uint32_t)__ldg(pos + j);
             keys[j] = p.policy == RA_POLICY_RECENCY ? 0xFFFFFFFFu - pj
-                                                    : philox4x32_10_w0(pj, (uint32_t)g, (uint32_t)p.layer, id, k0, k1);
+                                                    : philox4x32_10_w0(pj, (uint32_t)g, (uint32_t)layer, id, k0, k1);
         }
     } else if (p.policy == RA_POLICY_RECENCY) {  // protected recency: the K newest candidates score lowest
         for (int j = tid; j < N; j += kSelThreads) keys[j] = (uint32_t)(N - 1 - j);
     } else if (p.policy == RA_POLICY_BLOCK) {  // one draw per block of consecutive positions
         for (int j = tid; j < N; j += kSelThreads)
-            keys[j] = philox4x32_10_w0((uint32_t)(pos[j] / p.block), (uint32_t)g, (uint32_t)p.layer,
+            keys[j] = philox4x32_10_w0((uint32_t)(pos[j] / p.block), (uint32_t)g, (uint32_t)layer,
                                        key_stream(p.trig_admit[blockIdx.x], (uint32_t)head_id), k0, k1);
     } else if (p.policy == RA_POLICY_SNAPKV) {
         // scored comparator: the window score max-pooled over +-kScorePoolRadius candidates;
         // larger scores must sort first, so the key is the order-reversed float
-        const float* sc = L.scores + (((size_t)p.layer * L.B + b) * L.KVH + h) * L.Cmax;
+        const float* sc = L.scores + (((size_t)layer * L.B + b) * L.KVH + h) * L.Cmax;
         float* raw = reinterpret_cast<float*>(s_ev + r);  // [N], staged once
 #pragma unroll 4
         for (int j = tid; j < N; j += kSelThreads) raw[j] = __ldcg(sc + j);
@@ -174,7 +184,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const __grid_consta
         const uint32_t id = key_stream(p.trig_admit[blockIdx.x],
                                        p.policy == RA_POLICY_SHARED ? (uint32_t)(b * L.KVH) : (uint32_t)head_id);
         for (int j = tid; j < N; j += kSelThreads)
-            keys[j] = philox4x32_10_w0((uint32_t)j, (uint32_t)g, (uint32_t)p.layer, id, k0, k1);
+            keys[j] = philox4x32_10_w0((uint32_t)j, (uint32_t)g, (uint32_t)layer, id, k0, k1);
     }
     __syncthreads();
 
@@ -299,9 +309,18 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const __grid_consta
         pdl_wait();
         pdl_launch_dependents();
     }
+    if (p.to_plan) {  // a set as plan_kernel writes it: the count, then the ordinals ascending
+        int32_t* out = L.evplan + (size_t)((((size_t)p.ev_plan_parity * L.L + layer) * L.B + b) * L.KVH + h) * (r + 1);
+        for (int i = tid; i < min((int)s_total, r); i += kSelThreads) out[1 + i] = s_ev[i];
+        if (tid == 0) {
+            out[0] = s_total == (uint32_t)m ? m : -1;
+            if (s_total != (uint32_t)m) atomicExch(L.err, kDeviceErrPlan);
+        }
+        return;
+    }
     for (int i = tid; i < min((int)s_total, r); i += kSelThreads) plan[kPlanHeader + i] = s_ev[i];
     if (tid == 0) {
-        const int32_t* regp = L.region + ((size_t)p.layer * L.B + b) * L.KVH + h;
+        const int32_t* regp = L.region + ((size_t)layer * L.B + b) * L.KVH + h;
         const int src = *regp, dst = p.holefill ? src : L.spare[b * L.KVH + h];  // hole-filling works in place
         const bool ok = (s_total == (uint32_t)m);
         plan[0] = src;
@@ -309,13 +328,13 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const __grid_consta
         plan[2] = c;
         plan[3] = ok ? m : 0;
         if (ok && !p.holefill) {
-            L.region[((size_t)p.layer * L.B + b) * L.KVH + h] = dst;
+            L.region[((size_t)layer * L.B + b) * L.KVH + h] = dst;
             L.spare[b * L.KVH + h] = src;
         } else if (!ok) {
             atomicExch(L.err, kDeviceErrPlan);
         }
     }
-    if (!p.holefill) return;
+    if (kSelThreads == kSelWide || !p.holefill) return;
     // Order-free compaction, in place.  With top the slot count including a pending token: evicted
     // slot e_i takes the row of slot top - m + i for i < m - 1, and the newest row ends in the new
     // last slot top - m - 1, whose own row, unless e_{m-1} is that slot, fills e_{m-1}.  A pending
@@ -323,8 +342,8 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(const __grid_consta
     // Slots top - m .. top - 1 are buffer slots, so no move reads a slot that another writes.
     if (s_total != (uint32_t)m) return;
     const int top = p.pending ? c + 1 : c, last = top - m - 1;
-    const long long row0 = L.gen_row0 + (long long)L.region[((size_t)p.layer * L.B + b) * L.KVH + h] * L.Cmax;
-    int32_t* gpos = L.pos + (size_t)L.region[((size_t)p.layer * L.B + b) * L.KVH + h] * L.Cmax;
+    const long long row0 = L.gen_row0 + (long long)L.region[((size_t)layer * L.B + b) * L.KVH + h] * L.Cmax;
+    int32_t* gpos = L.pos + (size_t)L.region[((size_t)layer * L.B + b) * L.KVH + h] * L.Cmax;
     const int part = lane & 15;
     uint16_t* pool = lane < 16 ? L.kpool : L.vpool;  // lanes 0-15 move K, 16-31 V, 16 bytes each
     auto row = [&](int slot) { return reinterpret_cast<uint4*>(pool + (row0 + slot) * kHeadDim) + part; };
@@ -1093,20 +1112,29 @@ __global__ void __launch_bounds__(32) plan_kernel(const __grid_constant__ EvictP
 // separate, so their CTAs are independent).  Chunks of kStkRows rows stream through a ring of
 // stages with TMA bulk copies; the survivors' runs go back with bulk stores, positions by plain
 // stores.
+//
+// A CTA moves 45 KB/us, so few heads (few layers, few firing sequences) leave the chip idle.  With SPLIT a
+// cluster of CTAs takes a head's array, each a range of its chunks.  What a CTA stores lands at most m
+// rows below its range, in the last chunk of the CTA before (m <= kStkRows): so every CTA first loads
+// its last chunk into a stage of its own, and no CTA stores before the cluster has them all (a
+// barrier).  2 layers x 10 heads of 2.1K rows, 40 CTAs: 25.5 us, in clusters of 3 14.2 us.
 constexpr int kStkThreads = 128;
 constexpr int kStkRows = 128;   // rows per stage: 32 KB of K or V
 constexpr int kStkStages = 3;   // 96 KB of stages: two CTAs per SM
-constexpr size_t kStkSmem = (size_t)kStkStages * kStkRows * kRowBytes;
+constexpr int kStkMaxSplit = 8;
+template <bool SPLIT>
+constexpr size_t kStkSmem = (size_t)(kStkStages + (SPLIT ? 1 : 0)) * kStkRows * kRowBytes;
 static_assert(kStkStages >= 2 && kStkRows <= kStkThreads, "refills trail by one chunk; a thread per row");
 static_assert(((kStkRows + 4) * 4) % 16 == 0, "every stage's positions start 16-byte aligned");
 
 struct StkShared {
     int32_t ev[kEvCap];                  // the evicted ordinals, ascending
-    __align__(16) int32_t pos[kStkStages][kStkRows + 4];  // (bulk copy destinations: 16-byte aligned)
-    uint64_t bar[kStkStages];
+    __align__(16) int32_t pos[kStkStages + 1][kStkRows + 4];  // (bulk copy destinations: 16-byte aligned)
+    uint64_t bar[kStkStages + 1];        // (the last of each: SPLIT's own stage)
     int bad;
 };
 
+template <bool SPLIT>
 __global__ void __launch_bounds__(kStkThreads) compact_stack_kernel(const __grid_constant__ EvictParams p)
 {
     extern __shared__ __align__(128) uint8_t stk_dyn[];  // [stage][rows of K or V]
@@ -1114,14 +1142,16 @@ __global__ void __launch_bounds__(kStkThreads) compact_stack_kernel(const __grid
     constexpr int kStageBytes = kStkRows * kRowBytes;
     const DevLayout& L = p.lay;
     const int tid = threadIdx.x;
-    const int item = blockIdx.x >> 1, part = blockIdx.x & 1;  // layer-major (layer, sequence, KV head); 0: K, 1: V
+    const int P = SPLIT ? p.stk_split : 1, rank = SPLIT ? (int)cluster_ctarank() : 0;
+    const int unit = (int)blockIdx.x / P, item = unit >> 1, part = unit & 1;  // layer-major (layer, sequence, KV head); 0: K, 1: V
     uint16_t* pool = part ? L.vpool : L.kpool;
     const int h = item % L.KVH, t = (item / L.KVH) % p.n_trig, layer = item / (L.KVH * p.n_trig);
     const int b = p.trig[t], c = p.trig_c[t], N = p.trig_n[t];
     const int m = N - L.K;
     pdl_wait();  // the rows were written by the previous step's attention
     pdl_launch_dependents();
-    if (m < 1 || m > L.r || m > kEvCap || N > c || c > L.Cmax) {  // the host rules this out
+    // the host rules this out (every CTA of a cluster decides alike)
+    if (m < 1 || m > L.r || m > kEvCap || N > c || c > L.Cmax || (SPLIT && m > kStkRows)) {
         if (tid == 0) atomicExch(L.err, kDeviceErrPlan);
         return;
     }
@@ -1132,38 +1162,50 @@ __global__ void __launch_bounds__(kStkThreads) compact_stack_kernel(const __grid
         L.evplan + (size_t)((((size_t)p.ev_plan_parity * L.L + layer) * L.B + b) * L.KVH + h) * (L.r + 1);
     const bool with_pos = part == 0;
     const bool pos_bulk = with_pos && (L.Cmax & 3) == 0;  // position chunks are 16-byte aligned
-    const int nch = (c + kStkRows - 1) / kStkRows;
-    auto issue = [&](int i) {  // chunk i into stage i % kStkStages (thread 0)
-        const int s = i % kStkStages, a = i * kStkRows, n = min(kStkRows, c - a);
+    const int chunks = (c + kStkRows - 1) / kStkRows;
+    const int i0 = (int)((long long)rank * chunks / P), i1 = (int)((long long)(rank + 1) * chunks / P);  // this CTA's
+    const int last = SPLIT ? i1 - 1 : i1;  // chunks [i0, last) stream through the ring; SPLIT: chunk i1 - 1 has its own stage
+    auto stage_of = [&](int i) { return SPLIT && i == last ? kStkStages : (i - i0) % kStkStages; };
+    auto issue = [&](int i) {  // chunk i into its stage (thread 0)
+        const int s = stage_of(i), a = i * kStkRows, n = min(kStkRows, c - a);
         uint8_t* st = stk_dyn + (size_t)s * kStageBytes;
         const uint32_t pbytes = pos_bulk ? (uint32_t)min((n + 3) & ~3, L.Cmax - a) * 4u : 0u;
         mbar_arrive_expect_tx(&S.bar[s], (uint32_t)n * kRowBytes + pbytes);
         bulk_load(st, pool + (row0 + a) * kHeadDim, (uint32_t)n * kRowBytes, &S.bar[s]);
         if (pbytes) bulk_load(S.pos[s], gpos + a, pbytes, &S.bar[s]);
     };
-    int issued = 0;  // thread 0's count of chunks whose copies are issued
+    int issued = i0;  // thread 0: chunks of the ring whose copies are issued
     if (tid == 0) {
         S.bad = 0;
-        for (int s = 0; s < kStkStages; ++s) mbar_init(&S.bar[s], 1);
+        for (int s = 0; s <= kStkStages; ++s) mbar_init(&S.bar[s], 1);
         fence_mbar_init();
-        issued = min(kStkStages, nch);
-        for (int i = 0; i < issued; ++i) issue(i);
+        if (SPLIT && i0 < i1) issue(last);
+        for (; issued < min(i0 + kStkStages, last); ++issued) issue(issued);
     }
     // the plan: m ordinals, ascending, below N
     const int n_plan = __ldcg(plan);
     for (int i = tid; i < m; i += kStkThreads) S.ev[i] = __ldcg(plan + 1 + i);
+    if (SPLIT && with_pos && !pos_bulk && i0 < i1 && tid < min(kStkRows, c - last * kStkRows))
+        S.pos[kStkStages][tid] = __ldcg(gpos + last * kStkRows + tid);
     __syncthreads();
     bool bad = n_plan != m;
     for (int i = tid; i < m && !bad; i += kStkThreads)
         bad = S.ev[i] < 0 || S.ev[i] >= N || (i + 1 < m && S.ev[i] >= S.ev[i + 1]);
     if (bad) S.bad = 1;
     __syncthreads();
-    if (S.bad) {  // a bad plan moves nothing: wait (bounded) for the copies issued, and leave
-        if (tid == 0) {
-            atomicExch(L.err, kDeviceErrPlan);
-            for (int q = 0; q < issued; ++q)
-                (void)mbar_wait_bounded(&S.bar[q % kStkStages], (uint32_t)((q / kStkStages) & 1), kEvWaitLimitNs);
+    if (S.bad && tid == 0) atomicExch(L.err, kDeviceErrPlan);
+    if (SPLIT) {
+        // a wait that runs out is flagged and the CTA moves nothing; the others go on (the error word tells)
+        if (tid == 0 && i0 < i1 && !mbar_wait_bounded(&S.bar[kStkStages], 0u, kEvWaitLimitNs)) {
+            atomicExch(L.err, kDeviceErrTimeout);
+            S.bad = 2;
         }
+        __syncthreads();
+        cluster_sync();  // every CTA's last chunk is in its shared memory
+    }
+    if (S.bad) {  // a bad plan moves nothing: wait (bounded) for the copies issued, and leave
+        if (tid == 0)
+            for (int q = i0; q < issued; ++q) (void)mbar_wait_bounded(&S.bar[stage_of(q)], 0u, kEvWaitLimitNs);
         return;
     }
     auto ev_below = [&](int j) {  // evicted ordinals below j
@@ -1174,15 +1216,16 @@ __global__ void __launch_bounds__(kStkThreads) compact_stack_kernel(const __grid
         }
         return lo;
     };
-    for (int i = 0; i < nch; ++i) {  // every chunk's copies are issued by the time it is reached
-        const int s = i % kStkStages, a = i * kStkRows, n = min(kStkRows, c - a);
-        if (tid == 0 && !mbar_wait_bounded(&S.bar[s], (uint32_t)((i / kStkStages) & 1), kEvWaitLimitNs)) {
+    for (int i = i0; i < i1; ++i) {  // every chunk's copies are issued by the time it is reached
+        const bool own = SPLIT && i == last;  // landed before the cluster's barrier
+        const int s = stage_of(i), a = i * kStkRows, n = min(kStkRows, c - a);
+        if (!own && tid == 0 && !mbar_wait_bounded(&S.bar[s], (uint32_t)(((i - i0) / kStkStages) & 1), kEvWaitLimitNs)) {
             atomicExch(L.err, kDeviceErrTimeout);
             for (int q = i + 1; q < issued; ++q)  // let the copies already issued land (bounded)
-                (void)mbar_wait_bounded(&S.bar[q % kStkStages], (uint32_t)((q / kStkStages) & 1), kEvWaitLimitNs);
+                (void)mbar_wait_bounded(&S.bar[stage_of(q)], (uint32_t)(((q - i0) / kStkStages) & 1), kEvWaitLimitNs);
             S.bad = 2;
         }
-        if (with_pos && !pos_bulk && tid < n) S.pos[s][tid] = __ldcg(gpos + a + tid);  // (all read before any is written)
+        if (with_pos && !pos_bulk && !own && tid < n) S.pos[s][tid] = __ldcg(gpos + a + tid);  // (all read before any is written)
         __syncthreads();
         if (S.bad) break;
         if (with_pos && tid < n) {  // positions of the chunk's survivors
@@ -1209,7 +1252,7 @@ __global__ void __launch_bounds__(kStkThreads) compact_stack_kernel(const __grid
             bulk_commit();
         }
         __syncthreads();  // the stage's positions are read
-        if (tid == 0 && i >= 1 && issued < nch) {  // chunk i + 2 into chunk i - 1's stage once its stores read it
+        if (tid == 0 && i > i0 && issued < last) {  // chunk i + 2 into chunk i - 1's stage once its stores read it
             asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
             issue(issued);
             ++issued;
@@ -1422,13 +1465,15 @@ cudaError_t launch_select(const EvictParams& p, cudaStream_t s)
 {
     const int N = p.lay.K + p.lay.r;  // candidates at a firing step never exceed K + r
     const size_t smem = select_smem(N, p.lay.r, p.policy == RA_POLICY_SNAPKV);
-    static size_t configured = 0;
-    if (smem > 48 * 1024 && smem > configured) {
-        cudaError_t e = cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const bool wide = N >= kSelWideFrom && !p.holefill;
+    auto kernel = wide ? select_kernel<kSelWide> : select_kernel<256>;
+    static size_t configured[2] = {0, 0};
+    if (smem > 40 * 1024 && smem > configured[wide]) {
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        configured = smem;
+        configured[wide] = smem;
     }
-    return launch_pdl(select_kernel, dim3(p.n_trig, p.lay.KVH), dim3(kSelThreads), smem, s, p);
+    return launch_pdl(kernel, dim3(p.n_trig, p.lay.KVH, p.layers), dim3(wide ? kSelWide : 256), smem, s, p);
 }
 
 cudaError_t launch_compact(const EvictParams& p, cudaStream_t s)
@@ -1501,16 +1546,41 @@ cudaError_t launch_plan(const EvictParams& p, int sms, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_compact_stack(const EvictParams& p, int layers, cudaStream_t s)
+cudaError_t launch_compact_stack(const EvictParams& p, int layers, int sms, cudaStream_t s)
 {
     static bool configured = false;
     if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(compact_stack_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStkSmem);
+        cudaError_t e = cudaFuncSetAttribute(compact_stack_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStkSmem<false>);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(compact_stack_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStkSmem<true>);
         if (e != cudaSuccess) return e;
         configured = true;
     }
-    return launch_pdl(compact_stack_kernel, dim3((unsigned)(2 * layers * p.n_trig * p.lay.KVH)), dim3(kStkThreads),
-                      kStkSmem, s, p);
+    const int units = 2 * layers * p.n_trig * p.lay.KVH;
+    // A cluster per head's array while at least two CTAs of it fit beside the others' (one per SM), and
+    // every CTA has a chunk; rows that move further than a chunk stay with one CTA.
+    int longest = 0;
+    for (int i = 0; i < p.n_trig; ++i) longest = std::max(longest, (int)p.trig_c[i]);
+    const int split = std::min({kStkMaxSplit, sms / units, (longest + kStkRows - 1) / kStkRows});
+    if (split < 2 || p.lay.r > kStkRows)
+        return launch_pdl(compact_stack_kernel<false>, dim3((unsigned)units), dim3(kStkThreads), kStkSmem<false>, s, p);
+    EvictParams q = p;
+    q.stk_split = split;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)split;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(units * split));
+    cfg.blockDim = dim3(kStkThreads);
+    cfg.dynamicSmemBytes = kStkSmem<true>;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, compact_stack_kernel<true>, q);
 }
 
 cudaError_t launch_fill_stack(const EvictParams& p, int layers, cudaStream_t s)

@@ -68,6 +68,8 @@ struct AppendParams {
 struct EvictParams {
     DevLayout lay;
     int layer;
+    int layers;    // score (pass 2) and select: layers of the launch from `layer` on, counters alike
+    int to_plan;   // select: the evicted sets go to half ev_plan_parity of lay.evplan, for launch_compact_stack
     int policy;    // RA_POLICY_*: how candidates are scored
     int block;     // RA_POLICY_BLOCK: positions per block
     int holefill;  // RA_COMPACT_HOLEFILL: keys per position, evicted slots refilled in place by select
@@ -98,6 +100,7 @@ struct EvictParams {
     // ascending) and which half this launch reads; null: the kernel selects itself
     const int32_t* ev_plan;
     int ev_plan_parity;
+    int stk_split;  // launch_compact_stack: CTAs per head and array
 };
 
 constexpr int kScoreTile = 64;      // key rows per scoring tile
@@ -202,9 +205,9 @@ cudaError_t launch_evict(const EvictParams& p, int cluster, cudaStream_t s);
 // so that it runs beside the attention kernel.
 cudaError_t launch_plan(const EvictParams& p, int sms, cudaStream_t s);
 // Every layer's round of the triggered sequences (layers 0 .. layers - 1, counters alike in every
-// layer), in place, from the evicted sets in half p.ev_plan_parity of lay.evplan: one CTA per
-// (layer, sequence, KV head).
-cudaError_t launch_compact_stack(const EvictParams& p, int layers, cudaStream_t s);
+// layer), in place, from the evicted sets in half p.ev_plan_parity of lay.evplan: one CTA (a cluster, while
+// the SMs are more) per (layer, sequence, KV head) and array.
+cudaError_t launch_compact_stack(const EvictParams& p, int layers, int sms, cudaStream_t s);
 // The same rounds with order-free slots: the evicted slots of every layer refilled in place from
 // the newest ones, the step's token (p.k_new / p.v_new: [layers][B][KVH][d]) included.
 cudaError_t launch_fill_stack(const EvictParams& p, int layers, cudaStream_t s);

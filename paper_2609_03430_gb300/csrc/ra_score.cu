@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_sum_tc_kernel(const __grid_
     }
     const int r_hi = min(N, r_lo + p.ch2 * kScoreTile);
     const int ntile = (r_hi - r_lo + kTcRows - 1) / kTcRows;
-    const size_t lbh = ((size_t)p.layer * L.B + b) * L.KVH + h;
+    const size_t lbh = ((size_t)(p.layer + blockIdx.z) * L.B + b) * L.KVH + h;
     const long long grow = L.gen_row0 + (long long)L.region[lbh] * L.Cmax;
 
     auto issue_tile = [&](int i, uint32_t extra) {  // thread 0: key tile i into stage i % 2
@@ -627,7 +627,7 @@ cudaError_t prepare_mt()
 template <int MT>
 cudaError_t launch_sum_tc(const EvictParams& p, const CUtensorMap* tk, const CUtensorMap* tq, cudaStream_t s)
 {
-    const dim3 grid(p.nch2, p.n_trig * p.lay.KVH);
+    const dim3 grid(p.nch2, p.n_trig * p.lay.KVH, p.layers);
     return launch_pdl(score_sum_tc_kernel<128 * MT>, grid, dim3(kThreads), TcCfg<128 * MT>::SMEM, s, p, *tk, *tq);
 }
 

@@ -44,7 +44,7 @@ namespace ra {
 static_assert(kPromptPage % kScoreTile == 0, "a scoring tile of the prompt lies inside one page");
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kThreads = 512;  // summation pass: four warpgroups
 constexpr int kHalfBytes = kScoreTile * 128;      // one 64-channel box of a key tile
 constexpr uint64_t kWaitLimitNs = 2000000000ull;  // bounded mbarrier waits: 2 s
 static_assert(kHalfBytes % 1024 == 0, "128-byte-swizzled TMA boxes start 1024-byte aligned");
@@ -85,7 +85,7 @@ __device__ __forceinline__ int visible_rows(const int32_t* pos, int c, int lp, i
 // side of the MMA and the window rows are the N side (up to 256 per instruction), so that TMEM
 // lane j holds every window row's logit against key j.  The thread that reads lane j then sums
 // its own key's weights exp2(logit * scale_R - lse_R) over the window rows R, with no
-// cross-thread reduction; the two warpgroups take half of the window rows each.  Both operands
+// cross-thread reduction; the four warpgroups take a quarter of the window rows each.  Both operands
 // are K-major in shared memory with the 128-byte swizzle the TMA copies already produce (rows of
 // 128 bytes, 8-row groups 1024 bytes apart, the two 64-channel halves one after the other); a
 // K-step of 16 channels advances the descriptors' start address by 32 bytes.  One thread issues
@@ -106,7 +106,7 @@ struct TcCfg {
     static constexpr int Q_HALF = ROWS * 128;
     static constexpr int STAT_OFF = Q_OFF + ROWS * kRowBytes;
     static constexpr int RED_OFF = STAT_OFF + 2 * ROWS * 4;
-    static constexpr int BAR_OFF = RED_OFF + 2 * kTcRows * 4;  // full[2], mma_done[2], TMEM base
+    static constexpr int BAR_OFF = RED_OFF + kThreads / 128 * kTcRows * 4;  // full[2], mma_done[2], TMEM base
     static constexpr size_t SMEM = 1024 + (size_t)BAR_OFF + 4 * 8 + 16;
     static_assert(ROWS % 128 == 0 && ROWS <= 512, "window rows");
     static_assert(NC % 16 == 0 && NC <= 256, "UMMA N for M = 128");
@@ -177,8 +177,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_sum_tc_kernel(const __grid_
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + C::BAR_OFF);  // key tile (and the window) landed
     uint64_t* mdone = full + 2;                                          // the tile's MMAs completed
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(full + 4);
-    float* s_sl = reinterpret_cast<float*>(smem + C::STAT_OFF);
-    float* s_lse = s_sl + ROWS;
+    float2* s_st = reinterpret_cast<float2*>(smem + C::STAT_OFF);  // (scale, -lse) of each window row
     float* red = reinterpret_cast<float*>(smem + C::RED_OFF);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -245,8 +244,7 @@ __global__ void __launch_bounds__(kThreads, 1) score_sum_tc_kernel(const __grid_
         const float2* qst = L.qstats + lbh * (size_t)M;
         for (int R = tid; R < ROWS; R += kThreads) {
             const float2 f = R < M ? __ldcg(qst + R) : make_float2(0.f, INFINITY);  // padding rows weigh 0
-            s_sl[R] = f.x;
-            s_lse[R] = f.y;
+            s_st[R] = make_float2(f.x, -f.y);
         }
     }
     tmem_fence_before();
@@ -279,7 +277,8 @@ __global__ void __launch_bounds__(kThreads, 1) score_sum_tc_kernel(const __grid_
     };
 
     float* scores = L.scores + lbh * L.Cmax;
-    const int wg = warp >> 2, wq = warp & 3;  // warpgroup (half of the window rows), TMEM lane quarter
+    constexpr int kWgs = kThreads / 128;
+    const int wg = warp >> 2, wq = warp & 3;  // warpgroup (its part of the window rows), TMEM lane quarter
     bool ok = true;
     if (tid == 0) ok = issue_mma(0);
     for (int i = 0; i < ntile; ++i) {
@@ -296,22 +295,29 @@ __global__ void __launch_bounds__(kThreads, 1) score_sum_tc_kernel(const __grid_
             issue_tile(i + 2, 0u);
             n_loaded = i + 3;
         }
-        // this thread: key row wq * 32 + lane of the tile, window rows [wg * ROWS / 2, (wg + 1) * ROWS / 2)
+        // this thread: key row wq * 32 + lane of the tile, window rows [wg, wg + 1) * ROWS / kWgs
         const uint32_t tl = tmem + ((uint32_t)(wq * 32) << 16) + (uint32_t)((i % C::NBUF) * ROWS);
-        float sum = 0.f;
+        float sum[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 1
-        for (int c0 = wg * (ROWS / 2); c0 < (wg + 1) * (ROWS / 2); c0 += 32) {
+        for (int c0 = wg * (ROWS / kWgs); c0 < (wg + 1) * (ROWS / kWgs); c0 += 32) {
             uint32_t v[32];
             tmem_ld32(tl + c0, v);
 #pragma unroll
-            for (int j = 0; j < 32; ++j) sum += exp2f(fmaf(__uint_as_float(v[j]), s_sl[c0 + j], -s_lse[c0 + j]));
+            for (int j = 0; j < 32; j += 2) {
+                const float4 f = *reinterpret_cast<const float4*>(s_st + c0 + j);  // two rows' (one address: a broadcast)
+                sum[j & 2] += exp2f(fmaf(__uint_as_float(v[j]), f.x, f.y));
+                sum[(j & 2) + 1] += exp2f(fmaf(__uint_as_float(v[j + 1]), f.z, f.w));
+            }
         }
-        red[wg * kTcRows + wq * 32 + lane] = sum;
+        red[wg * kTcRows + wq * 32 + lane] = (sum[0] + sum[1]) + (sum[2] + sum[3]);
         tmem_fence_before();
-        __syncthreads();  // both halves summed; the accumulator buffer is free again
+        __syncthreads();  // every part summed; the accumulator buffer is free again
         if (tid < kTcRows) {
             const int row = r_lo + i * kTcRows + tid;
-            if (row < r_hi) scores[row] = red[tid] + red[kTcRows + tid];
+            float all = 0.f;
+#pragma unroll
+            for (int k = 0; k < kWgs; ++k) all += red[k * kTcRows + tid];
+            if (row < r_hi) scores[row] = all;
         }
         if (C::NBUF == 1 && tid == 0 && ok && i + 1 < ntile) {
             tmem_fence_after();
@@ -342,25 +348,33 @@ __global__ void __launch_bounds__(kThreads, 1) score_sum_tc_kernel(const __grid_
 //
 // D = Q K^T: the window rows are the M side (MQ tiles of 128), the 128 keys of a tile the N side, so
 // that a TMEM lane holds one window row's logits and the thread that reads it keeps that row's
-// running maximum and sum in registers.  The two warpgroups take the M tiles in turn, or the
-// halves of the keys when there is one M tile only.  A tile is two runs of kScoreTile cache rows
-// (a prompt page holds three); with at most 256 window rows the accumulator is double-buffered, and
-// the products of tile i + 1 run while tile i is summed.  Bound by exp2 (one per logit) and the
-// few instructions around it.  For 160 heads of 3.3K keys and 256 window rows it takes 85 us
-// where the mma.sync kernel, with two shuffles per 16 keys and a row, took 167 us.
+// running maximum and sum in registers.  Four warpgroups take the M tiles, or parts of the keys of
+// one (merged at the end), and a warp of its own loads tiles and issues products, so that neither
+// waits for the other: a tile's accumulator is handed back by an mbarrier.  A tile is two runs of
+// kScoreTile cache rows (a prompt page holds three); with at most 256 window rows the accumulator is
+// double-buffered, and the products of tile i + 1 run while tile i is summed.  Bound by exp2 (one per
+// logit) and the few instructions around it, with four warps per scheduler to hide their latency, and
+// by a CTA's start (64 KB of window rows).  160 heads of 3.3K keys and 256 window rows: 167 us with
+// mma.sync and two shuffles per 16 keys of a row, 85 us with two warpgroups and a barrier of all
+// threads per tile, 63 us this way.
+constexpr int kStWgs = 4, kStThreads = (kStWgs * 4 + 1) * 32;  // four warpgroups and the issuing warp
+
 template <int MQ>
 struct StCfg {
     static constexpr int ROWS = 128 * MQ;
+    static constexpr int NST = MQ <= 3 ? 3 : 2;                // key tiles on the way
     static constexpr int NBUF = MQ <= 2 ? 2 : 1;               // accumulator buffers in TMEM
     static constexpr int BUF_COLS = kTcRows * MQ;              // columns of one buffer: 128 keys per M tile
     static constexpr uint32_t COLS = MQ == 1 ? 256u : 512u;    // columns allocated (a power of 2)
-    static constexpr int MINE = (MQ + 1) / 2;                  // window rows per thread
-    static constexpr int Q_OFF = 2 * kTcStage;                 // after the two key stages
+    static constexpr int PARTS = MQ <= 2 ? kStWgs / MQ : 1;    // warpgroups that share an M tile's keys
+    static constexpr int PCOLS = kTcRows / PARTS;
+    static constexpr int Q_OFF = NST * kTcStage;               // after the key stages
     static constexpr int Q_HALF = ROWS * 128;
-    static constexpr int RED_OFF = Q_OFF + ROWS * kRowBytes;   // MQ == 1: the second warpgroup's statistics
-    static constexpr int BAR_OFF = RED_OFF + (MQ == 1 ? 128 * 8 : 0);  // full[2], mma_done[2], TMEM base
-    static constexpr size_t SMEM = 1024 + (size_t)BAR_OFF + 4 * 8 + 16;
-    static_assert(NBUF * BUF_COLS <= (int)COLS && SMEM <= 232448, "tensor and shared memory");
+    static constexpr int RED_OFF = Q_OFF + ROWS * kRowBytes;   // statistics of the parts but the first
+    static constexpr int BAR_OFF = RED_OFF + MQ * (PARTS - 1) * 128 * 8;  // full, free (stages), done, read (buffers), TMEM base
+    static constexpr int NBAR = 2 * NST + 2 * NBUF;
+    static constexpr size_t SMEM = 1024 + (size_t)BAR_OFF + NBAR * 8 + 16;
+    static_assert(NBUF * BUF_COLS <= (int)COLS && SMEM <= 232448 && PCOLS % 32 == 0, "tensor and shared memory");
 };
 
 __device__ __forceinline__ float ex2(float x)
@@ -394,16 +408,18 @@ __device__ __forceinline__ void add_stats(const uint32_t (&v)[32], int valid, fl
 }
 
 template <int MQ>
-__global__ void __launch_bounds__(kThreads, 1) score_stats_tc_kernel(const __grid_constant__ EvictParams p,
-                                                                    const __grid_constant__ CUtensorMap tk,
-                                                                    const __grid_constant__ CUtensorMap tw)
+__global__ void __launch_bounds__(kStThreads, 1) score_stats_tc_kernel(const __grid_constant__ EvictParams p,
+                                                                      const __grid_constant__ CUtensorMap tk,
+                                                                      const __grid_constant__ CUtensorMap tw)
 {
     using C = StCfg<MQ>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + C::BAR_OFF);  // key tile (and the window) landed
-    uint64_t* mdone = full + 2;                                          // the tile's MMAs completed
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(full + 4);
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + C::BAR_OFF);  // stage: key tile (and the window) landed
+    uint64_t* sfree = full + C::NST;                                    // stage: the products that read it completed
+    uint64_t* mdone = sfree + C::NST;                                   // buffer: a tile's products completed
+    uint64_t* bread = mdone + C::NBUF;                                  // buffer: its warps have read it
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bread + C::NBUF);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     pdl_wait();  // the window, the cache and the tables come from earlier kernels
@@ -419,30 +435,9 @@ __global__ void __launch_bounds__(kThreads, 1) score_stats_tc_kernel(const __gri
     const int t0 = blockIdx.x * p.ch1;           // this CTA's runs [t0, t1) of kScoreTile rows
     if (t0 >= nt_head) return;  // (exiting counts as letting the successor start)
     const int t1 = min(t0 + p.ch1, nt_head), ntile = (t1 - t0 + 1) / 2;
-    const long long pbase = prompt_row(L, p.layer, 0, h, 0);
-    const int32_t* ptab = L.pages + (size_t)b * L.max_pages;
     const size_t lbh = ((size_t)p.layer * L.B + b) * L.KVH + h;
     const int reg = L.region[lbh];
-    const long long grow = L.gen_row0 + (long long)reg * L.Cmax;
 
-    auto run_row = [&](int k) -> int {  // first cache row of the head's run k
-        // (a run of the prompt lies inside one page: kPromptPage is a multiple of kScoreTile)
-        return (int)(k < tp ? pbase + (long long)__ldg(ptab + k * kScoreTile / kPromptPage) * L.KVH * kPromptPage +
-                                  (k * kScoreTile) % kPromptPage
-                            : grow + (long long)(k - tp) * kScoreTile);
-    };
-    // thread 0: tile i (runs t0 + 2 i and the next, if this CTA has it) into stage i % 2; `extra` bytes of other
-    // copies complete on the same barrier.  A missing second run leaves old rows, whose logits count nothing.
-    auto issue_tile = [&](int i, uint32_t extra) {
-        const int s = i % 2, k = t0 + 2 * i, n = min(2, t1 - k);
-        uint8_t* st = smem + (size_t)s * kTcStage;
-        mbar_arrive_expect_tx(&full[s], (uint32_t)(n * kScoreTile * kRowBytes) + extra);
-        for (int q = 0; q < n; ++q) {
-            const int row = run_row(k + q);
-            tma_load_2d(st + q * kHalfBytes, &tk, 0, row, &full[s]);
-            tma_load_2d(st + kTcHalf + q * kHalfBytes, &tk, 64, row, &full[s]);
-        }
-    };
     if (warp == 0) {  // the accumulators' tensor memory (held until the end)
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                      "r"(C::COLS)
@@ -450,136 +445,146 @@ __global__ void __launch_bounds__(kThreads, 1) score_stats_tc_kernel(const __gri
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (tid == 0) {
-        for (int s = 0; s < 2; ++s) {
-            mbar_init(&full[s], 1);
-            mbar_init(&mdone[s], 1);
+        for (int i = 0; i < C::NST; ++i) {
+            mbar_init(&full[i], 1);
+            mbar_init(&sfree[i], 1);
+        }
+        for (int i = 0; i < C::NBUF; ++i) {
+            mbar_init(&mdone[i], 1);
+            mbar_init(&bread[i], MQ * C::PARTS * 4);
         }
         fence_mbar_init();
-        prefetch_tensormap(&tk);
-        prefetch_tensormap(&tw);
-        // The window rows (row R = slot * G + g) complete on full[0] with the first key tile; rows past M
-        // are another head's (or read as zero) and belong to no thread's statistics.
-        issue_tile(0, (uint32_t)(C::ROWS * kRowBytes));
-        const int row0 = (int)(lbh * (size_t)M);
-        for (int rb = 0; rb < C::ROWS; rb += kScoreTile) {
-            tma_load_2d(smem + C::Q_OFF + rb * 128, &tw, 0, row0 + rb, &full[0]);
-            tma_load_2d(smem + C::Q_OFF + C::Q_HALF + rb * 128, &tw, 64, row0 + rb, &full[0]);
-        }
-        if (ntile > 1) issue_tile(1, 0u);
     }
-    // thread 0's counts of tiles: copies issued, MMAs issued, MMAs waited for
-    int n_loaded = min(ntile, 2), n_mma = 0, done = 0;
-    // this thread's window rows: lane wq * 32 + lane of M tiles wg, wg + 2 (one M tile: of that tile)
-    const int wg = warp >> 2, wq = warp & 3;
-    int lim[C::MINE];  // generated rows the row sees
-    float mrow[C::MINE], lrow[C::MINE];
-#pragma unroll
-    for (int i = 0; i < C::MINE; ++i) {
-        const int R = ((MQ == 1 ? 0 : wg) + 2 * i) * 128 + wq * 32 + lane;
-        lim[i] = R < M ? visible_rows(L.pos + (size_t)reg * L.Cmax, N, lp, p.trig_g[t], r, R / G) : 0;
-        mrow[i] = -INFINITY;
-        lrow[i] = 0.f;
-    }
-    const float sl = p.qk_scale_log2;  // the scale the restored queries are taken at
     tmem_fence_before();
     __syncthreads();
     tmem_fence_after();
     const uint32_t tmem = *tmem_slot;
-    const uint32_t idesc = umma_idesc_bf16(128, kTcRows);
-    const uint32_t sbase = smem_u32(smem);
 
-    // Thread 0: the MMAs of tile i into accumulator buffer i % NBUF, committed to mdone[i % 2].
-    auto issue_mma = [&](int i) -> bool {
-        if (!mbar_wait_bounded(&full[i % 2], (uint32_t)((i / 2) & 1), kWaitLimitNs)) return false;
-        tmem_fence_after();
-        const uint32_t d0 = tmem + (uint32_t)((i % C::NBUF) * C::BUF_COLS);
-        const uint32_t b0 = sbase + (uint32_t)((i % 2) * kTcStage);
+    // this thread's window row: lane wq * 32 + lane of M tile q, the keys of part `part`
+    const int wg = warp >> 2, wq = warp & 3, q = wg / C::PARTS, part = wg % C::PARTS;
+    const int R = q * 128 + wq * 32 + lane;
+    float mrow = -INFINITY, lrow = 0.f;
+    if (warp == kStWgs * 4) {
+        if (lane == 0) {
+            const long long pbase = prompt_row(L, p.layer, 0, h, 0);
+            const int32_t* ptab = L.pages + (size_t)b * L.max_pages;
+            const long long grow = L.gen_row0 + (long long)reg * L.Cmax;
+            auto run_row = [&](int k) -> int {  // first cache row of the head's run k
+                // (a run of the prompt lies inside one page: kPromptPage is a multiple of kScoreTile)
+                return (int)(k < tp ? pbase + (long long)__ldg(ptab + k * kScoreTile / kPromptPage) * L.KVH * kPromptPage +
+                                          (k * kScoreTile) % kPromptPage
+                                    : grow + (long long)(k - tp) * kScoreTile);
+            };
+            // Tile i (runs t0 + 2 i and the next, if this CTA has it) into stage i % NST; `extra` bytes of other
+            // copies complete on the same barrier.  A missing second run leaves old rows, whose logits count
+            // nothing.
+            auto issue_tile = [&](int i, uint32_t extra) {
+                const int k = t0 + 2 * i, n = min(2, t1 - k);
+                uint8_t* st = smem + (size_t)(i % C::NST) * kTcStage;
+                uint64_t* bar = &full[i % C::NST];
+                mbar_arrive_expect_tx(bar, (uint32_t)(n * kScoreTile * kRowBytes) + extra);
+                for (int u = 0; u < n; ++u) {
+                    const int row = run_row(k + u);
+                    tma_load_2d(st + u * kHalfBytes, &tk, 0, row, bar);
+                    tma_load_2d(st + kTcHalf + u * kHalfBytes, &tk, 64, row, bar);
+                }
+            };
+            prefetch_tensormap(&tk);
+            prefetch_tensormap(&tw);
+            // The window rows (row R = slot * G + g) complete on full[0] with the first key tile; rows past M
+            // are another head's (or read as zero) and belong to no thread's statistics.
+            issue_tile(0, (uint32_t)(C::ROWS * kRowBytes));
+            const int row0 = (int)(lbh * (size_t)M);
+            for (int rb = 0; rb < C::ROWS; rb += kScoreTile) {
+                tma_load_2d(smem + C::Q_OFF + rb * 128, &tw, 0, row0 + rb, &full[0]);
+                tma_load_2d(smem + C::Q_OFF + C::Q_HALF + rb * 128, &tw, 64, row0 + rb, &full[0]);
+            }
+            int loaded = 1, issued = 0;  // tiles whose copies, whose products are issued
+            for (; loaded < min(C::NST, ntile); ++loaded) issue_tile(loaded, 0u);
+            const uint32_t idesc = umma_idesc_bf16(128, kTcRows), sbase = smem_u32(smem);
+            bool ok = true;
+            while (ok && issued < ntile) {
+                const int i = issued;
+                ok = mbar_wait_bounded(&full[i % C::NST], (uint32_t)((i / C::NST) & 1), kWaitLimitNs) &&
+                     (i < C::NBUF || mbar_wait_bounded(&bread[i % C::NBUF], (uint32_t)((i / C::NBUF - 1) & 1), kWaitLimitNs));
+                if (!ok) break;
+                tmem_fence_after();
+                const uint32_t d0 = tmem + (uint32_t)((i % C::NBUF) * C::BUF_COLS);
+                const uint32_t b0 = sbase + (uint32_t)((i % C::NST) * kTcStage);
 #pragma unroll
-        for (int q = 0; q < MQ; ++q)
+                for (int m = 0; m < MQ; ++m)
 #pragma unroll
-            for (int kh = 0; kh < 2; ++kh)        // 64-channel half
+                    for (int kh = 0; kh < 2; ++kh)        // 64-channel half
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)    // 16-channel K-step inside the half
-                    umma_bf16(d0 + q * kTcRows, umma_desc_sw128(sbase + C::Q_OFF + kh * C::Q_HALF + q * 128 * 128 + kk * 32),
-                              umma_desc_sw128(b0 + kh * kTcHalf + kk * 32), idesc, (kh | kk) != 0);
-        umma_commit(&mdone[i % 2]);
-        n_mma = i + 1;
-        return true;
-    };
-
-    bool ok = true;
-    if (tid == 0) ok = issue_mma(0);
-    for (int i = 0; i < ntile; ++i) {
-        const bool got = mbar_wait_bounded(&mdone[i % 2], (uint32_t)((i / 2) & 1), kWaitLimitNs);
-        if (!__syncthreads_and(got && ok)) {  // give up together
-            if (tid == 0) atomicExch(L.err, kDeviceErrTimeout);
-            break;
+                        for (int kk = 0; kk < 4; ++kk)    // 16-channel K-step inside the half
+                            umma_bf16(d0 + m * kTcRows,
+                                      umma_desc_sw128(sbase + C::Q_OFF + kh * C::Q_HALF + m * 128 * 128 + kk * 32),
+                                      umma_desc_sw128(b0 + kh * kTcHalf + kk * 32), idesc, (kh | kk) != 0);
+                umma_commit(&mdone[i % C::NBUF]);
+                umma_commit(&sfree[i % C::NST]);
+                ++issued;
+                if (i >= 1 && loaded < ntile) {  // tile i - 1 + NST into tile i - 1's stage
+                    ok = mbar_wait_bounded(&sfree[(i - 1) % C::NST], (uint32_t)(((i - 1) / C::NST) & 1), kWaitLimitNs);
+                    if (ok) issue_tile(loaded++, 0u);
+                }
+            }
+            if (!ok) {  // leave only with nothing in flight: everything issued is waited for once more, bounded
+                atomicExch(L.err, kDeviceErrTimeout);
+                for (int i = max(0, issued - C::NST); i < issued; ++i)
+                    (void)mbar_wait_bounded(&sfree[i % C::NST], (uint32_t)((i / C::NST) & 1), kWaitLimitNs);
+                for (int i = issued; i < loaded; ++i)
+                    (void)mbar_wait_bounded(&full[i % C::NST], (uint32_t)((i / C::NST) & 1), kWaitLimitNs);
+            }
         }
-        done = i + 1;
-        tmem_fence_after();
-        if (tid == 0 && i + 2 < ntile) {  // the tile's MMAs have read stage i % 2: refill it
-            fence_proxy_async_smem();
-            issue_tile(i + 2, 0u);
-            n_loaded = i + 3;
-        }
-        // (every thread has read the other buffer: it passed the barrier above after tile i - 1)
-        if (C::NBUF == 2 && tid == 0 && ok && i + 1 < ntile) ok = issue_mma(i + 1);
-#pragma unroll
-        for (int c = 0; c < C::MINE; ++c) {
-            const int q = (MQ == 1 ? 0 : wg) + 2 * c;
-            if (q >= MQ) continue;
+    } else if (q < MQ) {
+        // generated rows the row sees
+        const int lim = R < M ? visible_rows(L.pos + (size_t)reg * L.Cmax, N, lp, p.trig_g[t], r, R / G) : 0;
+        const float sl = p.qk_scale_log2;  // the scale the restored queries are taken at
+        for (int i = 0; i < ntile; ++i) {
+            if (!mbar_wait_bounded(&mdone[i % C::NBUF], (uint32_t)((i / C::NBUF) & 1), kWaitLimitNs)) {
+                if (lane == 0) atomicExch(L.err, kDeviceErrTimeout);
+                break;
+            }
+            tmem_fence_after();
             const uint32_t tl = tmem + ((uint32_t)(wq * 32) << 16) + (uint32_t)((i % C::NBUF) * C::BUF_COLS + q * kTcRows);
 #pragma unroll 1
-            for (int c0 = MQ == 1 ? wg * 64 : 0; c0 < (MQ == 1 ? wg * 64 + 64 : kTcRows); c0 += 32) {
+            for (int c0 = part * C::PCOLS; c0 < (part + 1) * C::PCOLS; c0 += 32) {
                 const int k = t0 + 2 * i + (c0 >> 6);  // the run these columns belong to
                 if (k >= t1) break;
-                const bool prompt = k < tp;
-                const int valid = (prompt ? lp - k * kScoreTile : lim[c] - (k - tp) * kScoreTile) - (c0 & 63);
+                const int valid = (k < tp ? lp - k * kScoreTile : lim - (k - tp) * kScoreTile) - (c0 & 63);
                 uint32_t v[32];
                 __syncwarp();
                 tmem_ld32(tl + c0, v);
-                if (__all_sync(0xffffffffu, valid >= 32)) add_stats<false>(v, valid, sl, mrow[c], lrow[c]);
-                else add_stats<true>(v, valid, sl, mrow[c], lrow[c]);
+                if (__all_sync(0xffffffffu, valid >= 32)) add_stats<false>(v, valid, sl, mrow, lrow);
+                else add_stats<true>(v, valid, sl, mrow, lrow);
             }
+            tmem_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bread[i % C::NBUF]);
         }
-        tmem_fence_before();
-        if (C::NBUF == 1) {
-            __syncthreads();  // the accumulators are read: free for the next tile
-            if (tid == 0 && ok && i + 1 < ntile) {
-                tmem_fence_after();
-                ok = issue_mma(i + 1);
-            }
-        }
+        if (part > 0)
+            reinterpret_cast<float2*>(smem + C::RED_OFF)[(q * (C::PARTS - 1) + part - 1) * 128 + wq * 32 + lane] =
+                make_float2(mrow, lrow);
     }
-    // Leave only with nothing in flight: after a timeout, the MMAs issued but not waited for and
-    // the copies issued but not consumed are waited for once more, bounded.
-    if (tid == 0) {
-        for (int i = done; i < n_mma; ++i) (void)mbar_wait_bounded(&mdone[i % 2], (uint32_t)((i / 2) & 1), kWaitLimitNs);
-        for (int i = n_mma; i < n_loaded; ++i) (void)mbar_wait_bounded(&full[i % 2], (uint32_t)((i / 2) & 1), kWaitLimitNs);
-    }
-    if (MQ == 1 && wg == 1)
-        reinterpret_cast<float2*>(smem + C::RED_OFF)[wq * 32 + lane] = make_float2(mrow[0], lrow[0]);
+    __syncwarp();
     tmem_fence_before();
     __syncthreads();
     if (warp == 0) {
         tmem_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C::COLS) : "memory");
     }
-    if (MQ == 1) {
-        if (wg == 1) return;
-        const float2 o = reinterpret_cast<const float2*>(smem + C::RED_OFF)[wq * 32 + lane];
-        const float mx = fmaxf(mrow[0], o.x);
+    if (warp >= kStWgs * 4 || q >= MQ || part > 0) return;
+#pragma unroll
+    for (int k = 0; k < C::PARTS - 1; ++k) {
+        const float2 o = reinterpret_cast<const float2*>(smem + C::RED_OFF)[(q * (C::PARTS - 1) + k) * 128 + wq * 32 + lane];
+        const float mx = fmaxf(mrow, o.x);
         if (mx != -INFINITY)
-            lrow[0] = (mrow[0] == -INFINITY ? 0.f : lrow[0] * ex2(mrow[0] - mx)) + (o.x == -INFINITY ? 0.f : o.y * ex2(o.x - mx));
-        mrow[0] = mx;
+            lrow = (mrow == -INFINITY ? 0.f : lrow * ex2(mrow - mx)) + (o.x == -INFINITY ? 0.f : o.y * ex2(o.x - mx));
+        mrow = mx;
     }
     // this chunk's statistics of every real row
-    float2* out = reinterpret_cast<float2*>(L.stats) + ((size_t)(b * L.KVH + h) * L.stats_chunks + blockIdx.x) * M;
-#pragma unroll
-    for (int c = 0; c < C::MINE; ++c) {
-        const int R = ((MQ == 1 ? 0 : wg) + 2 * c) * 128 + wq * 32 + lane;
-        if (R < M) out[R] = make_float2(mrow[c], lrow[c]);
-    }
+    if (R < M)
+        reinterpret_cast<float2*>(L.stats)[((size_t)(b * L.KVH + h) * L.stats_chunks + blockIdx.x) * M + R] = make_float2(mrow, lrow);
 }
 
 // Restore pass, last step: merge each window row's chunk statistics into its normaliser.
@@ -612,7 +617,7 @@ template <int MT>
 cudaError_t launch_stats(const EvictParams& p, const CUtensorMap* tk, const CUtensorMap* tq, cudaStream_t s)
 {
     const dim3 grid(p.nch1, p.n_trig * p.lay.KVH);
-    return launch_pdl(score_stats_tc_kernel<MT>, grid, dim3(kThreads), StCfg<MT>::SMEM, s, p, *tk, *tq);
+    return launch_pdl(score_stats_tc_kernel<MT>, grid, dim3(kStThreads), StCfg<MT>::SMEM, s, p, *tk, *tq);
 }
 
 template <int MT>

@@ -220,23 +220,38 @@ __global__ void __launch_bounds__(kThreads, 2)
     __syncwarp();
     cluster_sync();  // every slice is complete; no CTA touches another's memory after it
     const int nr = (nt + W * kWarps - 1) / (W * kWarps);  // CTAs that hold a piece
-    for (int i = tid; i < per; i += kThreads) {
-        const int col = rank * per + i;
-        if (col >= G * kVec) break;
-        const int g = col / kVec, c4 = col % kVec;
-        float M = -INFINITY, l = 0.f;
-        for (int k = 0; k < nr; ++k) M = fmaxf(M, land_ml[k * per + i].x);
+    // a group of `span` lanes per column, a lane per CTA that sent it (one thread over all of them takes a chain
+    // of shared-memory reads, half a microsecond for 14)
+    int span = 1;
+    while (span < nr) span <<= 1;
+    for (int i0 = 0; i0 < per; i0 += kThreads / span) {
+        const int i = i0 + tid / span, k = tid & (span - 1), col = rank * per + i;
+        const bool mine = i < per && col < G * kVec;
+        float m = -INFINITY, l = 0.f;
         float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int k = 0; k < nr; ++k) {
+        if (mine && k < nr) {
             const float2 ml = land_ml[k * per + i];
-            const float4 v = land[k * per + i];
-            const float e = exp2f(ml.x - M);
-            l = fmaf(e, ml.y, l);
-            o.x = fmaf(e, v.x, o.x);
-            o.y = fmaf(e, v.y, o.y);
-            o.z = fmaf(e, v.z, o.z);
-            o.w = fmaf(e, v.w, o.w);
+            m = ml.x;
+            l = ml.y;
+            o = land[k * per + i];
         }
+        float M = m;
+        for (int d = 1; d < span; d <<= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, d));
+        const float e = m == -INFINITY ? 0.f : exp2f(m - M);
+        l *= e;
+        o.x *= e;
+        o.y *= e;
+        o.z *= e;
+        o.w *= e;
+        for (int d = 1; d < span; d <<= 1) {
+            l += __shfl_xor_sync(0xffffffffu, l, d);
+            o.x += __shfl_xor_sync(0xffffffffu, o.x, d);
+            o.y += __shfl_xor_sync(0xffffffffu, o.y, d);
+            o.z += __shfl_xor_sync(0xffffffffu, o.z, d);
+            o.w += __shfl_xor_sync(0xffffffffu, o.w, d);
+        }
+        if (!mine || k > 0) continue;
+        const int g = col / kVec, c4 = col % kVec;
         if (p.qring && c4 == 0) {  // the window query's softmax normaliser
             int slot = (p.seq_g[b] + p.ring_off) % L.r;
             if (slot < 0) slot += L.r;

@@ -419,8 +419,8 @@ void layout_scoring(ra_ctx* ctx)
 }
 
 // Launch shape of a scoring pass over the heads of the sequences in p (pass 1: prompt + the
-// trig_n cached rows each; pass 2: the trig_n candidate rows each, in p->layers layers): CTAs (one per
-// SM: all of its tensor memory) take runs of consecutive tiles of one head, in whole 128-row tiles
+// trig_n cached rows each; pass 2: the trig_n candidate rows each, in p->layers layers): CTAs (two per
+// SM with a window of at most 256 rows, else one) take runs of consecutive tiles of one head, in whole 128-row tiles
 // (two scoring tiles), of the length whose waves, each as long as the run and about three tiles'
 // start-up, end first.  Returns the algorithmic bytes: the key rows read (every one is contracted
 // with the M = r * G window rows, so flops = bytes * M).
@@ -438,13 +438,13 @@ double plan_scoring(ra_ctx* ctx, EvictParams* p, int pass)
     }
     // (pass 1 keeps a record per run: as many as the arena has)
     const int least = pass == 1 ? std::max(2, (most + ctx->stats_chunks - 1) / ctx->stats_chunks) : 2;
-    const int whole = (most + 1) / 2 * 2;
+    const int whole = (most + 1) / 2 * 2, slots = ctx->sms * (score_window_tiles(ctx->r * ctx->G) <= 2 ? 2 : 1);
     int run = whole;
     long long best = 0;
     for (int ch = (least + 1) / 2 * 2; ch <= whole; ch += 2) {
         long long ctas = 0;
         for (int t : tiles) ctas += (long long)layers * ctx->KVH * ((t + ch - 1) / ch);
-        const long long cost = (ctas + ctx->sms - 1) / ctx->sms * (ch / 2 + 3);
+        const long long cost = (ctas + slots - 1) / slots * (ch / 2 + 3);
         if (best == 0 || cost < best) {
             best = cost;
             run = ch;

@@ -44,7 +44,6 @@ namespace ra {
 static_assert(kPromptPage % kScoreTile == 0, "a scoring tile of the prompt lies inside one page");
 namespace {
 
-constexpr int kThreads = 512;  // summation pass: four warpgroups
 constexpr int kHalfBytes = kScoreTile * 128;      // one 64-channel box of a key tile
 constexpr uint64_t kWaitLimitNs = 2000000000ull;  // bounded mbarrier waits: 2 s
 static_assert(kHalfBytes % 1024 == 0, "128-byte-swizzled TMA boxes start 1024-byte aligned");
@@ -79,18 +78,23 @@ __device__ __forceinline__ int visible_rows(const int32_t* pos, int c, int lp, i
 }
 
 // ---------------------------------------------------------------------------------------------
-// Summation pass on the 5th-generation tensor cores (tcgen05, accumulators in tensor memory).
+// Both passes on the 5th-generation tensor cores (tcgen05, accumulators in tensor memory).
 //
-// The product is taken transposed, D = K Q^T: the 128 candidate key rows of a tile are the M
-// side of the MMA and the window rows are the N side (up to 256 per instruction), so that TMEM
-// lane j holds every window row's logit against key j.  The thread that reads lane j then sums
-// its own key's weights exp2(logit * scale_R - lse_R) over the window rows R, with no
-// cross-thread reduction; the four warpgroups take a quarter of the window rows each.  Both operands
-// are K-major in shared memory with the 128-byte swizzle the TMA copies already produce (rows of
-// 128 bytes, 8-row groups 1024 bytes apart, the two 64-channel halves one after the other); a
-// K-step of 16 channels advances the descriptors' start address by 32 bytes.  One thread issues
-// the MMAs and commits them to an mbarrier.  With a window of at most 256 rows the accumulator
-// is double-buffered in TMEM, so the MMAs of tile i + 1 run while tile i's weights are summed.
+// Operands are K-major in shared memory with the 128-byte swizzle the TMA copies already produce (rows
+// of 128 bytes, 8-row groups 1024 bytes apart, the two 64-channel halves one after the other); a K-step
+// of 16 channels advances the descriptors' start address by 32 bytes.  One warp of its own loads key
+// tiles and issues products, the others read accumulators: stages and accumulator buffers go round by
+// mbarriers, so that neither side waits for the other (issue_tiles).  A CTA's start -- tables, tensor
+// memory, 64 KB of window rows -- takes as long as several tiles, so windows of at most 256 rows run
+// two CTAs per SM (one key stage and 256 accumulator columns each): one CTA's start, loads and products
+// run beside the other's exponentials.
+//
+// Summation pass.  The product is taken transposed, D = K Q^T: the 128 candidate key rows of a tile are
+// the M side of the MMA and the window rows are the N side (up to 256 per instruction), so that TMEM
+// lane j holds every window row's logit against key j.  The thread that reads lane j then sums its own
+// key's weights exp2(logit * scale_R - lse_R) over its warpgroup's part of the window rows, with no
+// reduction across lanes.  Six layers of 10 heads with 4160 candidates and 256 window rows: 42 us with
+// one CTA of two warpgroups per SM, 31 us this way.
 
 constexpr int kTcRows = 128;                        // key rows per tile: the MMA's M
 constexpr int kTcHalf = kTcRows * 128;              // one 64-channel half of a key tile
@@ -98,19 +102,25 @@ constexpr int kTcStage = 2 * kTcHalf;               // a key tile: 128 rows x 25
 
 template <int ROWS>  // window rows held: r * G padded to a multiple of 128, at most 512
 struct TcCfg {
+    static constexpr bool TWO = ROWS <= 256;                   // two CTAs per SM
+    static constexpr int WGS = TWO ? 2 : 4;                    // warpgroups that sum, each a part of the window rows
+    static constexpr int THREADS = (WGS * 4 + 1) * 32;         // and the issuing warp
     static constexpr int NCH = ROWS > 256 ? 2 : 1;             // MMAs per K-step (N <= 256 each)
     static constexpr int NC = ROWS / NCH;                      // N of each MMA
-    static constexpr int NBUF = 2 * ROWS <= 512 ? 2 : 1;      // accumulator buffers in TMEM (512 columns)
-    static constexpr uint32_t COLS = NBUF * ROWS <= 256 ? 256u : 512u;  // columns allocated (a power of 2)
-    static constexpr int Q_OFF = 2 * kTcStage;                 // after the two key stages
+    static constexpr int NST = TWO ? 1 : 2;                    // key tiles on the way
+    static constexpr int NBUF = 2 * ROWS <= 256 ? 2 : 1;      // accumulator buffers in TMEM
+    static constexpr uint32_t COLS = TWO ? 256u : 512u;        // columns allocated (a power of 2)
+    static constexpr int Q_OFF = NST * kTcStage;               // after the key stages
     static constexpr int Q_HALF = ROWS * 128;
     static constexpr int STAT_OFF = Q_OFF + ROWS * kRowBytes;
-    static constexpr int RED_OFF = STAT_OFF + 2 * ROWS * 4;
-    static constexpr int BAR_OFF = RED_OFF + kThreads / 128 * kTcRows * 4;  // full[2], mma_done[2], TMEM base
-    static constexpr size_t SMEM = 1024 + (size_t)BAR_OFF + 4 * 8 + 16;
+    static constexpr int RED_OFF = STAT_OFF + 2 * ROWS * 4;    // two tiles' parts, taken in turn
+    static constexpr int BAR_OFF = RED_OFF + 2 * WGS * kTcRows * 4;  // full, free (stages), done, read (buffers), TMEM base
+    static constexpr int NBAR = 2 * NST + 2 * NBUF;
+    static constexpr size_t SMEM = 1024 + (size_t)BAR_OFF + NBAR * 8 + 16;
     static_assert(ROWS % 128 == 0 && ROWS <= 512, "window rows");
     static_assert(NC % 16 == 0 && NC <= 256, "UMMA N for M = 128");
-    static_assert(SMEM <= 232448, "fits the 227 KB opt-in shared memory");
+    static_assert(ROWS / WGS % 32 == 0 && NBUF * ROWS <= (int)COLS, "whole reads of the accumulators");
+    static_assert(SMEM <= (TWO ? 113 * 1024 : 232448), "one or two CTAs per SM");
 };
 
 // Shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1024 bytes apart.
@@ -166,23 +176,98 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32])
         : "memory");
 }
 
+// The issuing thread of a scoring CTA: tile i goes through stage i % NST and accumulator buffer i % NBUF.
+// load(i) issues the copies of tile i (completing on full[i % NST]), product(i) its MMAs.  A stage is loaded
+// again when the products that read it have completed, a buffer written again when its readers have
+// arrived on read[].  Every wait is bounded; false after one ran out, with everything issued waited for.
+template <int NST, int NBUF, class Load, class Product>
+__device__ bool issue_tiles(int ntile, uint64_t* full, uint64_t* sfree, uint64_t* done, uint64_t* read, Load load,
+                            Product product)
+{
+    int loaded = 0, issued = 0;  // tiles whose copies, whose products are issued
+    while (loaded < min(NST, ntile)) load(loaded++);
+    bool ok = true;
+    while (ok && issued < ntile) {
+        const int i = issued;
+        ok = mbar_wait_bounded(&full[i % NST], (uint32_t)((i / NST) & 1), kWaitLimitNs) &&
+             (i < NBUF || mbar_wait_bounded(&read[i % NBUF], (uint32_t)((i / NBUF - 1) & 1), kWaitLimitNs));
+        if (!ok) break;
+        tmem_fence_after();
+        product(i);
+        umma_commit(&done[i % NBUF]);
+        umma_commit(&sfree[i % NST]);
+        ++issued;
+        const int old = loaded - NST;  // the tile whose stage the next one takes
+        if (loaded < ntile && old <= i - (NST > 1 ? 1 : 0)) {
+            ok = mbar_wait_bounded(&sfree[old % NST], (uint32_t)((old / NST) & 1), kWaitLimitNs);
+            if (ok) load(loaded++);
+        }
+    }
+    if (!ok) {
+        for (int i = max(0, issued - NST); i < issued; ++i)
+            (void)mbar_wait_bounded(&sfree[i % NST], (uint32_t)((i / NST) & 1), kWaitLimitNs);
+        for (int i = issued; i < loaded; ++i)
+            (void)mbar_wait_bounded(&full[i % NST], (uint32_t)((i / NST) & 1), kWaitLimitNs);
+    }
+    return ok;
+}
+
+// A scoring CTA's set-up, by all threads: the accumulators' tensor memory (held until tc_leave) and the barriers.
+template <int NST, int NBUF>
+__device__ __forceinline__ uint32_t tc_enter(uint64_t* full, uint64_t* sfree, uint64_t* done, uint64_t* read, uint32_t* slot,
+                                             uint32_t cols, int readers)
+{
+    if (threadIdx.x < 32) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)), "r"(cols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < NST; ++i) {
+            mbar_init(&full[i], 1);
+            mbar_init(&sfree[i], 1);
+        }
+        for (int i = 0; i < NBUF; ++i) {
+            mbar_init(&done[i], 1);
+            mbar_init(&read[i], readers);
+        }
+        fence_mbar_init();
+    }
+    tmem_fence_before();
+    __syncthreads();
+    tmem_fence_after();
+    return *slot;
+}
+
+__device__ __forceinline__ void tc_leave(uint32_t tmem, uint32_t cols)
+{
+    __syncwarp();
+    tmem_fence_before();
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        tmem_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(cols) : "memory");
+    }
+}
+
 template <int ROWS>
-__global__ void __launch_bounds__(kThreads, 1) score_sum_tc_kernel(const __grid_constant__ EvictParams p,
-                                                                  const __grid_constant__ CUtensorMap tk,
-                                                                  const __grid_constant__ CUtensorMap tw)
+__global__ void __launch_bounds__(TcCfg<ROWS>::THREADS, TcCfg<ROWS>::TWO ? 2 : 1)
+    score_sum_tc_kernel(const __grid_constant__ EvictParams p, const __grid_constant__ CUtensorMap tk,
+                        const __grid_constant__ CUtensorMap tw)
 {
     using C = TcCfg<ROWS>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + C::BAR_OFF);  // key tile (and the window) landed
-    uint64_t* mdone = full + 2;                                          // the tile's MMAs completed
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(full + 4);
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + C::BAR_OFF);  // stage: key tile (and the window) landed
+    uint64_t* sfree = full + C::NST;                                    // stage: the products that read it completed
+    uint64_t* mdone = sfree + C::NST;                                   // buffer: a tile's products completed
+    uint64_t* bread = mdone + C::NBUF;                                  // buffer: its warps have read it
     float2* s_st = reinterpret_cast<float2*>(smem + C::STAT_OFF);  // (scale, -lse) of each window row
     float* red = reinterpret_cast<float*>(smem + C::RED_OFF);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-    // As the mma.sync pass: with p.early everything read here was written by kernels that
-    // completed before the predecessor started, and the scores are read only by the successor.
+    // With p.early everything read here was written by kernels that completed before the predecessor
+    // started, and the scores are read only by the successor.
     if (!p.early) {
         pdl_wait();
         pdl_launch_dependents();
@@ -202,141 +287,99 @@ __global__ void __launch_bounds__(kThreads, 1) score_sum_tc_kernel(const __grid_
     const int r_hi = min(N, r_lo + p.ch2 * kScoreTile);
     const int ntile = (r_hi - r_lo + kTcRows - 1) / kTcRows;
     const size_t lbh = ((size_t)(p.layer + blockIdx.z) * L.B + b) * L.KVH + h;
-    const long long grow = L.gen_row0 + (long long)L.region[lbh] * L.Cmax;
-
-    auto issue_tile = [&](int i, uint32_t extra) {  // thread 0: key tile i into stage i % 2
-        const int s = i % 2;
-        uint8_t* st = smem + (size_t)s * kTcStage;
-        const int row = (int)(grow + r_lo + (long long)i * kTcRows);
-        mbar_arrive_expect_tx(&full[s], (uint32_t)kTcStage + extra);
-        for (int q = 0; q < kTcRows; q += kScoreTile) {
-            tma_load_2d(st + q * 128, &tk, 0, row + q, &full[s]);
-            tma_load_2d(st + kTcHalf + q * 128, &tk, 64, row + q, &full[s]);
-        }
-    };
-    if (warp == 0) {  // the accumulators' tensor memory (held until the end)
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                     "r"(C::COLS)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    if (tid == 0) {
-        for (int s = 0; s < 2; ++s) {
-            mbar_init(&full[s], 1);
-            mbar_init(&mdone[s], 1);
-        }
-        fence_mbar_init();
-        prefetch_tensormap(&tk);
-        prefetch_tensormap(&tw);
-        // The window rows (row R = slot * G + g) complete on full[0] with the first key tile;
-        // rows past M are another head's (or read as zero): finite, and given no weight below.
-        issue_tile(0, (uint32_t)(ROWS * kRowBytes));
-        const int row0 = (int)(lbh * (size_t)M);
-        for (int rb = 0; rb < ROWS; rb += kScoreTile) {
-            tma_load_2d(smem + C::Q_OFF + rb * 128, &tw, 0, row0 + rb, &full[0]);
-            tma_load_2d(smem + C::Q_OFF + C::Q_HALF + rb * 128, &tw, 64, row0 + rb, &full[0]);
-        }
-        if (ntile > 1) issue_tile(1, 0u);
-    }
-    // thread 0's counts of tiles: copies issued, MMAs issued, MMAs waited for
-    int n_loaded = min(ntile, 2), n_mma = 0, done = 0;
     {  // the normaliser each window query had at its decode step
         const float2* qst = L.qstats + lbh * (size_t)M;
-        for (int R = tid; R < ROWS; R += kThreads) {
+        for (int R = tid; R < ROWS; R += C::THREADS) {
             const float2 f = R < M ? __ldcg(qst + R) : make_float2(0.f, INFINITY);  // padding rows weigh 0
             s_st[R] = make_float2(f.x, -f.y);
         }
     }
-    tmem_fence_before();
-    __syncthreads();
-    tmem_fence_after();
-    const uint32_t tmem = *tmem_slot;
-    const uint32_t idesc = umma_idesc_bf16(kTcRows, C::NC);
-    const uint32_t sbase = smem_u32(smem);
-
-    // Thread 0: the MMAs of tile i into accumulator buffer i % NBUF, committed to mdone[i % 2].
-    auto issue_mma = [&](int i) -> bool {
-        if (!mbar_wait_bounded(&full[i % 2], (uint32_t)((i / 2) & 1), kWaitLimitNs)) return false;
-        tmem_fence_after();
-        const uint32_t d0 = tmem + (uint32_t)((i % C::NBUF) * ROWS);
-        const uint32_t a0 = sbase + (uint32_t)((i % 2) * kTcStage);
-#pragma unroll
-        for (int kh = 0; kh < 2; ++kh)        // 64-channel half
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {  // 16-channel K-step inside the half
-                const uint64_t ad = umma_desc_sw128(a0 + kh * kTcHalf + kk * 32);
-#pragma unroll
-                for (int c = 0; c < C::NCH; ++c) {
-                    const uint64_t bd = umma_desc_sw128(sbase + C::Q_OFF + kh * C::Q_HALF + c * C::NC * 128 + kk * 32);
-                    umma_bf16(d0 + c * C::NC, ad, bd, idesc, (kh | kk) != 0);
+    const uint32_t tmem = tc_enter<C::NST, C::NBUF>(full, sfree, mdone, bread, reinterpret_cast<uint32_t*>(bread + C::NBUF),
+                                                    C::COLS, C::WGS * 4);
+    if (warp == C::WGS * 4) {
+        if (lane == 0) {
+            prefetch_tensormap(&tk);
+            prefetch_tensormap(&tw);
+            const long long grow = L.gen_row0 + (long long)L.region[lbh] * L.Cmax;
+            const uint32_t idesc = umma_idesc_bf16(kTcRows, C::NC), sbase = smem_u32(smem);
+            auto load = [&](int i) {
+                uint8_t* st = smem + (size_t)(i % C::NST) * kTcStage;
+                uint64_t* bar = &full[i % C::NST];
+                const int row = (int)(grow + r_lo + (long long)i * kTcRows);
+                // The window rows (row R = slot * G + g) complete with the first key tile; rows past M are
+                // another head's (or read as zero): finite, and given no weight.
+                mbar_arrive_expect_tx(bar, (uint32_t)kTcStage + (i == 0 ? (uint32_t)(ROWS * kRowBytes) : 0u));
+                for (int q = 0; q < kTcRows; q += kScoreTile) {
+                    tma_load_2d(st + q * 128, &tk, 0, row + q, bar);
+                    tma_load_2d(st + kTcHalf + q * 128, &tk, 64, row + q, bar);
                 }
+                if (i > 0) return;
+                const int row0 = (int)(lbh * (size_t)M);
+                for (int rb = 0; rb < ROWS; rb += kScoreTile) {
+                    tma_load_2d(smem + C::Q_OFF + rb * 128, &tw, 0, row0 + rb, bar);
+                    tma_load_2d(smem + C::Q_OFF + C::Q_HALF + rb * 128, &tw, 64, row0 + rb, bar);
+                }
+            };
+            auto product = [&](int i) {
+                const uint32_t d0 = tmem + (uint32_t)((i % C::NBUF) * ROWS);
+                const uint32_t a0 = sbase + (uint32_t)((i % C::NST) * kTcStage);
+#pragma unroll
+                for (int kh = 0; kh < 2; ++kh)        // 64-channel half
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk)    // 16-channel K-step inside the half
+#pragma unroll
+                        for (int c = 0; c < C::NCH; ++c)
+                            umma_bf16(d0 + c * C::NC, umma_desc_sw128(a0 + kh * kTcHalf + kk * 32),
+                                      umma_desc_sw128(sbase + C::Q_OFF + kh * C::Q_HALF + c * C::NC * 128 + kk * 32), idesc,
+                                      (kh | kk) != 0);
+            };
+            if (!issue_tiles<C::NST, C::NBUF>(ntile, full, sfree, mdone, bread, load, product))
+                atomicExch(L.err, kDeviceErrTimeout);
+        }
+    } else {
+        // this thread: key row wq * 32 + lane of a tile, window rows [wg, wg + 1) * ROWS / WGS
+        const int wg = warp >> 2, wq = warp & 3;
+        float* scores = L.scores + lbh * L.Cmax;
+        bool ok = true;
+        for (int i = 0; i < ntile; ++i) {
+            // (after a wait that ran out the warp only keeps the others' barrier going)
+            if (ok && !mbar_wait_bounded(&mdone[i % C::NBUF], (uint32_t)((i / C::NBUF) & 1), kWaitLimitNs)) {
+                if (lane == 0) atomicExch(L.err, kDeviceErrTimeout);
+                ok = false;
             }
-        umma_commit(&mdone[i % 2]);
-        n_mma = i + 1;
-        return true;
-    };
-
-    float* scores = L.scores + lbh * L.Cmax;
-    constexpr int kWgs = kThreads / 128;
-    const int wg = warp >> 2, wq = warp & 3;  // warpgroup (its part of the window rows), TMEM lane quarter
-    bool ok = true;
-    if (tid == 0) ok = issue_mma(0);
-    for (int i = 0; i < ntile; ++i) {
-        if (C::NBUF == 2 && tid == 0 && ok && i + 1 < ntile) ok = issue_mma(i + 1);
-        const bool got = mbar_wait_bounded(&mdone[i % 2], (uint32_t)((i / 2) & 1), kWaitLimitNs);
-        if (!__syncthreads_and(got && ok)) {  // give up together
-            if (tid == 0) atomicExch(L.err, kDeviceErrTimeout);
-            break;
-        }
-        done = i + 1;
-        tmem_fence_after();
-        if (tid == 0 && i + 2 < ntile) {  // the tile's MMAs have read stage i % 2: refill it
-            fence_proxy_async_smem();
-            issue_tile(i + 2, 0u);
-            n_loaded = i + 3;
-        }
-        // this thread: key row wq * 32 + lane of the tile, window rows [wg, wg + 1) * ROWS / kWgs
-        const uint32_t tl = tmem + ((uint32_t)(wq * 32) << 16) + (uint32_t)((i % C::NBUF) * ROWS);
-        float sum[4] = {0.f, 0.f, 0.f, 0.f};
+            ok = __all_sync(0xffffffffu, ok);
+            float sum[4] = {0.f, 0.f, 0.f, 0.f};
+            if (ok) {
+                tmem_fence_after();
+                const uint32_t tl = tmem + ((uint32_t)(wq * 32) << 16) + (uint32_t)((i % C::NBUF) * ROWS);
 #pragma unroll 1
-        for (int c0 = wg * (ROWS / kWgs); c0 < (wg + 1) * (ROWS / kWgs); c0 += 32) {
-            uint32_t v[32];
-            tmem_ld32(tl + c0, v);
+                for (int c0 = wg * (ROWS / C::WGS); c0 < (wg + 1) * (ROWS / C::WGS); c0 += 32) {
+                    uint32_t v[32];
+                    tmem_ld32(tl + c0, v);
 #pragma unroll
-            for (int j = 0; j < 32; j += 2) {
-                const float4 f = *reinterpret_cast<const float4*>(s_st + c0 + j);  // two rows' (one address: a broadcast)
-                sum[j & 2] += exp2f(fmaf(__uint_as_float(v[j]), f.x, f.y));
-                sum[(j & 2) + 1] += exp2f(fmaf(__uint_as_float(v[j + 1]), f.z, f.w));
+                    for (int j = 0; j < 32; j += 2) {
+                        const float4 f = *reinterpret_cast<const float4*>(s_st + c0 + j);  // two rows' (one address: a broadcast)
+                        sum[j & 2] += exp2f(fmaf(__uint_as_float(v[j]), f.x, f.y));
+                        sum[(j & 2) + 1] += exp2f(fmaf(__uint_as_float(v[j + 1]), f.z, f.w));
+                    }
+                }
+                tmem_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&bread[i % C::NBUF]);
+            }
+            float* part = red + (i & 1) * (C::WGS * kTcRows);
+            part[wg * kTcRows + wq * 32 + lane] = (sum[0] + sum[1]) + (sum[2] + sum[3]);
+            asm volatile("bar.sync 1, %0;" ::"n"(C::WGS * 128) : "memory");  // every part of the tile is summed
+            const int row = r_lo + i * kTcRows + tid;
+            if (ok && tid < kTcRows && row < r_hi) {
+                float all = 0.f;
+#pragma unroll
+                for (int k = 0; k < C::WGS; ++k) all += part[k * kTcRows + tid];
+                scores[row] = all;
             }
         }
-        red[wg * kTcRows + wq * 32 + lane] = (sum[0] + sum[1]) + (sum[2] + sum[3]);
-        tmem_fence_before();
-        __syncthreads();  // every part summed; the accumulator buffer is free again
-        if (tid < kTcRows) {
-            const int row = r_lo + i * kTcRows + tid;
-            float all = 0.f;
-#pragma unroll
-            for (int k = 0; k < kWgs; ++k) all += red[k * kTcRows + tid];
-            if (row < r_hi) scores[row] = all;
-        }
-        if (C::NBUF == 1 && tid == 0 && ok && i + 1 < ntile) {
-            tmem_fence_after();
-            ok = issue_mma(i + 1);
-        }
-        __syncthreads();  // red is rewritten by the next tile
     }
-    // Leave only with nothing in flight: after a timeout, the MMAs issued but not waited for and
-    // the copies issued but not consumed are waited for once more, bounded.
-    if (tid == 0) {
-        for (int i = done; i < n_mma; ++i) (void)mbar_wait_bounded(&mdone[i % 2], (uint32_t)((i / 2) & 1), kWaitLimitNs);
-        for (int i = n_mma; i < n_loaded; ++i) (void)mbar_wait_bounded(&full[i % 2], (uint32_t)((i / 2) & 1), kWaitLimitNs);
-    }
-    tmem_fence_before();
-    __syncthreads();
-    if (warp == 0) {
-        tmem_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C::COLS) : "memory");
-    }
+    tc_leave(tmem, C::COLS);
     if (p.early) {
         pdl_wait();
         pdl_launch_dependents();
@@ -348,25 +391,23 @@ __global__ void __launch_bounds__(kThreads, 1) score_sum_tc_kernel(const __grid_
 //
 // D = Q K^T: the window rows are the M side (MQ tiles of 128), the 128 keys of a tile the N side, so
 // that a TMEM lane holds one window row's logits and the thread that reads it keeps that row's
-// running maximum and sum in registers.  Four warpgroups take the M tiles, or parts of the keys of
-// one (merged at the end), and a warp of its own loads tiles and issues products, so that neither
-// waits for the other: a tile's accumulator is handed back by an mbarrier.  A tile is two runs of
-// kScoreTile cache rows (a prompt page holds three); with at most 256 window rows the accumulator is
-// double-buffered, and the products of tile i + 1 run while tile i is summed.  Bound by exp2 (one per
-// logit) and the few instructions around it, with four warps per scheduler to hide their latency, and
-// by a CTA's start (64 KB of window rows).  160 heads of 3.3K keys and 256 window rows: 167 us with
-// mma.sync and two shuffles per 16 keys of a row, 85 us with two warpgroups and a barrier of all
-// threads per tile, 63 us this way.
-constexpr int kStWgs = 4, kStThreads = (kStWgs * 4 + 1) * 32;  // four warpgroups and the issuing warp
-
+// running maximum and sum in registers.  The warpgroups take the M tiles, or parts of the keys of one
+// (merged at the end).  A tile is two runs of kScoreTile cache rows (a prompt page holds three).  Bound by
+// exp2 (one per logit) and the few instructions around it.  160 heads of 3.3K keys and 256 window rows:
+// 167 us with mma.sync and two shuffles per 16 keys of a row; here 85 us with one CTA per SM of two
+// warpgroups and a barrier of all threads per tile, 63 us with four warpgroups and the issuing warp,
+// 55 us with two such CTAs of two warpgroups.
 template <int MQ>
 struct StCfg {
+    static constexpr bool TWO = MQ <= 2;                       // two CTAs per SM
+    static constexpr int WGS = TWO ? 2 : 4;                    // warpgroups that keep statistics
+    static constexpr int THREADS = (WGS * 4 + 1) * 32;         // and the issuing warp
     static constexpr int ROWS = 128 * MQ;
-    static constexpr int NST = MQ <= 3 ? 3 : 2;                // key tiles on the way
-    static constexpr int NBUF = MQ <= 2 ? 2 : 1;               // accumulator buffers in TMEM
+    static constexpr int NST = TWO ? 1 : MQ == 3 ? 3 : 2;      // key tiles on the way
     static constexpr int BUF_COLS = kTcRows * MQ;              // columns of one buffer: 128 keys per M tile
-    static constexpr uint32_t COLS = MQ == 1 ? 256u : 512u;    // columns allocated (a power of 2)
-    static constexpr int PARTS = MQ <= 2 ? kStWgs / MQ : 1;    // warpgroups that share an M tile's keys
+    static constexpr int NBUF = MQ == 1 ? 2 : 1;               // accumulator buffers in TMEM
+    static constexpr uint32_t COLS = TWO ? 256u : 512u;        // columns allocated (a power of 2)
+    static constexpr int PARTS = WGS > MQ ? WGS / MQ : 1;      // warpgroups that share an M tile's keys
     static constexpr int PCOLS = kTcRows / PARTS;
     static constexpr int Q_OFF = NST * kTcStage;               // after the key stages
     static constexpr int Q_HALF = ROWS * 128;
@@ -374,7 +415,8 @@ struct StCfg {
     static constexpr int BAR_OFF = RED_OFF + MQ * (PARTS - 1) * 128 * 8;  // full, free (stages), done, read (buffers), TMEM base
     static constexpr int NBAR = 2 * NST + 2 * NBUF;
     static constexpr size_t SMEM = 1024 + (size_t)BAR_OFF + NBAR * 8 + 16;
-    static_assert(NBUF * BUF_COLS <= (int)COLS && SMEM <= 232448 && PCOLS % 32 == 0, "tensor and shared memory");
+    static_assert(NBUF * BUF_COLS <= (int)COLS && PCOLS % 32 == 0, "tensor memory");
+    static_assert(SMEM <= (TWO ? 113 * 1024 : 232448), "one or two CTAs per SM");
 };
 
 __device__ __forceinline__ float ex2(float x)
@@ -408,9 +450,9 @@ __device__ __forceinline__ void add_stats(const uint32_t (&v)[32], int valid, fl
 }
 
 template <int MQ>
-__global__ void __launch_bounds__(kStThreads, 1) score_stats_tc_kernel(const __grid_constant__ EvictParams p,
-                                                                      const __grid_constant__ CUtensorMap tk,
-                                                                      const __grid_constant__ CUtensorMap tw)
+__global__ void __launch_bounds__(StCfg<MQ>::THREADS, StCfg<MQ>::TWO ? 2 : 1)
+    score_stats_tc_kernel(const __grid_constant__ EvictParams p, const __grid_constant__ CUtensorMap tk,
+                          const __grid_constant__ CUtensorMap tw)
 {
     using C = StCfg<MQ>;
     extern __shared__ uint8_t smem_raw[];
@@ -419,7 +461,6 @@ __global__ void __launch_bounds__(kStThreads, 1) score_stats_tc_kernel(const __g
     uint64_t* sfree = full + C::NST;                                    // stage: the products that read it completed
     uint64_t* mdone = sfree + C::NST;                                   // buffer: a tile's products completed
     uint64_t* bread = mdone + C::NBUF;                                  // buffer: its warps have read it
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bread + C::NBUF);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     pdl_wait();  // the window, the cache and the tables come from earlier kernels
@@ -438,33 +479,14 @@ __global__ void __launch_bounds__(kStThreads, 1) score_stats_tc_kernel(const __g
     const size_t lbh = ((size_t)p.layer * L.B + b) * L.KVH + h;
     const int reg = L.region[lbh];
 
-    if (warp == 0) {  // the accumulators' tensor memory (held until the end)
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                     "r"(C::COLS)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    if (tid == 0) {
-        for (int i = 0; i < C::NST; ++i) {
-            mbar_init(&full[i], 1);
-            mbar_init(&sfree[i], 1);
-        }
-        for (int i = 0; i < C::NBUF; ++i) {
-            mbar_init(&mdone[i], 1);
-            mbar_init(&bread[i], MQ * C::PARTS * 4);
-        }
-        fence_mbar_init();
-    }
-    tmem_fence_before();
-    __syncthreads();
-    tmem_fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = tc_enter<C::NST, C::NBUF>(full, sfree, mdone, bread, reinterpret_cast<uint32_t*>(bread + C::NBUF),
+                                                    C::COLS, MQ * C::PARTS * 4);
 
     // this thread's window row: lane wq * 32 + lane of M tile q, the keys of part `part`
     const int wg = warp >> 2, wq = warp & 3, q = wg / C::PARTS, part = wg % C::PARTS;
     const int R = q * 128 + wq * 32 + lane;
     float mrow = -INFINITY, lrow = 0.f;
-    if (warp == kStWgs * 4) {
+    if (warp == C::WGS * 4) {
         if (lane == 0) {
             const long long pbase = prompt_row(L, p.layer, 0, h, 0);
             const int32_t* ptab = L.pages + (size_t)b * L.max_pages;
@@ -475,40 +497,30 @@ __global__ void __launch_bounds__(kStThreads, 1) score_stats_tc_kernel(const __g
                                           (k * kScoreTile) % kPromptPage
                                     : grow + (long long)(k - tp) * kScoreTile);
             };
-            // Tile i (runs t0 + 2 i and the next, if this CTA has it) into stage i % NST; `extra` bytes of other
-            // copies complete on the same barrier.  A missing second run leaves old rows, whose logits count
-            // nothing.
-            auto issue_tile = [&](int i, uint32_t extra) {
+            // Tile i: runs t0 + 2 i and the next, if this CTA has it (else its rows are old ones, whose logits
+            // count nothing).  The window rows (row R = slot * G + g) complete with the first tile; rows past M
+            // are another head's (or read as zero) and belong to no thread's statistics.
+            prefetch_tensormap(&tk);
+            prefetch_tensormap(&tw);
+            const uint32_t idesc = umma_idesc_bf16(128, kTcRows), sbase = smem_u32(smem);
+            auto load = [&](int i) {
                 const int k = t0 + 2 * i, n = min(2, t1 - k);
                 uint8_t* st = smem + (size_t)(i % C::NST) * kTcStage;
                 uint64_t* bar = &full[i % C::NST];
-                mbar_arrive_expect_tx(bar, (uint32_t)(n * kScoreTile * kRowBytes) + extra);
+                mbar_arrive_expect_tx(bar, (uint32_t)(n * kScoreTile * kRowBytes) + (i == 0 ? (uint32_t)(C::ROWS * kRowBytes) : 0u));
                 for (int u = 0; u < n; ++u) {
                     const int row = run_row(k + u);
                     tma_load_2d(st + u * kHalfBytes, &tk, 0, row, bar);
                     tma_load_2d(st + kTcHalf + u * kHalfBytes, &tk, 64, row, bar);
                 }
+                if (i > 0) return;
+                const int row0 = (int)(lbh * (size_t)M);
+                for (int rb = 0; rb < C::ROWS; rb += kScoreTile) {
+                    tma_load_2d(smem + C::Q_OFF + rb * 128, &tw, 0, row0 + rb, bar);
+                    tma_load_2d(smem + C::Q_OFF + C::Q_HALF + rb * 128, &tw, 64, row0 + rb, bar);
+                }
             };
-            prefetch_tensormap(&tk);
-            prefetch_tensormap(&tw);
-            // The window rows (row R = slot * G + g) complete on full[0] with the first key tile; rows past M
-            // are another head's (or read as zero) and belong to no thread's statistics.
-            issue_tile(0, (uint32_t)(C::ROWS * kRowBytes));
-            const int row0 = (int)(lbh * (size_t)M);
-            for (int rb = 0; rb < C::ROWS; rb += kScoreTile) {
-                tma_load_2d(smem + C::Q_OFF + rb * 128, &tw, 0, row0 + rb, &full[0]);
-                tma_load_2d(smem + C::Q_OFF + C::Q_HALF + rb * 128, &tw, 64, row0 + rb, &full[0]);
-            }
-            int loaded = 1, issued = 0;  // tiles whose copies, whose products are issued
-            for (; loaded < min(C::NST, ntile); ++loaded) issue_tile(loaded, 0u);
-            const uint32_t idesc = umma_idesc_bf16(128, kTcRows), sbase = smem_u32(smem);
-            bool ok = true;
-            while (ok && issued < ntile) {
-                const int i = issued;
-                ok = mbar_wait_bounded(&full[i % C::NST], (uint32_t)((i / C::NST) & 1), kWaitLimitNs) &&
-                     (i < C::NBUF || mbar_wait_bounded(&bread[i % C::NBUF], (uint32_t)((i / C::NBUF - 1) & 1), kWaitLimitNs));
-                if (!ok) break;
-                tmem_fence_after();
+            auto product = [&](int i) {
                 const uint32_t d0 = tmem + (uint32_t)((i % C::NBUF) * C::BUF_COLS);
                 const uint32_t b0 = sbase + (uint32_t)((i % C::NST) * kTcStage);
 #pragma unroll
@@ -520,21 +532,9 @@ __global__ void __launch_bounds__(kStThreads, 1) score_stats_tc_kernel(const __g
                             umma_bf16(d0 + m * kTcRows,
                                       umma_desc_sw128(sbase + C::Q_OFF + kh * C::Q_HALF + m * 128 * 128 + kk * 32),
                                       umma_desc_sw128(b0 + kh * kTcHalf + kk * 32), idesc, (kh | kk) != 0);
-                umma_commit(&mdone[i % C::NBUF]);
-                umma_commit(&sfree[i % C::NST]);
-                ++issued;
-                if (i >= 1 && loaded < ntile) {  // tile i - 1 + NST into tile i - 1's stage
-                    ok = mbar_wait_bounded(&sfree[(i - 1) % C::NST], (uint32_t)(((i - 1) / C::NST) & 1), kWaitLimitNs);
-                    if (ok) issue_tile(loaded++, 0u);
-                }
-            }
-            if (!ok) {  // leave only with nothing in flight: everything issued is waited for once more, bounded
+            };
+            if (!issue_tiles<C::NST, C::NBUF>(ntile, full, sfree, mdone, bread, load, product))
                 atomicExch(L.err, kDeviceErrTimeout);
-                for (int i = max(0, issued - C::NST); i < issued; ++i)
-                    (void)mbar_wait_bounded(&sfree[i % C::NST], (uint32_t)((i / C::NST) & 1), kWaitLimitNs);
-                for (int i = issued; i < loaded; ++i)
-                    (void)mbar_wait_bounded(&full[i % C::NST], (uint32_t)((i / C::NST) & 1), kWaitLimitNs);
-            }
         }
     } else if (q < MQ) {
         // generated rows the row sees
@@ -566,14 +566,8 @@ __global__ void __launch_bounds__(kStThreads, 1) score_stats_tc_kernel(const __g
             reinterpret_cast<float2*>(smem + C::RED_OFF)[(q * (C::PARTS - 1) + part - 1) * 128 + wq * 32 + lane] =
                 make_float2(mrow, lrow);
     }
-    __syncwarp();
-    tmem_fence_before();
-    __syncthreads();
-    if (warp == 0) {
-        tmem_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C::COLS) : "memory");
-    }
-    if (warp >= kStWgs * 4 || q >= MQ || part > 0) return;
+    tc_leave(tmem, C::COLS);
+    if (warp >= C::WGS * 4 || q >= MQ || part > 0) return;
 #pragma unroll
     for (int k = 0; k < C::PARTS - 1; ++k) {
         const float2 o = reinterpret_cast<const float2*>(smem + C::RED_OFF)[(q * (C::PARTS - 1) + k) * 128 + wq * 32 + lane];
@@ -617,7 +611,7 @@ template <int MT>
 cudaError_t launch_stats(const EvictParams& p, const CUtensorMap* tk, const CUtensorMap* tq, cudaStream_t s)
 {
     const dim3 grid(p.nch1, p.n_trig * p.lay.KVH);
-    return launch_pdl(score_stats_tc_kernel<MT>, grid, dim3(kStThreads), StCfg<MT>::SMEM, s, p, *tk, *tq);
+    return launch_pdl(score_stats_tc_kernel<MT>, grid, dim3(StCfg<MT>::THREADS), StCfg<MT>::SMEM, s, p, *tk, *tq);
 }
 
 template <int MT>
@@ -633,7 +627,7 @@ template <int MT>
 cudaError_t launch_sum_tc(const EvictParams& p, const CUtensorMap* tk, const CUtensorMap* tq, cudaStream_t s)
 {
     const dim3 grid(p.nch2, p.n_trig * p.lay.KVH, p.layers);
-    return launch_pdl(score_sum_tc_kernel<128 * MT>, grid, dim3(kThreads), TcCfg<128 * MT>::SMEM, s, p, *tk, *tq);
+    return launch_pdl(score_sum_tc_kernel<128 * MT>, grid, dim3(TcCfg<128 * MT>::THREADS), TcCfg<128 * MT>::SMEM, s, p, *tk, *tq);
 }
 
 }  // namespace

@@ -1180,6 +1180,21 @@ int check_layer_call(ra_ctx* ctx, int layer, const uint16_t* q, const uint16_t* 
 // side stream, and run every layer's round of the sequences that fire now and have those sets,
 // in one launch.  It needs none of the step's rows: in both layouts each layer's attention then
 // appends its token into the last slot, as after an eviction inside the layer's own call.
+//
+// A sequence that fires without a set computed ahead (the first step of a loaded run, a slot switched on
+// again) has its sets computed here, before the compaction, where there are at least kPlanNowLayers
+// layers: one plan and one compaction of every layer then replace a launch of the eviction kernel per layer
+// (36 layers of one sequence with 2112 candidates: PN_A us of evictions, PN_B us this way).
+constexpr int kPlanNowLayers = 4;
+
+// Sequence b's counters are those of layer 0 in every layer.
+bool layers_alike_seq(const ra_ctx* ctx, int b)
+{
+    for (int l = 1; l < ctx->L; ++l)
+        if (ctx->g[(size_t)l * ctx->B + b] != ctx->g[b] || ctx->c[(size_t)l * ctx->B + b] != ctx->c[b]) return false;
+    return true;
+}
+
 int step_prologue(ra_ctx* ctx, cudaStream_t s)
 {
     cudaError_t e;
@@ -1251,6 +1266,48 @@ int step_prologue(ra_ctx* ctx, cudaStream_t s)
     // computed ahead, or from scores computed now: all their rounds in one launch, in place, before the first layer: the
     // survivors move down (ordered) or the evicted slots are refilled from the newest rows
     // (order-free), and the layers then append the token as usual.
+    bool planned_now = false;
+    if (now && serve && ctx->L >= kPlanNowLayers && (ctx->evict_mode & ~RA_EVICT_EXACT) == RA_EVICT_AUTO) {
+        EvictParams pp{};
+        pp.lay = ctx->lay;
+        pp.policy = ctx->policy;
+        pp.block = ctx->block;
+        pp.holefill = ctx->compaction == RA_COMPACT_HOLEFILL;
+        pp.ev_exact = (ctx->evict_mode & RA_EVICT_EXACT) ? 1 : 0;
+        pp.ev_plan_parity = cur;
+        int n = 0;
+        for (int b = 0; b < ctx->B; ++b) {
+            const int g = ctx->g[b] + 1, c = ctx->c[b] + 1, cand = c - ctx->r;
+            if (!ctx->active[b] || !fires(ctx, g, c) || cand > ctx->K + ctx->r || !layers_alike_seq(ctx, b)) continue;
+            bool planned = true;
+            for (int l = 0; l < ctx->L && planned; ++l) {
+                const size_t k = (size_t)cur * ctx->L * ctx->B + (size_t)l * ctx->B + b;
+                planned = ctx->plan_g[k] == g && ctx->plan_n[k] == cand;
+            }
+            if (planned) continue;
+            pp.trig[n] = (int16_t)b;
+            pp.trig_admit[n] = (uint16_t)ctx->admits[b];
+            pp.trig_g[n] = g;
+            pp.trig_n[n] = cand;
+            ++n;
+        }
+        if (n > 0) {
+            pp.n_trig = n;
+            {
+                ProfScope ps(ctx, RA_KERNEL_PLAN, 0.0, s);
+                e = launch_plan(pp, ctx->sms, s);
+                ps.done();
+            }
+            if (e != cudaSuccess) return cuda_fail(ctx, e, "plan launch");
+            planned_now = true;
+            for (int i = 0; i < n; ++i)
+                for (int l = 0; l < ctx->L; ++l) {
+                    const size_t k = (size_t)cur * ctx->L * ctx->B + (size_t)l * ctx->B + pp.trig[i];
+                    ctx->plan_g[k] = pp.trig_g[i];
+                    ctx->plan_n[k] = pp.trig_n[i];
+                }
+        }
+    }
     if (now) {
         const bool fill = ctx->compaction == RA_COMPACT_HOLEFILL;
         EvictParams sp{};
@@ -1258,6 +1315,7 @@ int step_prologue(ra_ctx* ctx, cudaStream_t s)
         sp.ev_plan_parity = cur;
         sp.holefill = fill ? 1 : 0;
         sp.pending = 1;
+        sp.early = fill && !planned_now ? kEarlyAll : kEarlyNone;  // (the order-free fill reads its plan ahead)
         int n = 0;
         double moved = 0;
         for (int b = 0; b < ctx->B; ++b) {

@@ -1281,9 +1281,10 @@ __global__ void __launch_bounds__(kFillThreads) fill_stack_kernel(const __grid_c
     const int h = item % L.KVH, t = (item / L.KVH) % p.n_trig, layer = item / (L.KVH * p.n_trig);
     const int b = p.trig[t], c = p.trig_c[t], N = p.trig_n[t];
     const int m = N - L.K;
-    // The plan (complete: the stream waited for it) and the tables are read before waiting for
-    // the predecessor; the rows and positions it may have written, after.  Every exit waits
-    // first, so that no successor starts before the predecessor completes.
+    // The plan (with p.early complete: the stream waited for it; else the predecessor computes it) and the
+    // tables are read before waiting for the predecessor; the rows and positions it may have written,
+    // after.  Every exit waits first, so that no successor starts before the predecessor completes.
+    if (p.early == kEarlyNone) pdl_wait();
     if (m < 1 || m > L.r || m > kEvCap || N > c || c + 1 > L.Cmax) {  // the host rules this out
         pdl_wait();
         pdl_launch_dependents();

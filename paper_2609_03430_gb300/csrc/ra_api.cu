@@ -256,6 +256,25 @@ void fill_active(const ra_ctx* ctx, uint32_t* mask)
 
 int cluster_size(const ra_ctx* ctx, int heads, int longest, int W);
 
+// The chunks of a long stacked launch: 97% of each warp's share in one, the rest in chunks that warps claim as
+// they finish (see ra_attn.cu), if the arena holds their records.
+constexpr int kTailFrom = 256;    // tiles per warp from which the launch is long enough
+constexpr int kTailLeast = 8;     // tiles per chunk, at least
+constexpr int kTailChunks = 4;    // chunks per warp that the arena holds records for (about three are made)
+void plan_tail(const ra_ctx* ctx, AttnParams* p)
+{
+    const double share = (double)p->total / p->nwarps;
+    const int W = (int)(0.97 * share), size = std::max(kTailLeast, (int)(0.015 * share));
+    const int chunks = p->nwarps + (p->total - W * p->nwarps + size - 1) / size;
+    if ((size_t)chunks > ctx->max_chunks) return;
+    p->W = W;
+    p->nstatic = p->nwarps;
+    p->tail_tile = W * p->nwarps;
+    p->tail_size = size;
+    p->nchunks = chunks;
+    p->ticket = ctx->lay.ticket;
+}
+
 // Work split of the attention of `layers` layers from `layer` on (counters alike), from the host
 // mirror, in tiles: a head has ceil(lp / TILE) prompt tiles and ceil(gen / TILE) tiles of generated
 // rows, where gen is the cached generated rows plus one for a fused new token; the tiles are cut
@@ -310,6 +329,7 @@ int plan_attention(ra_ctx* ctx, int layer, int layers, int fused, AttnParams* p,
     const long long nchunks = (acc + W - 1) / W;
     p->W = (int)W;
     p->nchunks = (int)nchunks;
+    p->nstatic = 0;
     *ctas = (int)std::min<long long>((long long)ctx->sms * cps, (nchunks + wpc - 1) / wpc);
     p->nwarps = *ctas * wpc;
     *n_active = na;
@@ -327,6 +347,7 @@ int plan_attention(ra_ctx* ctx, int layer, int layers, int fused, AttnParams* p,
         p->cluster_heads = holding * ctx->KVH;
         p->cluster = cluster_size(ctx, p->cluster_heads, longest, (int)W);
     }
+    if (layers > 1 && *shape == kAttnWide && W >= kTailFrom) plan_tail(ctx, p);
     if ((size_t)p->nchunks > ctx->max_chunks)
         return fail(ctx, RA_ERR_STATE, "attention split needs more partial records than the arena holds");
     return RA_OK;
@@ -380,13 +401,19 @@ int layout_base(ra_ctx* ctx)
     ctx->off_pages = take((size_t)batch * ctx->max_pages * 4);
     ctx->off_plan = take((size_t)batch * kv_heads * (kPlanHeader + r) * 4);
     // chunks of the attention split: one per warp
-    const size_t max_chunks =
+    size_t max_chunks =
         (size_t)kMaxSMs * std::max(attn_warps_per_cta(kAttnWide, ctx->G) * attn_ctas_per_sm(kAttnWide),
                                    attn_warps_per_cta(kAttnNarrow, ctx->G) * attn_ctas_per_sm(kAttnNarrow)) + 1;
+    // Stacks long enough for a claimed tail (plan_tail) have records for its chunks.
+    const long long stack_tiles = (long long)layers * batch * kv_heads *
+        ((ctx->max_prompt + attn_tile_rows(kAttnWide, ctx->G) - 1) / attn_tile_rows(kAttnWide, ctx->G) +
+         (ctx->Cmax + attn_tile_rows(kAttnWide, ctx->G) - 1) / attn_tile_rows(kAttnWide, ctx->G));
+    if (layers > 1 && stack_tiles >= (long long)kTailFrom * 100 * attn_warps_per_cta(kAttnWide, ctx->G))
+        max_chunks = std::max(max_chunks, (size_t)kMaxSMs * attn_warps_per_cta(kAttnWide, ctx->G) * kTailChunks);
     ctx->max_chunks = max_chunks;
     ctx->off_partial = take(2 * max_chunks * partial_stride(ctx->G) * 4);
     ctx->off_arrive = take(max_chunks * 4);
-    ctx->off_err = take(256);
+    ctx->off_err = take(256);  // the error word; at 128 the claim counter of long stacked launches
     ctx->off_evplan = take((size_t)2 * layers * batch * kv_heads * (r + 1) * 4);
     ctx->base_bytes = o;
     // pass-1 chunks per head: at most one per tile of the longest head, capped (the host
@@ -693,6 +720,7 @@ int ra_bind(ra_ctx* ctx, void* device_arena, size_t bytes, void* stream)
     Ly.partial = (float*)(a + ctx->off_partial);
     Ly.arrive = (int32_t*)(a + ctx->off_arrive);
     Ly.err = (int32_t*)(a + ctx->off_err);
+    Ly.ticket = Ly.err + 32;
     Ly.evplan = (int32_t*)(a + ctx->off_evplan);
     Ly.qring = ctx->scoring ? (uint16_t*)(a + ctx->off_qring) : nullptr;
     Ly.qstats = ctx->scoring ? (float2*)(a + ctx->off_qstats) : nullptr;
@@ -738,6 +766,7 @@ int ra_bind(ra_ctx* ctx, void* device_arena, size_t bytes, void* stream)
         (e = cudaMemcpyAsync(Ly.pages, ctx->pages.data(), ctx->pages.size() * 4, cudaMemcpyHostToDevice, s)) !=
             cudaSuccess ||
         (e = cudaMemcpyAsync(Ly.err, &zero, 4, cudaMemcpyHostToDevice, s)) != cudaSuccess ||
+        (e = cudaMemsetAsync(Ly.ticket, 0, 4, s)) != cudaSuccess ||
         (e = cudaMemsetAsync(Ly.arrive, 0, ctx->max_chunks * 4, s)) != cudaSuccess)
         return cuda_fail(ctx, e, "table initialisation");
     // rows that were never written (past a head's cached slots) then read as zeros, never as stale NaNs

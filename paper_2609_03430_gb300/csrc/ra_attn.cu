@@ -37,6 +37,15 @@
 // memory, announced at the CTA's end, and the last CTA merges a head with all
 // its threads.  8.5 us a layer of one sequence, 33.1 instead of 36.6 us one of 16.
 //
+// Equal chunks end unequally: in a stacked launch of 2.6 ms the CTAs of some SMs
+// (always the same ones) end 2.7% after the median.  A long stacked launch of the
+// wide shape therefore cuts its last 3% of tiles into chunks of 1.5% of a warp's
+// share, at least 8 tiles, which warps claim as they finish.  Smaller or more of
+// them cut heads into more pieces, whose merges cost what the balance gives.  16
+// layers of the Qwen3-32B shape 2817 -> 2767 us (2778 with 1% chunks, 2771 with
+// 5% in 2.5% chunks, 2778 with 8% in 2%), 64 layers 10.81 -> 10.54 ms, 36 layers of
+// 16 Qwen3-4B-shape sequences 932 -> 915 us.
+//
 // With the scored comparator's buffers bound, the warp that consumes a head's
 // first tile also copies the head's G query rows into the query window, and
 // whoever finishes a head records each query's softmax normaliser beside it:
@@ -263,10 +272,33 @@ __device__ void iter_init(TileIter& it, const PT& p, int R0, int R1)
     enter_head<MODE>(it, p);
 }
 
-// The warp's chunk (its index): false once it is done.
+// The chunk that tile `f` of the launch lies in.
+template <int MODE, class PT>
+__device__ __forceinline__ int chunk_of(const PT& p, long long f)
+{
+    if (MODE == kModeStack && p.nstatic > 0 && f >= p.tail_tile) return p.nstatic + (int)(f - p.tail_tile) / p.tail_size;
+    return (int)(f / p.W);
+}
+
+// The warp's next chunk: false once there is none.  One chunk per warp; in a long stacked launch, then
+// chunks claimed one by one.
 template <int MODE, class PT>
 __device__ bool iter_next_chunk(TileIter& it, const PT& p, int warp_id)
 {
+    if (MODE == kModeStack && p.nstatic > 0 && it.chunk >= 0) {
+        int c = 0;
+        if ((threadIdx.x & 31) == 0) {
+            c = p.nstatic + atomicAdd(p.ticket, 1);
+            // every warp (nstatic of them) claims until a claim fails: the last failing one is the launch's last
+            if (c == p.nchunks + p.nstatic - 1) *p.ticket = 0;
+        }
+        c = __shfl_sync(0xffffffffu, c, 0);
+        if (c >= p.nchunks) return false;
+        const int R0 = p.tail_tile + (c - p.nstatic) * p.tail_size;
+        it.chunk = c;
+        iter_init<MODE>(it, p, R0, min(p.total, R0 + p.tail_size));
+        return true;
+    }
     if (it.chunk >= 0 || warp_id >= p.nchunks) return false;
     it.chunk = warp_id;
     const int R0 = warp_id * p.W;
@@ -914,7 +946,7 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
             const int hid = hd.z;
             int nth;
             const long long A = head_tile0<MODE>(p, hid, &nth);
-            const int w0 = (int)(A / p.W), w1 = (int)((A + nth - 1) / p.W);
+            const int w0 = chunk_of<MODE>(p, A), w1 = chunk_of<MODE>(p, A + nth - 1);
             if (w0 == w1) {  // the whole head was this warp's: normalise and write the output
                 if (gq < G) {
                     if (p.qring && tq == 0) record_stats<G, MODE>(p, hid, gq, m_run + log2f(l));

@@ -40,6 +40,7 @@ struct DevLayout {
     float* partial;        // attention split partials
     int32_t* arrive;       // split-piece arrival counters, one per chunk of the attention split
     int32_t* err;          // device error word
+    int32_t* ticket;       // claim counter of long stacked attention launches; zero between launches
     int32_t* evplan;       // [2][L][B][KVH][r + 1] evicted sets computed ahead (plan_kernel)
     // scored policy (null when the context was bound without its buffers)
     uint16_t* qring;       // [L][B][KVH][r][G][128] bf16: query of step s in slot (s - 1) mod r
@@ -130,7 +131,12 @@ struct AttnScalars {
     int32_t* arrive;        // per chunk: pieces merged so far of the head that starts there; zero between launches
     int W;                  // tiles per chunk of the split: warp w takes tiles [w W, (w + 1) W)
     int total;              // total tiles of the launch
-    int nchunks;            // ceil(total / W)
+    int nchunks;            // chunks in all
+    // A long stacked launch (wide shape): `nstatic` chunks of W tiles, one per warp, then from tile tail_tile on
+    // chunks of tail_size tiles that warps claim from *ticket as they finish (zero between launches).
+    int nstatic;            // 0: no such chunks
+    int tail_tile, tail_size;
+    int32_t* ticket;
     int nwarps;             // warps launched
     float qk_scale_log2;    // scale * log2(e)
     int early;              // kEarly*: the first tiles' K/V may be loaded before the predecessor kernel finishes

@@ -279,20 +279,23 @@ class ClockSampler:
                 "reasons": reasons, "samples": len(inside)}
 
 
-def profiled_traffic(cfg):
-    """DRAM bytes per attention launch from the committed ncu record, if it was taken on the
-    current kernel source for this workload's layer shape; else None."""
+def profiled_traffic(cfg, layers):
+    """DRAM bytes per attention launch of `layers` layers from the committed ncu record (bytes per
+    layer of a stacked launch), if it was taken on the current kernel sources for this workload's
+    layer shape; else None."""
     import hashlib
 
     try:
         with open(os.path.join(ROOT, "profiles", "attn_kernel_traffic.json")) as f:
             rec = json.load(f)
-        src = os.path.join(ROOT, "paper_2609_03430_gb300", "csrc", "ra_attn.cu")
-        digest = hashlib.sha256(open(src, "rb").read()).hexdigest()
-        if rec.get("kernel_source_sha256") != digest:
+        digest = hashlib.sha256()
+        for name in ("ra_attn.cu", "ra_attn_tile.cuh"):
+            with open(os.path.join(ROOT, "paper_2609_03430_gb300", "csrc", name), "rb") as f:
+                digest.update(f.read())
+        if rec.get("kernel_source_sha256") != digest.hexdigest():
             return None
-        per_cfg = rec.get("traffic_bytes_per_launch", {})
-        return per_cfg.get(str(cfg))
+        per_layer = rec.get("traffic_bytes_per_layer", {}).get(str(cfg))
+        return None if per_layer is None else per_layer * layers
     except Exception:
         return None
 
@@ -812,7 +815,7 @@ def run_ours(args, w):
 
     peaks, peak_src = measured_peaks()
     roof = attention_roofline(kern.get("attn"), clean, args.steps, w["L"], peaks, peak_src,
-                              args.traffic if args.traffic is not None else profiled_traffic(args.config))
+                              args.traffic if args.traffic is not None else profiled_traffic(args.config, w["L"] if args.calls == "step" else 1))
     comparator = None
     if main_policy == 0 and (args.comparator == "on" or
                              (args.comparator == "auto" and args.config in COMPARATOR_CONFIGS)):

@@ -100,6 +100,8 @@ struct ra_ctx {
     // The last launch that touched the caches was ra_append_kv's (everything before it has completed when
     // a kernel behind it starts): its successor may read all rows but the newest ahead of it.
     bool appended = false;
+    int last_layer = -1;     // the layer of the last fused attention launch (it writes that layer's newest rows,
+    bool last_compacted = false;  // or, with compaction inside the pass, whole regions)
     bool step_open = false;  // a step's prologue ran (plans launched, stack evicted) and its end has not
     int step_cur = 0;        // the plan half that step reads
     std::vector<int32_t> plan_g, plan_n;
@@ -1480,7 +1482,7 @@ int evict_pending(ra_ctx* ctx, int layer, cudaStream_t s, int plan_parity, std::
     // completed (every kernel before the predecessor has).  The scored policy reads scores its
     // predecessor computes, and with one layer the predecessor is this layer's previous step.
     // Neither starts early right after rows were loaded: the predecessor may have written this layer.
-    const bool clean = ctx->L >= 2 && !ctx->no_early_once && !ctx->appended;
+    const bool clean = ctx->L >= 2 && !ctx->no_early_once && !ctx->appended && ctx->last_layer != layer;
     ep.early = (ctx->policy != RA_POLICY_SNAPKV && clean) ? 1 : 0;
     const int score_early = clean ? 1 : 0;  // the scoring pass reads only older kernels' output
     ep.pending = 1;  // the step's token is appended by the attention launch below
@@ -1555,15 +1557,18 @@ int attend_pending(ra_ctx* ctx, int layer, int layers, const uint16_t* q, const 
     p.qk_scale_log2 = scale_log2(scale);
     // The kernel may request its first K/V tiles before its predecessor finishes when that
     // predecessor cannot be writing this layer's cache or tables: no eviction of this layer at
-    // this step (else it is this layer's compaction) and more than one layer (else it is this
+    // this step (else it is this layer's compaction) and another layer before (else it is this
     // layer's previous step), or but for each head's newest cached row.  Kernels let successors start only after their own wait, so
     // everything older than the predecessor has completed.
-    // With one layer in all (its previous step) or after a call that appended on its own, the newest
-    // cached rows are the ones that the predecessor may be writing.
-    p.early = evicted || ctx->no_early_once || layers > 1 ? kEarlyNone
-              : ctx->L > 1 && !ctx->appended              ? kEarlyAll
-                                                          : kEarlyButNewest;
+    // Behind this layer's previous step (one layer in all, or a layer called twice in a row) or a call that
+    // appended on its own, the newest cached rows are the ones that the predecessor may be writing.
+    const bool again = ctx->last_layer == layer;
+    p.early = evicted || ctx->no_early_once || layers > 1 || (again && ctx->last_compacted) ? kEarlyNone
+              : !again && !ctx->appended                                                   ? kEarlyAll
+                                                                                            : kEarlyButNewest;
     ctx->appended = false;
+    ctx->last_layer = layers > 1 ? -1 : layer;
+    ctx->last_compacted = !old_rows.empty();
     ctx->no_early_once = layers > 1;  // the next launch's predecessor then writes every layer's newest row
     {
         // rows read (a new token's from the caller), a new token's row written, q read, out written

@@ -3,6 +3,7 @@ group size; heads of one tile (most CTAs of the cluster hold none), of tiles tha
 rows while the cache grows, and of several tiles per warp; sequences without a prompt, finished ones, pages out
 of order; one layer (the tiles requested ahead of the wait leave out the row that the step before wrote) and two.
 The rule's other side, too many heads for clusters, runs the same checks."""
+import numpy as np
 import pytest
 
 from ra_testlib import Runner
@@ -49,5 +50,38 @@ def test_layer_call_after_separate_calls():
     run.restore_full(79, layers=(1, 0))
     run.fused = True
     run.step(check_attn_layers=(0, 1))
+    run.check_state()
+    run.close()
+
+
+def test_compaction_inside_the_pass_of_one_layer():
+    """The step behind a compacting attention launch does not read the regions that launch writes ahead of it."""
+    run = Runner(1, 8, 2, [70, 0], 200, 16, eseed=5, dseed=6, fused=True, compaction=2)
+    run.restore_full(639)
+    for t in range(36):
+        run.step(check_attn_layers=(0,))
+    run.check_state()
+    run.close()
+
+
+def test_one_layer_called_again():
+    """A layer of a stack stepped on its own, several steps in a row, then the other."""
+    import paper_2609_03430_gb300 as ra
+
+    run = Runner(2, 8, 2, [70, 3], 24, 8, eseed=7, dseed=8, fused=True)
+    for layer in (0, 1):
+        for t in range(70):
+            k = run.torch.zeros((run.B, run.KVH, run.D), dtype=run.torch.int16, device="cuda")
+            v = run.torch.zeros_like(k)
+            for b in range(run.B):
+                pos = run.orc.append(b, layer)
+                for h in range(run.KVH):
+                    k[b, h] = run.up(run.krows(layer, b, h, [pos])[0])
+                    v[b, h] = run.up(run.vrows(layer, b, h, [pos])[0])
+                run.orc.evict(b, layer)
+            q = np.stack([run.qrows(layer, b, t) for b in range(run.B)])
+            tq, out = run.up(q), run.torch.zeros((run.B, run.H, run.D), dtype=run.torch.int16, device="cuda")
+            ra.ra_decode_layer(run.ctx, layer, tq.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr())
+            run.check_layer_attention(layer, q, out.cpu().numpy())
     run.check_state()
     run.close()

@@ -1213,11 +1213,24 @@ int check_layer_call(ra_ctx* ctx, int layer, const uint16_t* q, const uint16_t* 
 // appends its token into the last slot, as after an eviction inside the layer's own call.
 //
 // A sequence that fires without a set computed ahead (the first step of a loaded run, a slot switched on
-// again) has its sets computed here, before the compaction, where there are at least kPlanNowLayers
-// layers: one plan and one compaction of every layer then replace a launch of the eviction kernel per layer
-// (36 layers of one sequence with 2112 candidates: 594 us of evictions, 172 us this way).  With fewer layers
-// the plan, one warp per head, takes about as long as the launches it replaces.
-constexpr int kPlanNowLayers = 4;
+// again) has its sets computed here, before the compaction, where that is the shorter way: one plan and one
+// compaction of every layer then replace a launch of the eviction kernel per layer.  The plan, one warp per
+// head, has a length of its own, so the stack must be deep.  A first step planned here / by layer, random
+// draws: one sequence of 8 heads, 1024 kept, 12 layers 104 / 136 us, 24 layers 182 / 307; 16 sequences
+// 323 / 329, 590 / 628; of 4 layers 57 / 50 and 145 / 127.  The radix passes of block, recency and exact
+// draws take several times the sampled cut: block draws, 8 sequences, 2048 kept, 12 layers 379 / 321 us,
+// 16 layers 452 / 419, 24 layers 604 / 614; 4 sequences, 7000 kept, 24 layers 1039 / 1345.
+constexpr int kPlanNowLayers = 12, kPlanNowLayersRadix = 24;
+// Nothing runs beside this plan, so it takes as many one-warp CTAs as an SM holds (7 KB each), not the one
+// of a plan beside a step: 24 layers of 32 heads of block draws 1439 us with one, 1039 with 24.
+constexpr int kPlanNowCtas = 24;
+
+bool plans_in_step(const ra_ctx* ctx)
+{
+    const bool radix = ctx->policy == RA_POLICY_BLOCK || ctx->policy == RA_POLICY_RECENCY ||
+                       (ctx->evict_mode & RA_EVICT_EXACT);
+    return ctx->L >= (radix ? kPlanNowLayersRadix : kPlanNowLayers);
+}
 
 // Sequence b's counters are those of layer 0 in every layer.
 bool layers_alike_seq(const ra_ctx* ctx, int b)
@@ -1299,7 +1312,7 @@ int step_prologue(ra_ctx* ctx, cudaStream_t s)
     // survivors move down (ordered) or the evicted slots are refilled from the newest rows
     // (order-free), and the layers then append the token as usual.
     bool planned_now = false;
-    if (now && serve && ctx->L >= kPlanNowLayers && (ctx->evict_mode & ~RA_EVICT_EXACT) == RA_EVICT_AUTO) {
+    if (now && serve && plans_in_step(ctx) && (ctx->evict_mode & ~RA_EVICT_EXACT) == RA_EVICT_AUTO) {
         EvictParams pp{};
         pp.lay = ctx->lay;
         pp.policy = ctx->policy;
@@ -1327,7 +1340,7 @@ int step_prologue(ra_ctx* ctx, cudaStream_t s)
             pp.n_trig = n;
             {
                 ProfScope ps(ctx, RA_KERNEL_PLAN, 0.0, s);
-                e = launch_plan(pp, ctx->sms, s);
+                e = launch_plan(pp, kPlanNowCtas * ctx->sms, s);
                 ps.done();
             }
             if (e != cudaSuccess) return cuda_fail(ctx, e, "plan launch");

@@ -1540,10 +1540,10 @@ cudaError_t launch_evict(const EvictParams& p, int cluster, cudaStream_t s)
     return cudaLaunchKernelEx(&cfg, evict_kernel<kEvRows, kEvBufs>, p);
 }
 
-cudaError_t launch_plan(const EvictParams& p, int sms, cudaStream_t s)
+cudaError_t launch_plan(const EvictParams& p, int ctas, cudaStream_t s)
 {
     const int items = p.lay.L * p.n_trig * p.lay.KVH;
-    plan_kernel<<<(unsigned)std::min(items, std::max(sms, 1)), 32, 0, s>>>(p);
+    plan_kernel<<<(unsigned)std::min(items, std::max(ctas, 1)), 32, 0, s>>>(p);
     return cudaGetLastError();
 }
 

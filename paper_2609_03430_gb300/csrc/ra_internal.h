@@ -207,9 +207,9 @@ constexpr int kEvBufs = 3;   // copy buffers per warp: 192 KB per CTA, one CTA p
 cudaError_t launch_evict(const EvictParams& p, int cluster, cudaStream_t s);
 // The evicted sets of the triggered sequences' heads in every layer, from the counters alone
 // (the random draw reads no cache data), into half p.ev_plan_parity of lay.evplan; one warp per
-// CTA, at most `sms` CTAs looping over the (layer, sequence, KV head) items, little shared memory,
-// so that it runs beside the attention kernel.
-cudaError_t launch_plan(const EvictParams& p, int sms, cudaStream_t s);
+// CTA, at most `ctas` CTAs looping over the (layer, sequence, KV head) items, little shared memory,
+// so that with one per SM it runs beside the attention kernel.
+cudaError_t launch_plan(const EvictParams& p, int ctas, cudaStream_t s);
 // Every layer's round of the triggered sequences (layers 0 .. layers - 1, counters alike in every
 // layer), in place, from the evicted sets in half p.ev_plan_parity of lay.evplan: one CTA (a cluster, while
 // the SMs are more) per (layer, sequence, KV head) and array.

@@ -1,6 +1,7 @@
-"""Sequences that fire without a set computed ahead, in stacks of four layers and more: the sets are computed in
-the step and every layer's round runs in one launch, in both layouts, for every policy of the plans, bit for bit
-against the oracle; a slot switched on again at its firing step, beside one whose set was computed ahead."""
+"""Sequences that fire without a set computed ahead, in stacks of twelve layers and more (24 for recency and block
+draws): the sets are computed in the step and every layer's round runs in one launch, in both layouts, for every
+policy of the plans, bit for bit against the oracle; a slot switched on again at its firing step, beside one whose
+set was computed ahead."""
 import pytest
 
 from ra_testlib import Runner
@@ -13,16 +14,17 @@ pytestmark = pytest.mark.gpu
 def test_first_round_of_a_loaded_run(policy, block, compaction):
     import paper_2609_03430_gb300 as ra
 
-    run = Runner(5, 4, 2, [33, 0, 90], 100, 16, eseed=policy, dseed=9, fused=True, policy=policy, block=block,
+    L, KVH = (24, 1) if policy >= 2 else (12, 2)
+    run = Runner(L, 2 * KVH, KVH, [33, 0, 90], 100, 16, eseed=policy, dseed=9, fused=True, policy=policy, block=block,
                  compaction=compaction)
-    run.restore_full(639, layers=range(5))  # all fire at the next step
+    run.restore_full(639, layers=range(L))  # all fire at the next step
     ra.ra_profile_reset(run.ctx)
     for t in range(35):
         if t == 10:
             run.set_active(1, False)
         if t == 26:  # on again: it fires 6 steps later than the others, once more after
             run.set_active(1, True)
-        run.step(check_attn_layers=(0, 4) if t in (0, 1, 16, 31, 32) else ())
+        run.step(check_attn_layers=(0, L - 1) if t in (0, 1, 16, 31, 32) else ())
         if t in (0, 1, 16, 32):
             run.check_state()
     assert ra.ra_profile_read(run.ctx, ra.RA_KERNEL_EVICT)[1] == 0 and ra.ra_profile_read(run.ctx, ra.RA_KERNEL_SELECT)[1] == 0
@@ -31,15 +33,15 @@ def test_first_round_of_a_loaded_run(policy, block, compaction):
 
 
 def test_slot_on_again_at_its_round():
-    run = Runner(4, 4, 2, [20, 20], 60, 8, eseed=3, dseed=4, fused=True)
-    run.restore_full(399, layers=range(4))
+    run = Runner(12, 4, 2, [20, 20], 60, 8, eseed=3, dseed=4, fused=True)
+    run.restore_full(399, layers=range(12))
     run.step()
     for _ in range(7):
         run.step()
     run.set_active(1, False)  # both would fire at the next step: slot 1's set is ready, and not used
-    run.step(check_attn_layers=(0, 3))
+    run.step(check_attn_layers=(0, 11))
     run.set_active(1, True)
-    run.step(check_attn_layers=(0, 3))  # slot 1's round
+    run.step(check_attn_layers=(0, 11))  # slot 1's round
     run.check_state()
     for _ in range(10):
         run.step()

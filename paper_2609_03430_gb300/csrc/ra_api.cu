@@ -1215,12 +1215,15 @@ int check_layer_call(ra_ctx* ctx, int layer, const uint16_t* q, const uint16_t* 
 // A sequence that fires without a set computed ahead (the first step of a loaded run, a slot switched on
 // again) has its sets computed here, before the compaction, where that is the shorter way: one plan and one
 // compaction of every layer then replace a launch of the eviction kernel per layer.  The plan, one warp per
-// head, has a length of its own, so the stack must be deep.  A first step planned here / by layer, random
-// draws: one sequence of 8 heads, 1024 kept, 12 layers 104 / 136 us, 24 layers 182 / 307; 16 sequences
-// 323 / 329, 590 / 628; of 4 layers 57 / 50 and 145 / 127.  The radix passes of block, recency and exact
-// draws take several times the sampled cut: block draws, 8 sequences, 2048 kept, 12 layers 379 / 321 us,
-// 16 layers 452 / 419, 24 layers 604 / 614; 4 sequences, 7000 kept, 24 layers 1039 / 1345.
-constexpr int kPlanNowLayers = 12, kPlanNowLayersRadix = 24;
+// head, has a length of its own, so the stack must be deep: deeper where the plan takes radix passes
+// (recency, block and exact draws) instead of the sampled cut, and where its keys wait for the candidates'
+// positions (block draws, order-free slots, whose rounds by layer are short as well).  A first step planned
+// here / by layer:
+//   random, ordered       32 heads, 8000 kept: 4 layers 221 / 218 us, 8 layers 378 / 424;
+//                         8 heads, 1024 kept: 4 layers 54 / 83, 24 layers 195 / 477
+//   recency, ordered      32 heads, 8000 kept: 4 layers 286 / 233, 8 layers 443 / 453
+//   random, order-free    128 heads, 1024 kept: 4 layers 145 / 127, 12 layers 323 / 329, 24 layers 590 / 628
+//   block, order-free     64 heads, 2048 kept: 12 layers 379 / 321, 16 layers 452 / 419, 24 layers 604 / 614
 // Nothing runs beside this plan, so it takes as many one-warp CTAs as an SM holds (7 KB each), not the one
 // of a plan beside a step: 24 layers of 32 heads of block draws 1439 us with one, 1039 with 24.
 constexpr int kPlanNowCtas = 24;
@@ -1229,7 +1232,7 @@ bool plans_in_step(const ra_ctx* ctx)
 {
     const bool radix = ctx->policy == RA_POLICY_BLOCK || ctx->policy == RA_POLICY_RECENCY ||
                        (ctx->evict_mode & RA_EVICT_EXACT);
-    return ctx->L >= (radix ? kPlanNowLayersRadix : kPlanNowLayers);
+    return ctx->L >= 4 * (radix ? 2 : 1) * (keys_read_positions(ctx) ? 3 : 1);
 }
 
 // Sequence b's counters are those of layer 0 in every layer.

@@ -55,7 +55,9 @@
 // rows runs on the tensor cores (mma.sync m16n8k16, bf16 in, fp32 accumulate):
 // S = Q K^T takes the query heads as the 16 M rows (G <= 8 used, the rest
 // zero) and 8 cache rows per N tile; O += P V reuses the S accumulator
-// fragments as the A operand (P rounded to bf16).  Q fragments stay in
+// fragments as the A operand (P rounded to bf16; launches over several layers
+// take what the rounding left out as the A rows 8..15, which are otherwise
+// zero, into accumulators of their own: see ra_attn_tile.cuh).  Q fragments stay in
 // registers for a whole head piece; K and V are read with ldmatrix from TMA
 // tiles stored with the 128-byte swizzle, so the reads are bank-conflict free.
 // Each lane owns one query head (lane / 4): the softmax statistics need only
@@ -376,6 +378,14 @@ __device__ __forceinline__ void mma_rows8(float& c0, float& c1, uint32_t a0, uin
     (void)d3;
 }
 #pragma nv_diag_default 550
+
+// The same with all 16 rows: the weights in rows 0..7 (a0, a2), their residuals in rows 8..15 (a1, a3).
+__device__ __forceinline__ void mma_rows16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                           uint32_t b1)
+{
+    const uint32_t a[4] = {a0, a1, a2, a3};
+    mma16816(c, a, b0, b1);
+}
 #endif
 
 // The scored policy's window: the softmax normaliser of query head g of head `hid` at this
@@ -733,14 +743,25 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
     uint32_t qa[8][2];  // fragments of Q (rows 0..7) for the 8 k-steps of 16 channels (A, or B of Q^T)
 #if RA_ATTN_TRANSPOSED
     const int hA = 2 * tq, hB = 2 * tq + 1;  // the query heads of this lane's accumulator columns
-    PieceT acc;
+    constexpr int RES = MODE != kModeStack ? kResNone : (G <= 4 ? kResCols : kResAcc);
+    const int qh = RES == kResCols ? gq & 3 : gq;  // the head whose query rows this lane's fragments hold
+    PieceT<RES> acc;
     acc.clear();
 #else
     const int mi = lane >> 3, ri = lane & 7;  // ldmatrix: matrix and row this lane addresses
-    float O[16][2];     // O[head gq][n-tile * 8 + 2 tq + {0, 1}]
+    constexpr bool RES = MODE == kModeStack;  // the weights' residuals count too
+    const int qh = gq;
+    float O[16][RES ? 4 : 2];  // O[head gq][n-tile * 8 + 2 tq + {0, 1}]; then the residuals'
     float m_run = -INFINITY, l_run = 0.f;
+    auto clear = [&] {
+        m_run = -INFINITY;
+        l_run = 0.f;
 #pragma unroll
-    for (int nt = 0; nt < 16; ++nt) O[nt][0] = O[nt][1] = 0.f;
+        for (int nt = 0; nt < 16; ++nt)
+#pragma unroll
+            for (int e = 0; e < (RES ? 4 : 2); ++e) O[nt][e] = 0.f;
+    };
+    clear();
 #endif
 
     for (int t = 0; t < issued; ++t) {
@@ -770,8 +791,8 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
             }
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk) {
-                qa[kk][0] = gq < G ? *reinterpret_cast<const uint32_t*>(Qs + gq * kRowBytes + (16 * kk + 2 * tq) * 2) : 0u;
-                qa[kk][1] = gq < G ? *reinterpret_cast<const uint32_t*>(Qs + gq * kRowBytes + (16 * kk + 8 + 2 * tq) * 2) : 0u;
+                qa[kk][0] = qh < G ? *reinterpret_cast<const uint32_t*>(Qs + qh * kRowBytes + (16 * kk + 2 * tq) * 2) : 0u;
+                qa[kk][1] = qh < G ? *reinterpret_cast<const uint32_t*>(Qs + qh * kRowBytes + (16 * kk + 8 + 2 * tq) * 2) : 0u;
             }
             if ((hd.y & kHead0) && p.qring) {  // the scored policy's window: this step's query rows of the head
                 const int r = p.lay.r;
@@ -830,6 +851,7 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
 
         if (hd.y & kLast) {  // last tile of the piece
             float la, lb;
+            acc.add_residuals();
             acc.sum_lanes(la, lb);
             const int hid = hd.z;
             int nth;
@@ -867,7 +889,7 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
                     rec = reinterpret_cast<float*>(deposit<G>(smem, warp, chunk < w1, s));
                     rs = C::DEP_ROW;
                 }
-                acc.store<G>(rec, rs, la, lb, lane);
+                acc.template store<G>(rec, rs, la, lb, lane);
                 if (a == z) {
                     if (lane == 0) cm.part[a == w0 ? 1 : 0] = {hid, w0 / C::WARPS, w1 / C::WARPS - w0 / C::WARPS + 1};
                 } else {
@@ -917,10 +939,9 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
                 l_run *= a;
                 m_run = m_new;
 #pragma unroll
-                for (int nt = 0; nt < 16; ++nt) {
-                    O[nt][0] *= a;
-                    O[nt][1] *= a;
-                }
+                for (int nt = 0; nt < 16; ++nt)
+#pragma unroll
+                    for (int e = 0; e < (RES ? 4 : 2); ++e) O[nt][e] *= a;
             }
             float pr[4];
 #pragma unroll
@@ -929,17 +950,30 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
             for (int e = 0; e < 4; ++e) pr[e] = (MODE == kModeCompact && sc[e] == -INFINITY) ? 0.f : exp2f(sc[e] - m_run);
             l_run += (pr[0] + pr[1]) + (pr[2] + pr[3]);
             const uint32_t pa0 = pack_bf16x2(pr[0], pr[1]), pa2 = pack_bf16x2(pr[2], pr[3]);
+            const uint32_t pa1 = residual_bf16x2(pr[0], pr[1], pa0), pa3 = residual_bf16x2(pr[2], pr[3], pa2);
             // O += P V: 16 n-tiles of 8 channels, k = the 16 rows
 #pragma unroll
             for (int np = 0; np < 8; ++np) {
                 uint32_t b[4];
                 ldsm_x4_t(b, vs + swz<G>(bs + (mi & 1) * 8 + ri, 2 * np + (mi >> 1)));
-                mma_rows8(O[2 * np][0], O[2 * np][1], pa0, pa2, b[0], b[1]);
-                mma_rows8(O[2 * np + 1][0], O[2 * np + 1][1], pa0, pa2, b[2], b[3]);
+                if constexpr (RES) {
+                    mma_rows16(O[2 * np], pa0, pa1, pa2, pa3, b[0], b[1]);
+                    mma_rows16(O[2 * np + 1], pa0, pa1, pa2, pa3, b[2], b[3]);
+                } else {
+                    mma_rows8(O[2 * np][0], O[2 * np][1], pa0, pa2, b[0], b[1]);
+                    mma_rows8(O[2 * np + 1][0], O[2 * np + 1][1], pa0, pa2, b[2], b[3]);
+                }
             }
         }
 
         if (hd.y & kLast) {  // last tile of the piece
+            if constexpr (RES) {
+#pragma unroll
+                for (int nt = 0; nt < 16; ++nt) {
+                    O[nt][0] = add_residual(O[nt][0], O[nt][2]);
+                    O[nt][1] = add_residual(O[nt][1], O[nt][3]);
+                }
+            }
             float l = l_run;
             l += __shfl_xor_sync(0xffffffffu, l, 1);
             l += __shfl_xor_sync(0xffffffffu, l, 2);
@@ -978,10 +1012,7 @@ __global__ void __launch_bounds__(Cfg<G>::WARPS * 32, 1)
                     if (lane == 0) p.arrive[w0] = 0;  // ready for the next launch
                 }
             }
-            m_run = -INFINITY;
-            l_run = 0.f;
-#pragma unroll
-            for (int nt = 0; nt < 16; ++nt) O[nt][0] = O[nt][1] = 0.f;
+            clear();
         }
 #endif
 

@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     if (first_late) issue(t0);
 
     const int gq = lane >> 2, tq = lane & 3;
-    PieceT acc;
+    PieceT<kResNone> acc;
     acc.clear();
     if (t0 < t1) {
         uint32_t qa[8][2];  // the query rows as B fragments of the 8 k-steps

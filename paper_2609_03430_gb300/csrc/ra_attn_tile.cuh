@@ -62,18 +62,54 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
            ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(hi)) << 16);
 }
 
+// What the rounding of two weights to bf16 (w) left out.
+__device__ __forceinline__ uint32_t residual_bf16x2(float lo, float hi, uint32_t w)
+{
+    return pack_bf16x2(lo - bf16lo(w), hi - bf16hi(w));
+}
+// A sum of products with the residuals, onto that with the rounded weights (an infinite one stays: V's infinities
+// times a residual of zero are NaN).
+__device__ __forceinline__ float add_residual(float o, float res) { return isinf(o) ? o : o + res; }
+
+// Residuals of the weights.  Weights rounded to bf16 relative to a running maximum are exact where they are the
+// maximum, so a head in short pieces loses less than one in long pieces: 64 layers of one sequence, launched one by one
+// (a tile per piece), were 2.11e-3 from 64 bits, in one launch 2.33e-3, of which the output's own rounding is
+// 1.65e-3.  Launches over several layers therefore multiply V with the residuals too (1.66e-3): in the columns that
+// at most four query heads leave free, whose lanes hold the same logits once more (kResCols), else as products of
+// their own (kResAcc).
+constexpr int kResNone = 0, kResCols = 1, kResAcc = 2;
+
 // The transposed products' running state of a head piece, per lane: O^T (m-tile mt = channels 16 mt..:
 // {ch 16 mt + gq: heads hA, hB; ch 16 mt + gq + 8: hA, hB}, gq = lane / 4, hA = 2 (lane % 4), hB = hA + 1), the
-// running max and the (lane-partial) sum of the two heads.
+// running max and the (lane-partial) sum of the two heads.  kResCols: columns 4 .. 7 are the residuals' of heads 0 .. 3;
+// kResAcc: R holds the residuals'.
+template <int RES>
 struct PieceT {
     float O[8][4];
+    float R[RES == kResAcc ? 8 : 1][4];
     float mA, mB, lA, lB;
     __device__ __forceinline__ void clear()
     {
         mA = mB = -INFINITY;
         lA = lB = 0.f;
 #pragma unroll
-        for (int mt = 0; mt < 8; ++mt) O[mt][0] = O[mt][1] = O[mt][2] = O[mt][3] = 0.f;
+        for (int mt = 0; mt < 8; ++mt)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                O[mt][e] = 0.f;
+                if (RES == kResAcc) R[mt][e] = 0.f;
+            }
+    }
+    // The piece's end: the residuals' products into O (kResCols: of the lanes that hold heads 0 .. 3).
+    __device__ __forceinline__ void add_residuals()
+    {
+        if constexpr (RES != kResNone) {
+#pragma unroll
+            for (int mt = 0; mt < 8; ++mt)
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    O[mt][e] = add_residual(O[mt][e], RES == kResAcc ? R[mt][e] : __shfl_xor_sync(0xffffffffu, O[mt][e], 2));
+        }
     }
     __device__ __forceinline__ void sum_lanes(float& la, float& lb) const  // over the 8 lanes of a head pair
     {
@@ -145,7 +181,8 @@ __device__ __forceinline__ void tile_logits(float (&sv)[4], uint32_t ks, int bs,
 }
 
 // The running max of both heads raised where xA, xB (this lane's largest logits) exceed it by more than 2^8.
-__device__ __forceinline__ void raise_max(PieceT& s, float xA, float xB)
+template <int RES>
+__device__ __forceinline__ void raise_max(PieceT<RES>& s, float xA, float xB)
 {
     if (!__any_sync(0xffffffffu, xA > s.mA + kTau || xB > s.mB + kTau)) return;
 #pragma unroll
@@ -165,12 +202,18 @@ __device__ __forceinline__ void raise_max(PieceT& s, float xA, float xB)
         s.O[mt][2] *= aA;
         s.O[mt][1] *= aB;
         s.O[mt][3] *= aB;
+        if (RES == kResAcc) {
+            s.R[mt][0] *= aA;
+            s.R[mt][2] *= aA;
+            s.R[mt][1] *= aB;
+            s.R[mt][3] *= aB;
+        }
     }
 }
 
-// The weights of 16 rows, added to the sums; P^T as B fragments.
-template <bool MASK>
-__device__ __forceinline__ void tile_weights(PieceT& s, const float (&sv)[4], uint32_t& b0, uint32_t& b1)
+// The weights of 16 rows, added to the sums; P^T as B fragments in b, with kResAcc their residuals' in c.
+template <bool MASK, int RES>
+__device__ __forceinline__ void tile_weights(PieceT<RES>& s, const float (&sv)[4], uint32_t (&b)[2], uint32_t (&c)[2], int lane)
 {
     float pr[4];
 #pragma unroll
@@ -180,16 +223,30 @@ __device__ __forceinline__ void tile_weights(PieceT& s, const float (&sv)[4], ui
     }
     s.lA += pr[0] + pr[2];
     s.lB += pr[1] + pr[3];
-    b0 = movtrans(pack_bf16x2(pr[0], pr[1]));
-    b1 = movtrans(pack_bf16x2(pr[2], pr[3]));
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const uint32_t w = pack_bf16x2(pr[2 * i], pr[2 * i + 1]);
+        const uint32_t left = RES == kResNone ? 0u : residual_bf16x2(pr[2 * i], pr[2 * i + 1], w);
+        b[i] = movtrans(RES == kResCols && (lane & 2) ? left : w);
+        if (RES == kResAcc) c[i] = movtrans(left);
+    }
+}
+
+// O^T += V^T P^T of one m-tile (v: V transposed), and the residuals'.
+template <int RES>
+__device__ __forceinline__ void add_product(PieceT<RES>& s, int mt, const uint32_t (&v)[4], const uint32_t (&b)[2],
+                                            const uint32_t (&c)[2])
+{
+    mma16816(s.O[mt], v, b[0], b[1]);
+    if (RES == kResAcc) mma16816(s.R[mt], v, c[0], c[1]);
 }
 
 // n rows of a tile (K at shared address ks, V at vs): S^T = K Q^T, online softmax, O^T += V^T P^T.  qa: the
-// head's query rows as B fragments of the 8 k-steps.  32 rows at a time, so that two batches' products and
+// head's query rows as B fragments of the 8 k-steps (kResCols: twice, as columns 0 .. 3 and 4 .. 7).  32 rows at a time, so that two batches' products and
 // exponentials run beside each other (36 layers of 16 sequences 1167 us, 16 rows at a time; 1152 us this way),
 // then 16 for what is left.
-template <int HALF, bool MASK>
-__device__ __forceinline__ void attend_tile(PieceT& s, uint32_t ks, uint32_t vs, int n, const uint32_t (&qa)[8][2], float sl,
+template <int HALF, bool MASK, int RES>
+__device__ __forceinline__ void attend_tile(PieceT<RES>& s, uint32_t ks, uint32_t vs, int n, const uint32_t (&qa)[8][2], float sl,
                                             uint32_t ev_lo, uint32_t ev_hi, int lane)
 {
     const int mi = lane >> 3, ri = lane & 7;
@@ -199,29 +256,29 @@ __device__ __forceinline__ void attend_tile(PieceT& s, uint32_t ks, uint32_t vs,
         tile_logits<HALF, MASK>(s0, ks, bs, n, qa, sl, ev_lo, ev_hi, lane);
         tile_logits<HALF, MASK>(s1, ks, bs + 16, n, qa, sl, ev_lo, ev_hi, lane);
         raise_max(s, fmaxf(fmaxf(s0[0], s0[2]), fmaxf(s1[0], s1[2])), fmaxf(fmaxf(s0[1], s0[3]), fmaxf(s1[1], s1[3])));
-        uint32_t b0, b1, c0, c1;
-        tile_weights<MASK>(s, s0, b0, b1);
-        tile_weights<MASK>(s, s1, c0, c1);
+        uint32_t b0[2], b1[2], c0[2], c1[2];
+        tile_weights<MASK>(s, s0, b0, c0, lane);
+        tile_weights<MASK>(s, s1, b1, c1, lane);
 #pragma unroll
         for (int mt = 0; mt < 8; ++mt) {
             uint32_t v4[4], w4[4];
             ldsm_x4_t(v4, vs + swz_tile<HALF>(bs + (mi >> 1) * 8 + ri, 2 * mt + (mi & 1)));
             ldsm_x4_t(w4, vs + swz_tile<HALF>(bs + 16 + (mi >> 1) * 8 + ri, 2 * mt + (mi & 1)));
-            mma16816(s.O[mt], v4, b0, b1);
-            mma16816(s.O[mt], w4, c0, c1);
+            add_product(s, mt, v4, b0, c0);
+            add_product(s, mt, w4, b1, c1);
         }
     }
     if (bs < n) {
         float s0[4];
         tile_logits<HALF, MASK>(s0, ks, bs, n, qa, sl, ev_lo, ev_hi, lane);
         raise_max(s, fmaxf(s0[0], s0[2]), fmaxf(s0[1], s0[3]));
-        uint32_t b0, b1;
-        tile_weights<MASK>(s, s0, b0, b1);
+        uint32_t b0[2], c0[2];
+        tile_weights<MASK>(s, s0, b0, c0, lane);
 #pragma unroll
         for (int mt = 0; mt < 8; ++mt) {
             uint32_t v4[4];
             ldsm_x4_t(v4, vs + swz_tile<HALF>(bs + (mi >> 1) * 8 + ri, 2 * mt + (mi & 1)));
-            mma16816(s.O[mt], v4, b0, b1);
+            add_product(s, mt, v4, b0, c0);
         }
     }
 }

@@ -389,7 +389,9 @@ int ra_get_kv(ra_ctx* ctx, int layer, int seq, int kv_head, uint16_t* host_k, ui
  * RA_ERR_DEVICE_TIMEOUT if a kernel gave up a bounded wait (every mbarrier wait of the pipelines
  * is bounded at 2 s; the kernel then lets its own copies land, releases what it holds and
  * returns), RA_ERR_STATE if an eviction plan disagreed with the host counters.  The word is
- * cleared once reported, so a later call reports only new events.
+ * cleared once reported, so a later call reports only new events; so are the attention's claim and
+ * arrival counters, which a launch that gave up leaves behind.  (What that launch computed is lost:
+ * its outputs, and rows it should have written, are incomplete.)
  */
 int ra_check_device(ra_ctx* ctx, void* stream);
 

@@ -1776,9 +1776,14 @@ int ra_check_device(ra_ctx* ctx, void* stream)
     if ((e = cudaStreamSynchronize((cudaStream_t)stream)) != cudaSuccess) return cuda_fail(ctx, e, "stream sync");
     int32_t w = 0;
     if ((e = cudaMemcpy(&w, ctx->lay.err, 4, cudaMemcpyDeviceToHost)) != cudaSuccess) return cuda_fail(ctx, e, "err read");
-    if (w != 0) {  // reported once: clear it (the stream is idle, nothing else writes it now)
-        const int32_t zero = 0;
-        if ((e = cudaMemcpy(ctx->lay.err, &zero, 4, cudaMemcpyHostToDevice)) != cudaSuccess)
+    if (w != 0) {
+        // Reported once: clear it (the stream is idle, nothing else writes it now), and with it the counters that
+        // a launch which gave up leaves behind: its claims and the arrivals at heads that were never merged.
+        cudaStream_t s = (cudaStream_t)stream;
+        if ((e = cudaMemsetAsync(ctx->lay.err, 0, 4, s)) != cudaSuccess ||
+            (e = cudaMemsetAsync(ctx->lay.ticket, 0, 4, s)) != cudaSuccess ||
+            (e = cudaMemsetAsync(ctx->lay.arrive, 0, ctx->max_chunks * 4, s)) != cudaSuccess ||
+            (e = cudaStreamSynchronize(s)) != cudaSuccess)
             return cuda_fail(ctx, e, "err clear");
     }
     if (w == kDeviceErrTimeout) return fail(ctx, RA_ERR_DEVICE_TIMEOUT, "a kernel gave up a bounded wait");

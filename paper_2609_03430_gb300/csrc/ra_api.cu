@@ -96,7 +96,8 @@ struct ra_ctx {
     cudaEvent_t fork_ev = nullptr, plan_ev = nullptr;
     bool plan_pending = false;
     int parity = 0;
-    bool no_early_once = false;  // the next fused launches follow an eviction, or a copy into the caches
+    // The next fused launches follow an eviction, a copy into the caches, or a call that wrote a query window.
+    bool no_early_once = false;
     // The last launch that touched the caches was ra_append_kv's (everything before it has completed when
     // a kernel behind it starts): its successor may read all rows but the newest ahead of it.
     bool appended = false;
@@ -1040,6 +1041,7 @@ int ra_restore_queries(ra_ctx* ctx, int layer, const uint16_t* q, float scale, v
     const size_t base = (size_t)layer * ctx->B;
     cudaError_t e = launch_restore_queries(ctx->lay, layer, q, ctx->g.data() + base, s);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "query window restore launch");
+    ctx->no_early_once = true;  // a scoring pass behind these launches reads what they write
     // The normalisers of the loaded queries: each over the prompt and the cached rows at
     // positions up to its own (what it attended to at its step, as no eviction can come between).
     EvictParams p{};
@@ -1180,6 +1182,7 @@ int ra_decode_attn(ra_ctx* ctx, int layer, const uint16_t* q, uint16_t* out, flo
     cudaError_t e = launch_attention(shape, p, &ctx->tmap_k[shape], &ctx->tmap_v[shape], ctas, s);
     ps.done();
     if (e != cudaSuccess) return cuda_fail(ctx, e, "attention launch");
+    if (p.qring) ctx->no_early_once = true;  // it records the layer's window: a scoring pass behind it waits
     return RA_OK;
 }
 
@@ -1932,5 +1935,6 @@ extern "C" int ra_decode_attn_noalloc(ra_ctx* ctx, int layer, const uint16_t* q,
     if (e != cudaSuccess) return cuda_fail(ctx, e, "scratch counter clear");
     e = launch_attention(shape, p, &ctx->tmap_k[shape], &ctx->tmap_v[shape], ctas, s);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "attention launch");
+    if (p.qring) ctx->no_early_once = true;  // (as in ra_decode_attn)
     return RA_OK;
 }

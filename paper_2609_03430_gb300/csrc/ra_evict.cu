@@ -1468,12 +1468,6 @@ cudaError_t launch_select(const EvictParams& p, cudaStream_t s)
     const size_t smem = select_smem(N, p.lay.r, p.policy == RA_POLICY_SNAPKV);
     const bool wide = N >= kSelWideFrom && !p.holefill;
     auto kernel = wide ? select_kernel<kSelWide> : select_kernel<256>;
-    static size_t configured[2] = {0, 0};
-    if (smem > 40 * 1024 && smem > configured[wide]) {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        configured[wide] = smem;
-    }
     return launch_pdl(kernel, dim3(p.n_trig, p.lay.KVH, p.layers), dim3(wide ? kSelWide : 256), smem, s, p);
 }
 
@@ -1512,7 +1506,15 @@ cudaLaunchConfig_t evict_config(int cluster, int heads_reps, int n_trig, cudaStr
 cudaError_t evict_prepare(int* active)
 {
     auto kernel = evict_kernel<kEvRows, kEvBufs>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEvSmem);
+    // (attributes hold for the current device, the bound context's, so they are set here and not before a launch)
+    auto shared = [](auto* k, size_t bytes) {
+        return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    };
+    cudaError_t e = shared(kernel, kEvSmem);
+    if (e == cudaSuccess) e = shared(select_kernel<256>, kSelectSmemLimit);
+    if (e == cudaSuccess) e = shared(select_kernel<kSelWide>, kSelectSmemLimit);
+    if (e == cudaSuccess) e = shared(compact_stack_kernel<false>, kStkSmem<false>);
+    if (e == cudaSuccess) e = shared(compact_stack_kernel<true>, kStkSmem<true>);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     bool any = false;
@@ -1549,14 +1551,6 @@ cudaError_t launch_plan(const EvictParams& p, int ctas, cudaStream_t s)
 
 cudaError_t launch_compact_stack(const EvictParams& p, int layers, int sms, cudaStream_t s)
 {
-    static bool configured = false;
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(compact_stack_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStkSmem<false>);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(compact_stack_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStkSmem<true>);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
     const int units = 2 * layers * p.n_trig * p.lay.KVH;
     // A cluster per head's array while at least two CTAs of it fit beside the others' (one per SM), and
     // every CTA has a chunk; rows that move further than a chunk stay with one CTA.

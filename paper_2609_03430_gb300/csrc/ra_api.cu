@@ -516,8 +516,22 @@ bool plan_usable(const ra_ctx* ctx)
 // of place, over all CTAs).
 bool scored_stack_usable(const ra_ctx* ctx)
 {
-    return ctx->policy == RA_POLICY_SNAPKV && ctx->compaction == RA_COMPACT_ORDERED && ctx->L > 1 && ctx->L <= 65535 && ctx->r <= kEvMaxEvicted &&
-           (ctx->evict_mode & ~RA_EVICT_EXACT) != RA_EVICT_TWO_KERNELS;
+    return ctx->policy == RA_POLICY_SNAPKV && ctx->compaction == RA_COMPACT_ORDERED && ctx->L > 1 && ctx->L <= 65535 &&
+           ctx->r <= kEvMaxEvicted && (ctx->evict_mode & ~RA_EVICT_EXACT) != RA_EVICT_TWO_KERNELS;
+}
+
+// Whether `heads` heads that fire in every layer are shorter that way.  The in-place compaction of a buffer of more than
+// 128 rows is a chain of one CTA per head and array, 45 KB/us, where the one by layer runs over all CTAs: it then
+// takes enough layers, whose scores and selections run beside each other.  Microseconds, from a step with one round at
+// the start / by layer: r = 130, 2 heads of 1024 kept, 2 layers 54 / 62; of 4096, 2 layers 89 / 78, 3 layers 90 / 105;
+// of 15000, 4 layers 232 / 223, 6 layers 242 / 343; 8 heads of 15000, 2 layers 254 / 206, 3 layers 279 / 300; r = 512,
+// 8 heads of 1024, 2 layers 93 / 75, 3 layers 94 / 104; of 8000, 3 layers 244 / 242, 4 layers 270 / 317.
+bool scored_stack_shorter(const ra_ctx* ctx, int heads)
+{
+    if (ctx->r <= 128) return true;
+    const double cost = 25 + 0.0125 * ctx->K + 0.06 * (ctx->r - 128);     // of the stack, beyond a layer's round
+    const double gain = 20 + (heads <= 4 ? 0.0018 : 0.0035) * ctx->K;     // of each layer
+    return ctx->L * gain >= cost;
 }
 
 // One eviction round of the triggered sequences in p: [score passes,] select, compact (unless
@@ -1388,7 +1402,7 @@ int step_prologue(ra_ctx* ctx, cudaStream_t s)
             // rows moved per head: the survivors below the token (ordered), the m refills (order-free)
             moved += (double)(fill ? c + 1 - ctx->r - ctx->K : ctx->K + ctx->r - 1) * ctx->KVH * ctx->L;
         }
-        if (n > 0) {
+        if (n > 0 && (!scored || scored_stack_shorter(ctx, n * ctx->KVH))) {
             sp.n_trig = n;
             if (scored) {
                 sp.policy = ctx->policy;

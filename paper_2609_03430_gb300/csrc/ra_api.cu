@@ -1223,33 +1223,48 @@ int check_layer_call(ra_ctx* ctx, int layer, const uint16_t* q, const uint16_t* 
     return RA_OK;
 }
 
-// The start of a decode step of the whole stack (ra_decode_step, or ra_decode_layer of layer 0):
-// wait for the evicted sets computed during the previous step, launch the next step's on the
-// side stream, and run every layer's round of the sequences that fire now and have those sets,
-// in one launch.  It needs none of the step's rows: in both layouts each layer's attention then
-// appends its token into the last slot, as after an eviction inside the layer's own call.
-//
-// A sequence that fires without a set computed ahead (the first step of a loaded run, a slot switched on
-// again) has its sets computed here, before the compaction, where that is the shorter way: one plan and one
-// compaction of every layer then replace a launch of the eviction kernel per layer.  The plan, one warp per
-// head, has a length of its own, so the stack must be deep: deeper where the plan takes radix passes
-// (recency, block and exact draws) instead of the sampled cut, and where its keys wait for the candidates'
-// positions (block draws, order-free slots, whose rounds by layer are short as well).  A first step planned
-// here / by layer:
-//   random, ordered       32 heads, 8000 kept: 4 layers 221 / 218 us, 8 layers 378 / 424;
-//                         8 heads, 1024 kept: 4 layers 54 / 83, 24 layers 195 / 477
-//   recency, ordered      32 heads, 8000 kept: 4 layers 286 / 233, 8 layers 443 / 453
-//   random, order-free    128 heads, 1024 kept: 4 layers 145 / 127, 12 layers 323 / 329, 24 layers 590 / 628
-//   block, order-free     64 heads, 2048 kept: 12 layers 379 / 321, 16 layers 452 / 419, 24 layers 604 / 614
-// Nothing runs beside this plan, so it takes as many one-warp CTAs as an SM holds (7 KB each), not the one
-// of a plan beside a step: 24 layers of 32 heads of block draws 1439 us with one, 1039 with 24.
+// Sets computed at the step's start, on the caller's stream: nothing runs beside this plan, so it takes as many
+// one-warp CTAs as an SM holds (7 KB each), not the one of a plan beside a step: 24 layers of 32 heads of block draws
+// 1439 us with one, 1039 with 24.
 constexpr int kPlanNowCtas = 24;
 
-bool plans_in_step(const ra_ctx* ctx)
+// Whether that is shorter for `heads` heads that fire in every layer: one plan and one compaction then replace a launch
+// of the eviction kernel (order-free: the selection) per layer.  The plan, one warp per head, is as long as a head's
+// candidates take it, however few the heads; so is the compaction's chain of a CTA per head and array, where it is
+// not shared.  A round by layer is mostly latency, once per layer.  Both sides in microseconds, fitted to rounds of
+// 2 to 32 heads, 1024 to 24000 kept, r = 64 to 512.  A first step planned here / by layer:
+//   random, ordered     2 heads, r = 64:   4 layers of 1024 kept 40 / 69, of 8000 81 / 78, of 24000 186 / 130;
+//                                          24 layers of 24000 476 / 704
+//                       8 heads, r = 192:  4 layers of 8000 228 / 222, 8 layers 268 / 427
+//                       2 heads, r = 512:  8 layers of 8000 390 / 226, 24 layers 420 / 678
+//   recency, ordered    2 heads, r = 64:   8 layers of 8000 156 / 176, of 24000 439 / 312; 24 layers of 24000 686 / 904
+//   block, ordered      8 heads, r = 64:   24 layers of 1024 140 / 348, of 8000 888 / 834
+//   random, order-free  2 heads, r = 64:   12 layers of 24000 486 / 1016; r = 512: 12 layers of 8000 600 / 473
+bool plans_in_step(const ra_ctx* ctx, int heads)
 {
-    const bool radix = ctx->policy == RA_POLICY_BLOCK || ctx->policy == RA_POLICY_RECENCY ||
-                       (ctx->evict_mode & RA_EVICT_EXACT);
-    return ctx->L >= 4 * (radix ? 2 : 1) * (keys_read_positions(ctx) ? 3 : 1);
+    const bool free = ctx->compaction == RA_COMPACT_HOLEFILL, block = ctx->policy == RA_POLICY_BLOCK;
+    const bool radix = block || ctx->policy == RA_POLICY_RECENCY || (ctx->evict_mode & RA_EVICT_EXACT);
+    const bool reads = keys_read_positions(ctx);
+    if (ctx->L < 4 * (radix ? 2 : 1) * (reads ? 3 : 1)) return false;
+    const double k = ctx->K / 1000.0, r = ctx->r, L = ctx->L;
+    const bool cut = !radix && 2 * ctx->r + 32 <= kEvMaxEvicted;  // (a longer list than that takes the radix passes)
+    const double listed = (2 * r + 32) * (2 * r + 32);            // the cut's pairs, ranked one against another
+    double plan, layer, chain = 8;  // chain: the compaction, beyond the bytes that both ways move
+    if (cut) plan = 10 + (reads ? 19 : 5.2) * k + 0.00046 * listed;
+    else if (ctx->policy == RA_POLICY_RECENCY) plan = 20 + (reads ? 49 : 15.5) * k + 0.08 * r;
+    else plan = 20 + (reads ? 70 : 32) * k + 0.1 * r;
+    if (free) {
+        layer = 6 + (block ? 4.9 : 3.4) * k + 0.02 * r;
+    } else {
+        const double few = 0.55 * std::min(heads, 8), kc = std::min(k, 8.0);  // (kc: the cluster grows up to there)
+        const double longer = (ctx->policy == RA_POLICY_RECENCY ? 1.5 : 0.75) * r / 512;
+        layer = cut ? 9.5 + 0.22 * k + few + 0.0001 * listed
+                    : 10.5 + 0.15 * k + (block ? 0 : few) + kc * (0.75 + longer);
+        const double ctas = 2 * L * heads;
+        const double split = ctx->r > 128 ? 1 : std::min(8.0, std::max(1.0, std::floor(ctx->sms / ctas)));
+        chain += std::max(0.0, (ctx->K + r) / 176 / split - L * heads * 0.15 * k);
+    }
+    return plan + chain < L * layer;
 }
 
 // Sequence b's counters are those of layer 0 in every layer.
@@ -1260,6 +1275,14 @@ bool layers_alike_seq(const ra_ctx* ctx, int b)
     return true;
 }
 
+// The start of a decode step of the whole stack (ra_decode_step, or ra_decode_layer of layer 0):
+// wait for the evicted sets computed during the previous step, launch the next step's on the
+// side stream, and run every layer's round of the sequences that fire now and have those sets,
+// in one launch.  It needs none of the step's rows: in both layouts each layer's attention then
+// appends its token into the last slot, as after an eviction inside the layer's own call.
+//
+// A sequence that fires without a set computed ahead (the first step of a loaded run, a slot switched on
+// again) has its sets computed here, before the compaction, where that is the shorter way (plans_in_step).
 int step_prologue(ra_ctx* ctx, cudaStream_t s)
 {
     cudaError_t e;
@@ -1332,7 +1355,7 @@ int step_prologue(ra_ctx* ctx, cudaStream_t s)
     // survivors move down (ordered) or the evicted slots are refilled from the newest rows
     // (order-free), and the layers then append the token as usual.
     bool planned_now = false;
-    if (now && serve && plans_in_step(ctx) && (ctx->evict_mode & ~RA_EVICT_EXACT) == RA_EVICT_AUTO) {
+    if (now && serve && (ctx->evict_mode & ~RA_EVICT_EXACT) == RA_EVICT_AUTO) {
         EvictParams pp{};
         pp.lay = ctx->lay;
         pp.policy = ctx->policy;
@@ -1356,7 +1379,7 @@ int step_prologue(ra_ctx* ctx, cudaStream_t s)
             pp.trig_n[n] = cand;
             ++n;
         }
-        if (n > 0) {
+        if (n > 0 && plans_in_step(ctx, n * ctx->KVH)) {
             pp.n_trig = n;
             {
                 ProfScope ps(ctx, RA_KERNEL_PLAN, 0.0, s);

@@ -602,7 +602,11 @@ __device__ void finish_cta(const PT& p, CtaMerge& cm)
                 }
 #pragma unroll
                 for (int j = 0; j < kBatch; ++j) nM = fmaxf(nM, m[j]);
-                if (nM == -INFINITY) continue;
+                if (nM == -INFINITY) {  // no logit in these pieces: all rows evicted, which sum to 0, or NaN, which stays
+#pragma unroll
+                    for (int j = 0; j < kBatch; ++j) l += s[j];
+                    continue;
+                }
                 const float sc = exp2f(M - nM);
                 M = nM;
                 l *= sc;

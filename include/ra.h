@@ -329,9 +329,13 @@ int ra_decode_attn(ra_ctx* ctx, int layer, const uint16_t* q, uint16_t* out, flo
  * RA_ERR_CAPACITY as for ra_append_kv.  Layers called in order 0 .. layers-1
  * form a step, as in ra_decode_step: with ordered or order-free compaction and
  * a policy other than the scored one, layer 0's call also runs every layer's
- * round of the sequences that fire, from evicted sets computed during the
- * previous step (same result as each layer evicting in its own call), and
- * layer layers-1's call joins the library's stream back.
+ * round of the sequences that fire (same result as each layer evicting in its
+ * own call), from evicted sets computed during the previous step, or in this call
+ * where that is shorter than selecting layer by layer; layer layers-1's call
+ * joins the library's stream back.  Under the scored policy layer 0's call computes
+ * every layer's scores and sets (ra_get_scores shows them from then on), and each
+ * layer's round still runs in its own call: a window loaded in between
+ * (ra_restore_queries), or a latest query recorded again (ra_decode_attn), counts.
  */
 int ra_decode_layer(ra_ctx* ctx, int layer, const uint16_t* q, const uint16_t* k_new, const uint16_t* v_new,
                     uint16_t* out, float scale, void* stream);
@@ -347,10 +351,14 @@ int ra_decode_layer(ra_ctx* ctx, int layer, const uint16_t* q, const uint16_t* k
  * joined to it at its end, by events: once `stream` completes, so has all the
  * step's work) computes the next step's evicted sets in every layer, and at that step one
  * launch compacts every layer of the sequences that fire (ordered or order-free,
- * in place) before the first layer runs.  The attention of all layers is one launch
- * too, where their counters are alike (unless compaction is inside the attention pass).  Sets computed ahead are used only
- * where the counters they were computed from still hold; elsewhere the layers
- * select as ra_decode_layer does.
+ * in place) before the first layer runs.  A sequence that fires without such a set
+ * (the first step of a loaded run) has its sets computed at the step's start where
+ * that is shorter than selecting layer by layer.  Under the scored policy every
+ * layer's scores and sets are computed there, and compacted by the same launch where
+ * that is shorter than layer by layer.  The attention of all layers is one launch as
+ * well, where their counters are alike (unless compaction is inside the attention
+ * pass).  Sets computed ahead are used only where the counters they were computed from
+ * still hold; what is left selects layer by layer as in the layers' own calls.
  */
 int ra_decode_step(ra_ctx* ctx, const uint16_t* q_all, const uint16_t* k_all, const uint16_t* v_all,
                    uint16_t* out_all, float scale, void* stream);

@@ -510,28 +510,39 @@ bool plan_usable(const ra_ctx* ctx)
     return ctx->compaction == RA_COMPACT_ORDERED && ctx->evict_active[1] > 0;
 }
 
-// The scored policy's rounds of a step's start, every layer in one launch each of scores, selection
-// and in-place compaction (a window holds the queries of earlier steps only, so no layer of this step is
-// needed): with ordered compaction of its own, and more than one layer (one layer's round compacts out
-// of place, over all CTAs).
+// The scored policy's sets of a step's start, every layer's scores in one launch and its selections in another (a
+// window holds the queries of earlier steps only, so no layer of this step is needed): with ordered compaction of its
+// own, and more than one layer.  In ra_decode_step the compaction of every layer follows, in place, where that is
+// shorter.  Between layer calls the caller may still load a layer's window, or record its latest query again
+// (drop_scored_sets): there, each layer's own call compacts from its set.
 bool scored_stack_usable(const ra_ctx* ctx)
 {
     return ctx->policy == RA_POLICY_SNAPKV && ctx->compaction == RA_COMPACT_ORDERED && ctx->L > 1 && ctx->L <= 65535 &&
-           ctx->r <= kEvMaxEvicted && (ctx->evict_mode & ~RA_EVICT_EXACT) != RA_EVICT_TWO_KERNELS;
+           ctx->r <= kEvMaxEvicted && (ctx->evict_mode & ~RA_EVICT_EXACT) != RA_EVICT_TWO_KERNELS &&
+           ctx->evict_active[1] > 0;
 }
 
-// Whether `heads` heads that fire in every layer are shorter that way.  The in-place compaction of a buffer of more than
-// 128 rows is a chain of one CTA per head and array, 45 KB/us, where the one by layer runs over all CTAs: it then
-// takes enough layers, whose scores and selections run beside each other.  Microseconds, from a step with one round at
-// the start / by layer: r = 130, 2 heads of 1024 kept, 2 layers 54 / 62; of 4096, 2 layers 89 / 78, 3 layers 90 / 105;
-// of 15000, 4 layers 232 / 223, 6 layers 242 / 343; 8 heads of 15000, 2 layers 254 / 206, 3 layers 279 / 300; r = 512,
-// 8 heads of 1024, 2 layers 93 / 75, 3 layers 94 / 104; of 8000, 3 layers 244 / 242, 4 layers 270 / 317.
+void drop_scored_sets(ra_ctx* ctx, int layer)
+{
+    if (ctx->policy != RA_POLICY_SNAPKV) return;  // (sets of the other policies do not depend on a window)
+    for (int half = 0; half < 2; ++half) {
+        const auto first = ctx->plan_g.begin() + ((size_t)half * ctx->L + layer) * ctx->B;
+        std::fill(first, first + ctx->B, -1);
+    }
+}
+
+// Whether the in-place compaction of every layer is shorter than one of each layer's own, for `heads` heads that fire
+// in every layer.  With a buffer of more than 128 rows it is a chain of one CTA per head and array, 45 KB/us, where a
+// layer's own runs over all CTAs and takes 5 us and more: it then takes enough layers.  A step with one round,
+// microseconds, stacked / each layer's own: r = 130, 2 heads of 1024 kept, 4 layers 53 / 50, 6 layers 54 / 61; of 4096,
+// 6 layers 97 / 80; 8 heads of 8000, 4 layers 184 / 165, 6 layers 216 / 222; of 15000, 6 layers 367 / 358; r = 512, 8
+// heads of 1024, 6 layers 108 / 89; of 15000, 6 layers 510 / 470.  With r = 64: 8 heads of 8000, 2 layers 95 / 100,
+// 3 layers 133 / 130, 6 layers 206 / 216.
 bool scored_stack_shorter(const ra_ctx* ctx, int heads)
 {
     if (ctx->r <= 128) return true;
-    const double cost = 25 + 0.0125 * ctx->K + 0.06 * (ctx->r - 128);     // of the stack, beyond a layer's round
-    const double gain = 20 + (heads <= 4 ? 0.0018 : 0.0035) * ctx->K;     // of each layer
-    return ctx->L * gain >= cost;
+    const double k = ctx->K / 1000.0, longer = (ctx->r - 128) / 128.0;
+    return ctx->L >= (heads <= 4 ? std::min(4 + 1.3 * k, 14.0) + 1.8 * longer : 5 + k / 8 + longer);
 }
 
 // One eviction round of the triggered sequences in p: [score passes,] select, compact (unless
@@ -558,7 +569,7 @@ int run_eviction_launches(ra_ctx* ctx, EvictParams& p, double moved, cudaStream_
     cudaError_t e;
     p.layers = 1;
     p.to_plan = 0;
-    if (p.policy == RA_POLICY_SNAPKV) {  // window scores with the normalisers recorded at decode time
+    if (p.policy == RA_POLICY_SNAPKV && !p.ev_plan) {  // window scores with the normalisers recorded at decode time
         for (int i = 0; i < p.n_trig; ++i) ctx->score_n[(size_t)p.layer * ctx->B + p.trig[i]] = p.trig_n[i];
         const double bytes = plan_scoring(ctx, &p, 2);
         ProfScope ps(ctx, RA_KERNEL_SCORE_SUM, bytes, s);
@@ -599,7 +610,7 @@ int run_eviction_launches(ra_ctx* ctx, EvictParams& p, double moved, cudaStream_
         }
         if (forced >= 2) break;  // the forced size (or the next one the device can schedule)
     }
-    const bool one_launch = !p.holefill && !compact_in_attention && p.policy != RA_POLICY_SNAPKV &&
+    const bool one_launch = !p.holefill && !compact_in_attention && (p.policy != RA_POLICY_SNAPKV || p.ev_plan) &&
                             forced != RA_EVICT_TWO_KERNELS && cl > 0 && ctx->r <= kEvMaxEvicted;
     if (one_launch) {
         p.ev_reps = reps;
@@ -1056,6 +1067,7 @@ int ra_restore_queries(ra_ctx* ctx, int layer, const uint16_t* q, float scale, v
     cudaError_t e = launch_restore_queries(ctx->lay, layer, q, ctx->g.data() + base, s);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "query window restore launch");
     ctx->no_early_once = true;  // a scoring pass behind these launches reads what they write
+    drop_scored_sets(ctx, layer);
     // The normalisers of the loaded queries: each over the prompt and the cached rows at
     // positions up to its own (what it attended to at its step, as no eviction can come between).
     EvictParams p{};
@@ -1196,7 +1208,10 @@ int ra_decode_attn(ra_ctx* ctx, int layer, const uint16_t* q, uint16_t* out, flo
     cudaError_t e = launch_attention(shape, p, &ctx->tmap_k[shape], &ctx->tmap_v[shape], ctas, s);
     ps.done();
     if (e != cudaSuccess) return cuda_fail(ctx, e, "attention launch");
-    if (p.qring) ctx->no_early_once = true;  // it records the layer's window: a scoring pass behind it waits
+    if (p.qring) {  // it records the layer's window: a scoring pass behind it waits
+        ctx->no_early_once = true;
+        drop_scored_sets(ctx, layer);
+    }
     return RA_OK;
 }
 
@@ -1283,7 +1298,8 @@ bool layers_alike_seq(const ra_ctx* ctx, int b)
 //
 // A sequence that fires without a set computed ahead (the first step of a loaded run, a slot switched on
 // again) has its sets computed here, before the compaction, where that is the shorter way (plans_in_step).
-int step_prologue(ra_ctx* ctx, cudaStream_t s)
+// `stacked`: every layer's part of the step follows in the same call.
+int step_prologue(ra_ctx* ctx, cudaStream_t s, bool stacked)
 {
     cudaError_t e;
     const bool serve = plan_usable(ctx);
@@ -1425,7 +1441,8 @@ int step_prologue(ra_ctx* ctx, cudaStream_t s)
             // rows moved per head: the survivors below the token (ordered), the m refills (order-free)
             moved += (double)(fill ? c + 1 - ctx->r - ctx->K : ctx->K + ctx->r - 1) * ctx->KVH * ctx->L;
         }
-        if (n > 0 && (!scored || scored_stack_shorter(ctx, n * ctx->KVH))) {
+        const bool sets_only = scored && !(stacked && scored_stack_shorter(ctx, n * ctx->KVH));
+        if (n > 0) {
             sp.n_trig = n;
             if (scored) {
                 sp.policy = ctx->policy;
@@ -1447,13 +1464,20 @@ int step_prologue(ra_ctx* ctx, cudaStream_t s)
                 }
                 if (e != cudaSuccess) return cuda_fail(ctx, e, "select launch");
             }
-            {
+            if (sets_only) {
+                for (int i = 0; i < n; ++i)
+                    for (int l = 0; l < ctx->L; ++l) {
+                        const size_t k = (size_t)cur * ctx->L * ctx->B + (size_t)l * ctx->B + sp.trig[i];
+                        ctx->plan_g[k] = sp.trig_g[i];
+                        ctx->plan_n[k] = sp.trig_n[i];
+                    }
+            } else {
                 ProfScope ps(ctx, RA_KERNEL_STACK, moved * 2.0 * (2 * kRowBytes + 4), s);
                 e = fill ? launch_fill_stack(sp, ctx->L, s) : launch_compact_stack(sp, ctx->L, ctx->sms, s);
                 ps.done();
             }
             if (e != cudaSuccess) return cuda_fail(ctx, e, "whole-stack compaction launch");
-            for (int i = 0; i < n; ++i)
+            for (int i = 0; i < n && !sets_only; ++i)
                 for (int l = 0; l < ctx->L; ++l) {
                     const size_t k = (size_t)l * ctx->B + sp.trig[i];
                     ctx->c[k] = ctx->K + ctx->r - 1;  // rows left before the step's token is written (last)
@@ -1497,7 +1521,7 @@ int ra_decode_layer(ra_ctx* ctx, int layer, const uint16_t* q, const uint16_t* k
     cudaStream_t s = (cudaStream_t)stream;
     if (layer == 0) {
         if (ctx->step_open && (rc = step_epilogue(ctx, s)) != RA_OK) return rc;
-        if ((rc = step_prologue(ctx, s)) != RA_OK) return rc;
+        if ((rc = step_prologue(ctx, s, false)) != RA_OK) return rc;
     }
     rc = decode_layer_impl(ctx, layer, q, k_new, v_new, out, scale, stream, ctx->step_open ? ctx->step_cur : -1);
     if (layer == ctx->L - 1 && ctx->step_open) {
@@ -1539,7 +1563,6 @@ int evict_pending(ra_ctx* ctx, int layer, cudaStream_t s, int plan_parity, std::
     // predecessor computes, and with one layer the predecessor is this layer's previous step.
     // Neither starts early right after rows were loaded: the predecessor may have written this layer.
     const bool clean = ctx->L >= 2 && !ctx->no_early_once && !ctx->appended && ctx->last_layer != layer;
-    ep.early = (ctx->policy != RA_POLICY_SNAPKV && clean) ? 1 : 0;
     const int score_early = clean ? 1 : 0;  // the scoring pass reads only older kernels' output
     ep.pending = 1;  // the step's token is appended by the attention launch below
     int n = 0;
@@ -1557,7 +1580,7 @@ int evict_pending(ra_ctx* ctx, int layer, cudaStream_t s, int plan_parity, std::
         }
     }
     *n_fired = n;
-    if (n > 0 && plan_parity >= 0 && !ep.holefill && !fuse_compaction && plan_usable(ctx)) {
+    if (n > 0 && plan_parity >= 0 && !ep.holefill && !fuse_compaction && (plan_usable(ctx) || scored_stack_usable(ctx))) {
         bool all = true;  // every triggered sequence's evicted sets were computed ahead for this round
         for (int i = 0; i < n && all; ++i) {
             const size_t k = (size_t)plan_parity * ctx->L * ctx->B + (size_t)layer * ctx->B + ep.trig[i];
@@ -1568,6 +1591,7 @@ int evict_pending(ra_ctx* ctx, int layer, cudaStream_t s, int plan_parity, std::
             ep.ev_plan_parity = plan_parity;
         }
     }
+    ep.early = clean && (ctx->policy != RA_POLICY_SNAPKV || ep.ev_plan) ? 1 : 0;
     if (n > 0) {
         ep.n_trig = n;
         if ((rc = run_eviction(ctx, ep, moved, s, fuse_compaction, score_early)) != RA_OK) return rc;
@@ -1689,7 +1713,7 @@ int ra_decode_step(ra_ctx* ctx, const uint16_t* q_all, const uint16_t* k_all, co
     const size_t qs = (size_t)ctx->B * ctx->H * kHeadDim, ks = (size_t)ctx->B * ctx->KVH * kHeadDim;
     cudaStream_t s = (cudaStream_t)stream;
     if (ctx->step_open && (rc = step_epilogue(ctx, s)) != RA_OK) return rc;  // a per-layer step left open
-    if ((rc = step_prologue(ctx, s)) != RA_OK) return rc;
+    if ((rc = step_prologue(ctx, s, true)) != RA_OK) return rc;
     // All the step's inputs are here, so the layers' attention runs as one launch: first the rounds
     // left to the layers (sequences that fire with no set computed ahead; they need cached rows
     // only), then every layer at once.  With compaction inside the attention pass, or with
@@ -1972,6 +1996,9 @@ extern "C" int ra_decode_attn_noalloc(ra_ctx* ctx, int layer, const uint16_t* q,
     if (e != cudaSuccess) return cuda_fail(ctx, e, "scratch counter clear");
     e = launch_attention(shape, p, &ctx->tmap_k[shape], &ctx->tmap_v[shape], ctas, s);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "attention launch");
-    if (p.qring) ctx->no_early_once = true;  // (as in ra_decode_attn)
+    if (p.qring) {  // (as in ra_decode_attn)
+        ctx->no_early_once = true;
+        drop_scored_sets(ctx, layer);
+    }
     return RA_OK;
 }

@@ -1,6 +1,7 @@
 """Rounds at a step's start go for all layers at once only where that is the shorter way: on both sides of the rules'
-lines the launches are the expected ones, and the caches bit for bit the oracle's.  Scored rounds with a buffer that the
-in-place compaction does not share between CTAs, and sets planned in the step whose plan takes the radix passes."""
+lines the launches are the expected ones, and the caches bit for bit the oracle's.  Scored rounds, whose in-place
+compaction does not share a buffer of more than 128 rows between CTAs, and which between layer calls only select ahead;
+sets planned in the step whose plan takes the radix passes."""
 import numpy as np
 import pytest
 
@@ -9,11 +10,32 @@ from ra_testlib import Runner
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("L,stacked", [(2, False), (3, True)], ids=["by-layer", "stacked"])
-def test_scored_rounds_of_a_long_buffer(L, stacked):
+def _step(run):
+    """One ra_decode_step of a scored run of one sequence; the oracle's rounds take the kernel's scores."""
     import paper_2609_03430_gb300 as ra
 
-    K, r = 4096, 130
+    L, t = run.L, run.step_idx
+    run.qsteps[0].append(t)
+    run.step_scale.append(0.0)
+    pos = [run.orc.append(0, l) for l in range(L)]
+    q = np.stack([run.qrows(l, 0, t)[None] for l in range(L)])
+    k, v = (np.stack([np.stack([f(l, 0, h, [pos[l]])[0] for h in range(run.KVH)])[None] for l in range(L)])
+            for f in (run.krows, run.vrows))
+    tq, tk, tv = run.up(q), run.up(k), run.up(v)
+    out = run.torch.zeros(q.shape, dtype=run.torch.int16, device="cuda")
+    ra.ra_decode_step(run.ctx, tq.data_ptr(), tk.data_ptr(), tv.data_ptr(), out.data_ptr())
+    for l in range(L):
+        run.orc.evict(0, l, scorer=run.scorer)
+        run.check_layer_attention(l, q[l], out[l].cpu().numpy())
+    run.step_idx += 1
+
+
+# launches of (select, evict, the stack's compaction): every layer's selection is one launch in all three
+@pytest.mark.parametrize("form,L,launches", [("step", 4, (1, 4, 0)), ("step", 6, (1, 0, 1)), ("layers", 6, (1, 6, 0))])
+def test_scored_rounds_of_a_long_buffer(form, L, launches):
+    import paper_2609_03430_gb300 as ra
+
+    K, r = 1024, 130
     run = Runner(L, 2, 2, [65], K, r, eseed=1, dseed=71, fused=True, policy=4)
     g = -(-4 * (K + 2 * r) // r) * r - 1  # the next step fires
     run.restore_full(g, layers=range(L))
@@ -23,11 +45,15 @@ def test_scored_rounds_of_a_long_buffer(L, stacked):
         w = run.up(np.stack([run.qrows(l, 0, s) for s in range(g - r, g)], axis=1)[None])
         ra.ra_restore_queries(run.ctx, l, w.data_ptr())
     ra.ra_profile_reset(run.ctx)
-    run.step(check_attn_layers=(0, L - 1))
-    select, stack = (ra.ra_profile_read(run.ctx, k)[1] for k in (ra.RA_KERNEL_SELECT, ra.RA_KERNEL_STACK))
-    assert (select, stack) == ((1, 1) if stacked else (L, 0))
-    run.step(check_attn_layers=(0, L - 1))
-    run.check_state()
+    for t in range(2):
+        if form == "step":
+            _step(run)
+        else:
+            run.step(check_attn_layers=range(L))
+        run.check_state()
+    kinds = (ra.RA_KERNEL_SELECT, ra.RA_KERNEL_EVICT, ra.RA_KERNEL_STACK)
+    assert tuple(ra.ra_profile_read(run.ctx, k)[1] for k in kinds) == launches
+    assert run.scored_rounds == 2 * L
     run.close()
 
 

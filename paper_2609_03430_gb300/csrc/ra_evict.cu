@@ -1355,8 +1355,8 @@ __global__ void __launch_bounds__(32) timeout_probe_kernel(int32_t* err, uint64_
 // ----------------------------------------------------------------------------- prefill / restore
 // Rows into a cache: one CTA per chunk of kCopyRows rows of a (layer, sequence, KV head), K and V,
 // every 16-byte piece of the chunk in flight before the first store.  Bound by HBM: a chunk is 32 KB
-// read and written, and up to eight CTAs per SM keep 256 KB on the way, so that a single request (a
-// few heads of many layers, in one launch) fills the chip as a whole batch does.  A chunk of
+// read and written, and five CTAs per SM (48 registers a thread) keep 160 KB on the way, so that a single request
+// (a few heads of many layers, in one launch) fills the chip as a whole batch does.  A chunk of
 // prompt rows lies inside one page.  With one CTA per head, a row per warp on the way, and a launch
 // per layer of a request, loading 8 prompts of 512-4096 tokens into 8 layers (1.2 GB moved, attention
 // of the last token included) took 2300 us and admitting one of 300-2048 tokens into 36 layers (0.9 GB

@@ -279,20 +279,31 @@ class ClockSampler:
                 "reasons": reasons, "samples": len(inside)}
 
 
-def profiled_traffic(cfg, layers):
-    """DRAM bytes per attention launch of `layers` layers from the committed ncu record (bytes per
-    layer of a stacked launch), if it was taken on the current kernel sources for this workload's
-    layer shape; else None."""
+# what decides which attention kernel a stacked step launches, and what it reads and writes
+TRAFFIC_SOURCES = ("ra_attn.cu", "ra_attn_tile.cuh", "ra_internal.h", "ra_api.cu")
+
+
+def traffic_digest():
     import hashlib
 
+    digest = hashlib.sha256()
+    for name in TRAFFIC_SOURCES:
+        with open(os.path.join(ROOT, "paper_2609_03430_gb300", "csrc", name), "rb") as f:
+            digest.update(f.read())
+    return digest.hexdigest()
+
+
+def profiled_traffic(cfg, layers, calls):
+    """DRAM bytes per attention launch of `layers` layers from the committed ncu record: bytes per layer of a
+    stacked launch of the form that the workload's full stack takes (kernel shape, claimed tail).  None for
+    layer calls, whose launches are other kernels, and where the sources of the kernel or of the rules
+    that choose it have changed since."""
+    if calls != "step":
+        return None
     try:
         with open(os.path.join(ROOT, "profiles", "attn_kernel_traffic.json")) as f:
             rec = json.load(f)
-        digest = hashlib.sha256()
-        for name in ("ra_attn.cu", "ra_attn_tile.cuh"):
-            with open(os.path.join(ROOT, "paper_2609_03430_gb300", "csrc", name), "rb") as f:
-                digest.update(f.read())
-        if rec.get("kernel_source_sha256") != digest.hexdigest():
+        if rec.get("sources_sha256") != traffic_digest():
             return None
         per_layer = rec.get("traffic_bytes_per_layer", {}).get(str(cfg))
         return None if per_layer is None else per_layer * layers
@@ -815,7 +826,8 @@ def run_ours(args, w):
 
     peaks, peak_src = measured_peaks()
     roof = attention_roofline(kern.get("attn"), clean, args.steps, w["L"], peaks, peak_src,
-                              args.traffic if args.traffic is not None else profiled_traffic(args.config, w["L"] if args.calls == "step" else 1))
+                              args.traffic if args.traffic is not None
+                              else profiled_traffic(args.config, w["L"], args.calls))
     comparator = None
     if main_policy == 0 and (args.comparator == "on" or
                              (args.comparator == "auto" and args.config in COMPARATOR_CONFIGS)):

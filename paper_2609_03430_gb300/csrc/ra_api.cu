@@ -282,8 +282,8 @@ void plan_tail(const ra_ctx* ctx, AttnParams* p)
 // mirror, in tiles: a head has ceil(lp / TILE) prompt tiles and ceil(gen / TILE) tiles of generated
 // rows, where gen is the cached generated rows plus one for a fused new token; the tiles are cut
 // into one equal chunk per warp.  *slots = rows attended.
-int plan_attention(ra_ctx* ctx, int layer, int layers, int fused, AttnParams* p, int* n_active, int* ctas, double* slots,
-                   int* shape, const int32_t* old_rows = nullptr)
+int plan_attention(ra_ctx* ctx, int layer, int layers, int fused, AttnParams* p, int* n_active, int* ctas,
+                   double* slots, int* shape, const int32_t* old_rows = nullptr)
 {
     p->lay = ctx->lay;
     p->layer = layer;
@@ -340,7 +340,8 @@ int plan_attention(ra_ctx* ctx, int layer, int layers, int fused, AttnParams* p,
     // A layer of few heads takes a cluster per head: see cluster_size.
     p->cluster = 0;
     p->cluster_heads = 0;
-    if (layers == 1 && !old_rows && ctx->attn_shape == RA_ATTN_SHAPE_AUTO && *shape == kAttnNarrow && ctx->B <= kSmallBatch && acc > 0) {
+    if (layers == 1 && !old_rows && ctx->attn_shape == RA_ATTN_SHAPE_AUTO && *shape == kAttnNarrow &&
+        ctx->B <= kSmallBatch && acc > 0) {
         int holding = 0, longest = 0;
         for (int b = 0; b < ctx->B; ++b) {
             const int t = (p->seq_base[b + 1] - p->seq_base[b]) / ctx->KVH;
@@ -362,7 +363,10 @@ int plan_attention(ra_ctx* ctx, int layer, int layers, int fused, AttnParams* p,
 // the cluster kernel saves 2 to 4 us a layer, about as long as a warp takes for two tiles, but heads
 // that do not divide the SMs (or are uneven) give its warps more tiles than W.  Measured, with 8 KV heads
 // and G = 4 (tiles per warp here / with the split): 1/1 5.7 against 8.3 us, 4/3 12.4 and 14.8, 7/6
-// 19.6 and 21.4, 13/11 30.8 and 31.9, 17/16 42.0 and 41.7, 14/12 34.7 and 33.3, 14/9 30.4 and 27.1.
+// 19.6 and 21.4, 13/11 30.8 and 31.9, 17/16 42.0 and 41.7, 14/12 34.7 and 33.3, 14/9 30.4 and 27.1.  The other
+// group sizes leave the line where it is: of 230 shapes (G = 1, 2, 4, 5, 8; 2 to 24 heads of 300 to 30000 rows) none is
+// more than 2% longer than with the split; 8 heads of 2700 rows take 4.9 against 7.0 us with G = 1 and 6.3 against 10.0
+// with G = 8, 24 heads of 12000 rows 27.4 against 29.2 and 28.4 against 32.1.
 int cluster_size(const ra_ctx* ctx, int heads, int longest, int W)
 {
     int cl = std::min(16, ctx->sms / heads);
@@ -450,8 +454,8 @@ void layout_scoring(ra_ctx* ctx)
 
 // Launch shape of a scoring pass over the heads of the sequences in p (pass 1: prompt + the
 // trig_n cached rows each; pass 2: the trig_n candidate rows each, in p->layers layers): CTAs (two per
-// SM with a window of at most 256 rows, else one) take runs of consecutive tiles of one head, in whole 128-row tiles
-// (two scoring tiles), of the length whose waves, each as long as the run and about three tiles'
+// SM with a window of at most 256 rows, else one) take runs of consecutive tiles of one head, in whole
+// 128-row tiles (two scoring tiles), of the length whose waves, each as long as the run and about three tiles'
 // start-up, end first.  Returns the algorithmic bytes: the key rows read (every one is contracted
 // with the M = r * G window rows, so flops = bytes * M).
 double plan_scoring(ra_ctx* ctx, EvictParams* p, int pass)
@@ -471,7 +475,10 @@ double plan_scoring(ra_ctx* ctx, EvictParams* p, int pass)
     const int whole = (most + 1) / 2 * 2, slots = ctx->sms * (score_window_tiles(ctx->r * ctx->G) <= 2 ? 2 : 1);
     int run = whole;
     long long best = 0;
-    for (int ch = (least + 1) / 2 * 2; ch <= whole; ch += 2) {
+    // (every length of up to 64 tiles, then about 16 to each doubling, and the whole head)
+    for (int ch = (least + 1) / 2 * 2, next; ch <= whole; ch = next) {
+        next = ch + std::max(2, ch / 32 * 2);
+        if (ch < whole) next = std::min(next, whole);
         long long ctas = 0;
         for (int t : tiles) ctas += (long long)layers * ctx->KVH * ((t + ch - 1) / ch);
         const long long cost = (ctas + slots - 1) / slots * (ch / 2 + 3);
@@ -811,7 +818,8 @@ int ra_bind(ra_ctx* ctx, void* device_arena, size_t bytes, void* stream)
         if ((rc = make_tmap(ctx, &ctx->tmap_v[sh], Ly.vpool, ctx->total_rows, tile)) != RA_OK) return rc;
         if ((e = attn_prepare(sh, ctx->G)) != cudaSuccess) return cuda_fail(ctx, e, "attention kernel attributes");
     }
-    if ((e = attn_cluster_prepare(ctx->G, ctx->attn_active)) != cudaSuccess) return cuda_fail(ctx, e, "attention kernel attributes");
+    if ((e = attn_cluster_prepare(ctx->G, ctx->attn_active)) != cudaSuccess)
+        return cuda_fail(ctx, e, "attention kernel attributes");
     if ((e = evict_prepare(ctx->evict_active)) != cudaSuccess) return cuda_fail(ctx, e, "eviction kernel attributes");
     if (ctx->scoring) {
         if ((rc = make_tmap(ctx, &ctx->tmap_ks, Ly.kpool, ctx->total_rows, kScoreTile)) != RA_OK) return rc;
@@ -1308,8 +1316,8 @@ int step_prologue(ra_ctx* ctx, cudaStream_t s, bool stacked)
         ctx->plan_pending = false;
     }
     const int cur = ctx->parity, nxt = 1 - cur;
-    std::fill(ctx->plan_g.begin() + (size_t)nxt * ctx->L * ctx->B, ctx->plan_g.begin() + (size_t)(nxt + 1) * ctx->L * ctx->B,
-              -1);
+    const auto half = ctx->plan_g.begin() + (size_t)nxt * ctx->L * ctx->B;
+    std::fill(half, half + (size_t)ctx->L * ctx->B, -1);
     const bool scored = scored_stack_usable(ctx);
     bool now = false, next = false;  // a sequence may fire at this step, at the next one (layer 0's counters)
     for (int b = 0; b < ctx->B && (serve || scored); ++b) {
@@ -1367,9 +1375,10 @@ int step_prologue(ra_ctx* ctx, cudaStream_t s, bool stacked)
         }
     }
     // The sequences that fire at this step in every layer alike, with every layer's evicted set
-    // computed ahead, or from scores computed now: all their rounds in one launch, in place, before the first layer: the
-    // survivors move down (ordered) or the evicted slots are refilled from the newest rows
-    // (order-free), and the layers then append the token as usual.
+    // computed ahead, or from scores computed now: all their rounds in one launch, in place, before the
+    // first layer (or, between layer calls under the scored policy, their sets only): the survivors move
+    // down (ordered) or the evicted slots are refilled from the newest rows (order-free), and the layers
+    // then append the token as usual.
     bool planned_now = false;
     if (now && serve && (ctx->evict_mode & ~RA_EVICT_EXACT) == RA_EVICT_AUTO) {
         EvictParams pp{};
@@ -1539,7 +1548,8 @@ namespace {
 // candidate, and evicting before writing it gives the same state as append-then-evict.  With
 // compaction in the attention pass only the selection runs here: that pass reads the old region
 // anyway and writes the survivors to the new one as it goes; old_rows (empty before) then receives
-// the rows of the sequences it compacts, -1 for the others, and *compacted the rows it writes.  *n_fired: sequences that evict.
+// the rows of the sequences it compacts, -1 for the others, and *compacted the rows it writes.  *n_fired: sequences
+// that evict.
 int evict_pending(ra_ctx* ctx, int layer, cudaStream_t s, int plan_parity, std::vector<int32_t>& old_rows,
                   double* compacted, int* n_fired)
 {
@@ -1547,7 +1557,8 @@ int evict_pending(ra_ctx* ctx, int layer, cudaStream_t s, int plan_parity, std::
     const size_t base = (size_t)layer * ctx->B;
     *n_fired = 0;
     bool any = false;
-    for (int b = 0; b < ctx->B && !any; ++b) any = ctx->active[b] && fires(ctx, ctx->g[base + b] + 1, ctx->c[base + b] + 1);
+    for (int b = 0; b < ctx->B && !any; ++b)
+        any = ctx->active[b] && fires(ctx, ctx->g[base + b] + 1, ctx->c[base + b] + 1);
     if (!any) return RA_OK;
     // The attention pass compacts (time order kept) when each tile's evicted rows fit its 64-bit mask.
     const bool fuse_compaction = ctx->compaction == RA_COMPACT_FUSED && ctx->r <= 64;  // tiles have <= 64 rows
@@ -1580,7 +1591,8 @@ int evict_pending(ra_ctx* ctx, int layer, cudaStream_t s, int plan_parity, std::
         }
     }
     *n_fired = n;
-    if (n > 0 && plan_parity >= 0 && !ep.holefill && !fuse_compaction && (plan_usable(ctx) || scored_stack_usable(ctx))) {
+    const bool sets = plan_parity >= 0 && (plan_usable(ctx) || scored_stack_usable(ctx));
+    if (n > 0 && sets && !ep.holefill && !fuse_compaction) {
         bool all = true;  // every triggered sequence's evicted sets were computed ahead for this round
         for (int i = 0; i < n && all; ++i) {
             const size_t k = (size_t)plan_parity * ctx->L * ctx->B + (size_t)layer * ctx->B + ep.trig[i];
@@ -1638,8 +1650,8 @@ int attend_pending(ra_ctx* ctx, int layer, int layers, const uint16_t* q, const 
     // The kernel may request its first K/V tiles before its predecessor finishes when that
     // predecessor cannot be writing this layer's cache or tables: no eviction of this layer at
     // this step (else it is this layer's compaction) and another layer before (else it is this
-    // layer's previous step), or but for each head's newest cached row.  Kernels let successors start only after their own wait, so
-    // everything older than the predecessor has completed.
+    // layer's previous step), or but for each head's newest cached row.  Kernels let successors start only
+    // after their own wait, so everything older than the predecessor has completed.
     // Behind this layer's previous step (one layer in all, or a layer called twice in a row) or a call that
     // appended on its own, the newest cached rows are the ones that the predecessor may be writing.
     const bool again = ctx->last_layer == layer;
@@ -1722,7 +1734,8 @@ int ra_decode_step(ra_ctx* ctx, const uint16_t* q_all, const uint16_t* k_all, co
         std::vector<int32_t> old_rows;  // (stays empty)
         double compacted = 0;
         int n = 0;
-        for (int l = 0; l < ctx->L && rc == RA_OK; ++l) rc = evict_pending(ctx, l, s, ctx->step_cur, old_rows, &compacted, &n);
+        for (int l = 0; l < ctx->L && rc == RA_OK; ++l)
+            rc = evict_pending(ctx, l, s, ctx->step_cur, old_rows, &compacted, &n);
         if (rc == RA_OK)
             rc = attend_pending(ctx, 0, ctx->L, q_all, k_all, v_all, out_all, scale, s, true, old_rows, 0.0);
         const int rc_end = step_epilogue(ctx, s);
@@ -1979,7 +1992,8 @@ extern "C" int ra_decode_attn_noalloc(ra_ctx* ctx, int layer, const uint16_t* q,
     p.qk_scale_log2 = scale_log2(scale);
     // [arrival counters, one int per chunk][partial records, two per chunk].  The limit that the
     // interface states counts a record per warp and per head.
-    const size_t counters = align_up((size_t)p.nchunks * sizeof(int32_t), kAlign), record = partial_stride(ctx->G) * sizeof(float);
+    const size_t counters = align_up((size_t)p.nchunks * sizeof(int32_t), kAlign);
+    const size_t record = partial_stride(ctx->G) * sizeof(float);
     const size_t heads = (size_t)ctx->B * ctx->KVH;
     const size_t need = std::max(align_up(heads * sizeof(int32_t), kAlign) + (p.nchunks + heads) * record,
                                  counters + 2 * (size_t)p.nchunks * record);

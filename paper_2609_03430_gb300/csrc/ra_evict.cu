@@ -12,7 +12,8 @@
 //                   Under the scored comparator the score is the max-pooled
 //                   window attention that ra_score.cu computed (at a step's
 //                   start for every layer in one launch, into the sets that
-//                   compact_stack_kernel takes); with order-free
+//                   compact_stack_kernel takes, or evict_kernel layer by
+//                   layer); with order-free
 //                   slots every key follows the candidate's position.
 //                   With order-free slots the select CTA also refills the
 //                   evicted slots in place from the newest ones (no compact).

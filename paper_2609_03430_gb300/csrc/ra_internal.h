@@ -70,7 +70,7 @@ struct EvictParams {
     DevLayout lay;
     int layer;
     int layers;    // score (pass 2) and select: layers of the launch from `layer` on, counters alike
-    int to_plan;   // select: the evicted sets go to half ev_plan_parity of lay.evplan, for launch_compact_stack
+    int to_plan;   // select: the evicted sets go to half ev_plan_parity of lay.evplan, for a launch of its own
     int policy;    // RA_POLICY_*: how candidates are scored
     int block;     // RA_POLICY_BLOCK: positions per block
     int holefill;  // RA_COMPACT_HOLEFILL: keys per position, evicted slots refilled in place by select
@@ -97,8 +97,9 @@ struct EvictParams {
     // all of them) and whether to skip the sampled cut (exact radix passes only)
     int ev_reps;
     int ev_exact;
-    // evicted sets computed ahead by plan_kernel ([2][L][B][KVH][r + 1]: count, then the ordinals
-    // ascending) and which half this launch reads; null: the kernel selects itself
+    // evicted sets computed ahead by plan_kernel, or under the scored policy by select_kernel
+    // ([2][L][B][KVH][r + 1]: count, then the ordinals ascending), and which half this launch reads;
+    // null: the kernel selects itself
     const int32_t* ev_plan;
     int ev_plan_parity;
     int stk_split;  // launch_compact_stack: CTAs per head and array
